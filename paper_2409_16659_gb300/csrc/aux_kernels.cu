@@ -396,14 +396,15 @@ __global__ void friction_eval_kernel(KParams P, long ncell, const float* __restr
                                      float* __restrict__ Rx, float* __restrict__ Ry) {
   for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell;
        c += (long)gridDim.x * blockDim.x) {
-    float hh[N], jx[N], jy[N], rx[N], ry[N];
+    float hh[N], ih[N], jx[N], jy[N], rx[N], ry[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       hh[i] = h[(long)i * ncell + c];
-      jx[i] = Jx[(long)i * ncell + c];
-      jy[i] = Jy ? Jy[(long)i * ncell + c] : 0.f;
+      ih[i] = rcp(hh[i]);
+      jx[i] = Jx[(long)i * ncell + c] * ih[i];  // mean velocities
+      jy[i] = Jy ? Jy[(long)i * ncell + c] * ih[i] : 0.f;
     }
-    friction<N>(P, hh, jx, jy, rx, ry);
+    friction<N, true>(P, hh, ih, jx, jy, rx, ry);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       Rx[(long)i * ncell + c] = rx[i];

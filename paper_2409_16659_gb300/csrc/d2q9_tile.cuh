@@ -9,196 +9,10 @@
 
 #include "kernels.h"
 #include "physics.cuh"
+#include "step_common.cuh"
 #include "tma.cuh"
 
 namespace mlsw {
-
-// ---------------------------------------------------------------------------
-// Bounds checks of the debug build (physics.cuh): a shared-memory pointer
-// must lie in the CTA's dynamic shared memory, an index in its array, a
-// global store in its buffer or plane. Out of range, the access is counted
-// and goes to the first element instead. Release builds pass through.
-// ---------------------------------------------------------------------------
-#ifdef MLSW_DEBUG
-extern __shared__ __align__(128) unsigned char dyn_smem_base[];
-__device__ __forceinline__ bool dyn_smem_ok(const void* p, int bytes) {
-  if (!__isShared(p)) return false;
-  uint32_t size;
-  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(size));
-  const uint32_t a = smem_addr(p), lo = smem_addr(dyn_smem_base);
-  return a >= lo && a + (uint32_t)bytes <= lo + size;
-}
-#endif
-template <class P>
-__device__ __forceinline__ P* chk_smem(P* p) {
-#ifdef MLSW_DEBUG
-  if (!dyn_smem_ok(p, (int)sizeof(P))) {
-    note_bounds_violation();
-    return reinterpret_cast<P*>(dyn_smem_base);
-  }
-#endif
-  return p;
-}
-__device__ __forceinline__ int chk_index(int i, int n) {
-#ifdef MLSW_DEBUG
-  if (i < 0 || i >= n) {
-    note_bounds_violation();
-    return 0;
-  }
-#endif
-  return i;
-}
-// offset of a global store inside its buffer or plane: i in [0, len)
-__device__ __forceinline__ long chk_offset(long i, long len) {
-#ifdef MLSW_DEBUG
-  if (i < 0 || i >= len) {
-    note_bounds_violation();
-    return 0;
-  }
-#endif
-  return i;
-}
-// global store target: p inside [base, base + len)
-__device__ __forceinline__ float* chk_global(float* base, float* p, long len) {
-#ifdef MLSW_DEBUG
-  const long i = p - base;
-  if (i < 0 || i >= len) {
-    note_bounds_violation();
-    return base;
-  }
-#endif
-  return p;
-}
-
-// ---------------------------------------------------------------------------
-// Stores of one post-collision population to its streamed destination
-// (dx, dy) (already periodic) and to the ghost cells that image it.
-// ---------------------------------------------------------------------------
-// Lattices with both sides >= 4 cells: a real column d has at most one
-// ghost image (d + n for d < 2, d - n for d >= n - 2), likewise rows, so a
-// population near an edge needs at most three extra stores.
-constexpr int kNoImage = -(1 << 28);
-
-__device__ __forceinline__ int image_of(int d, int n) {
-  return d < 2 ? d + n : (d >= n - 2 ? d - n : kNoImage);
-}
-
-__device__ __forceinline__ void store_edge(float* __restrict__ plane_base, const Layout& L,
-                                           int dx, int dy, int xi, int yi, float v) {
-  // indices into the plane (not derived pointers), so that the stores keep
-  // the base pointer's no-alias guarantee
-  const long r0 = (long)(dy + L.gy) * L.pitch;
-  plane_base[chk_offset(r0 + dx + L.gx, L.plane)] = v;
-  if (xi != kNoImage) plane_base[chk_offset(r0 + xi + L.gx, L.plane)] = v;
-  if (yi != kNoImage) {
-    const long r1 = (long)(yi + L.gy) * L.pitch;
-    plane_base[chk_offset(r1 + dx + L.gx, L.plane)] = v;
-    if (xi != kNoImage) plane_base[chk_offset(r1 + xi + L.gx, L.plane)] = v;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The rest population after the collision, g0* = g0 + delta: the stored rest
-// population g0 (shifted by H, O(h - H)) plus a small change (the incoming
-// moving populations less the outgoing equilibria, times omega when tau !=
-// 1). Rounding g0 + delta to FP32 loses up to half an ulp of g0 per cell
-// and step, and in a slowly changing film (a dewetted precursor far from H)
-// that loss has the same sign step after step. The exact rounding error
-// (Fast2Sum, |g0| >= |delta| in the cells where it matters) is passed on
-// instead, half to each of two opposite moving populations: their ulp is
-// orders of magnitude finer, the momentum they carry is unchanged, and the
-// cell's populations sum to the incoming mass to their rounding.
-// ---------------------------------------------------------------------------
-template <class T>
-__device__ __forceinline__ T rest_update(T g0, T delta, T& fa, T& fb) {
-  const T out = g0 + delta;
-  const T r = delta - (out - g0);  // exact: the part of delta the sum dropped
-  fa = fmav(r, 0.5f, fa);
-  fb = fmav(r, 0.5f, fb);
-  return out;
-}
-
-// Equilibrium, BGK with forcing for one layer at one cell; fs[k] receives
-// the post-collision populations (rest one stored shifted by H).
-// g0: the stored rest population; small: the sum of the stored moving ones
-// (h - H = g0 + small); f_old (read only when !TAU1) holds the stored
-// pre-collision populations.
-template <int LAT, bool TAU1>
-__device__ __forceinline__ void collide(const KParams& P, float h, float g0, float small,
-                                        float jx, float jy, float Fx, float Fy,
-                                        const float* f_old, float (&fs)[Lattice<LAT>::Q]) {
-  using Lt = Lattice<LAT>;
-  const float inv_h = rcp(h);
-  const float ux = jx * inv_h, uy = jy * inv_h;
-  const float u2 = ux * ux + uy * uy;
-  float sum_eq = 0.f;
-#pragma unroll
-  for (int k = 1; k < Lt::Q; ++k) {
-    const float cu = (float)Lt::cx(k) * ux + (float)Lt::cy(k) * uy;
-    // w_k h (c.U / cs^2 + (c.U)^2 / (2 cs^4) - U^2 / (2 cs^2)), cs^2 = 1/3
-    const float feq = Lt::w(k) * h * (3.f * cu + 4.5f * cu * cu - 1.5f * u2);
-    sum_eq += feq;
-    float v = TAU1 ? feq : f_old[k] + P.omega * (feq - f_old[k]);
-    v += 3.f * Lt::w(k) * ((float)Lt::cx(k) * Fx + (float)Lt::cy(k) * Fy);
-    fs[k] = v;
-  }
-  // rest population: h - sum of the moving equilibria, which equals
-  // h (1 - w_0 U^2 / (2 cs^2)) and keeps the cell's mass exact in the sum;
-  // stored shifted by H: g0 + (small - sum_eq), relaxed by omega when
-  // tau != 1 (the moving populations then keep 1 - omega of small)
-  const float d = small - sum_eq;
-  fs[0] = rest_update(g0, TAU1 ? d : P.omega * d, fs[1], fs[2]);
-}
-
-// ---------------------------------------------------------------------------
-// D2Q9 collision with the opposite directions paired: for c_{k+4} = -c_k the
-// equilibria share w_k h (4.5 (c.U)^2 - 1.5 U^2) and differ in the sign of
-// 3 w_k h c.U, and the forcing terms 3 w_k c.F are odd, so each pair costs
-// one symmetric and one antisymmetric part. Directions: 1 (1,0), 2 (1,1),
-// 3 (0,1), 4 (-1,1); 5..8 are their opposites.
-// ---------------------------------------------------------------------------
-template <bool TAU1, class T>
-__device__ __forceinline__ void collide_d2q9(const KParams& P, T h, T g0, T small, T jx, T jy,
-                                             T Fx, T Fy, const T* f_old, T (&fs)[9]) {
-  const T ih = rcp(h);
-  const T ux = jx * ih, uy = jy * ih;
-  const T u15 = 1.5f * fmav(ux, ux, uy * uy);
-  T sumsym = Num<T>::splat(0.f);
-  const T cus[4] = {ux, ux + uy, uy, uy - ux};
-  const T cfs[4] = {Fx, Fx + Fy, Fy, Fy - Fx};
-  const float ws[4] = {1.f / 9.f, 1.f / 36.f, 1.f / 9.f, 1.f / 36.f};
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const T A = ws[q] * h;
-    const T cu = cus[q];
-    const T sym = A * fmav(4.5f * cu, cu, -u15);
-    sumsym += sym;
-    if constexpr (TAU1) {
-      const T anti = 3.f * fmav(A, cu, ws[q] * cfs[q]);
-      fs[q + 1] = sym + anti;
-      fs[q + 5] = sym - anti;
-    } else {
-      const T aeq = (3.f * A) * cu, afr = (3.f * ws[q]) * cfs[q];
-      fs[q + 1] = fmav(P.omega, (sym + aeq) - f_old[q + 1], f_old[q + 1]) + afr;
-      fs[q + 5] = fmav(P.omega, (sym - aeq) - f_old[q + 5], f_old[q + 5]) - afr;
-    }
-  }
-  // rest population h - (sum of moving equilibria) = h (1 - w_0 U^2/(2 cs^2)),
-  // stored shifted by H: g0 + (small - 2 sumsym), relaxed by omega when
-  // tau != 1 (see rest_update)
-  const T d = fmav(-2.f, sumsym, small);
-  fs[0] = rest_update(g0, TAU1 ? d : P.omega * d, fs[1], fs[5]);
-}
-
-// Sum of the eight stored moving populations of one layer at a cell: the
-// opposite directions first (their moving parts nearly cancel), then the
-// diagonals with the axes. The layer's h - H is the rest population plus
-// this sum, added last: adding the small populations to the O(h - H) rest
-// population one by one would drop their low bits one direction at a time.
-template <class T>
-__device__ __forceinline__ T moving_sum(const T (&v)[9]) {
-  return ((v[1] + v[5]) + (v[3] + v[7])) + ((v[2] + v[6]) + (v[4] + v[8]));
-}
 
 // Loads / stores of one cell (float) or of a pair of cells (f2) at two
 // addresses.
@@ -228,7 +42,7 @@ template <> struct Lanes<f2> {
 //   zs    [N][TY + 4][36]    interface-height deviations z_i - sum_{j<=i} H_j
 //                            on the two-ring region (their differences give
 //                            the layer thicknesses)
-//   ps    [N][TY + 2][34]    p_i on the one-ring region
+//   ps    [N][TY + 2][34]    q_i = p_atm - p_i on the one-ring region
 //   js    [2][N][TY][32]     fluxes J_i of the tile cells
 //   bar                      mbarrier (8 bytes)
 //   next_tile                (int)
@@ -261,11 +75,6 @@ struct D2Tile {
   // reserved blocks fill the 228 KB of an SM
   static_assert(2 * (kSmem + 1024) <= 233472, "two CTAs per SM");
 };
-
-// Kernel modes: the general step for tau != 1 and for tau = 1, and a fast
-// step for the case the paper runs (tau = 1, wetting exponents (3, 2),
-// spreading coefficients only between neighbouring interfaces).
-enum StepMode { kGeneral = 0, kTau1 = 1, kFast = 2 };
 
 // One tile of work: its parameters, the tensor map of its input buffer, its
 // output buffer and its position in the tile grid of its lattice.
@@ -577,9 +386,9 @@ __device__ __forceinline__ int d2q9_tile_loop(const Tiles& tiles, int* __restric
             z0c = LU::ld2(zc[0], zc[1]);
             sg0 = LU::ld2(sg[0], sg[1]);
           }
-          layer_pressures_dev<N, W32, U, NN>(P, zd, gzx, gzy, lz, p, z0c, sg0);
+          neg_pressures<N, W32, U, NN>(P, zd, gzx, gzy, lz, p, &z0c, &sg0);
         } else {
-          layer_pressures_dev<N, W32, U, NN>(P, zd, gzx, gzy, lz, p);
+          neg_pressures<N, W32, U, NN>(P, zd, gzx, gzy, lz, p);
         }
 #pragma unroll
         for (int i = 0; i < N; ++i)
@@ -622,8 +431,14 @@ __device__ __forceinline__ int d2q9_tile_loop(const Tiles& tiles, int* __restric
             jy[i] = Ln::ld(js + ((1 * N + i) * TY + iyA) * TX + ix, js + ((1 * N + i) * TY + iyB) * TX + ix);
           }
         }
-        T Rx[N], Ry[N];
-        friction<N>(P, hh, jx, jy, Rx, Ry);
+        T ih[N], ux[N], uy[N], Rx[N], Ry[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          ih[i] = rcp(hh[i]);
+          ux[i] = jx[i] * ih[i];
+          uy[i] = jy[i] * ih[i];
+        }
+        friction<N, true>(P, hh, ih, ux, uy, Rx, Ry);
         // A tile at least three cells from every edge streams without
         // wrap-around or ghost images: all nine destinations are fixed,
         // warp-uniform offsets from one base per cell.
@@ -719,11 +534,11 @@ __device__ __forceinline__ int d2q9_tile_loop(const Tiles& tiles, int* __restric
           const T pN = Ln::ld(a + PW, b + PW), pS = Ln::ld(a - PW, b - PW);
           const T pNE = Ln::ld(a + PW + 1, b + PW + 1), pNW = Ln::ld(a + PW - 1, b + PW - 1);
           const T pSE = Ln::ld(a - PW + 1, b - PW + 1), pSW = Ln::ld(a - PW - 1, b - PW - 1);
-          const T gpx = fmav(pE - pW, 1.f / 3.f, ((pNE - pNW) + (pSE - pSW)) * (1.f / 12.f));
-          const T gpy = fmav(pN - pS, 1.f / 3.f, ((pNE - pSE) + (pNW - pSW)) * (1.f / 12.f));
+          const T gqx = fmav(pE - pW, 1.f / 3.f, ((pNE - pNW) + (pSE - pSW)) * (1.f / 12.f));
+          const T gqy = fmav(pN - pS, 1.f / 3.f, ((pNE - pSE) + (pNW - pSW)) * (1.f / 12.f));
           const T h = hh[i];
-          const T Fx = fmav(-h, gpx, Rx[i]);
-          const T Fy = fmav(-h, gpy, Ry[i]);
+          const T Fx = fmav(h, gqx, Rx[i]);
+          const T Fy = fmav(h, gqy, Ry[i]);
 #pragma unroll
           for (int l = 0; l < W; ++l)
             if (valid[l])
@@ -736,7 +551,7 @@ __device__ __forceinline__ int d2q9_tile_loop(const Tiles& tiles, int* __restric
             for (int k = 0; k < Q; ++k) fo[k] = Ln::ld(sA + (i * Q + k) * BH * BW, sB + (i * Q + k) * BH * BW);
           }
           T fs[Q];
-          collide_d2q9<TAU1>(P, h, g0s[i], sms[i], jx[i], jy[i], Fx, Fy, fo, fs);
+          collide_d2q9<TAU1>(P, g0s[i], sms[i], jx[i], jy[i], ux[i], uy[i], Fx, Fy, fo, fs);
           if (inner) {
 #pragma unroll
             for (int l = 0; l < W; ++l) {

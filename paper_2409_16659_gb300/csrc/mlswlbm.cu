@@ -119,6 +119,13 @@ double spectral_radius_I_plus_K(const mlsw_params& p, const double* h) {
   return std::exp((logscale + 0.5 * std::log(fro)) / std::ldexp(1.0, squarings));
 }
 
+// friction coefficients of layer i, rounded to FP32 once
+void set_friction(KParams& k, int i, double mu, double beta) {
+  k.fr_visc[i] = (float)(-1.0 / (6.0 * mu));
+  k.fr_slip[i] = (float)(beta / mu);
+  k.fr_slip2[i] = (float)(beta * beta / (2.0 * mu));
+}
+
 KParams make_kparams(const mlsw_params& p) {
   KParams k;
   std::memset(&k, 0, sizeof(k));
@@ -128,8 +135,7 @@ KParams make_kparams(const mlsw_params& p) {
   k.omega = (float)(1.0 / p.tau);
   for (int i = 0; i < p.n_layers; ++i) {
     k.gamma[i] = (float)p.gamma[i];
-    k.mu_inv[i] = (float)(1.0 / p.mu[i]);
-    k.beta[i] = (float)p.beta[i];
+    set_friction(k, i, p.mu[i], p.beta[i]);
     for (int kk = 1; kk <= p.n_layers - i; ++kk) k.S[i][kk - 1] = (float)p.spread[i][kk - 1];
   }
   k.hstar = (float)p.hstar;
@@ -138,6 +144,8 @@ KParams make_kparams(const mlsw_params& p) {
   if (p.wet_kind == 0) {
     k.c_phi = (float)(1.0 / (p.wet_n - p.wet_m));
     k.c_dphi = (float)((double)p.wet_n * p.wet_m / (p.wet_n - p.wet_m));
+    for (int i = 0; i < p.n_layers; ++i)
+      k.Sd[i] = (float)(p.spread[i][0] * p.wet_n * p.wet_m / (p.wet_n - p.wet_m));
   }
   k.wet_kind = p.wet_kind;
   k.kappa = (float)p.wet_kappa;
@@ -933,8 +941,7 @@ int mlswlbm_friction_eval(const mlsw_params* p, long ncell, const float* hh, con
   std::memset(&k, 0, sizeof(k));
   k.n = n;
   for (int i = 0; i < n; ++i) {
-    k.mu_inv[i] = (float)(1.0 / p->mu[i]);
-    k.beta[i] = (float)p->beta[i];
+    set_friction(k, i, p->mu[i], p->beta[i]);
   }
   CU(mlsw::launch_friction_eval(k, ncell, hh, Jx, Jy, Rx, Ry, (cudaStream_t)stream));
   return MLSW_OK;

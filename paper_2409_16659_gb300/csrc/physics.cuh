@@ -81,8 +81,9 @@ struct KParams {
   float omega;                       // 1 / tau
   float gamma[kMaxLayers];           // gamma_{i,i+1}
   float S[kMaxLayers][kMaxLayers];   // S[l][k-1] = S_{lk}
-  float mu_inv[kMaxLayers];          // 1 / mu_i
-  float beta[kMaxLayers];            // beta_i
+  float Sd[kMaxLayers];              // S_{l1} nw mw / (nw - mw)
+  // friction (see friction()): -1 / (6 mu_i), beta_i / mu_i, beta_i^2 / (2 mu_i)
+  float fr_visc[kMaxLayers], fr_slip[kMaxLayers], fr_slip2[kMaxLayers];
   float hstar;
   int nw, mw;
   float c_phi;                       // 1 / (nw - mw)
@@ -194,9 +195,15 @@ __device__ __forceinline__ f2 fmav(float a, f2 b, f2 c) { return fmav(mk2(a, a),
 __device__ __forceinline__ f2 fmav(f2 a, f2 b, float c) { return fmav(a, b, mk2(c, c)); }
 __device__ __forceinline__ f2 fmav(f2 a, float b, float c) { return fmav(a, mk2(b, b), mk2(c, c)); }
 
-// fast reciprocal: the __fdividef intrinsic (at most 2 ulp for the O(1e-2 ..
-// 1e2) arguments used here: layer thicknesses, friction pivots)
-__device__ __forceinline__ float rcp(float x) { return __fdividef(1.f, x); }
+// fast reciprocal: the hardware's approximation, at most 1 ulp for normal
+// arguments (here layer thicknesses and friction pivots, far from the ends
+// of the FP32 range). Division intrinsics add five instructions of range
+// scaling to it, which no argument here needs.
+__device__ __forceinline__ float rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ f2 rcp(f2 x) { return mk2(rcp(x.v.x), rcp(x.v.y)); }
 __device__ __forceinline__ float expv(float x) { return expf(x); }
 __device__ __forceinline__ f2 expv(f2 x) { return mk2(expf(x.v.x), expf(x.v.y)); }
@@ -208,22 +215,11 @@ __device__ __forceinline__ T ipow(T r, int e) {
   return a;
 }
 
-// r^mw and r^nw: the common exponent pair (3, 2) at compile time (W32), any
-// other pair with a run-time loop
-template <bool W32, class T>
-__device__ __forceinline__ void wet_powers(const KParams& P, T r, T& rm, T& rn) {
-  if (W32) {
-    rm = r * r;
-    rn = rm * r;
-  } else {
-    rm = ipow(r, P.mw);
-    rn = ipow(r, P.nw);
-  }
-}
-
 // ---------------------------------------------------------------------------
-// Layer pressures p_i - p_atm at one cell (Eqs. Laplace_pressure,
-// disjoining_pressure; p_i = sum_{j>=i} (Lambda_j + Pi_j)).
+// Layer pressures at one cell, with the sign turned: q_i = p_atm - p_i (Eqs.
+// Laplace_pressure, disjoining_pressure; p_i = sum_{j>=i} (Lambda_j + Pi_j)),
+// so that the force of the next phase is F_i = R_i + h_i grad q_i without a
+// negation (a packed pair has no sign modifier on its operands).
 // Every interface pair (l, m = l + k), 0 <= l < m <= N, enters once with
 // the thickness d = z_m - z_l between them: E = S_lk phi'_k(d)
 // (1 + |grad z_l|^2 / 2) is subtracted from Pi_l and added to Pi_m, and
@@ -236,217 +232,141 @@ __device__ __forceinline__ void wet_powers(const KParams& P, T r, T& rm, T& rn) 
 // ---------------------------------------------------------------------------
 // NN: only nearest-neighbour pairs (k = 1) carry a spreading coefficient
 // (S_{lk} = 0 for k >= 2, as in the paper's three-layer runs); the pair loop
-// is then branch-free.
+// is then branch-free. With W32 (exponents 3, 2) the power law is evaluated
+// as phi = r^2 (3 - 2 r), phi' = 6 r^2 (r - 1) / d.
 // z0, sg0: the substrate height z_0 (on the scale of zd) and 1 + |grad z_0|^2 / 2
-// at the cell; 0 and 1 for the flat substrate.
+// at the cell; null for the flat substrate (0 and 1).
 template <int N, bool W32, class T, bool NN = false>
-__device__ __forceinline__ void layer_pressures_dev(const KParams& P, const T (&zd)[N],
-                                                    const T (&gx)[N], const T (&gy)[N],
-                                                    const T (&lz)[N], T (&p)[N],
-                                                    T z0 = Num<T>::splat(0.f),
-                                                    T sg0 = Num<T>::splat(1.f)) {
-  T ten[N], pi[N], sg[N];
+__device__ __forceinline__ void neg_pressures(const KParams& P, const T (&zd)[N], const T (&gx)[N],
+                                              const T (&gy)[N], const T (&lz)[N], T (&q)[N],
+                                              const T* z0 = nullptr, const T* sg0 = nullptr) {
+  T ten[N], pi[N];  // tension of the interface; -Pi of the layer
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     ten[i] = Num<T>::splat(P.gamma[i]);
     pi[i] = Num<T>::splat(0.f);
-    sg[i] = fmav(0.5f, fmav(gx[i], gx[i], gy[i] * gy[i]), Num<T>::splat(1.f));
   }
 #pragma unroll
   for (int l = 0; l < N; ++l) {
-    const T sgl = (l == 0) ? sg0 : sg[l > 0 ? l - 1 : 0];
-    const T zl = (l == 0) ? z0 : zd[l > 0 ? l - 1 : 0];
+    T sgl;
+    if (l > 0) {
+      const int i = l > 0 ? l - 1 : 0;
+      sgl = fmav(0.5f, fmav(gx[i], gx[i], gy[i] * gy[i]), Num<T>::splat(1.f));
+    }
 #pragma unroll
     for (int m = l + 1; m <= (NN ? l + 1 : N); ++m) {
       const int k = m - l;
       const float s = P.S[l][k - 1];
       if (NN || s != 0.f) {
-        const T d = (zd[m - 1] - zl) + P.Hsum[l][m];
-        T phi, dphi;
+        T d;
+        if (l > 0)
+          d = (zd[m - 1] - zd[l > 0 ? l - 1 : 0]) + P.Hsum[l][m];
+        else if (z0)
+          d = (zd[m - 1] - *z0) + P.Hsum[l][m];
+        else
+          d = zd[m - 1] + P.Hsum[l][m];
+        T phi, e;  // e = S phi'
         if (!W32 && P.wet_kind == 1) {
           // charged surfaces: a = e^{-kappa (d - k h*)}, phi = 2 a - a^2,
           // phi' = 2 kappa a (a - 1)
           const T a = expv(fmav(d, -P.kappa, P.kappa * ((float)k * P.hstar)));
           phi = a * (2.f - a);
-          dphi = (2.f * P.kappa) * (a * (a - 1.f));
+          e = s * ((2.f * P.kappa) * (a * (a - 1.f)));
         } else {
           const T inv_d = rcp(d);
           const T r = ((float)k * P.hstar) * inv_d;
-          T rm, rn;
-          wet_powers<W32>(P, r, rm, rn);
-          phi = W32 ? fmav(rm, 3.f, -2.f * rn)
-                    : (fmav(rm, (float)P.nw, -(float)P.mw * rn)) * P.c_phi;
-          dphi = (P.c_dphi * (rn - rm)) * inv_d;
+          if constexpr (W32) {
+            const T r2 = r * r;
+            phi = r2 * fmav(r, -2.f, 3.f);
+            e = (NN ? P.Sd[l] : s * P.c_dphi) * ((r2 * (r - 1.f)) * inv_d);
+          } else {
+            const T rm = ipow(r, P.mw), rn = rm * ipow(r, P.nw - P.mw);
+            phi = fmav(rm, (float)P.nw, -(float)P.mw * rn) * P.c_phi;
+            e = s * ((P.c_dphi * (rn - rm)) * inv_d);
+          }
         }
-        const T se = s * dphi;
         // explicit fused updates, so one cell and a packed pair of cells
         // round identically
-        if (l >= 1) {
-          ten[l > 0 ? l - 1 : 0] = fmav(s, phi, ten[l > 0 ? l - 1 : 0]);
-          pi[l > 0 ? l - 1 : 0] = fmav(-se, sgl, pi[l > 0 ? l - 1 : 0]);
+        if (l > 0) {
+          const int i = l > 0 ? l - 1 : 0;
+          e = e * sgl;
+          ten[i] = fmav(s, phi, ten[i]);
+          pi[i] = pi[i] + e;
+        } else if (sg0) {
+          e = e * *sg0;
         }
-        pi[m - 1] = fmav(se, sgl, pi[m - 1]);
+        pi[m - 1] = pi[m - 1] - e;
       }
     }
   }
   T acc = Num<T>::splat(0.f);
 #pragma unroll
   for (int i = N - 1; i >= 0; --i) {
-    acc = acc + fmav(-ten[i], lz[i], pi[i]);
-    p[i] = acc;
+    const T own = fmav(ten[i], lz[i], pi[i]);
+    acc = i == N - 1 ? own : acc + own;
+    q[i] = acc;
   }
 }
 
 // ---------------------------------------------------------------------------
-// Friction 2 mu_i h_i a_i (Eq. friction_force) by shear-stress integration.
+// Friction R_i = 2 mu_i h_i a_i (Eq. friction_force) from the thicknesses
+// and the layers' mean velocities U_i = J_i / h_i.
 //
-// In Stokes layers with pressure gradient G_i, mu_i u'' = G_i. Integrating
-// the stress down from the stress-free top (Eq. viscous_boundary with
-// mu_{n+1} = 0) gives, in layer i, sigma(z) = G_i (z - z_i) - sum_{j>i} h_j G_j.
-// Integrating u = sigma / mu_i upward from the substrate, the slip condition
-// of Eq. (no_slip) -- the parabola of layer i continued a distance beta_i
-// below z_{i-1} meets u_{i-1}(z_{i-1}) -- adds the jump
-// (beta_i / mu_i) sigma_i(z_{i-1} - beta_i / 2). Integrating u over each
-// layer (Eq. flux) gives J = L G with an N x N matrix L built column by
-// column in O(N^2). Force balance of the thin-sheet equation,
-// 0 = -h_i G_i + 2 mu_i h_i a_i, then gives the friction R_i = h_i G_i with
-// G = L^-1 J: one factorisation, two right-hand sides (x and y), by the
-// adjugate for N <= 3 and by elimination with row pivoting for N = 4, 5 (L is
-// not symmetric in general: the slip convention breaks reciprocity; the
-// pivoted form is scalar only).
+// In Stokes layers with pressure gradient G_i, mu_i u'' = G_i; the force
+// balance 0 = -h_i G_i + 2 mu_i h_i a_i makes R_i = h_i G_i. Integrating the
+// stress down from the stress-free top (Eq. viscous_boundary with mu_{n+1} =
+// 0), the interface above layer i carries -T_{i+1} and the one below it
+// -T_i, with T_i = sum_{j>=i} R_j (T_{n+1} = 0). Integrating u upward through
+// layer i from the velocity w_i of the interface below it, with the slip
+// condition of Eq. (no_slip) (the parabola continued a distance beta_i below
+// the interface meets w_i),
+//   mean velocity  U_i = w_i - (b_i + c_i / h_i) T_i + (c_i / h_i) T_{i+1}
+//                          - (h_i / mu_i) (T_i / 3 + T_{i+1} / 6)
+//   next interface w_{i+1} - U_i = -(h_i / mu_i) (T_i / 6 + T_{i+1} / 3)
+// with b_i = beta_i / mu_i, c_i = beta_i^2 / (2 mu_i). Subtracting
+// neighbouring layers eliminates the w_i (w_1 = 0) and leaves a tridiagonal
+// system for T: with a_i = h_i / (6 mu_i), s_i = c_i / h_i,
+//   a_{i-1} T_{i-1} + (2 a_{i-1} + 2 a_i + b_i + s_i) T_i + (a_i - s_i) T_{i+1}
+//     = U_{i-1} - U_i        (a_0 = U_0 = 0).
+// Its rows are strictly diagonally dominant (a, b, s >= 0, a > 0), so
+// elimination needs no pivoting for any n, thicknesses and slips. Solving
+// the full n x n flux-gradient matrix took 2.5 times the arithmetic at n = 3
+// (adjugate), and a pivoted elimination on single cells at n = 4, 5.
+// ih: 1 / h. TWO: both components (else the y ones are left alone).
 // ---------------------------------------------------------------------------
-// Solves L G = J for two right-hand sides with the adjugate of L
-// (N = 1, 2, 3). Unused for larger N.
-template <int N, class T>
-__device__ __forceinline__ void solve_small(const T (&L)[N][N], const T (&Jx)[N],
-                                            const T (&Jy)[N], T (&Gx)[N], T (&Gy)[N]) {
-  if constexpr (N == 1) {
-    const T r = rcp(L[0][0]);
-    Gx[0] = Jx[0] * r;
-    Gy[0] = Jy[0] * r;
-  } else if constexpr (N == 2) {
-    const T r = rcp(fmav(L[0][0], L[1][1], -(L[0][1] * L[1][0])));
-    Gx[0] = fmav(L[1][1], Jx[0], -(L[0][1] * Jx[1])) * r;
-    Gx[1] = fmav(L[0][0], Jx[1], -(L[1][0] * Jx[0])) * r;
-    Gy[0] = fmav(L[1][1], Jy[0], -(L[0][1] * Jy[1])) * r;
-    Gy[1] = fmav(L[0][0], Jy[1], -(L[1][0] * Jy[0])) * r;
-  } else if constexpr (N == 3) {
-    const T a = L[0][0], b = L[0][1], c = L[0][2];
-    const T d = L[1][0], e = L[1][1], f = L[1][2];
-    const T g = L[2][0], hh = L[2][1], k = L[2][2];
-    const T A00 = fmav(e, k, -(f * hh)), A01 = fmav(c, hh, -(b * k)), A02 = fmav(b, f, -(c * e));
-    const T A10 = fmav(f, g, -(d * k)), A11 = fmav(a, k, -(c * g)), A12 = fmav(c, d, -(a * f));
-    const T A20 = fmav(d, hh, -(e * g)), A21 = fmav(b, g, -(a * hh)), A22 = fmav(a, e, -(b * d));
-    const T r = rcp(fmav(a, A00, fmav(b, A10, c * A20)));
-    Gx[0] = fmav(A00, Jx[0], fmav(A01, Jx[1], A02 * Jx[2])) * r;
-    Gx[1] = fmav(A10, Jx[0], fmav(A11, Jx[1], A12 * Jx[2])) * r;
-    Gx[2] = fmav(A20, Jx[0], fmav(A21, Jx[1], A22 * Jx[2])) * r;
-    Gy[0] = fmav(A00, Jy[0], fmav(A01, Jy[1], A02 * Jy[2])) * r;
-    Gy[1] = fmav(A10, Jy[0], fmav(A11, Jy[1], A12 * Jy[2])) * r;
-    Gy[2] = fmav(A20, Jy[0], fmav(A21, Jy[1], A22 * Jy[2])) * r;
+template <int N, bool TWO, class T>
+__device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], const T (&ih)[N],
+                                         const T (&Ux)[N], const T (&Uy)[N], T (&Rx)[N],
+                                         T (&Ry)[N]) {
+  T piv[N], nsup[N], bx[N], by[N];
+  T na_prev;  // -a_{i-1}
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const T na = h[i] * P.fr_visc[i], s = ih[i] * P.fr_slip2[i];
+    T diag = fmav(na, -2.f, s + P.fr_slip[i]);
+    nsup[i] = na + s;
+    if (i == 0) {
+      bx[0] = Ux[0] * -1.f;
+      if constexpr (TWO) by[0] = Uy[0] * -1.f;
+    } else {
+      const int j = i > 0 ? i - 1 : 0;
+      const T nf = na_prev * piv[j];
+      diag = fmav(nf, nsup[j] * -1.f, fmav(na_prev, -2.f, diag));
+      bx[i] = fmav(nf, bx[j], Ux[j] - Ux[i]);
+      if constexpr (TWO) by[i] = fmav(nf, by[j], Uy[j] - Uy[i]);
+    }
+    piv[i] = rcp(diag);
+    na_prev = na;
   }
-}
-
-template <int N, class T>
-__device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], const T (&Jx)[N],
-                                         const T (&Jy)[N], T (&Rx)[N], T (&Ry)[N]) {
-  T L[N][N];
+  T tx, ty;  // T_{i+1}
 #pragma unroll
-  for (int j = 0; j < N; ++j) {
-    T ub = Num<T>::splat(0.f);  // velocity at the bottom of layer i for unit G_j
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const float mi = P.mu_inv[i], bi = P.beta[i];
-      const T hi = h[i];
-      if (j > i) {
-        // unit gradient in a layer above: only the stress s = -h_j acts
-        const T s = -h[j];
-        ub = fmav(s, bi * mi, ub);
-        L[i][j] = fmav(hi, ub, (mi * 0.5f) * (hi * hi) * s);
-        ub = fmav(mi * hi, s, ub);
-      } else if (j == i) {
-        // unit gradient in this layer (g = 1, s = 0)
-        ub = fmav(-(bi * mi), hi + 0.5f * bi, ub);
-        L[i][j] = fmav(hi, ub, (-mi / 3.f) * (hi * hi) * hi);
-        ub = fmav(-0.5f * mi, hi * hi, ub);
-      } else {
-        L[i][j] = hi * ub;  // layers above the forced one move with it
-      }
-    }
-  }
-  if constexpr (N <= 3) {
-    // adjugate (Cramer) solution of the 1x1 / 2x2 / 3x3 system
-    T Gx[N], Gy[N];
-    solve_small<N>(L, Jx, Jy, Gx, Gy);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      Rx[i] = h[i] * Gx[i];
-      Ry[i] = h[i] * Gy[i];
-    }
-    return;
-  } else {
-    static_assert(sizeof(T) == sizeof(float), "pivoted elimination is scalar");
-    float bx[N], by[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      bx[i] = Jx[i];
-      by[i] = Jy[i];
-    }
-    float inv_piv[N];
-#pragma unroll
-    for (int c = 0; c < N; ++c) {
-      int piv = c;
-      float best = fabsf(L[c][c]);
-#pragma unroll
-      for (int r = c + 1; r < N; ++r) {
-        const float a = fabsf(L[r][c]);
-        if (a > best) {
-          best = a;
-          piv = r;
-        }
-      }
-      // the row exchange as selects on fixed indices, so that the system
-      // stays in registers
-#pragma unroll
-      for (int r = c + 1; r < N; ++r) {
-        const bool sw = (piv == r);
-#pragma unroll
-        for (int q = c; q < N; ++q) {
-          const float a = L[c][q], b = L[r][q];
-          L[c][q] = sw ? b : a;
-          L[r][q] = sw ? a : b;
-        }
-        const float ax = bx[c], bxr = bx[r], ay = by[c], byr = by[r];
-        bx[c] = sw ? bxr : ax;
-        bx[r] = sw ? ax : bxr;
-        by[c] = sw ? byr : ay;
-        by[r] = sw ? ay : byr;
-      }
-      inv_piv[c] = rcp(L[c][c]);
-#pragma unroll
-      for (int r = c + 1; r < N; ++r) {
-        const float l = L[r][c] * inv_piv[c];
-#pragma unroll
-        for (int q = c + 1; q < N; ++q) L[r][q] -= l * L[c][q];
-        bx[r] -= l * bx[c];
-        by[r] -= l * by[c];
-      }
-    }
-#pragma unroll
-    for (int c = N - 1; c >= 0; --c) {
-      float sx = bx[c], sy = by[c];
-#pragma unroll
-      for (int q = c + 1; q < N; ++q) {
-        sx -= L[c][q] * bx[q];
-        sy -= L[c][q] * by[q];
-      }
-      bx[c] = sx * inv_piv[c];
-      by[c] = sy * inv_piv[c];
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      Rx[i] = h[i] * bx[i];
-      Ry[i] = h[i] * by[i];
+  for (int i = N - 1; i >= 0; --i) {
+    const T ox = tx, oy = ty;
+    tx = (i == N - 1 ? bx[i] : fmav(nsup[i], ox, bx[i])) * piv[i];
+    Rx[i] = i == N - 1 ? tx : tx - ox;
+    if constexpr (TWO) {
+      ty = (i == N - 1 ? by[i] : fmav(nsup[i], oy, by[i])) * piv[i];
+      Ry[i] = i == N - 1 ? ty : ty - oy;
     }
   }
 }

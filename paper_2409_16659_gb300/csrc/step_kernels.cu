@@ -28,6 +28,7 @@
 
 #include "kernels.h"
 #include "physics.cuh"
+#include "step_common.cuh"
 #include "d2q9_tile.cuh"
 
 namespace mlsw {
@@ -49,7 +50,7 @@ __global__ void __launch_bounds__(256, 2)
 // D1Q3 cell arithmetic shared by the tiled and the persistent kernels, so
 // both give the same bits.
 // ---------------------------------------------------------------------------
-// p_i of one cell from z deviations at x - 1, x, x + 1
+// q_i = p_atm - p_i of one cell from z deviations at x - 1, x, x + 1
 // z0w, z0c, z0e: the substrate at x - 1, x, x + 1 (all 0 when flat)
 template <int N, bool W32>
 __device__ __forceinline__ void d1q3_pressures(const KParams& P, const float (&zw)[N],
@@ -67,9 +68,10 @@ __device__ __forceinline__ void d1q3_pressures(const KParams& P, const float (&z
   }
   if (P.sub_amp != 0.f) {
     const float g0 = 0.5f * (z0e - z0w);
-    layer_pressures_dev<N, W32>(P, zd, gxz, gyz, lz, p, z0c, fmaf(0.5f, g0 * g0, 1.f));
+    const float sg0 = fmaf(0.5f, g0 * g0, 1.f);
+    neg_pressures<N, W32>(P, zd, gxz, gyz, lz, p, &z0c, &sg0);
   } else {
-    layer_pressures_dev<N, W32>(P, zd, gxz, gyz, lz, p);
+    neg_pressures<N, W32>(P, zd, gxz, gyz, lz, p);
   }
 }
 
@@ -83,18 +85,21 @@ __device__ __forceinline__ bool d1q3_collide_cell(const KParams& P, const float 
                                                   const float (&pw)[N], const float (&pc)[N],
                                                   const float (&pe)[N], const float (&f_old)[N][3],
                                                   float (&fs)[N][3]) {
-  float zero[N], Rx[N], Ry[N];
+  float ih[N], ux[N], Rx[N];
 #pragma unroll
-  for (int i = 0; i < N; ++i) zero[i] = 0.f;
-  friction<N>(P, hh, jx, zero, Rx, Ry);
+  for (int i = 0; i < N; ++i) {
+    ih[i] = rcp(hh[i]);
+    ux[i] = jx[i] * ih[i];
+  }
+  friction<N, false>(P, hh, ih, ux, ux, Rx, Rx);
   bool bad = false;
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const float gpx = 0.5f * ((pe[i] - pc[i]) - (pw[i] - pc[i]));
+    const float gqx = 0.5f * ((pe[i] - pc[i]) - (pw[i] - pc[i]));
     const float h = hh[i];
-    const float Fx = fmav(-h, gpx, Rx[i]);
+    const float Fx = fmav(h, gqx, Rx[i]);
     bad |= !(h > 0.f) || !isfinite(Fx) || !isfinite(jx[i]);
-    collide<1, TAU1>(P, h, g0[i], sm[i], jx[i], 0.f, Fx, 0.f, f_old[i], fs[i]);
+    collide_d1q3<TAU1>(P, g0[i], sm[i], jx[i], ux[i], Fx, f_old[i], fs[i]);
   }
   return bad;
 }
