@@ -38,7 +38,10 @@
  *     fluxes of precursor films representable in FP32. mlswlbm_get_state /
  *     mlswlbm_set_state convert to and from the true populations;
  *     mlswlbm_save_state / mlswlbm_load_state move the
- *     internal representation unchanged (bit-exact checkpoints).
+ *     internal representation unchanged (bit-exact checkpoints). A D2Q9 lattice
+ *     with tau = 1 is kept as the moments its next step reads (rest population,
+ *     sum of the moving ones, flux); the calls that read its populations form
+ *     them from the moments one step back, with the step's own arithmetic.
  */
 #ifndef MLSWLBM_H
 #define MLSWLBM_H
@@ -130,8 +133,8 @@ int mlswlbm_spreading_from_tensions(int n_layers, const double* gamma_full,
 int mlswlbm_check_params(const mlsw_params* p);
 
 /*
- * Creates a solver: validates p, allocates two population buffers of
- * n*Q*nx*ny floats plus small scratch on the current CUDA device, uploads
+ * Creates a solver: validates p, allocates two state buffers and room for the
+ * populations (at most 2*n*Q*nx*ny padded floats in all) plus small scratch on the current CUDA device, uploads
  * h_init (host, [n][ny][nx], every value finite and > 0) and sets
  * f = f_eq(h_init, U = 0) (Eq. equilibrium_distribution), i.e. the rest
  * population carries h and the moving ones are zero.
@@ -363,15 +366,12 @@ int mlswlbm_diagnostics_noalloc(const mlsw_params* p, const float* f, const floa
  * ------------------------------------------------------------------------
  * Batches: many independent D2Q9 lattices (e.g. the instances of a
  * stability or equilibrium sweep: layer counts, sizes and parameters may all
- * differ) advanced together. One step of a batch is one persistent kernel
- * launch over a table of every instance's tiles, in which the instances
- * sharing the layer count, the kernel mode (tau = 1 or not, exponents
- * (3, 2), spreading only between neighbouring interfaces) and the tile
- * height (a group) form a contiguous range; CTAs draw tiles from one
- * counter and pass from range to range without waiting for each other.
- * The launch is captured once in a CUDA graph per buffer parity and
- * replayed. Each instance is stepped with exactly the arithmetic of
- * mlswlbm_step (section LBM, Eq. BGK).
+ * differ) advanced together. One step of a batch is one kernel launch over a
+ * table of every instance's units of work (strips of some rows), in which the
+ * instances sharing the layer count, the kernel mode (tau = 1 or not,
+ * exponents (3, 2), spreading only between neighbouring interfaces) and the
+ * tile height (a group) form a contiguous range. Each instance is stepped
+ * with exactly the arithmetic of mlswlbm_step (section LBM, Eq. BGK).
  * ------------------------------------------------------------------------
  */
 typedef struct mlsw_batch mlsw_batch;
@@ -443,9 +443,8 @@ int mlswlbm_batch_tile_rows(const mlsw_batch* b, int index);
  * out of range, a repeated index, or nsel outside [0, count]. */
 int mlswlbm_batch_select(mlsw_batch* b, int nsel, const int* indices);
 
-/* Kernel launches issued since create (graph replays counted by the
- * kernels they contain: one per step), and groups (ranges of the step's
- * tile table). */
+/* Kernel launches issued since create (one per step), and groups (ranges of
+ * the step's unit table). */
 long mlswlbm_batch_launch_count(const mlsw_batch* b);
 int mlswlbm_batch_groups(const mlsw_batch* b);
 

@@ -17,9 +17,14 @@ CSRC = os.path.join(PKG, "csrc")
 OUT_DIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT_DIR, "libmlswlbm.so")
 DEBUG_LIB = os.path.join(OUT_DIR, "libmlswlbm_debug.so")
-SOURCES = ["mlswlbm.cu", "step_kernels.cu", "batch_kernels.cu", "aux_kernels.cu", "noalloc.cu",
-           "batch.cu", "analysis.cu", "unet.cu"]
-HEADERS = ["physics.cuh", "step_common.cuh", "d2q9_tile.cuh", "kernels.h", "tma.cuh", "tcgen05.cuh", "host.h"]
+# (source, defines): the D2Q9 step is compiled once per layer count, the batch
+# step once per largest layer count, so that their kernels compile in parallel
+UNITS = ([("batch_kernels.cu", ["-DMLSW_BATCH_N=%d" % n]) for n in (5, 3)]
+         + [("step_d2q9.cu", ["-DMLSW_N=%d" % n]) for n in (5, 4, 3, 2, 1)]
+         + [(s, []) for s in ("unet.cu", "step_kernels.cu", "aux_kernels.cu", "mlswlbm.cu",
+                              "noalloc.cu", "batch.cu", "analysis.cu")])
+HEADERS = ["physics.cuh", "step_common.cuh", "march.cuh", "kernels.h", "tma.cuh", "tcgen05.cuh",
+           "host.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 CFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",
@@ -27,7 +32,7 @@ CFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",
 
 
 def _deps():
-    files = [os.path.join(CSRC, f) for f in SOURCES + HEADERS]
+    files = [os.path.join(CSRC, f) for f in sorted({s for s, _ in UNITS}) + HEADERS]
     files.append(os.path.join(ROOT, "include", "mlswlbm.h"))
     files.append(os.path.abspath(__file__))
     return files
@@ -40,9 +45,11 @@ def _stale(lib):
     return any(os.path.getmtime(f) > t for f in _deps())
 
 
-def _compile(src, extra, obj_dir=OUT_DIR):
-    obj = os.path.join(obj_dir, os.path.splitext(src)[0] + ".o")
-    cmd = [NVCC, *ARCH, *CFLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+def _compile(unit, extra, obj_dir=OUT_DIR):
+    src, defines = unit
+    tag = "".join("_" + d.split("=")[1] for d in defines)
+    obj = os.path.join(obj_dir, os.path.splitext(src)[0] + tag + ".o")
+    cmd = [NVCC, *ARCH, *CFLAGS, *defines, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("nvcc failed for %s:\n%s%s" % (src, r.stdout, r.stderr))
@@ -58,8 +65,8 @@ def build(force=False, verbose=False, extra=(), debug=False):
     obj_dir = os.path.join(OUT_DIR, "debug") if debug else OUT_DIR
     os.makedirs(obj_dir, exist_ok=True)
     flags = list(extra) + (["-DMLSW_DEBUG"] if debug else [])
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        results = list(ex.map(lambda s: _compile(s, flags, obj_dir), SOURCES))
+    with cf.ThreadPoolExecutor(max_workers=len(UNITS)) as ex:
+        results = list(ex.map(lambda u: _compile(u, flags, obj_dir), UNITS))
     if verbose:
         for _, err in results:
             if err:

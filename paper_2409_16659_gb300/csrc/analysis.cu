@@ -50,15 +50,15 @@ __device__ void fft_inplace(float2* a, int bits, int count) {
 }
 
 // One CTA per (row y, layer i): the row of h_i - H_i (the sum of the stored
-// populations, whose rest population is shifted by H_i), transformed.
-template <int Q>
+// planes, PL per layer of which the first Q add up to it), transformed.
+template <int Q, int PL>
 __global__ void __launch_bounds__(256)
     spectrum_rows_kernel(Layout L, const float* __restrict__ f, int bits_x,
                          float2* __restrict__ work) {
   extern __shared__ float2 row[];
   const int nx = L.nx, ny = L.ny;
   const int y = blockIdx.x, i = blockIdx.y;
-  const float* src = f + L.at(i * Q, 0, y);
+  const float* src = f + L.at(i * PL, 0, y);
   for (int x = threadIdx.x; x < nx; x += blockDim.x) {
     float d = 0.f;
 #pragma unroll
@@ -137,19 +137,12 @@ cudaError_t launch_spectrum(int Q, int n, const Layout& L, const float* f, int n
   const size_t row_smem = (size_t)nx * sizeof(float2);
   const int rthreads = nx / 2 < 32 ? 32 : (nx / 2 > 256 ? 256 : nx / 2);
   cudaError_t e;
-  if (Q == 9) {
-    e = cudaFuncSetAttribute(spectrum_rows_kernel<9>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)row_smem);
-    if (e != cudaSuccess) return e;
-    spectrum_rows_kernel<9><<<dim3(ny, n), rthreads, row_smem, st>>>(L, f, bx, work);
-  } else if (Q == 3) {
-    e = cudaFuncSetAttribute(spectrum_rows_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)row_smem);
-    if (e != cudaSuccess) return e;
-    spectrum_rows_kernel<3><<<dim3(ny, n), rthreads, row_smem, st>>>(L, f, bx, work);
-  } else {
-    return cudaErrorInvalidValue;
-  }
+  auto rows = Q == 9 ? spectrum_rows_kernel<9, 9>
+                     : (Q == 3 ? spectrum_rows_kernel<3, 3> : spectrum_rows_kernel<2, kMomPlanes>);
+  if (Q != 9 && Q != 3 && Q != kMomPlanes) return cudaErrorInvalidValue;
+  e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem);
+  if (e != cudaSuccess) return e;
+  rows<<<dim3(ny, n), rthreads, row_smem, st>>>(L, f, bx, work);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // columns per CTA: up to 8, at most 8192 complex values in shared memory
@@ -174,7 +167,7 @@ cudaError_t launch_spectrum(int Q, int n, const Layout& L, const float* f, int n
 // in FP64. One thread per cell, FP64 atomics into sums[m][nbins] and
 // counts[nbins].
 // ---------------------------------------------------------------------------
-template <int Q>
+template <int Q, int PL>
 __global__ void __launch_bounds__(256)
     radial_profile_kernel(int n, Layout L, const float* __restrict__ f, KShift sh,
                           ProfileParams A, double* __restrict__ sums,
@@ -200,7 +193,7 @@ __global__ void __launch_bounds__(256)
   }
   atomicAdd(sums + b, z);
   for (int i = 0; i < n; ++i) {
-    const float* src = f + L.at(i * Q, x, y);
+    const float* src = f + L.at(i * PL, x, y);
     float d = 0.f;
 #pragma unroll
     for (int k = 0; k < Q; ++k) d += src[(long)k * L.plane];
@@ -217,9 +210,11 @@ cudaError_t launch_radial_profile(int Q, int n, const Layout& L, const float* f,
   if (A.nbins < 1 || n < 1 || cells < 1) return cudaErrorInvalidValue;
   const unsigned grid = (unsigned)((cells + 255) / 256);
   if (Q == 9)
-    radial_profile_kernel<9><<<grid, 256, 0, st>>>(n, L, f, sh, A, sums, counts);
+    radial_profile_kernel<9, 9><<<grid, 256, 0, st>>>(n, L, f, sh, A, sums, counts);
   else if (Q == 3)
-    radial_profile_kernel<3><<<grid, 256, 0, st>>>(n, L, f, sh, A, sums, counts);
+    radial_profile_kernel<3, 3><<<grid, 256, 0, st>>>(n, L, f, sh, A, sums, counts);
+  else if (Q == kMomPlanes)
+    radial_profile_kernel<2, kMomPlanes><<<grid, 256, 0, st>>>(n, L, f, sh, A, sums, counts);
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();

@@ -6,8 +6,9 @@
 #include <cstdint>
 
 #include "kernels.h"
-#include "tma.cuh"
 #include "physics.cuh"
+#include "step_common.cuh"
+#include "tma.cuh"
 
 namespace mlsw {
 
@@ -76,26 +77,24 @@ struct Row<4> {
 };
 
 // ---------------------------------------------------------------------------
-// f = f_eq(h, U = 0) (Eq. equilibrium_distribution at rest): f_0 = h, else 0.
+// f = f_eq(h, U = 0) (Eq. equilibrium_distribution at rest): f_0 = h, else 0;
+// in moment form (Q = kMomPlanes) the same: g_0 = h - H, the other three 0.
 // One thread owns V cells of a padded row of one layer, reads their heights
 // once and writes all Q planes. The x range [-4, nx + 4) covers the ghost
-// ring and the two alignment columns on each side, and y runs over
-// [-2, ny + 2) when ghosts_y: every ghost takes its periodic image, so no
-// separate ghost pass is needed. R rows are in flight per thread, which
-// matters when h is page-locked host memory read across the host link.
+// columns: every ghost takes its periodic image, so no separate ghost pass
+// is needed. R rows are in flight per thread, which matters when h is
+// page-locked host memory read across the host link.
 // ---------------------------------------------------------------------------
 template <int Q, int V>
 __global__ void __launch_bounds__(kRowThreads)
-    init_kernel(int n, Layout L, int ghosts_y, const float* __restrict__ h,
-                float* __restrict__ f, KShift sh, int* __restrict__ status) {
+    init_kernel(int n, Layout L, const float* __restrict__ h, float* __restrict__ f, KShift sh,
+                int* __restrict__ status) {
   using Rw = Row<V>;
   using T = typename Rw::T;
   constexpr int R = 4;
   const int nx = L.nx, ny = L.ny;
   const int groups = (nx + 8) / V;
-  const int yrows = ghosts_y ? ny + 4 : 1;
-  const int y0 = ghosts_y ? 2 : 0;
-  const long nrows = (long)n * yrows;
+  const long nrows = (long)n * ny;
   const int gi = blockIdx.x * blockDim.x + threadIdx.x;
   if (gi >= groups) return;
   const int x = gi * V - 4;
@@ -107,19 +106,13 @@ __global__ void __launch_bounds__(kRowThreads)
 #pragma unroll
     for (int u = 0; u < R; ++u) {
       const long r = r0 + (long)u * gridDim.y;
-      if (r < nrows) {
-        const int i = (int)(r / yrows);
-        const int y = (int)(r - (long)i * yrows) - y0;
-        const int sy = ghosts_y ? ((y >= 0 && y < ny) ? y : wrap_any(y, ny)) : 0;
-        hv[u] = Rw::load(h + ((long)i * ny + sy) * nx + sx);
-      }
+      if (r < nrows) hv[u] = Rw::load(h + r * nx + sx);
     }
 #pragma unroll
     for (int u = 0; u < R; ++u) {
       const long r = r0 + (long)u * gridDim.y;
       if (r < nrows) {
-        const int i = (int)(r / yrows);
-        const int y = (int)(r - (long)i * yrows) - y0;
+        const int i = (int)(r / ny), y = (int)(r - (long)i * ny);
         bad |= !Rw::ok(hv[u]);
         float* dst = f + L.at(i * Q, x, y);
         Rw::store(dst, Rw::sub(hv[u], sh.H[i]));  // rest population, shifted by H_i
@@ -132,71 +125,100 @@ __global__ void __launch_bounds__(kRowThreads)
 }
 
 template <int Q>
-static void init_q(const dim3& g, int V, int n, const Layout& L, int gy, const float* h,
-                   float* f, const KShift& sh, int* status, cudaStream_t st) {
+static void init_q(const dim3& g, int V, int n, const Layout& L, const float* h, float* f,
+                   const KShift& sh, int* status, cudaStream_t st) {
   if (V == 4)
-    init_kernel<Q, 4><<<g, kRowThreads, 0, st>>>(n, L, gy, h, f, sh, status);
+    init_kernel<Q, 4><<<g, kRowThreads, 0, st>>>(n, L, h, f, sh, status);
   else
-    init_kernel<Q, 1><<<g, kRowThreads, 0, st>>>(n, L, gy, h, f, sh, status);
+    init_kernel<Q, 1><<<g, kRowThreads, 0, st>>>(n, L, h, f, sh, status);
 }
 
-cudaError_t launch_init(int Q, int n, const Layout& L, bool ghosts_y, const float* h, float* f,
-                        const KShift& sh, int* status, cudaStream_t st) {
-  // the written x range [-4, nx + 4) and y range [-2, ny + 2) must lie
-  // inside the padding
-  if (L.gx != 4 || L.pitch < L.nx + 8 || (ghosts_y && (L.gy != 2 || L.rows < L.ny + 4)))
-    return cudaErrorInvalidValue;
+cudaError_t launch_init(int Q, int n, const Layout& L, const float* h, float* f, const KShift& sh,
+                        int* status, cudaStream_t st) {
+  // the written x range [-4, nx + 4) must lie inside the padding
+  if (L.gx < 4 || L.pitch < L.gx + L.nx + 4 || L.rows < L.ny) return cudaErrorInvalidValue;
   const bool vec = L.nx % 4 == 0 && L.nx >= 4 && (reinterpret_cast<uintptr_t>(h) & 15) == 0 &&
                    (reinterpret_cast<uintptr_t>(f) & 15) == 0 && L.pitch % 4 == 0 &&
-                   L.gx == 4 && L.plane % 4 == 0;
+                   L.gx % 4 == 0 && L.plane % 4 == 0;
   const int V = vec ? 4 : 1;
-  const long nrows = (long)n * (ghosts_y ? L.ny + 4 : 1);
-  const dim3 g = row_grid((L.nx + 8) / V, nrows);
-  if (Q == 9)
-    init_q<9>(g, V, n, L, ghosts_y ? 1 : 0, h, f, sh, status, st);
-  else if (Q == 3)
-    init_q<3>(g, V, n, L, ghosts_y ? 1 : 0, h, f, sh, status, st);
-  else
-    return cudaErrorInvalidValue;
+  const dim3 g = row_grid((L.nx + 8) / V, (long)n * L.ny);
+  switch (Q) {
+    case 9: init_q<9>(g, V, n, L, h, f, sh, status, st); break;
+    case 3: init_q<3>(g, V, n, L, h, f, sh, status, st); break;
+    case kMomPlanes: init_q<kMomPlanes>(g, V, n, L, h, f, sh, status, st); break;
+    default: return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// ghost images: rows y in {-2, -1, ny, ny + 1} over x in [-2, nx + 2) and
-// columns x in {-2, -1, nx, nx + 1} over y in [0, ny) (x only: the columns
-// over y = 0)
+// ghost images: columns x in [-4, 0) and [nx, nx + 4)
 // ---------------------------------------------------------------------------
-__global__ void fill_ghosts_kernel(int nplanes, Layout L, int ghosts_y, float* __restrict__ f) {
-  const int nx = L.nx, ny = L.ny;
-  const long rows_part = ghosts_y ? 4L * (nx + 4) : 0;  // four ghost rows
-  const long cols_part = 4L * (ghosts_y ? ny : 1);      // four ghost columns
-  const long per_plane = rows_part + cols_part;
-  const long total = per_plane * nplanes;
+__global__ void fill_ghosts_kernel(int nplanes, Layout L, float* __restrict__ f) {
+  const int nx = L.nx;
+  const long per_plane = 8L * L.ny, total = per_plane * nplanes;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
        t += (long)gridDim.x * blockDim.x) {
     const int p = (int)(t / per_plane);
     const long u = t % per_plane;
-    int x, y;
-    if (u < rows_part) {
-      const int g = (int)(u / (nx + 4));
-      x = (int)(u % (nx + 4)) - 2;
-      y = g == 0 ? -2 : (g == 1 ? -1 : (g == 2 ? ny : ny + 1));
-    } else {
-      const long v = u - rows_part;
-      const int g = (int)(v & 3);
-      y = (int)(v >> 2);
-      x = g == 0 ? -2 : (g == 1 ? -1 : (g == 2 ? nx : nx + 1));
-    }
-    const int sx = wrap_any(x, nx), sy = ghosts_y ? wrap_any(y, ny) : 0;
-    f[L.at(p, x, y)] = f[L.at(p, sx, sy)];
+    const int g = (int)(u & 7), y = (int)(u >> 3);
+    const int x = g < 4 ? g - 4 : nx + g - 4;
+    f[L.at(p, x, y)] = f[L.at(p, wrap_any(x, nx), y)];
   }
 }
 
-cudaError_t launch_fill_ghosts(int nplanes, const Layout& L, bool ghosts_y, float* f,
-                               cudaStream_t st) {
-  const long per_plane = (ghosts_y ? 4L * (L.nx + 4) + 4L * L.ny : 4L);
-  fill_ghosts_kernel<<<grid_for(per_plane * nplanes, 256), 256, 0, st>>>(nplanes, L,
-                                                                         ghosts_y ? 1 : 0, f);
+cudaError_t launch_fill_ghosts(int nplanes, const Layout& L, float* f, cudaStream_t st) {
+  fill_ghosts_kernel<<<grid_for(8L * L.ny * nplanes, 256), 256, 0, st>>>(nplanes, L, f);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// D2Q9 populations to moments (the same arithmetic on the same values as a
+// step that forms them), ghost columns included, and the populations of a
+// state at rest from its moments (real cells).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kRowThreads)
+    moments_kernel(int n, Layout L, const float* __restrict__ f, float* __restrict__ m) {
+  const int nx = L.nx, ny = L.ny;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= nx) return;
+  for (long r = blockIdx.y; r < (long)n * ny; r += gridDim.y) {
+    const int i = (int)(r / ny), y = (int)(r - (long)i * ny);
+    float v[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) v[k] = f[L.at(i * 9 + k, x, y)];
+    const Moments<float> q = moments_of(v);
+    const float out[kMomPlanes] = {q.g0, q.s, q.jx, q.jy};
+#pragma unroll
+    for (int k = 0; k < kMomPlanes; ++k) {
+      m[L.at(i * kMomPlanes + k, x, y)] = out[k];
+      if (x < 4) m[L.at(i * kMomPlanes + k, x + nx, y)] = out[k];
+      if (x >= nx - 4) m[L.at(i * kMomPlanes + k, x - nx, y)] = out[k];
+    }
+  }
+}
+
+cudaError_t launch_moments(int n, const Layout& L, const float* f, float* m, cudaStream_t st) {
+  moments_kernel<<<row_grid(L.nx, (long)n * L.ny), kRowThreads, 0, st>>>(n, L, f, m);
+  return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(kRowThreads)
+    rest_populations_kernel(int n, Layout L, const float* __restrict__ m, float* __restrict__ f) {
+  const int nx = L.nx, ny = L.ny;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= nx) return;
+  for (long r = blockIdx.y; r < (long)n * ny; r += gridDim.y) {
+    const int i = (int)(r / ny), y = (int)(r - (long)i * ny);
+    f[L.at(i * 9, x, y)] = m[L.at(i * kMomPlanes, x, y)];
+#pragma unroll
+    for (int k = 1; k < 9; ++k) f[L.at(i * 9 + k, x, y)] = 0.f;
+  }
+}
+
+cudaError_t launch_rest_populations(int n, const Layout& L, const float* m, float* f,
+                                    cudaStream_t st) {
+  rest_populations_kernel<<<row_grid(L.nx, (long)n * L.ny), kRowThreads, 0, st>>>(n, L, m, f);
   return cudaGetLastError();
 }
 
@@ -204,7 +226,8 @@ cudaError_t launch_fill_ghosts(int nplanes, const Layout& L, bool ghosts_y, floa
 // read-out and representation shifts (real cells only; one row = one layer
 // row y of the lattice)
 // ---------------------------------------------------------------------------
-template <int Q, int V>
+// PL planes per layer, of which the first Q add up to h_i - H_i
+template <int Q, int PL, int V>
 __global__ void __launch_bounds__(kRowThreads)
     heights_kernel(int n, Layout L, const float* __restrict__ f, KShift sh,
                    float* __restrict__ h, const int* __restrict__ st_in,
@@ -218,7 +241,7 @@ __global__ void __launch_bounds__(kRowThreads)
   if (x >= nx) return;
   for (long r = blockIdx.y; r < (long)n * ny; r += gridDim.y) {
     const int i = (int)(r / ny), y = (int)(r - (long)i * ny);
-    const float* src = f + L.at(i * Q, x, y);
+    const float* src = f + L.at(i * PL, x, y);
     T v[Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) v[k] = Rw::load(src + (long)k * L.plane);
@@ -230,14 +253,14 @@ __global__ void __launch_bounds__(kRowThreads)
   }
 }
 
-template <int Q>
+template <int Q, int PL>
 static void heights_q(const dim3& g, int V, int n, const Layout& L, const float* f,
                       const KShift& sh, float* h, const int* st_in, int* st_out,
                       cudaStream_t st) {
   if (V == 4)
-    heights_kernel<Q, 4><<<g, kRowThreads, 0, st>>>(n, L, f, sh, h, st_in, st_out);
+    heights_kernel<Q, PL, 4><<<g, kRowThreads, 0, st>>>(n, L, f, sh, h, st_in, st_out);
   else
-    heights_kernel<Q, 1><<<g, kRowThreads, 0, st>>>(n, L, f, sh, h, st_in, st_out);
+    heights_kernel<Q, PL, 1><<<g, kRowThreads, 0, st>>>(n, L, f, sh, h, st_in, st_out);
 }
 
 cudaError_t launch_heights(int Q, int n, const Layout& L, const float* f, const KShift& sh,
@@ -247,12 +270,14 @@ cudaError_t launch_heights(int Q, int n, const Layout& L, const float* f, const 
                    L.gx % 4 == 0 && L.plane % 4 == 0;
   const int V = vec ? 4 : 1;
   const dim3 g = row_grid(L.nx / V, (long)n * L.ny);
-  if (Q == 9)
-    heights_q<9>(g, V, n, L, f, sh, h, st_in, st_out, st);
-  else if (Q == 3)
-    heights_q<3>(g, V, n, L, f, sh, h, st_in, st_out, st);
-  else
-    return cudaErrorInvalidValue;
+  switch (Q) {
+    case 9: heights_q<9, 9>(g, V, n, L, f, sh, h, st_in, st_out, st); break;
+    case 3: heights_q<3, 3>(g, V, n, L, f, sh, h, st_in, st_out, st); break;
+    case kMomPlanes:
+      heights_q<2, kMomPlanes>(g, V, n, L, f, sh, h, st_in, st_out, st);
+      break;
+    default: return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 
@@ -313,8 +338,9 @@ template <int LAT>
 __global__ void __launch_bounds__(kDiagThreads)
     diag_partial_kernel(int n, Layout L, const float* __restrict__ f, KShift sh,
                         double* __restrict__ partials) {
-  using Lt = Lattice<LAT>;
-  constexpr int Q = Lt::Q;
+  // LAT 0: a D2Q9 state in moment form
+  using Lt = Lattice<(LAT == 0 ? 2 : LAT)>;
+  constexpr int Q = LAT == 0 ? kMomPlanes : Lt::Q;
   __shared__ double red[kDiagThreads / 32][kMaxLayers + 2];
   const long ncell = (long)L.nx * L.ny;
   double mass[kMaxLayers];
@@ -325,12 +351,18 @@ __global__ void __launch_bounds__(kDiagThreads)
     const int x = (int)(c % L.nx), y = (int)(c / L.nx);
     for (int i = 0; i < n; ++i) {
       float dh = 0.f, jx = 0.f, jy = 0.f;
+      if constexpr (LAT == 0) {
+        dh = f[L.at(i * Q, x, y)] + f[L.at(i * Q + 1, x, y)];
+        jx = f[L.at(i * Q + 2, x, y)];
+        jy = f[L.at(i * Q + 3, x, y)];
+      } else {
 #pragma unroll
-      for (int k = 0; k < Q; ++k) {
-        const float v = f[L.at(i * Q + k, x, y)];
-        dh += v;
-        jx += (float)Lt::cx(k) * v;
-        jy += (float)Lt::cy(k) * v;
+        for (int k = 0; k < Q; ++k) {
+          const float v = f[L.at(i * Q + k, x, y)];
+          dh += v;
+          jx += (float)Lt::cx(k) * v;
+          jy += (float)Lt::cy(k) * v;
+        }
       }
       const double h = (double)sh.H[i] + (double)dh;
       mass[i] += h;
@@ -374,11 +406,13 @@ __global__ void diag_final_kernel(int n, int nblk, const double* __restrict__ pa
   out[q] = acc;
 }
 
-cudaError_t launch_diagnostics(int lattice, int n, const Layout& L, const float* f,
+cudaError_t launch_diagnostics(int Q, int n, const Layout& L, const float* f,
                                const KShift& sh, double* partials, int nblk, double* out,
                                cudaStream_t st) {
-  if (lattice == 2)
+  if (Q == 9)
     diag_partial_kernel<2><<<nblk, kDiagThreads, 0, st>>>(n, L, f, sh, partials);
+  else if (Q == kMomPlanes)
+    diag_partial_kernel<0><<<nblk, kDiagThreads, 0, st>>>(n, L, f, sh, partials);
   else
     diag_partial_kernel<1><<<nblk, kDiagThreads, 0, st>>>(n, L, f, sh, partials);
   cudaError_t e = cudaGetLastError();
@@ -453,6 +487,7 @@ __global__ void __launch_bounds__(kModeThreads)
     return;
   }
   const Layout& L = P.L;
+  const bool moments = b.kind % 3 != kGeneral;
   const float* __restrict__ f = b.f[cur];
   const int nx = P.nx, ny = P.ny;
   const long ncell = (long)nx * ny;
@@ -460,10 +495,16 @@ __global__ void __launch_bounds__(kModeThreads)
   double re = 0.0, im = 0.0;
   for (long c = threadIdx.x; c < ncell; c += kModeThreads) {
     const int y = (int)(c / nx), x = (int)(c - (long)y * nx);
-    const float* src = f + L.at(i * 9, x, y);
-    float d = 0.f;
+    float d;
+    if (moments) {
+      const float* src = f + L.at(i * kMomPlanes, x, y);
+      d = src[0] + src[L.plane];
+    } else {
+      const float* src = f + L.at(i * 9, x, y);
+      d = 0.f;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) d += src[(long)k * L.plane];
+      for (int k = 0; k < 9; ++k) d += src[(long)k * L.plane];
+    }
     const double h = (double)(P.H[i] + d);
     // phase / (2 pi) = m / (nx ny), m exact
     const long m = ((qx * x) % nx * ny + (qy * y) % ny * nx) % ncell;
@@ -503,7 +544,7 @@ cudaError_t launch_batch_modes(const BatchInst* inst, int count, int cur, const 
 
 // heights of one instance of a batch (layout of its buffers)
 cudaError_t launch_batch_heights(const BatchInst* inst_host, int cur, float* h, cudaStream_t st) {
-  return launch_heights(9, inst_host->P.n, inst_host->P.L, inst_host->f[cur],
+  return launch_heights(step_moments(inst_host->P) ? kMomPlanes : 9, inst_host->P.n, inst_host->P.L, inst_host->f[cur],
                         KShift{{inst_host->P.H[0], inst_host->P.H[1], inst_host->P.H[2],
                                 inst_host->P.H[3], inst_host->P.H[4]}},
                         h, st);

@@ -1,10 +1,9 @@
 // batch.cu -- batches of independent D2Q9 lattices (the C ABI's
 // mlswlbm_batch_*): one population arena, per-instance device descriptors,
-// one tile table in which the instances that share layer count, kernel mode
-// and tile height (a group) have a contiguous range, one persistent launch
-// per step over the whole table (batch_kernels.cu), captured once in a CUDA
-// graph, and a timing autotuner for the tile height of every class of
-// alike instances.
+// one unit table in which the instances that share layer count, kernel mode
+// and tile height (a group) have a contiguous range, one launch per step
+// over the whole table (batch_kernels.cu), and a timing autotuner for the
+// tile height of every class of alike instances.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -23,11 +22,10 @@ using mlsw::KParams;
 namespace {
 
 constexpr int kQ = 9;
-constexpr int kMaxGroups = mlsw::kBatchKinds;  // n x mode x variant
 
 struct Group {
   int n, mode, variant;
-  int offset, ntiles;  // slice of the tile table
+  int offset, nunits;  // slice of the unit table
 };
 
 }  // namespace
@@ -42,16 +40,17 @@ struct mlsw_batch {
   std::vector<int> home;
   std::vector<Group> groups;
   BatchInst* dinst;
-  int2* dtable;  // the tile table, sorted by kind
+  int2* dtable;  // the unit table, sorted by kind
+  int nunits, nmax;    // its length, the largest layer count in it
+  unsigned kinds;      // kinds in it
+  std::vector<int> tiny;  // selected instances whose ghosts need a pass of their own
   float* arena;
-  int* dstatus;  // [0] error bits, [1], [2] the step kernel's tile counters
+  int* dstatus;  // error bits
   float* hbuf;   // heights of the largest instance (upload, read-out)
   int* dk;       // 2 count mode numbers
   double* dmode; // 2 kMaxLayers count doubles
   int cur;
   cudaStream_t stream;   // the caller's stream
-  cudaStream_t cap;      // private stream the step graph is captured on
-  cudaGraphExec_t gexec[2];  // one step from buffer 0, from buffer 1
   long launches;
   int num_sms;
 };
@@ -63,9 +62,18 @@ namespace {
     if ((call) != cudaSuccess) return MLSW_ERR_CUDA; \
   } while (0)
 
-int tiles_of(const BatchInst& b, int variant) {
-  const int ty = mlsw::batch_tile_rows(variant);
-  return b.ntx * ((b.P.ny + ty - 1) / ty);
+// planes per layer of an instance's buffers
+int planes_of(const KParams& P) { return mlsw::step_moments(P) ? mlsw::kMomPlanes : kQ; }
+
+int units_of(const BatchInst& b, int rows) { return b.strips * ((b.P.ny + rows - 1) / rows); }
+
+// Tiles a unit spans: as many (up to 8) as leave three waves of the resident
+// warps. A unit costs its rows plus about five rows of warm-up, and the
+// waves even out the instances' different costs.
+int span_for(long units_one_tile, int warps) {
+  int span = 8;
+  while (span > 1 && units_one_tile / span < 3L * warps) span /= 2;
+  return span;
 }
 
 // the buffer that holds instance j's state now
@@ -80,7 +88,7 @@ int align_buffers(mlsw_batch* b) {
     if (b->selected[j] || b->home[j] == b->cur) continue;
     BatchInst& bi = b->hinst[j];
     std::swap(bi.f[0], bi.f[1]);
-    for (int v = 0; v < mlsw::kBatchVariants; ++v) std::swap(bi.map[v][0], bi.map[v][1]);
+    std::swap(bi.map[0], bi.map[1]);
     b->home[j] = b->cur;
     changed = true;
   }
@@ -99,7 +107,7 @@ int init_all(mlsw_batch* b, const float* const* h_init) {
     mlsw::KShift sh;
     for (int i = 0; i < mlsw::kMaxLayers; ++i) sh.H[i] = P.H[i];
     CUB(cudaMemcpyAsync(b->hbuf, h_init[j], bytes, cudaMemcpyHostToDevice, b->stream));
-    CUB(mlsw::launch_init(kQ, P.n, P.L, true, b->hbuf, b->hinst[j].f[0], sh, b->dstatus,
+    CUB(mlsw::launch_init(planes_of(P), P.n, P.L, b->hbuf, b->hinst[j].f[0], sh, b->dstatus,
                           b->stream));
     b->launches += 1;
     b->home[j] = 0;
@@ -108,91 +116,63 @@ int init_all(mlsw_batch* b, const float* const* h_init) {
   return MLSW_OK;
 }
 
-// ends of the groups' ranges of the tile table, per kind (the groups come
-// in kind order: the map below orders them by (n, mode, variant))
-mlsw::BatchEnds ends_of(const mlsw_batch* b) {
-  mlsw::BatchEnds E;
-  int g = 0, end = 0;
-  for (int k = 0; k < mlsw::kBatchKinds; ++k) {
-    if (g < (int)b->groups.size()) {
-      const Group& G = b->groups[g];
-      if (mlsw::batch_kind(G.n, G.mode, G.variant) == k) {
-        end = G.offset + G.ntiles;
-        ++g;
-      }
-    }
-    E.end[k] = end;
-  }
-  return E;
-}
-
-// the tile table of the groups for the current variant choice, sorted by
-// kind
+// the unit table of the groups for the current variant choice, sorted by
+// kind (layer count descending: the dearest units first, so that the last
+// ones to run are short), and the unit rows in the descriptors
 int build_groups(mlsw_batch* b) {
   std::map<std::tuple<int, int, int>, std::vector<int>> members;
+  long tiles = 0;
+  b->nmax = 0;
+  b->kinds = 0;
+  b->tiny.clear();
   for (int j = 0; j < b->count; ++j) {
     if (!b->selected[j]) continue;
-    const KParams& P = b->hinst[j].P;
-    members[std::make_tuple(P.n, mlsw::step_mode(P), b->variant[j])].push_back(j);
+    const BatchInst& bi = b->hinst[j];
+    members[std::make_tuple(-bi.P.n, mlsw::step_mode(bi.P), b->variant[j])].push_back(j);
+    tiles += units_of(bi, mlsw::batch_tile_rows(b->variant[j]));
+    b->nmax = std::max(b->nmax, bi.P.n);
+    b->kinds |= 1u << bi.kind;
+    if (bi.P.tiny) b->tiny.push_back(j);
   }
+  const int span = span_for(tiles, b->num_sms * mlsw::batch_warps_per_sm(b->nmax));
   std::vector<int2> table;
   b->groups.clear();
   for (auto& kv : members) {
     Group g;
-    g.n = std::get<0>(kv.first);
+    g.n = -std::get<0>(kv.first);
     g.mode = std::get<1>(kv.first);
     g.variant = std::get<2>(kv.first);
     g.offset = (int)table.size();
     for (int j : kv.second) {
-      const int nt = tiles_of(b->hinst[j], g.variant);
-      for (int t = 0; t < nt; ++t) table.push_back(make_int2(j, t));
+      b->hinst[j].rows = mlsw::batch_tile_rows(g.variant) * span;
+      const int nu = units_of(b->hinst[j], b->hinst[j].rows);
+      for (int t = 0; t < nu; ++t) table.push_back(make_int2(j, t));
     }
-    g.ntiles = (int)table.size() - g.offset;
+    g.nunits = (int)table.size() - g.offset;
     b->groups.push_back(g);
   }
-  if (b->groups.size() > (size_t)kMaxGroups) return MLSW_ERR_UNSUPPORTED;
-  // the ranges must cover the table in kind order
-  if (ends_of(b).end[mlsw::kBatchKinds - 1] != (int)table.size()) return MLSW_ERR_UNSUPPORTED;
+  b->nunits = (int)table.size();
   if (b->dtable) cudaFree(b->dtable);
   b->dtable = nullptr;
   if (cudaMalloc(&b->dtable, std::max<size_t>(1, table.size()) * sizeof(int2)) != cudaSuccess)
     return MLSW_ERR_NOMEM;
   CUB(cudaMemcpy(b->dtable, table.data(), table.size() * sizeof(int2), cudaMemcpyHostToDevice));
+  CUB(cudaMemcpy(b->dinst, b->hinst.data(), (size_t)b->count * sizeof(BatchInst),
+                 cudaMemcpyHostToDevice));
   return MLSW_OK;
 }
 
-// the step launch over the groups' table, from buffer cur
-mlsw::BatchLaunch step_launch(const mlsw_batch* b, int cur) {
+// the launch of a step over the groups' table, from buffer cur
+mlsw::BatchLaunch step_launch(const mlsw_batch* b) {
   mlsw::BatchLaunch a;
   a.inst = b->dinst;
   a.table = b->dtable;
-  a.ends = ends_of(b);
-  a.cur = cur;
+  a.nunits = b->nunits;
+  a.nmax = b->nmax;
+  a.kinds = b->kinds;
+  a.cur = b->cur;
   a.status = b->dstatus;
-  a.sched = b->dstatus + 1;
-  a.num_sms = b->num_sms;
   return a;
-}
-
-// Captures one step (from buffer cur) as a graph of its one launch.
-int capture_step(mlsw_batch* b, int cur, cudaGraphExec_t* exec) {
-  // configure the kernel (shared-memory limit) outside capture
-  mlsw::BatchLaunch a = step_launch(b, cur);
-  mlsw::BatchLaunch none = a;
-  for (int k = 0; k < mlsw::kBatchKinds; ++k) none.ends.end[k] = 0;
-  CUB(mlsw::launch_batch_step(none, b->cap));
-  CUB(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-  const bool ok = mlsw::launch_batch_step(a, b->cap) == cudaSuccess;
-  cudaGraph_t graph = nullptr;
-  const cudaError_t e = cudaStreamEndCapture(b->cap, &graph);
-  if (!ok || e != cudaSuccess || !graph) {
-    if (graph) cudaGraphDestroy(graph);
-    cudaGetLastError();
-    return MLSW_ERR_CUDA;
-  }
-  const cudaError_t ei = cudaGraphInstantiate(exec, graph, 0);
-  cudaGraphDestroy(graph);
-  return ei == cudaSuccess ? MLSW_OK : MLSW_ERR_CUDA;
 }
 
 // Timing autotuner: for every class of instances with the same n (<= 3),
@@ -219,25 +199,28 @@ int autotune(mlsw_batch* b) {
     int best_v = 0;
     for (int v = 0; v < mlsw::kBatchVariants && rc == MLSW_OK; ++v) {
       std::vector<int2> table;
+      long tiles = 0;
+      for (int j : kv.second) tiles += units_of(b->hinst[j], mlsw::batch_tile_rows(v));
+      const int span = span_for(tiles, b->num_sms * mlsw::batch_warps_per_sm(n));
+      for (int j : kv.second) b->hinst[j].rows = mlsw::batch_tile_rows(v) * span;
       for (int j : kv.second)
-        for (int t = 0; t < tiles_of(b->hinst[j], v); ++t) table.push_back(make_int2(j, t));
+        for (int t = 0; t < units_of(b->hinst[j], b->hinst[j].rows); ++t)
+          table.push_back(make_int2(j, t));
       if (dt) cudaFree(dt);
       dt = nullptr;
       if (cudaMalloc(&dt, table.size() * sizeof(int2)) != cudaSuccess ||
           cudaMemcpy(dt, table.data(), table.size() * sizeof(int2), cudaMemcpyHostToDevice) !=
-              cudaSuccess) {
+              cudaSuccess ||
+          cudaMemcpy(b->dinst, b->hinst.data(), (size_t)b->count * sizeof(BatchInst),
+                     cudaMemcpyHostToDevice) != cudaSuccess) {
         rc = MLSW_ERR_CUDA;
         break;
       }
-      mlsw::BatchLaunch a;
-      a.inst = b->dinst;
+      mlsw::BatchLaunch a = step_launch(b);
       a.table = dt;
-      // one range: kinds before this one end at 0, the others at the end
-      const int kind = mlsw::batch_kind(n, mode, v);
-      for (int k = 0; k < mlsw::kBatchKinds; ++k) a.ends.end[k] = k < kind ? 0 : (int)table.size();
-      a.status = b->dstatus;
-      a.sched = b->dstatus + 1;
-      a.num_sms = b->num_sms;
+      a.nunits = (int)table.size();
+      a.nmax = n;
+      a.kinds = 1u << mlsw::batch_kind(n, mode);
       constexpr int kWarm = 2, kTimed = 6;
       float ms = 0.f;
       for (int s = 0; s < kWarm + kTimed && rc == MLSW_OK; ++s) {
@@ -270,11 +253,7 @@ extern "C" {
 
 void mlswlbm_batch_destroy(mlsw_batch* b) {
   if (!b) return;
-  if (b->cap) cudaStreamSynchronize(b->cap);
   cudaStreamSynchronize(b->stream);
-  for (int k = 0; k < 2; ++k)
-    if (b->gexec[k]) cudaGraphExecDestroy(b->gexec[k]);
-  if (b->cap) cudaStreamDestroy(b->cap);
   cudaFree(b->dinst);
   cudaFree(b->dtable);
   cudaFree(b->arena);
@@ -316,8 +295,9 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
     mlsw::KShift sh;
     rc = mlsw_host::prepare_instance(params[j], h_init[j], bi.P, sh);
     if (rc != MLSW_OK) break;
-    bi.ntx = (bi.P.nx + 31) / 32;
-    const size_t flen = (size_t)bi.P.n * kQ * bi.P.L.plane;
+    bi.kind = mlsw::batch_kind(bi.P.n, mlsw::step_mode(bi.P));
+    bi.strips = mlsw::march_strips(bi.P.nx);
+    const size_t flen = (size_t)bi.P.n * planes_of(bi.P) * bi.P.L.plane;
     off[j] = arena_floats;
     arena_floats += 2 * ((flen + 63) / 64 * 64);  // two buffers, 256-byte aligned
     max_heights = std::max(max_heights, (size_t)bi.P.n * bi.P.nx * bi.P.ny);
@@ -334,10 +314,9 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
     return MLSW_ERR_CUDA;
   }
   b->num_sms = sms > 0 ? sms : 1;
-  const int nstat = 3;
   bool ok = cudaMalloc(&b->arena, arena_floats * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&b->dinst, (size_t)count * sizeof(BatchInst)) == cudaSuccess &&
-            cudaMalloc(&b->dstatus, nstat * sizeof(int)) == cudaSuccess &&
+            cudaMalloc(&b->dstatus, sizeof(int)) == cudaSuccess &&
             cudaMalloc(&b->hbuf, max_heights * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&b->dk, 2 * (size_t)count * sizeof(int)) == cudaSuccess &&
             cudaMalloc(&b->dmode, 2 * (size_t)mlsw::kMaxLayers * count * sizeof(double)) ==
@@ -347,22 +326,17 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
     mlswlbm_batch_destroy(b);
     return MLSW_ERR_NOMEM;
   }
-  ok = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) == cudaSuccess;
-  // zero padding (cells outside the real domains and their ghost rings are
-  // read by edge tiles but feed no real cell) and the status words
-  ok = ok && cudaMemsetAsync(b->dstatus, 0, nstat * sizeof(int), b->stream) == cudaSuccess &&
+  // zero padding (columns outside the real domains and their ghosts are
+  // read by edge strips but feed no real cell) and the status word
+  ok = cudaMemsetAsync(b->dstatus, 0, sizeof(int), b->stream) == cudaSuccess &&
        cudaMemsetAsync(b->arena, 0, arena_floats * sizeof(float), b->stream) == cudaSuccess;
   for (int j = 0; j < count && ok; ++j) {
     BatchInst& bi = b->hinst[j];
-    const size_t flen = (size_t)bi.P.n * kQ * bi.P.L.plane;
+    const size_t flen = (size_t)bi.P.n * planes_of(bi.P) * bi.P.L.plane;
     bi.f[0] = b->arena + off[j];
     bi.f[1] = b->arena + off[j] + (flen + 63) / 64 * 64;
-    for (int v = 0; v < mlsw::kBatchVariants && ok; ++v) {
-      if (v == 0 && bi.P.n > 3) continue;  // 16-row tiles need n <= 3
-      for (int k = 0; k < 2 && ok; ++k)
-        ok = mlsw_host::make_tile_map(&bi.map[v][k], bi.f[k], bi.P.L, bi.P.n * kQ, 40,
-                                      mlsw::batch_tile_rows(v) + 4);
-    }
+    for (int k = 0; k < 2 && ok; ++k)
+      ok = mlsw_host::make_row_map(&bi.map[k], bi.f[k], bi.P.L, bi.P.n * planes_of(bi.P));
   }
   ok = ok && cudaMemcpy(b->dinst, b->hinst.data(), (size_t)count * sizeof(BatchInst),
                         cudaMemcpyHostToDevice) == cudaSuccess;
@@ -378,8 +352,6 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
   }
   if (rc == MLSW_OK) rc = build_groups(b);
   if (rc == MLSW_OK && cudaStreamSynchronize(b->stream) != cudaSuccess) rc = MLSW_ERR_CUDA;
-  if (rc == MLSW_OK) rc = capture_step(b, 0, &b->gexec[0]);
-  if (rc == MLSW_OK) rc = capture_step(b, 1, &b->gexec[1]);
   if (rc == MLSW_OK) {
     // a non-finite or non-positive height in h_init was flagged by init
     int flag = 0;
@@ -400,9 +372,14 @@ int mlswlbm_batch_step(mlsw_batch* b, long nsteps) {
   if (!b || nsteps < 0) return MLSW_ERR_ARG;
   if (b->groups.empty()) return MLSW_OK;  // no instance selected
   for (long s = 0; s < nsteps; ++s) {
-    CUB(cudaGraphLaunch(b->gexec[b->cur], b->stream));
+    CUB(mlsw::launch_batch_step(step_launch(b), b->stream));
     b->launches += 1;
     b->cur ^= 1;
+    for (int j : b->tiny) {
+      const BatchInst& bi = b->hinst[j];
+      CUB(mlsw::launch_fill_ghosts(bi.P.n * kQ, bi.P.L, bi.f[b->cur], b->stream));
+      b->launches += 1;
+    }
   }
   return MLSW_OK;
 }
@@ -441,7 +418,7 @@ int mlswlbm_batch_set_heights_device(mlsw_batch* b, int index, const float* dev_
   const KParams& P = b->hinst[index].P;
   mlsw::KShift sh;
   for (int i = 0; i < mlsw::kMaxLayers; ++i) sh.H[i] = P.H[i];
-  CUB(mlsw::launch_init(kQ, P.n, P.L, true, dev_in, b->hinst[index].f[state_buffer(b, index)],
+  CUB(mlsw::launch_init(planes_of(P), P.n, P.L, dev_in, b->hinst[index].f[state_buffer(b, index)],
                         sh, b->dstatus, b->stream));
   b->launches += 1;
   return MLSW_OK;
@@ -474,7 +451,7 @@ int mlswlbm_batch_set_heights_device_many(mlsw_batch* b, int count, const int* i
     const KParams& P = b->hinst[j].P;
     mlsw::KShift sh;
     for (int i = 0; i < mlsw::kMaxLayers; ++i) sh.H[i] = P.H[i];
-    CUB(mlsw::launch_init(kQ, P.n, P.L, true, dev_in + off, b->hinst[j].f[state_buffer(b, j)],
+    CUB(mlsw::launch_init(planes_of(P), P.n, P.L, dev_in + off, b->hinst[j].f[state_buffer(b, j)],
                           sh, b->dstatus, b->stream));
     b->launches += 1;
     off += (size_t)P.n * P.nx * P.ny;
@@ -513,17 +490,9 @@ int mlswlbm_batch_select(mlsw_batch* b, int nsel, const int* indices) {
     b->selected[j] = want[j];
     b->home[j] = b->cur;
   }
-  // the step graphs read the tile table being replaced
+  // steps in flight read the unit table being replaced
   CUB(cudaStreamSynchronize(b->stream));
-  for (int k = 0; k < 2; ++k)
-    if (b->gexec[k]) {
-      cudaGraphExecDestroy(b->gexec[k]);
-      b->gexec[k] = nullptr;
-    }
-  rc = build_groups(b);
-  if (rc == MLSW_OK && !b->groups.empty()) rc = capture_step(b, 0, &b->gexec[0]);
-  if (rc == MLSW_OK && !b->groups.empty()) rc = capture_step(b, 1, &b->gexec[1]);
-  return rc;
+  return build_groups(b);
 }
 
 int mlswlbm_batch_tile_rows(const mlsw_batch* b, int index) {

@@ -1,132 +1,113 @@
 // batch_kernels.cu -- one D2Q9 step of every instance of a batch in one
-// persistent launch.
+// launch. This file is compiled once per MLSW_BATCH_N, the largest layer
+// count its kernel holds.
 //
-// The tile table lists (instance, tile) pairs sorted by kind (layer count,
-// kernel mode, tile height), so the tiles of each kind form one range. A CTA
-// starts on tile blockIdx.x and draws later tiles from one counter shared by
-// the whole table, so the tiles it takes increase and it passes through the
-// ranges in order: it runs the tile loop of each range it has tiles in
-// (section LBM, the same loop as the single-lattice step, d2q9_tile.cuh)
-// and hands the first tile it drew beyond a range to the next one. No CTA
-// waits for another between ranges, so the ranges of a step overlap as the
-// tiles of one range do.
-// The dynamic shared memory of a launch is the largest of its ranges' tile
-// loops, which each fit two CTAs per SM.
+// The unit table lists (instance, unit) pairs sorted by kind (layer count,
+// kernel mode); a CTA is one warp that marches down one unit (section LBM,
+// the same code as the single-lattice step, march.cuh). Neighbouring CTAs
+// run the same kind, so the warps of an SM share its instructions.
 #include <algorithm>
 
-#include "d2q9_tile.cuh"
+#include "march.cuh"
+
+#ifndef MLSW_BATCH_N
+#error "MLSW_BATCH_N: the largest layer count of the kernel"
+#endif
 
 namespace mlsw {
 
 namespace {
 
-// The tiles of kind K, when this CTA's tile t is among them (t < 0: a
-// bounded wait ran out, nothing more runs), then those of the next kinds.
-// The kinds' tile loops follow one another in straight-line code: inlined
-// in a loop over the ranges instead, they spill registers, and compiled as
-// separate functions they lose the uniform registers and constant operands
-// of a kernel's parameters (both measured slower than kernels of their own).
+constexpr size_t kParBytes = (sizeof(KParams) + 127) / 128 * 128;
+static_assert(sizeof(KParams) % 4 == 0, "parameters are copied as words");
+
+// Warps per SM, as for the single lattice (step_d2q9.cu).
+constexpr int kWarps = MLSW_BATCH_N <= 3 ? 12 : 8;
+
+// The unit, if its kind is K, else the next kinds. Straight-line code: as
+// separate functions the kinds would lose the registers that carry rows.
 template <int K>
-__device__ __forceinline__ void run_kinds(const BatchInst* __restrict__ inst,
-                                          const int2* __restrict__ table, const BatchEnds& E,
-                                          int cur, int* __restrict__ status,
-                                          int* __restrict__ sched, int& t) {
-  constexpr int V = K % kBatchVariants, M = (K / kBatchVariants) % 3;
-  constexpr int N = K / (3 * kBatchVariants) + 1;
-  if constexpr (V == 1 || N <= 3) {
-    if (t >= 0 && t < E.end[K]) {
-      const BatchTiles tiles{inst, table, cur, E.end[K], V};
-      t = d2q9_tile_loop<N, M, V == 0 ? 2 : 1>(tiles, status, sched, t);
-    }
+__device__ __forceinline__ void run_kind(int kind, const KParams& P, const BatchInst& b, int cur,
+                                         int x0, int ya, int yb, unsigned char* sm,
+                                         int* __restrict__ status) {
+  constexpr int N = K / 3 + 1, M = K % 3;
+  if (kind == K) {
+    float* fout = b.f[cur ^ 1];
+    __builtin_assume(__isGlobal(fout));
+    march_unit<N, M, M == kGeneral>(P, &b.map[cur], fout, x0, ya, yb, sm, status);
+  } else if constexpr (K + 1 < 3 * MLSW_BATCH_N) {
+    run_kind<K + 1>(kind, P, b, cur, x0, ya, yb, sm, status);
   }
-  if constexpr (K + 1 < kBatchKinds) run_kinds<K + 1>(inst, table, E, cur, status, sched, t);
+}
+
+// dynamic shared memory of a launch over the given kinds
+template <int K>
+size_t smem_from(unsigned kinds) {
+  constexpr int N = K / 3 + 1, M = K % 3;
+  size_t s = (kinds >> K) & 1u ? MarchShape<N, M, M == kGeneral>::kSmem : 0;
+  if constexpr (K + 1 < 3 * MLSW_BATCH_N) s = std::max(s, smem_from<K + 1>(kinds));
+  return s;
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(256, 2)
-    step_d2q9_batch(const BatchInst* __restrict__ inst, const int2* __restrict__ table,
-                    const __grid_constant__ BatchEnds E, int cur, int* __restrict__ status,
-                    int* __restrict__ sched) {
-  int t = blockIdx.x;
-  run_kinds<0>(inst, table, E, cur, status, sched, t);
-  tile_loop_finish(sched);
+// The instance's parameters are read from a copy in shared memory: in global
+// memory every use after a store would load them again.
+template <int NMAX>
+__global__ void __launch_bounds__(32, kWarps)
+    step_d2q9_batch(const BatchInst* __restrict__ inst, const int2* __restrict__ table, int cur,
+                    int* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int2 e = table[blockIdx.x];
+  const BatchInst& b = inst[e.x];
+  int* dst = reinterpret_cast<int*>(smem_raw);
+  const int* src = reinterpret_cast<const int*>(&b.P);
+  for (int w = threadIdx.x; w < (int)(sizeof(KParams) / 4); w += 32) *chk_smem(dst + w) = src[w];
+  __syncwarp();
+  const KParams& P = *reinterpret_cast<const KParams*>(smem_raw);
+  const int strip = e.y % b.strips, ya = e.y / b.strips * b.rows;
+  run_kind<0>(b.kind, P, b, cur, strip * kMarchOut, ya, min(ya + b.rows, P.ny),
+                      smem_raw + kParBytes, status);
 }
 
-bool batch_kind_valid(int n, int mode, int variant) {
-  return n >= 1 && n <= kMaxLayers && mode >= kGeneral && mode <= kFast && variant >= 0 &&
-         variant < kBatchVariants && (variant == 1 || n <= 3);
-}
-
-size_t batch_kind_smem(int n, int variant) {
-  if (variant == 0) {
-    switch (n) {
-      case 1: return D2Tile<1, 2>::kSmem;
-      case 2: return D2Tile<2, 2>::kSmem;
-      default: return D2Tile<3, 2>::kSmem;
-    }
-  }
-  switch (n) {
-    case 1: return D2Tile<1, 1>::kSmem;
-    case 2: return D2Tile<2, 1>::kSmem;
-    case 3: return D2Tile<3, 1>::kSmem;
-    case 4: return D2Tile<4, 1>::kSmem;
-    default: return D2Tile<5, 1>::kSmem;
-  }
-}
-
-cudaError_t launch_batch_step(const BatchLaunch& a, cudaStream_t st) {
-  // once per device: the kernel's shared-memory limit (the largest tile
-  // loop any range can need) and its CTAs per SM at each range kind's
-  // shared memory, so that a launch being captured calls no other API
+template <>
+cudaError_t launch_batch_step_n<MLSW_BATCH_N>(const BatchLaunch& a, cudaStream_t st) {
+  if (a.nunits <= 0) return cudaSuccess;
+  auto kern = step_d2q9_batch<MLSW_BATCH_N>;
+  // once per device: the largest shared memory any kind can need
   static unsigned long long configured = 0;
-  static int per_sm[64][kMaxLayers][kBatchVariants];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 64) return cudaErrorInvalidDevice;
   if (!((configured >> dev) & 1ull)) {
-    size_t most = 0;
-    for (int n = 1; n <= kMaxLayers; ++n)
-      for (int v = 0; v < kBatchVariants; ++v)
-        if (batch_kind_valid(n, kGeneral, v)) most = std::max(most, batch_kind_smem(n, v));
-    e = cudaFuncSetAttribute(step_d2q9_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)most);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kParBytes + smem_from<0>(~0u)));
     if (e != cudaSuccess) return e;
-    for (int n = 1; n <= kMaxLayers; ++n)
-      for (int v = 0; v < kBatchVariants; ++v) {
-        int nb = 0;
-        if (batch_kind_valid(n, kGeneral, v)) {
-          e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, step_d2q9_batch, 256,
-                                                            batch_kind_smem(n, v));
-          if (e != cudaSuccess) return e;
-        }
-        per_sm[dev][n - 1][v] = nb > 0 ? nb : 1;
-      }
     configured |= 1ull << dev;
   }
-  // the largest shared memory of the kinds present sets the launch's CTAs
-  // per SM
-  const BatchEnds& E = a.ends;
-  size_t smem = 0;
-  int blocks = 1 << 30, prev = 0;
-  for (int k = 0; k < kBatchKinds; ++k) {
-    if (E.end[k] < prev) return cudaErrorInvalidValue;
-    if (E.end[k] == prev) continue;  // no tiles of kind k
-    const int v = k % kBatchVariants, m = (k / kBatchVariants) % 3, n = k / (3 * kBatchVariants) + 1;
-    if (!batch_kind_valid(n, m, v)) return cudaErrorInvalidValue;
-    prev = E.end[k];
-    smem = std::max(smem, batch_kind_smem(n, v));
-    blocks = std::min(blocks, per_sm[dev][n - 1][v]);
-  }
-  const int ntiles = prev;
-  if (ntiles <= 0) return cudaSuccess;
-  const int slots = a.num_sms * blocks;
-  const int grid = ntiles < slots ? ntiles : slots;
-  step_d2q9_batch<<<grid, 256, smem, st>>>(a.inst, a.table, E, a.cur, a.status, a.sched);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)a.nunits);
+  cfg.blockDim = dim3(32);
+  cfg.dynamicSmemBytes = kParBytes + smem_from<0>(a.kinds);
+  cfg.stream = st;
+  // a programmatic dependent of the previous kernel (see march_unit)
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a.inst, a.table, a.cur, a.status);
 }
 
-MLSW_DEFINE_BOUNDS_READER(bounds_violations_batch)
+#if MLSW_BATCH_N == 5
+cudaError_t launch_batch_step(const BatchLaunch& a, cudaStream_t st) {
+  return a.nmax <= 3 ? launch_batch_step_n<3>(a, st) : launch_batch_step_n<5>(a, st);
+}
+
+int batch_warps_per_sm(int nmax) { return nmax <= 3 ? 12 : 8; }
+#endif
+
+MLSW_DEFINE_BOUNDS_READER(MLSW_CAT(bounds_violations_batch_, MLSW_BATCH_N))
 
 }  // namespace mlsw

@@ -14,6 +14,16 @@ namespace mlsw {
 constexpr int kStatusNonfinite = 1;  // h <= 0 or a non-finite value
 constexpr int kStatusTimeout = 2;    // a bounded mbarrier wait ran out
 
+// D2Q9 step: a warp marches down a strip of kMarchCols columns, of which the
+// kMarchHalo on each side only feed the stencils (march.cuh).
+constexpr int kMarchCols = 64, kMarchHalo = 4, kMarchOut = kMarchCols - 2 * kMarchHalo;
+inline int march_strips(int nx) { return (nx + kMarchOut - 1) / kMarchOut; }
+// A D2Q9 state with tau = 1 is stored as moments: plane 4 i + q holds g_0, s,
+// J_x, J_y (q = 0..3) of layer i; another tau (and a lattice whose ghosts need
+// a pass of their own) as populations, plane 9 i + k. Both in the layout of
+// KParams::L.
+constexpr int kMomPlanes = 4;
+
 // Per-layer rest-population shift (see KParams).
 struct KShift {
   float H[kMaxLayers];
@@ -24,14 +34,23 @@ struct StepLaunch {
   int lattice;                  // 1 = D1Q3, 2 = D2Q9
   const float* fin;
   float* fout;
-  const CUtensorMap* fin_map;   // D2Q9: 3-D tensor map of fin (box of one tile)
+  const CUtensorMap* fin_map;   // D2Q9: row map of fin (see mlsw_host::make_row_map)
   KParams P;
+  int to_populations;           // D2Q9, moments in: write the populations after the step
   int* status;
-  int* sched;                   // D2Q9: two zero-initialised tile-scheduler counters
   int num_sms;
-  int reverse;                  // D2Q9: 1 = tiles in reverse order (see SingleTiles)
 };
 cudaError_t launch_step(const StepLaunch& a, cudaStream_t st);
+// the D2Q9 step of n = N layers (step_d2q9.cu)
+template <int N>
+cudaError_t launch_step_d2q9(const StepLaunch& a, cudaStream_t st);
+template <> cudaError_t launch_step_d2q9<1>(const StepLaunch& a, cudaStream_t st);
+template <> cudaError_t launch_step_d2q9<2>(const StepLaunch& a, cudaStream_t st);
+template <> cudaError_t launch_step_d2q9<3>(const StepLaunch& a, cudaStream_t st);
+template <> cudaError_t launch_step_d2q9<4>(const StepLaunch& a, cudaStream_t st);
+template <> cudaError_t launch_step_d2q9<5>(const StepLaunch& a, cudaStream_t st);
+// Cells of a D1Q3 tile (the padded layout covers whole tiles).
+int step_d1q3_cols();
 
 // D1Q3 lattices small enough for one CTA's shared memory run many steps in
 // one persistent launch: bytes of shared memory it needs (0: not possible
@@ -45,58 +64,50 @@ cudaError_t launch_step_persistent(const StepLaunch& a, int nsteps, cudaStream_t
 // over one tile table, in which the tiles of instances that share n, kernel
 // mode and tile height form a contiguous range (batch_kernels.cu).
 // ---------------------------------------------------------------------------
-// Tile heights a batch can use: variant 0 = 16 rows with two rows per
-// thread (n <= 3 only), variant 1 = 8 rows with one row per thread.
+// Tile heights a batch can use: variant 0 = 16 rows (n <= 3 only), variant
+// 1 = 8 rows. A warp's unit of work is a strip of `rows` rows, whole tiles.
 constexpr int kBatchVariants = 2;
-__host__ __device__ constexpr int batch_variant(int rows_per_thread) {
-  return rows_per_thread == 2 ? 0 : 1;
-}
 __host__ __device__ constexpr int batch_tile_rows(int variant) { return variant == 0 ? 16 : 8; }
 
 // Device descriptor of one instance (aligned as its tensor maps require).
 struct BatchInst {
-  CUtensorMap map[kBatchVariants][2];  // [variant][input buffer]: box of one tile + halo
+  CUtensorMap map[2];  // row maps of the two buffers
   KParams P;
-  float* f[2];  // population buffers
-  int ntx;      // tile columns (tiles are 32 cells wide)
+  float* f[2];  // buffers, moments or populations
+  int kind;     // batch_kind
+  int strips;   // strips of kMarchOut columns
+  int rows;     // rows of a unit
 };
 
 // Kernel mode of a parameter set: 0 general, 1 tau = 1, 2 fast (tau = 1,
 // exponents (3, 2), spreading only between neighbouring interfaces).
 int step_mode(const KParams& P);
+// Whether a D2Q9 state is stored as moments (else populations).
+bool step_moments(const KParams& P);
 
-// Kind of a range of tiles: layer count n (1..5), kernel mode, tile-height
-// variant (16-row tiles only for n <= 3).
-constexpr int kBatchKinds = 5 * 3 * kBatchVariants;
-__host__ __device__ constexpr int batch_kind(int n, int mode, int variant) {
-  return ((n - 1) * 3 + mode) * kBatchVariants + variant;
-}
-bool batch_kind_valid(int n, int mode, int variant);
-// dynamic shared memory of the tile loop of one kind
-size_t batch_kind_smem(int n, int variant);
+// Kernel of an instance: layer count n (1..5) and kernel mode.
+constexpr int kBatchKinds = 5 * 3;
+__host__ __device__ constexpr int batch_kind(int n, int mode) { return (n - 1) * 3 + mode; }
 
-// Ends of the ranges of a tile table sorted by kind: the tiles of kind k are
-// the entries [end[k - 1], end[k]) (end[-1] = 0), so end is non-decreasing
-// and a kind without tiles repeats the previous end.
-struct BatchEnds {
-  int end[kBatchKinds];
-};
-
-// One batch step of every instance in a tile table (device, entries of
-// (instance, tile) in ranges), buffers cur -> cur ^ 1: one launch.
+// One batch step, buffers cur -> cur ^ 1, of every instance in a table of
+// (instance, unit) entries, one warp each: one launch.
 struct BatchLaunch {
   const BatchInst* inst;
   const int2* table;
-  BatchEnds ends;
+  int nunits;
+  int nmax;        // largest layer count in the table
+  unsigned kinds;  // bit k: instances of kind k are in the table
   int cur;
   int* status;
-  int* sched;  // two zero-initialised counters
-  int num_sms;
 };
-// With an empty table (every end 0) it only configures the kernel
-// (shared-memory limit, occupancy) on the current device, so that a later
-// launch can be captured.
+// warps of a batch step resident on one SM
+int batch_warps_per_sm(int nmax);
 cudaError_t launch_batch_step(const BatchLaunch& a, cudaStream_t st);
+// the kernel for at most NMAX layers (3: more warps fit an SM; 5)
+template <int NMAX>
+cudaError_t launch_batch_step_n(const BatchLaunch& a, cudaStream_t st);
+template <> cudaError_t launch_batch_step_n<3>(const BatchLaunch& a, cudaStream_t st);
+template <> cudaError_t launch_batch_step_n<5>(const BatchLaunch& a, cudaStream_t st);
 
 // out[2 (j kMaxLayers + i) + {0, 1}] = real and imaginary part of
 // sum_x h_i(x) exp(-2 pi i (kx[j] x / nx + ky[j] y / ny)) for every instance
@@ -132,22 +143,24 @@ cudaError_t launch_radial_profile(int Q, int n, const Layout& L, const float* f,
                                   const ProfileParams& A, double* sums,
                                   unsigned long long* counts, cudaStream_t st);
 
-// Tile shape of the step kernels (the padded layout covers whole tiles).
-int step_tile_cols(int lattice);
-int step_tile_rows(int n, int lattice);
+// The launches below take a state's planes per layer as Q: 9 (D2Q9) or 3
+// (D1Q3) populations, or kMomPlanes for moments.
 
-// f = f_eq(h, U = 0) on the real cells and their ghost images (x only
-// when ghosts_y is false): rest population h - H_i, moving populations 0;
-// h dense [n][ny][nx]. status |= kStatusNonfinite where h <= 0 or h is not
-// finite.
-cudaError_t launch_init(int Q, int n, const Layout& L, bool ghosts_y, const float* h, float* f,
-                        const KShift& sh, int* status, cudaStream_t st);
+// f = f_eq(h, U = 0) on the real cells and their ghost images: rest
+// population h - H_i, everything else 0; h dense [n][ny][nx]. status |=
+// kStatusNonfinite where h <= 0 or h is not finite.
+cudaError_t launch_init(int Q, int n, const Layout& L, const float* h, float* f, const KShift& sh,
+                        int* status, cudaStream_t st);
 
-// Periodic images: every ghost cell within two cells of the real domain
-// (x only when ghosts_y is false) copies its real cell, for all nplanes
-// planes.
-cudaError_t launch_fill_ghosts(int nplanes, const Layout& L, bool ghosts_y, float* f,
-                               cudaStream_t st);
+// Periodic images: every ghost cell within four columns of the real domain
+// copies its real cell, for all nplanes planes.
+cudaError_t launch_fill_ghosts(int nplanes, const Layout& L, float* f, cudaStream_t st);
+
+// Moments m (ghosts included) of D2Q9 populations f; the populations f (real
+// cells) of a D2Q9 state at rest with moments m.
+cudaError_t launch_moments(int n, const Layout& L, const float* f, float* m, cudaStream_t st);
+cudaError_t launch_rest_populations(int n, const Layout& L, const float* m, float* f,
+                                    cudaStream_t st);
 
 // h dense [n][ny][nx] = H_i + sum_k g[i][k]
 // With st_out (a device view of page-locked host memory), the first thread
@@ -168,7 +181,7 @@ cudaError_t launch_rest_planes(int Q, int n, const Layout& L, const float* f, co
 // Two-pass deterministic reduction of per-layer mass, kinetic energy and
 // min h over the real cells. partials: nblk * (n + 2) doubles; out: n + 2
 // doubles (mass[0..n-1], kinetic, hmin).
-cudaError_t launch_diagnostics(int lattice, int n, const Layout& L, const float* f,
+cudaError_t launch_diagnostics(int Q, int n, const Layout& L, const float* f,
                                const KShift& sh, double* partials, int nblk, double* out,
                                cudaStream_t st);
 
@@ -203,7 +216,6 @@ inline Layout dense_layout(int nx, int ny, int nplanes = 0) {
   L.nx = nx;
   L.ny = ny;
   L.gx = 0;
-  L.gy = 0;
   L.pitch = nx;
   L.rows = ny;
   L.plane = (long)nx * ny;
@@ -217,6 +229,12 @@ inline Layout dense_layout(int nx, int ny, int nplanes = 0) {
 unsigned bounds_violations_step();
 unsigned bounds_violations_aux();
 unsigned bounds_violations_analysis();
-unsigned bounds_violations_batch();
+unsigned bounds_violations_d2q9_1();
+unsigned bounds_violations_d2q9_2();
+unsigned bounds_violations_d2q9_3();
+unsigned bounds_violations_d2q9_4();
+unsigned bounds_violations_d2q9_5();
+unsigned bounds_violations_batch_3();
+unsigned bounds_violations_batch_5();
 
 }  // namespace mlsw

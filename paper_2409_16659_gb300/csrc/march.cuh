@@ -1,0 +1,511 @@
+// march.cuh -- the fused D2Q9 step (section LBM: moments, interfaces and
+// pressures, force, BGK with forcing, streaming) as one warp marching down
+// the rows of a strip of 64 columns, shared by the single-lattice kernels
+// (step_kernels.cu) and the batch kernels (batch_kernels.cu).
+//
+// A lane holds two neighbouring columns as one FP32x2 pair. Column
+// neighbours come by warp shuffles, row neighbours from registers carried
+// from row to row, so a unit of work needs no barrier with any other warp
+// and no field goes through shared memory; only the input rows do, copied
+// by TMA into a ring a few rows ahead. Of the 64 columns 56 are written: the
+// 4 on each side feed the stencils (z three columns out, p two, the streamed
+// populations one), and 56 columns are whole 32-byte sectors.
+//
+// With row r arriving:
+//   z(r)                 interface deviations z_i - sum_{j<=i} H_j
+//   p(r - 1)             needs z of rows r - 2 .. r
+//   collision(r - 2)     needs p of rows r - 3 .. r - 1
+//   output(r - 3)        needs the populations of rows r - 4 .. r - 2
+//
+// State. With tau = 1 the collision forgets the populations: a step reads,
+// per layer and cell, only the rest population g_0, the sum s of the moving
+// ones (h - H = g_0 + s, kept apart because adding them would round s to the
+// resolution of g_0) and the flux J = (J_x, J_y). These four moments are the
+// state a lattice with tau = 1 is stored in ("moment form", 16 bytes instead
+// of 36 per layer and cell, a quarter of the planes to write being whole
+// rows); its populations at a time follow from the moments one step earlier
+// by the same kernel with populations as its output (OP). Another tau keeps
+// populations.
+#pragma once
+
+#include "kernels.h"
+#include "physics.cuh"
+#include "step_common.cuh"
+#include "tma.cuh"
+
+namespace mlsw {
+
+constexpr unsigned kFullWarp = 0xffffffffu;
+
+template <int N, int MODE, bool OP>
+struct MarchShape {
+  static constexpr bool TAU1 = MODE != kGeneral;
+  static_assert(TAU1 || OP, "tau != 1 steps from populations to populations");
+  static constexpr int PL = (TAU1 ? kMomPlanes : 9) * N;  // planes of an input row
+  static constexpr int ROW = PL * kMarchCols;             // floats of a ring row
+  // Ring rows: three are live (the newest down to the one collided) and one
+  // is in flight, which a row's time (about 2000 cycles) covers.
+  static constexpr int RS = 4;
+  // five layers: the older row of upward populations is parked in shared
+  // memory (in registers it spills: 90 against 47 us a step at 1024^2)
+  static constexpr bool PARK = N >= 5 && !OP;
+  static constexpr size_t kOffPark = (size_t)RS * ROW * 4;
+  static constexpr size_t kOffBar = kOffPark + (PARK ? (size_t)3 * N * kMarchCols * 4 : 0);
+  static constexpr size_t kSmem = (kOffBar + 8 * RS + 127) / 128 * 128;
+};
+
+__device__ __forceinline__ f2 ld_pair(const float* a) {
+  const float2 v = *reinterpret_cast<const float2*>(chk_smem(reinterpret_cast<const float2*>(a)));
+  return mk2(v.x, v.y);
+}
+__device__ __forceinline__ void st_pair(float* a, f2 v) {
+  *chk_smem(reinterpret_cast<float2*>(a)) = v.v;
+}
+
+// the columns left and right of a pair: .x the column before v.x, .y the one
+// after v.y (garbage in the outermost lanes, which feed no output)
+__device__ __forceinline__ float2 beside(f2 v) {
+  return make_float2(__shfl_up_sync(kFullWarp, v.v.y, 1), __shfl_down_sync(kFullWarp, v.v.x, 1));
+}
+
+// Lattice derivatives of a field at the centre row of three, from the centre
+// values c and the differences A = north - c and B = c - south:
+// with V = north + south - 2 c = A - B and D = north - south = A + B,
+//   d/dx = (c_E - c_W) / 2 + (V_E - V_W) / 12
+//   d/dy = D / 3 + (D_E + D_W) / 12
+//   lap  = (c_E + c_W - 2 c) + 2/3 V + (V_E + V_W) / 6,
+// the isotropic stencils (weights 1/3, 1/12 and 2/3, 1/6) written in
+// differences of neighbours, so no large values cancel and a constant field
+// gives exact zeros.
+template <bool LAP>
+__device__ __forceinline__ void lattice_derivatives(f2 c, f2 A, f2 B, f2& gx, f2& gy, f2& lap) {
+  const f2 V = A - B, D = A + B;
+  const float2 cb = beside(c), vb = beside(V), db = beside(D);
+  const f2 vd = mk2(V.v.y - vb.x, vb.y - V.v.x);
+  const f2 ds = mk2(D.v.y + db.x, db.y + D.v.x);
+  gy = fmav(D, 1.f / 3.f, ds * (1.f / 12.f));
+  if constexpr (LAP) {
+    const f2 fwd = mk2(c.v.y - c.v.x, cb.y - c.v.y), back = mk2(c.v.x - cb.x, c.v.y - c.v.x);
+    const f2 vs = mk2(V.v.y + vb.x, vb.y + V.v.x);
+    gx = fmav(fwd + back, 0.5f, vd * (1.f / 12.f));
+    lap = fmav(V, 2.f / 3.f, fmav(vs, 1.f / 6.f, fwd - back));
+  } else {
+    gx = fmav(mk2(c.v.y - cb.x, cb.y - c.v.x), 0.5f, vd * (1.f / 12.f));
+  }
+}
+
+// A pair of output values (columns ca, ca + 1; `row` points at column 0) and
+// their periodic images in the ghost columns [-4, 0) and [nx, nx + 4). Most
+// strips have neither images nor columns beyond the lattice: they store with
+// one predicate and a 32-bit lane offset from a warp-uniform address.
+struct PairStore {
+  bool own, own2;        // the pair's first / second column belongs to the lattice
+  bool plain;            // (warp-uniform) no image, no column beyond the lattice
+  bool im[2][2];         // [column][0: + nx, 1: - nx]
+  int ca, nx;
+  unsigned off;          // bytes from column 0 (lanes that own a column)
+  __device__ PairStore(int x0, int lane, int nx_) {
+    nx = nx_;
+    ca = x0 - kMarchHalo + 2 * lane;
+    const bool in = lane >= kMarchHalo / 2 && lane < 32 - kMarchHalo / 2;
+    own = in && ca < nx;
+    own2 = in && ca + 1 < nx;
+    plain = x0 >= 4 && x0 + kMarchOut <= nx - 4;
+    off = (unsigned)(ca < 0 ? 0 : ca) * 4u;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const bool o = c ? own2 : own;
+      im[c][0] = o && ca + c < 4;
+      im[c][1] = o && ca + c >= nx - 4;
+    }
+  }
+  __device__ __forceinline__ void fast(float* buf, long len, float* row, f2 v) const {
+    if (own)
+      *reinterpret_cast<float2*>(
+          chk_global(buf, reinterpret_cast<float*>(reinterpret_cast<char*>(row) + off), len, 2)) = v.v;
+  }
+  __device__ __forceinline__ void slow(float* buf, long len, float* row, f2 v) const {
+    if (own) *chk_global(buf, row + ca, len) = v.v.x;
+    if (own2) *chk_global(buf, row + ca + 1, len) = v.v.y;
+    if (im[0][0]) *chk_global(buf, row + ca + nx, len) = v.v.x;
+    if (im[1][0]) *chk_global(buf, row + ca + 1 + nx, len) = v.v.y;
+    if (im[0][1]) *chk_global(buf, row + ca - nx, len) = v.v.x;
+    if (im[1][1]) *chk_global(buf, row + ca + 1 - nx, len) = v.v.y;
+  }
+};
+
+// The phase of the substrate at a pair of columns, in whole units of
+// 1 / (nx ny), carried from row to row; height() gives substrate_at's values.
+struct SubstratePhase {
+  long col[2], row;
+  __device__ SubstratePhase() {}
+  __device__ SubstratePhase(const KParams& P, int x, int y) {
+    const long nx = P.nx, ny = P.ny, nc = nx * ny;
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+      long m = ((long)P.sub_kx * (x + c) % nx) * ny;
+      if (m < 0) m += nc;
+      (c ? col[1] : col[0]) = m;
+    }
+    row = ((long)P.sub_ky * y % ny) * nx;
+    if (row < 0) row += nc;
+  }
+  __device__ float height(const KParams& P, int c) const {
+    const long nc = (long)P.nx * P.ny;
+    long m = col[c] + row;
+    if (m >= nc) m -= nc;
+    return substrate_height(P, m, nc);
+  }
+  __device__ void next_row(const KParams& P) {
+    const long nc = (long)P.nx * P.ny;
+    row += (long)(P.sub_ky % P.ny) * P.nx;
+    if (row >= nc) row -= nc;
+    if (row < 0) row += nc;
+  }
+};
+
+// One unit of work: the output rows [ya, yb) of the strip that starts at
+// column x0, by one warp. sm: MarchShape::kSmem bytes, 128-byte aligned.
+// wait: the programmatic-launch wait for the previous grid (every global
+// access comes after it).
+template <int N, int MODE, bool OP>
+__device__ __forceinline__ void march_unit(const KParams& P, const CUtensorMap* map,
+                                           float* __restrict__ fout, int x0, int ya, int yb,
+                                           unsigned char* sm, int* __restrict__ status) {
+  using S = MarchShape<N, MODE, OP>;
+  constexpr bool TAU1 = S::TAU1, W32 = MODE == kFast, NN = MODE == kFast;
+  constexpr int Q = 9, RS = S::RS, CW = kMarchCols;
+  constexpr int kTwoRows = N <= 3 ? 2 : 1;  // rows a turn of the main loop (four layers: spills)
+  float* ring = reinterpret_cast<float*>(sm);
+  float* park = reinterpret_cast<float*>(sm + S::kOffPark) + 2 * (threadIdx.x & 31);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + S::kOffBar);
+  const int lane = threadIdx.x & 31;
+  const Layout& L = P.L;
+  const int nx = P.nx, ny = P.ny;
+  // collision rows: the output rows, and one more on each side when the
+  // output gathers its populations from them
+  const int cA = OP ? ya : ya - 1, cB = OP ? yb : yb + 1;
+  const int r0 = cA - 2, T = cB - cA + 4;  // input rows r0 .. r0 + T - 1
+
+  auto wrap_row = [&](int y) {
+    y %= ny;
+    return y < 0 ? y + ny : y;
+  };
+  auto issue = [&](int t) {  // lane 0
+    uint64_t* b = bar + t % RS;
+    const int x = x0 + L.gx - kMarchHalo, y = wrap_row(r0 + t);
+#ifdef MLSW_DEBUG
+    // the copy must start on a 16-byte boundary inside the buffer (columns
+    // beyond the row's end read as zeros); a bad one is not issued (the
+    // barrier completes without data)
+    if (x % 4 != 0 || x < 0 || x >= L.pitch || y < 0 || y >= L.rows) {
+      note_bounds_violation();
+      mbar_arrive_expect_tx(b, 0u);
+      return;
+    }
+#endif
+    mbar_arrive_expect_tx(b, (uint32_t)(S::ROW * 4));
+    tma_load_3d(ring + (t % RS) * S::ROW, map, b, x, y, 0);
+  };
+  if (lane == 0) {
+    for (int s = 0; s < RS; ++s) mbar_init(bar + s, 1);
+    mbar_init_fence();
+  }
+  // Programmatic dependent launch: the next step's warps are scheduled as
+  // this grid's exit, and wait here. They are not let in earlier (no
+  // launch_dependents): warps that arrive while an SM still runs its share
+  // crowd onto the SMs that finish first (three layers, 128^2: 8.2 us a step
+  // with an early trigger, 5.2 without; 1024^2: 30.2 and 28.7).
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  __syncwarp();
+  int issued = RS < T ? RS : T;  // input rows whose copies were started
+  if (lane == 0)
+    for (int t = 0; t < issued; ++t) issue(t);
+  // starts the copy of the next row, into the slot of the oldest one, which
+  // every lane has read
+  auto refill = [&]() {
+    if (issued < T) {
+      __syncwarp();
+      if (lane == 0) {
+        fence_proxy_async_smem();
+        issue(issued);
+      }
+      ++issued;
+    }
+  };
+
+  const bool sub = MODE != kFast && P.sub_amp != 0.f;
+  SubstratePhase sub_phase;
+  if (sub) sub_phase = SubstratePhase(P, x0 - kMarchHalo + 2 * lane, r0);
+  const PairStore put(x0, lane, nx);
+  const f2 zero = mk2(0.f, 0.f);
+  f2 zc[N], zB[N], pc[N], pB[N];  // previous row, and its difference to the row before
+  f2 sc = zero, sB = zero;        // the same of the substrate
+  f2 up1[N][3], up2[S::PARK ? 1 : N][3], mid[N][3];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    zc[i] = zB[i] = pc[i] = pB[i] = zero;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      up1[i][k] = mid[i][k] = zero;
+      if constexpr (S::PARK)
+        st_pair(park + (3 * i + k) * CW, zero);
+      else
+        up2[i][k] = zero;
+    }
+  }
+  // smallest height so far; 0, or NaN once a force was not finite (0 * inf and
+  // 0 * NaN are NaN): looked at once, at the end
+  f2 hlow = mk2(1.f, 1.f), fall = zero;
+  int slot = 0;  // of the next input row
+  uint32_t parity = 0;
+
+  // Row t arrives: its z; returns false when the bounded wait ran out.
+  auto arrive = [&](int t, f2 (&zn)[N], f2& sn) {
+    if (!mbar_wait_bounded(bar + slot, parity)) return false;
+    const float* src = ring + slot * S::ROW + 2 * lane;
+    f2 z = zero;
+    if (sub) {
+      z = sn = mk2(sub_phase.height(P, 0), sub_phase.height(P, 1));
+      sub_phase.next_row(P);
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if constexpr (!TAU1) {
+        f2 v[Q];
+#pragma unroll
+        for (int k = 0; k < Q; ++k) v[k] = ld_pair(src + (i * Q + k) * CW);
+        z = z + (v[0] + moving_sum(v));
+      } else {
+        z = z + (ld_pair(src + 4 * i * CW) + ld_pair(src + (4 * i + 1) * CW));
+      }
+      zn[i] = z;
+    }
+    if (++slot == RS) {
+      slot = 0;
+      parity ^= 1u;
+    }
+    return true;
+  };
+  // Pressures at the centre row (the previous z) from the new row's z.
+  auto pressures = [&](const f2 (&zn)[N], f2 sn, f2 (&pn)[N]) {
+    f2 gx[N], gy[N], lz[N], zd[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const f2 A = zn[i] - zc[i];
+      lattice_derivatives<true>(zc[i], A, zB[i], gx[i], gy[i], lz[i]);
+      zd[i] = zc[i];
+    }
+    if (sub) {
+      f2 g0x, g0y, l0;
+      lattice_derivatives<true>(sc, sn - sc, sB, g0x, g0y, l0);
+      const f2 sg0 = fmav(0.5f, fmav(g0x, g0x, g0y * g0y), mk2(1.f, 1.f));
+      neg_pressures<N, W32, f2, NN>(P, zd, gx, gy, lz, pn, &sc, &sg0);
+    } else {
+      neg_pressures<N, W32, f2, NN>(P, zd, gx, gy, lz, pn);
+    }
+  };
+  auto roll_z = [&](const f2 (&zn)[N], f2 sn) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      zB[i] = zn[i] - zc[i];
+      zc[i] = zn[i];
+    }
+    sB = sn - sc;
+    sc = sn;
+  };
+  auto roll_p = [&](const f2 (&pn)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      pB[i] = pn[i] - pc[i];
+      pc[i] = pn[i];
+    }
+  };
+
+  // Collision of row r0 + t - 2, between the pressures of the two rows before
+  // and pn, and the output it completes.
+  auto collision = [&](int t, const f2 (&pn)[N]) {
+    const int tc = t - 2, y = r0 + tc;
+    f2 g0[N], sm_[N], jx[N], jy[N], hh[N], ih[N], ux[N], uy[N], Rx[N], Ry[N];
+    const int cslot = tc % RS;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if constexpr (!TAU1) {
+        const float* src = ring + cslot * S::ROW + i * Q * CW + 2 * lane;
+        f2 v[Q];
+#pragma unroll
+        for (int k = 0; k < Q; ++k) v[k] = ld_pair(src + k * CW);
+        const Moments<f2> m = moments_of(v);
+        g0[i] = m.g0;
+        sm_[i] = m.s;
+        jx[i] = m.jx;
+        jy[i] = m.jy;
+      } else {
+        const float* src = ring + cslot * S::ROW + 4 * i * CW + 2 * lane;
+        g0[i] = ld_pair(src);
+        sm_[i] = ld_pair(src + CW);
+        jx[i] = ld_pair(src + 2 * CW);
+        jy[i] = ld_pair(src + 3 * CW);
+      }
+      hh[i] = (g0[i] + sm_[i]) + P.H[i];
+      ih[i] = rcp(hh[i]);
+      ux[i] = jx[i] * ih[i];
+      uy[i] = jy[i] * ih[i];
+    }
+    friction<N, true>(P, hh, ih, ux, uy, Rx, Ry);
+    // rows of the output
+    float* rowp[3];
+    float* mrow = nullptr;
+    const bool write = OP || t >= 6;
+    if constexpr (OP) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+        rowp[d] = fout + (long)wrap_row(y + d - 1) * L.pitch + L.gx;
+    } else {
+      mrow = fout + (long)(y - 1) * L.pitch + L.gx;
+    }
+    Moments<f2> om[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      f2 gqx, gqy, none;
+      lattice_derivatives<false>(pc[i], pn[i] - pc[i], pB[i], gqx, gqy, none);
+      const f2 Fx = fmav(hh[i], gqx, Rx[i]), Fy = fmav(hh[i], gqy, Ry[i]);
+      hlow = mk2(fminf(hlow.v.x, hh[i].v.x), fminf(hlow.v.y, hh[i].v.y));
+      fall = fmav(Fx + Fy, 0.f, fall);
+      f2 fo[Q], fs[Q];
+      if constexpr (!TAU1) {
+        const float* src = ring + cslot * S::ROW + i * Q * CW + 2 * lane;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) fo[k] = ld_pair(src + k * CW);
+      }
+      collide_d2q9<TAU1>(P, g0[i], sm_[i], jx[i], jy[i], ux[i], uy[i], Fx, Fy, fo, fs);
+      // streaming along x: the pair takes what arrives at its columns
+      f2 v[Q];
+      v[0] = fs[0];
+      v[3] = fs[3];
+      v[7] = fs[7];
+#pragma unroll
+      for (int k = 1; k < Q; ++k) {
+        if (Lattice<2>::cx(k) > 0)
+          v[k] = mk2(__shfl_up_sync(kFullWarp, fs[k].v.y, 1), fs[k].v.x);
+        else if (Lattice<2>::cx(k) < 0)
+          v[k] = mk2(fs[k].v.y, __shfl_down_sync(kFullWarp, fs[k].v.x, 1));
+      }
+      if constexpr (OP) {
+        if (put.plain) {
+#pragma unroll
+          for (int k = 0; k < Q; ++k)
+            put.fast(fout, (long)Q * N * L.plane, rowp[Lattice<2>::cy(k) + 1] + (long)(i * Q + k) * L.plane, v[k]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < Q; ++k)
+            put.slow(fout, (long)Q * N * L.plane, rowp[Lattice<2>::cy(k) + 1] + (long)(i * Q + k) * L.plane, v[k]);
+        }
+      } else {
+        f2 below[3];  // moving up, from the row below the output row
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          if constexpr (S::PARK)
+            below[k] = ld_pair(park + (3 * i + k) * CW);
+          else
+            below[k] = up2[i][k];
+        }
+        const f2 w[Q] = {mid[i][0], mid[i][1], below[0], below[1], below[2],
+                         mid[i][2], v[6],      v[7],     v[8]};
+        om[i] = moments_of(w);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          if constexpr (S::PARK)
+            st_pair(park + (3 * i + k) * CW, up1[i][k]);
+          else
+            up2[i][k] = up1[i][k];
+          up1[i][k] = v[2 + k];
+        }
+        mid[i][0] = v[0];
+        mid[i][1] = v[1];
+        mid[i][2] = v[5];
+      }
+    }
+    if constexpr (!OP) {
+      if (write) {
+        const long len = (long)kMomPlanes * N * L.plane;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          float* d = mrow + (long)(kMomPlanes * i) * L.plane;
+          if (put.plain) {
+            put.fast(fout, len, d, om[i].g0);
+            put.fast(fout, len, d + L.plane, om[i].s);
+            put.fast(fout, len, d + 2 * L.plane, om[i].jx);
+            put.fast(fout, len, d + 3 * L.plane, om[i].jy);
+          } else {
+            put.slow(fout, len, d, om[i].g0);
+            put.slow(fout, len, d + L.plane, om[i].s);
+            put.slow(fout, len, d + 2 * L.plane, om[i].jx);
+            put.slow(fout, len, d + 3 * L.plane, om[i].jy);
+          }
+        }
+      }
+    }
+  };
+
+  bool ok = true;
+  int t = 0;
+  if constexpr (MODE == kFast && !OP) {
+    // the steps of a long call: the warm-up rows apart, so that a full row is
+    // one block of straight-line code, two rows at a time (the carried rows
+    // then change names instead of moving; 31.2 -> 30.3 us a step at 1024^2)
+#pragma unroll 1
+    for (; t < 4; ++t) {
+      f2 zn[N], pn[N], sn = zero;
+      ok = arrive(t, zn, sn);
+      if (!ok) break;
+      if (t >= 2) {
+        refill();  // row t - 2 gave its z and is not collided
+        pressures(zn, sn, pn);
+        roll_p(pn);
+      }
+      roll_z(zn, sn);
+    }
+#pragma unroll kTwoRows
+    for (; t < T && ok; ++t) {
+      f2 zn[N], pn[N], sn = zero;
+      ok = arrive(t, zn, sn);
+      if (!ok) break;
+      pressures(zn, sn, pn);
+      roll_z(zn, sn);
+      collision(t, pn);
+      roll_p(pn);
+      refill();
+    }
+  } else {
+#pragma unroll 1
+    for (; t < T; ++t) {
+      f2 zn[N], pn[N], sn = zero;
+      ok = arrive(t, zn, sn);
+      if (!ok) break;
+      if (t >= 2) {
+        pressures(zn, sn, pn);
+        if (t >= 4) collision(t, pn);
+        roll_p(pn);
+        refill();  // row t - 2 is used up
+      }
+      roll_z(zn, sn);
+    }
+  }
+  if (!ok) {
+    // a bounded wait ran out: report, and let this warp's copies land
+    if (lane == 0) atomicOr(status, kStatusTimeout);
+    for (; t < issued; ++t) {
+      mbar_wait_bounded(bar + slot, parity, 1u << 16);
+      if (++slot == RS) {
+        slot = 0;
+        parity ^= 1u;
+      }
+    }
+  }
+  const bool bad = (put.own && (!(hlow.v.x > 0.f) || isnan(fall.v.x))) ||
+                   (put.own2 && (!(hlow.v.y > 0.f) || isnan(fall.v.y)));
+  if (bad) atomicOr(status, kStatusNonfinite);
+}
+
+}  // namespace mlsw

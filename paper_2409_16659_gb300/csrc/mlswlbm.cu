@@ -20,11 +20,18 @@ struct mlsw_handle {
   KParams kp;         // includes the padded layout kp.L
   int Q;
   long ncell;
-  size_t flen;        // floats per (padded) population buffer
+  // State buffers: populations, or moments (D2Q9, tau = 1; see kernels.h).
   float* f[2];
   int cur;            // index of the buffer holding the current state
+  bool moments;
+  // Moment form only. pop: room for the populations, which the state calls
+  // exchange with the host. They are in there (kGiven), or follow from the
+  // moments: zero moving populations (kAtRest), or one step on from the other
+  // buffer, which holds the moments before the last step (kStepped).
+  float* pop;
+  enum Origin { kAtRest, kGiven, kStepped } origin;
   float* hbuf;        // n * ncell heights (upload / read-out)
-  int* status;        // [0] OR of kernel error bits; [1], [2] tile scheduler
+  int* status;        // [0] OR of kernel error bits; [1] of kernels that only read out
   double* partials;   // diagnostics partials
   double* dout;       // diagnostics result, n + 2 doubles
   int nblk_diag;
@@ -33,7 +40,7 @@ struct mlsw_handle {
   mlsw::KShift sh;    // rest-population shift H_i (also in kp.H)
   int num_sms;
   size_t psmem;       // D1Q3 persistent launch: shared memory bytes (0: not used)
-  CUtensorMap map[2]; // D2Q9: tensor map of each buffer, box = one tile + halo
+  CUtensorMap map[2]; // D2Q9: row map of each buffer
   int* status_host;   // page-locked mirror of status[0], written by the read-out
   int* status_mirror; // its device address
 };
@@ -137,6 +144,8 @@ KParams make_kparams(const mlsw_params& p) {
     k.gamma[i] = (float)p.gamma[i];
     set_friction(k, i, p.mu[i], p.beta[i]);
     for (int kk = 1; kk <= p.n_layers - i; ++kk) k.S[i][kk - 1] = (float)p.spread[i][kk - 1];
+    for (int kk = 2; kk <= p.n_layers - i; ++kk)
+      if (k.S[i][kk - 1] != 0.f) k.far_pairs = 1;
   }
   k.hstar = (float)p.hstar;
   k.nw = p.wet_n;
@@ -174,32 +183,26 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 mlsw::Layout make_layout(const mlsw_params& p) {
   mlsw::Layout L;
-  const int tx = mlsw::step_tile_cols(p.lattice);
-  const int ty = mlsw::step_tile_rows(p.n_layers, p.lattice);
+  const bool d2 = p.lattice == MLSW_D2Q9;
   L.nx = p.nx;
   L.ny = p.ny;
-  L.gx = 4;  // two ghost columns plus two for 16-byte alignment of tile boxes
-  L.gy = (p.lattice == MLSW_D2Q9) ? 2 : 0;
-  L.pitch = round_up(p.nx, tx) + 8;
-  L.rows = (p.lattice == MLSW_D2Q9) ? round_up(p.ny, ty) + 4 : 1;
+  L.gx = d2 ? 8 : 4;
+  L.pitch = d2 ? round_up(8 + p.nx + 4, 8) : round_up(p.nx, mlsw::step_d1q3_cols()) + 8;
+  L.rows = p.ny;
   L.plane = (long)L.pitch * L.rows;
   L.nplanes = p.n_layers * Qof(p.lattice);
   return L;
 }
 
-int wrap_host(int v, int n) {
-  v %= n;
-  return v < 0 ? v + n : v;
-}
-
-void set_ghost_tables(KParams& k, const mlsw_params& p) {
-  const int gx[4] = {-2, -1, p.nx, p.nx + 1};
-  const int gy[4] = {-2, -1, p.ny, p.ny + 1};
-  for (int g = 0; g < 4; ++g) {
-    k.gsrcx[g] = wrap_host(gx[g], p.nx);
-    k.gsrcy[g] = (p.lattice == MLSW_D2Q9) ? wrap_host(gy[g], p.ny) : -1000;
-  }
-  k.tiny = (p.nx < 4 || (p.lattice == MLSW_D2Q9 && p.ny < 4)) ? 1 : 0;
+// A layer's planes are limited to 2^31 - 1 floats, counted with the margins
+// of 32-column, 16- or 8-row tiles.
+bool too_large(const mlsw_params& p) {
+  double plane;
+  if (p.lattice == MLSW_D2Q9)
+    plane = (double)(round_up(p.nx, 32) + 8) * (round_up(p.ny, p.n_layers <= 3 ? 16 : 8) + 4);
+  else
+    plane = (double)(round_up(p.nx, mlsw::step_d1q3_cols()) + 8);
+  return plane * Qof(p.lattice) >= 2147483647.0;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -222,15 +225,15 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 3-D map (x: pitch, y: rows, z: planes) whose box is one D2Q9 tile with
-// its halo: 40 x (TY + 4) x all planes.
-bool make_tile_map(CUtensorMap* m, float* base, const mlsw::Layout& L, int nplanes, int box_cols,
-                   int box_rows) {
+// A row map's box is one row of a warp's columns in every plane. Rows are
+// copied one by one (box height 1), so that a warp can wrap them around the
+// periodic lattice.
+bool make_row_map(CUtensorMap* m, float* base, const mlsw::Layout& L, int planes) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)L.pitch, (cuuint64_t)L.rows, (cuuint64_t)nplanes};
+  cuuint64_t dims[3] = {(cuuint64_t)L.pitch, (cuuint64_t)L.rows, (cuuint64_t)planes};
   cuuint64_t strides[2] = {(cuuint64_t)L.pitch * 4, (cuuint64_t)L.plane * 4};
-  cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)nplanes};
+  cuuint32_t box[3] = {(cuuint32_t)mlsw::kMarchCols, 1, (cuuint32_t)planes};
   cuuint32_t es[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -254,6 +257,48 @@ cudaError_t copy_planes(mlsw_handle* h, float* host, const float* dev, bool to_h
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+// planes per layer of the state buffers, as the read-out launches take them
+int state_planes(const mlsw_handle* h) { return h->moments ? mlsw::kMomPlanes : h->Q; }
+
+// The state for an analysis: populations while they are at hand (given by
+// the caller, or the form the lattice is stored in), else moments.
+struct StateView {
+  const float* f;
+  int Q;
+};
+StateView view(const mlsw_handle* h) {
+  if (h->moments && h->origin == mlsw_handle::kGiven) return {h->pop, h->Q};
+  return {h->f[h->cur], state_planes(h)};
+}
+
+// The populations of the current state (on the handle's stream).
+cudaError_t populations(mlsw_handle* h, const float** f) {
+  *f = h->moments ? h->pop : h->f[h->cur];
+  if (!h->moments || h->origin == mlsw_handle::kGiven) return cudaSuccess;
+  h->launches += 1;
+  if (h->origin == mlsw_handle::kAtRest)
+    return mlsw::launch_rest_populations(h->p.n_layers, h->kp.L, h->f[h->cur], h->pop, h->stream);
+  mlsw::StepLaunch a;
+  a.lattice = h->p.lattice;
+  a.P = h->kp;
+  a.status = h->status + 1;
+  a.num_sms = h->num_sms;
+  a.fin = h->f[h->cur ^ 1];
+  a.fin_map = &h->map[h->cur ^ 1];
+  a.fout = h->pop;
+  a.to_populations = 1;
+  return mlsw::launch_step(a, h->stream);
+}
+
+// After populations were written to *f (real cells): the state is theirs.
+cudaError_t adopt_populations(mlsw_handle* h) {
+  h->launches += 1;
+  if (!h->moments)
+    return mlsw::launch_fill_ghosts(h->p.n_layers * h->Q, h->kp.L, h->f[h->cur], h->stream);
+  h->origin = mlsw_handle::kGiven;
+  return mlsw::launch_moments(h->p.n_layers, h->kp.L, h->pop, h->f[h->cur], h->stream);
 }
 
 void set_shift(KParams& kp, mlsw::KShift& sh, int n, const float* H) {
@@ -325,9 +370,8 @@ int prepare_instance(const mlsw_params& p, const float* h_init, KParams& kp, mls
   }
   kp = make_kparams(p);
   kp.L = make_layout(p);
-  // the step kernels address a layer's planes with 32-bit offsets
-  if ((double)kp.L.plane * Qof(p.lattice) >= 2147483647.0) return MLSW_ERR_UNSUPPORTED;
-  set_ghost_tables(kp, p);
+  if (too_large(p)) return MLSW_ERR_UNSUPPORTED;
+  kp.tiny = p.nx < 4 ? 1 : 0;
   set_shift(kp, sh, n, shift);
   return MLSW_OK;
 }
@@ -418,6 +462,7 @@ void mlswlbm_destroy(mlsw_handle* h) {
   cudaStreamSynchronize(h->stream);
   cudaFree(h->f[0]);
   cudaFree(h->f[1]);
+  cudaFree(h->pop);
   cudaFree(h->hbuf);
   cudaFree(h->status);
   cudaFree(h->partials);
@@ -446,7 +491,8 @@ int mlswlbm_create(const mlsw_params* p, const float* h_init, void* stream, mlsw
   h->sh = sh;
   h->Q = Qof(p->lattice);
   h->ncell = ncell;
-  h->flen = (size_t)n * h->Q * h->kp.L.plane;
+  h->moments = p->lattice == MLSW_D2Q9 && mlsw::step_moments(kp);
+  const size_t flen = (size_t)n * state_planes(h) * kp.L.plane;
   h->stream = (cudaStream_t)stream;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -456,13 +502,6 @@ int mlswlbm_create(const mlsw_params* p, const float* h_init, void* stream, mlsw
   }
   h->num_sms = sms > 0 ? sms : 1;
   h->nblk_diag = 2 * h->num_sms;
-  {
-    // a buffer that fits in 90 % of the L2 is kept there between steps
-    int l2 = 0;
-    if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) l2 = 0;
-    const double buf = (double)h->flen * sizeof(float);
-    h->kp.l2_policy = (l2 > 0 && buf <= 0.9 * l2) ? mlsw::kL2Resident : mlsw::kL2Stream;
-  }
   if (!(p->flags & MLSW_FLAG_NO_PERSISTENT)) {
     int optin = 0;
     const size_t need = mlsw::step_persistent_smem(n, p->lattice, p->nx);
@@ -471,10 +510,12 @@ int mlswlbm_create(const mlsw_params* p, const float* h_init, void* stream, mlsw
         need <= (size_t)optin)
       h->psmem = need;
   }
-  bool ok = cudaMalloc(&h->f[0], h->flen * sizeof(float)) == cudaSuccess &&
-            cudaMalloc(&h->f[1], h->flen * sizeof(float)) == cudaSuccess &&
+  bool ok = cudaMalloc(&h->f[0], flen * sizeof(float)) == cudaSuccess &&
+            cudaMalloc(&h->f[1], flen * sizeof(float)) == cudaSuccess &&
+            (!h->moments ||
+             cudaMalloc(&h->pop, (size_t)n * h->Q * kp.L.plane * sizeof(float)) == cudaSuccess) &&
             cudaMalloc(&h->hbuf, (size_t)n * ncell * sizeof(float)) == cudaSuccess &&
-            cudaMalloc(&h->status, 4 * sizeof(int)) == cudaSuccess &&
+            cudaMalloc(&h->status, 2 * sizeof(int)) == cudaSuccess &&
             cudaMalloc(&h->partials, (size_t)h->nblk_diag * (n + 2) * sizeof(double)) ==
                 cudaSuccess &&
             cudaMalloc(&h->dout, (size_t)(n + 2) * sizeof(double)) == cudaSuccess &&
@@ -485,22 +526,20 @@ int mlswlbm_create(const mlsw_params* p, const float* h_init, void* stream, mlsw
     mlswlbm_destroy(h);
     return MLSW_ERR_NOMEM;
   }
-  // zero padding: cells outside the real domain and its ghost ring are read
-  // by edge tiles but never feed a real cell
-  if (cudaMemsetAsync(h->status, 0, 4 * sizeof(int), h->stream) != cudaSuccess ||
-      cudaMemsetAsync(h->f[0], 0, h->flen * sizeof(float), h->stream) != cudaSuccess ||
-      cudaMemsetAsync(h->f[1], 0, h->flen * sizeof(float), h->stream) != cudaSuccess) {
+  // zero padding: columns outside the real domain and its ghosts are read by
+  // edge strips but never feed a real cell
+  if (cudaMemsetAsync(h->status, 0, 2 * sizeof(int), h->stream) != cudaSuccess ||
+      cudaMemsetAsync(h->f[0], 0, flen * sizeof(float), h->stream) != cudaSuccess ||
+      cudaMemsetAsync(h->f[1], 0, flen * sizeof(float), h->stream) != cudaSuccess) {
     mlswlbm_destroy(h);
     return MLSW_ERR_CUDA;
   }
   if (p->lattice == MLSW_D2Q9) {
-    const int bc = mlsw::step_tile_cols(p->lattice) + 8;
-    const int br = mlsw::step_tile_rows(n, p->lattice) + 4;
-    if (!make_tile_map(&h->map[0], h->f[0], h->kp.L, n * h->Q, bc, br) ||
-        !make_tile_map(&h->map[1], h->f[1], h->kp.L, n * h->Q, bc, br)) {
-      mlswlbm_destroy(h);
-      return MLSW_ERR_CUDA;
-    }
+    for (int k = 0; k < 2; ++k)
+      if (!make_row_map(&h->map[k], h->f[k], h->kp.L, n * state_planes(h))) {
+        mlswlbm_destroy(h);
+        return MLSW_ERR_CUDA;
+      }
   }
   rc = mlswlbm_set_heights(h, h_init);
   if (rc == MLSW_OK && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = MLSW_ERR_CUDA;
@@ -522,16 +561,18 @@ int mlswlbm_set_heights(mlsw_handle* h, const float* h_in) {
     CU(cudaMemcpyAsync(h->hbuf, h_in, bytes, cudaMemcpyHostToDevice, h->stream));
     src = h->hbuf;
   }
-  CU(mlsw::launch_init(h->Q, h->p.n_layers, h->kp.L, h->p.lattice == MLSW_D2Q9, src,
-                       h->f[h->cur], h->sh, h->status, h->stream));
+  CU(mlsw::launch_init(state_planes(h), h->p.n_layers, h->kp.L, src, h->f[h->cur], h->sh,
+                       h->status, h->stream));
+  h->origin = mlsw_handle::kAtRest;
   h->launches += 1;
   return MLSW_OK;
 }
 
 int mlswlbm_set_heights_device(mlsw_handle* h, const float* dev_in) {
   if (!h || !dev_in) return MLSW_ERR_ARG;
-  CU(mlsw::launch_init(h->Q, h->p.n_layers, h->kp.L, h->p.lattice == MLSW_D2Q9, dev_in,
-                       h->f[h->cur], h->sh, h->status, h->stream));
+  CU(mlsw::launch_init(state_planes(h), h->p.n_layers, h->kp.L, dev_in, h->f[h->cur], h->sh,
+                       h->status, h->stream));
+  h->origin = mlsw_handle::kAtRest;
   h->launches += 1;
   return MLSW_OK;
 }
@@ -542,9 +583,8 @@ int mlswlbm_step(mlsw_handle* h, long nsteps) {
   a.lattice = h->p.lattice;
   a.P = h->kp;
   a.status = h->status;
-  a.sched = h->status + 1;
   a.num_sms = h->num_sms;
-  a.reverse = 0;
+  a.to_populations = 0;
   if (h->psmem) {
     // whole lattice in one CTA: chunks of steps per launch
     constexpr long kChunk = 16384;
@@ -563,21 +603,16 @@ int mlswlbm_step(mlsw_handle* h, long nsteps) {
     a.fin = h->f[h->cur];
     a.fout = h->f[h->cur ^ 1];
     a.fin_map = &h->map[h->cur];
-    // unless a whole buffer stays in the L2, steps from buffer 1 run their
-    // tiles in reverse order: every step then begins with the rows its
-    // predecessor wrote last, which the L2 still holds (the results do not
-    // depend on the order)
-    a.reverse = h->kp.l2_policy == mlsw::kL2Stream ? h->cur : 0;
     CU(mlsw::launch_step(a, h->stream));
     h->launches += 1;
     if (h->kp.tiny) {
-      // a side below 4 cells: a real cell can have several ghost images,
+      // fewer than 4 columns: a real cell can have several ghost images,
       // which a separate pass refreshes
-      CU(mlsw::launch_fill_ghosts(h->p.n_layers * h->Q, h->kp.L, h->p.lattice == MLSW_D2Q9,
-                                  a.fout, h->stream));
+      CU(mlsw::launch_fill_ghosts(h->p.n_layers * h->Q, h->kp.L, a.fout, h->stream));
       h->launches += 1;
     }
     h->cur ^= 1;
+    h->origin = mlsw_handle::kStepped;
   }
   return MLSW_OK;
 }
@@ -596,7 +631,7 @@ int mlswlbm_status(mlsw_handle* h) {
 
 int mlswlbm_get_heights_device(mlsw_handle* h, float* dev_out) {
   if (!h || !dev_out) return MLSW_ERR_ARG;
-  CU(mlsw::launch_heights(h->Q, h->p.n_layers, h->kp.L, h->f[h->cur], h->sh, dev_out,
+  CU(mlsw::launch_heights(state_planes(h), h->p.n_layers, h->kp.L, h->f[h->cur], h->sh, dev_out,
                           h->stream));
   h->launches += 1;
   return MLSW_OK;
@@ -608,7 +643,7 @@ int mlswlbm_get_heights(mlsw_handle* h, float* out) {
   // kernel also mirrors the status word to the host, so one
   // synchronisation serves both
   float* mapped = static_cast<float*>(const_cast<void*>(mapped_host_ptr(out)));
-  CU(mlsw::launch_heights(h->Q, h->p.n_layers, h->kp.L, h->f[h->cur], h->sh,
+  CU(mlsw::launch_heights(state_planes(h), h->p.n_layers, h->kp.L, h->f[h->cur], h->sh,
                           mapped ? mapped : h->hbuf, h->stream, h->status, h->status_mirror));
   h->launches += 1;
   if (!mapped) {
@@ -627,9 +662,11 @@ int mlswlbm_get_state(mlsw_handle* h, float* f_out) {
   const size_t plane = (size_t)h->ncell;
   // rest planes H_i + g_0 into the height buffer, all planes raw to the host,
   // then the rest planes over their raw copies
-  CU(mlsw::launch_rest_planes(h->Q, n, h->kp.L, h->f[h->cur], h->sh, h->hbuf, h->stream));
+  const float* f;
+  CU(populations(h, &f));
+  CU(mlsw::launch_rest_planes(h->Q, n, h->kp.L, f, h->sh, h->hbuf, h->stream));
   h->launches += 1;
-  CU(copy_planes(h, f_out, h->f[h->cur], true));
+  CU(copy_planes(h, f_out, f, true));
   for (int i = 0; i < n; ++i)
     CU(cudaMemcpyAsync(f_out + (size_t)i * h->Q * plane, h->hbuf + (size_t)i * plane,
                        plane * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
@@ -639,11 +676,11 @@ int mlswlbm_get_state(mlsw_handle* h, float* f_out) {
 
 int mlswlbm_set_state(mlsw_handle* h, const float* f_in) {
   if (!h || !f_in) return MLSW_ERR_ARG;
-  CU(copy_planes(h, const_cast<float*>(f_in), h->f[h->cur], false));
-  CU(mlsw::launch_shift(h->Q, h->p.n_layers, h->kp.L, h->f[h->cur], h->sh, -1.f, h->stream));
-  CU(mlsw::launch_fill_ghosts(h->p.n_layers * h->Q, h->kp.L, h->p.lattice == MLSW_D2Q9,
-                              h->f[h->cur], h->stream));
-  h->launches += 2;
+  float* f = h->moments ? h->pop : h->f[h->cur];
+  CU(copy_planes(h, const_cast<float*>(f_in), f, false));
+  CU(mlsw::launch_shift(h->Q, h->p.n_layers, h->kp.L, f, h->sh, -1.f, h->stream));
+  h->launches += 1;
+  CU(adopt_populations(h));
   CU(cudaStreamSynchronize(h->stream));
   return MLSW_OK;
 }
@@ -651,7 +688,9 @@ int mlswlbm_set_state(mlsw_handle* h, const float* f_in) {
 int mlswlbm_save_state(mlsw_handle* h, float* H_out, float* g_out) {
   if (!h || !H_out || !g_out) return MLSW_ERR_ARG;
   for (int i = 0; i < h->p.n_layers; ++i) H_out[i] = h->sh.H[i];
-  CU(copy_planes(h, g_out, h->f[h->cur], true));
+  const float* f;
+  CU(populations(h, &f));
+  CU(copy_planes(h, g_out, f, true));
   CU(cudaStreamSynchronize(h->stream));
   return MLSW_OK;
 }
@@ -662,10 +701,8 @@ int mlswlbm_load_state(mlsw_handle* h, const float* H_in, const float* g_in) {
     if (!std::isfinite(H_in[i])) return MLSW_ERR_ARG;
   CU(cudaStreamSynchronize(h->stream));
   set_shift(h, H_in);
-  CU(copy_planes(h, const_cast<float*>(g_in), h->f[h->cur], false));
-  CU(mlsw::launch_fill_ghosts(h->p.n_layers * h->Q, h->kp.L, h->p.lattice == MLSW_D2Q9,
-                              h->f[h->cur], h->stream));
-  h->launches += 1;
+  CU(copy_planes(h, const_cast<float*>(g_in), h->moments ? h->pop : h->f[h->cur], false));
+  CU(adopt_populations(h));
   CU(cudaStreamSynchronize(h->stream));
   return MLSW_OK;
 }
@@ -673,7 +710,8 @@ int mlswlbm_load_state(mlsw_handle* h, const float* H_in, const float* g_in) {
 int mlswlbm_get_diagnostics(mlsw_handle* h, double* mass, double* kinetic, double* hmin) {
   if (!h) return MLSW_ERR_ARG;
   const int n = h->p.n_layers;
-  CU(mlsw::launch_diagnostics(h->p.lattice, n, h->kp.L, h->f[h->cur], h->sh, h->partials,
+  const StateView v = view(h);
+  CU(mlsw::launch_diagnostics(v.Q, n, h->kp.L, v.f, h->sh, h->partials,
                               h->nblk_diag, h->dout, h->stream));
   h->launches += 2;
   double res[MLSW_MAX_LAYERS + 2];
@@ -708,7 +746,8 @@ int mlswlbm_get_free_energy(mlsw_handle* h, double* F) {
   E.sub_amp = p.sub_amp;
   E.sub_kx = p.sub_kx;
   E.sub_ky = p.sub_ky;
-  CU(mlsw::launch_heights(h->Q, p.n_layers, h->kp.L, h->f[h->cur], h->sh, h->hbuf, h->stream));
+  const StateView v = view(h);
+  CU(mlsw::launch_heights(v.Q, p.n_layers, h->kp.L, v.f, h->sh, h->hbuf, h->stream));
   CU(mlsw::launch_free_energy(E, h->hbuf, h->partials, h->nblk_diag, h->dout, h->stream));
   h->launches += 3;
   CU(cudaMemcpyAsync(F, h->dout, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -739,7 +778,7 @@ int mlswlbm_get_spectrum(mlsw_handle* h, int nbins, double* out) {
   std::vector<unsigned long long> hc(nbins);
   ok = cudaMemsetAsync(bins, 0, (size_t)n * nbins * sizeof(double), st) == cudaSuccess &&
        cudaMemsetAsync(counts, 0, (size_t)nbins * sizeof(unsigned long long), st) == cudaSuccess &&
-       mlsw::launch_spectrum(h->Q, n, h->kp.L, h->f[h->cur], nbins, work, bins, counts, st) ==
+       mlsw::launch_spectrum(view(h).Q, n, h->kp.L, view(h).f, nbins, work, bins, counts, st) ==
            cudaSuccess &&
        cudaMemcpyAsync(hb.data(), bins, hb.size() * sizeof(double), cudaMemcpyDeviceToHost, st) ==
            cudaSuccess &&
@@ -787,7 +826,7 @@ int mlswlbm_get_radial_profile(mlsw_handle* h, double cx, double cy, int nbins, 
   std::vector<unsigned long long> hc(nbins);
   ok = cudaMemsetAsync(sums, 0, nsum * sizeof(double), st) == cudaSuccess &&
        cudaMemsetAsync(cnt, 0, (size_t)nbins * sizeof(unsigned long long), st) == cudaSuccess &&
-       mlsw::launch_radial_profile(h->Q, n, h->kp.L, h->f[h->cur], h->sh, A, sums, cnt, st) ==
+       mlsw::launch_radial_profile(view(h).Q, n, h->kp.L, view(h).f, h->sh, A, sums, cnt, st) ==
            cudaSuccess &&
        cudaMemcpyAsync(hs.data(), sums, nsum * sizeof(double), cudaMemcpyDeviceToHost, st) ==
            cudaSuccess &&
@@ -904,9 +943,12 @@ int mlswlbm_debug_bounds_violations(unsigned long long* count) {
   if (!count) return MLSW_ERR_ARG;
 #ifdef MLSW_DEBUG
   if (cudaDeviceSynchronize() != cudaSuccess) return MLSW_ERR_CUDA;
-  const unsigned parts[4] = {mlsw::bounds_violations_step(), mlsw::bounds_violations_aux(),
-                             mlsw::bounds_violations_analysis(),
-                             mlsw::bounds_violations_batch()};
+  const unsigned parts[] = {
+      mlsw::bounds_violations_step(),   mlsw::bounds_violations_aux(),
+      mlsw::bounds_violations_analysis(), mlsw::bounds_violations_d2q9_1(),
+      mlsw::bounds_violations_d2q9_2(), mlsw::bounds_violations_d2q9_3(),
+      mlsw::bounds_violations_d2q9_4(), mlsw::bounds_violations_d2q9_5(),
+      mlsw::bounds_violations_batch_3(), mlsw::bounds_violations_batch_5()};
   unsigned long long total = 0;
   for (unsigned v : parts) {
     if (v == ~0u) return MLSW_ERR_CUDA;

@@ -57,6 +57,7 @@ extern "C" int mlswlbm_diagnostics_noalloc(const mlsw_params* p, const float* f,
   if (!p || !f || !out) return MLSW_ERR_ARG;
   if (mlswlbm_check_params(p) != MLSW_OK) return MLSW_ERR_ARG;
   const int n = p->n_layers;
+  const int Q = p->lattice == MLSW_D1Q3 ? 3 : 9;
   const long ncell = (long)p->nx * p->ny;
   const long nblk = (ncell + kNoallocCellsPerBlock - 1) / kNoallocCellsPerBlock;
   if (nblk > kNoallocBlocks) return MLSW_ERR_UNSUPPORTED;  // beyond the static scratch
@@ -72,7 +73,7 @@ extern "C" int mlswlbm_diagnostics_noalloc(const mlsw_params* p, const float* f,
   if (scratch_of_device(dev, &scratch) != cudaSuccess) return MLSW_ERR_CUDA;
   // every block writes its own partials, so nothing needs clearing first
   const cudaError_t e =
-      mlsw::launch_diagnostics(p->lattice, n, mlsw::dense_layout(p->nx, p->ny, n * (p->lattice == MLSW_D1Q3 ? 3 : 9)), f, sh,
-                               scratch, (int)nblk, out, (cudaStream_t)stream);
+      mlsw::launch_diagnostics(Q, n, mlsw::dense_layout(p->nx, p->ny, n * Q), f, sh, scratch,
+                               (int)nblk, out, (cudaStream_t)stream);
   return e == cudaSuccess ? MLSW_OK : MLSW_ERR_CUDA;
 }

@@ -20,6 +20,8 @@ constexpr int kMaxLayers = 5;
 // them through mlswlbm_debug_bounds_violations. Release builds compile
 // none of this.
 // ---------------------------------------------------------------------------
+#define MLSW_CAT2(a, b) a##b
+#define MLSW_CAT(a, b) MLSW_CAT2(a, b)
 #ifdef MLSW_DEBUG
 static __device__ unsigned int g_bounds_violations;
 __device__ __forceinline__ void note_bounds_violation() { atomicAdd(&g_bounds_violations, 1u); }
@@ -46,30 +48,30 @@ __device__ __forceinline__ void note_bounds_violation() { atomicAdd(&g_bounds_vi
 // storing f_0 itself loses the capillary signal; the shift keeps ~1e-10.
 // The arithmetic of the scheme is unchanged: only the representation of
 // f_0 moves by a constant.
-// Device layout of a population buffer: every plane (layer i, direction k,
-// plane index i * Q + k) is a padded 2-D array of `rows` rows of `pitch`
-// floats; the real cell (x, y) sits at row y + gy, column x + gx. The ring
-// of ghost cells within two cells of the real domain (x in [-2, nx + 2),
-// y in [-2, ny + 2) for D2Q9; x only for D1Q3) holds the periodic images of
-// the real cells, so the step kernels read a tile plus its halo without
-// any wrap-around arithmetic. gx = 4 keeps every tile's box 16-byte aligned
-// for the tensor-memory-access unit; pitch and rows cover whole tiles.
+// Device layout of a state buffer: every plane (layer i, direction k: plane
+// i * Q + k; or moment q: plane 4 i + q) is a padded 2-D array of `rows` rows
+// of `pitch` floats; the real cell (x, y) sits at row y, column x + gx. The
+// ghost columns [-4, 0) and [nx, nx + 4) hold the periodic images of the real
+// ones, so the step kernels read a strip plus its halo without any
+// wrap-around arithmetic; rows are wrapped by the reader. gx keeps every row
+// copy 16-byte aligned for the tensor-memory-access unit and, on D2Q9, every
+// strip's stores on whole 32-byte sectors.
 struct Layout {
   int nx, ny;    // real lattice
-  int gx, gy;    // padded position of the real cell (0, 0)
+  int gx;        // padded column of the real cell (0, 0)
   int pitch;     // floats per padded row (multiple of 4)
   int rows;      // padded rows per plane
   long plane;    // pitch * rows
   int nplanes;   // planes of a buffer (0: not known, planes are then not checked)
   __host__ __device__ long at(int p, int x, int y) const {
 #if defined(MLSW_DEBUG) && defined(__CUDA_ARCH__)
-    if (x + gx < 0 || x + gx >= pitch || y + gy < 0 || y + gy >= rows || p < 0 ||
+    if (x + gx < 0 || x + gx >= pitch || y < 0 || y >= rows || p < 0 ||
         (nplanes > 0 && p >= nplanes)) {
       note_bounds_violation();
       return 0;
     }
 #endif
-    return (long)p * plane + (long)(y + gy) * pitch + (x + gx);
+    return (long)p * plane + (long)y * pitch + (x + gx);
   }
   // floats of one buffer (0 when the plane count is not known)
   __host__ __device__ long length() const { return (long)nplanes * plane; }
@@ -82,6 +84,7 @@ struct KParams {
   float gamma[kMaxLayers];           // gamma_{i,i+1}
   float S[kMaxLayers][kMaxLayers];   // S[l][k-1] = S_{lk}
   float Sd[kMaxLayers];              // S_{l1} nw mw / (nw - mw)
+  int far_pairs;                     // 1: some S_{lk} with k >= 2 is not zero
   // friction (see friction()): -1 / (6 mu_i), beta_i / mu_i, beta_i^2 / (2 mu_i)
   float fr_visc[kMaxLayers], fr_slip[kMaxLayers], fr_slip2[kMaxLayers];
   float hstar;
@@ -92,12 +95,9 @@ struct KParams {
   // Hsum[l][m] = H_{l+1} + ... + H_m (1-based layers, 0 <= l < m <= n): the
   // reference part of the thickness z_m - z_l between interfaces l and m
   float Hsum[kMaxLayers + 1][kMaxLayers + 1];
-  Layout L;                          // padded layout of both population buffers
-  // periodic images: ghost column gcol[g] (g = 0..3 for x = -2, -1, nx,
-  // nx + 1) holds real column gsrcx[g]; likewise rows
-  int gsrcx[4], gsrcy[4];
-  // 1 when a side of the lattice is shorter than 4 cells: a real column or
-  // row can then have several ghost images
+  Layout L;                          // padded layout of the state buffers
+  // 1 when the lattice has fewer than 4 columns: a real column can then have
+  // several ghost images
   int tiny;
   // substrate z_0(x, y) = sub_amp cos(2 pi (sub_kx x / nx + sub_ky y / ny));
   // sub_amp = 0 is the flat substrate
@@ -107,15 +107,14 @@ struct KParams {
   // phi_k(d) = 2 a - a^2, a = e^{-kappa (d - k h*)}
   int wet_kind;
   float kappa;
-  // L2 cache policy of the D2Q9 step (see d2q9_tile_loop): kL2None,
-  // kL2Stream or kL2Resident
-  int l2_policy;
 };
 
-// kL2None: no cache hints (batches, whose many lattices stream through);
-// kL2Stream: a lattice larger than the L2, output kept as long as possible;
-// kL2Resident: one population buffer fits in the L2 and stays there.
-enum L2Policy { kL2None = 0, kL2Stream = 1, kL2Resident = 2 };
+// Substrate height at phase 2 pi m / nc, 0 <= m < nc
+__device__ __forceinline__ float substrate_height(const KParams& P, long m, long nc) {
+  float s, c;
+  sincospif(2.f * (float)((double)m / (double)nc), &s, &c);
+  return P.sub_amp * c;
+}
 
 // Substrate height at lattice cell (x, y) (any integers: the cosine is
 // periodic); the phase is reduced exactly in integers.
@@ -124,9 +123,7 @@ __device__ __forceinline__ float substrate_at(const KParams& P, int x, int y) {
   long m = ((long)P.sub_kx * x % nx) * ny + ((long)P.sub_ky * y % ny) * nx;
   m %= nc;
   if (m < 0) m += nc;
-  float s, c;
-  sincospif(2.f * (float)((double)m / (double)nc), &s, &c);
-  return P.sub_amp * c;
+  return substrate_height(P, m, nc);
 }
 
 // ---------------------------------------------------------------------------
@@ -208,10 +205,28 @@ __device__ __forceinline__ f2 rcp(f2 x) { return mk2(rcp(x.v.x), rcp(x.v.y)); }
 __device__ __forceinline__ float expv(float x) { return expf(x); }
 __device__ __forceinline__ f2 expv(f2 x) { return mk2(expf(x.v.x), expf(x.v.y)); }
 
+// v or exactly 0
+__device__ __forceinline__ float keep_if(bool c, float v) { return c ? v : 0.f; }
+__device__ __forceinline__ f2 keep_if(bool c, f2 v) {
+  return mk2(c ? v.v.x : 0.f, c ? v.v.y : 0.f);
+}
+
+// r^e, e >= 0 a uniform run-time exponent: squares, with the factors of the
+// low three bits chosen by selects (exponents in use are small) and a loop
+// for the rest
 template <class T>
 __device__ __forceinline__ T ipow(T r, int e) {
-  T a = Num<T>::splat(1.f);
-  for (int i = 0; i < e; ++i) a = a * r;
+  const T one = Num<T>::splat(1.f), r2 = r * r, r4 = r2 * r2;
+  T a = ((e & 1) ? r : one) * ((e & 2) ? r2 : one);
+  a = a * ((e & 4) ? r4 : one);
+  if (e >= 8) {
+    T s = r4 * r4;
+#pragma unroll 1
+    for (e >>= 3;; s = s * s) {
+      if (e & 1) a = a * s;
+      if ((e >>= 1) == 0) break;
+    }
+  }
   return a;
 }
 
@@ -236,68 +251,95 @@ __device__ __forceinline__ T ipow(T r, int e) {
 // as phi = r^2 (3 - 2 r), phi' = 6 r^2 (r - 1) / d.
 // z0, sg0: the substrate height z_0 (on the scale of zd) and 1 + |grad z_0|^2 / 2
 // at the cell; null for the flat substrate (0 and 1).
+//
+// Without NN or W32 the options are run-time values, but uniform ones: the
+// pairs are evaluated in straight-line code for one combination (with or
+// without far pairs, either potential), chosen once, so that the latencies
+// of the pairs overlap. A pair without a coefficient contributes exactly
+// nothing, whatever its potential evaluates to.
+enum PairForm { kPower32, kPower, kExponential };
+
+template <int N, bool FAR, int FORM, class T>
+__device__ __forceinline__ void interface_pairs(const KParams& P, const T (&zd)[N],
+                                                const T (&sg)[N], const T* z0, const T* sg0,
+                                                T (&ten)[N], T (&pi)[N]) {
+#pragma unroll
+  for (int l = 0; l < N; ++l) {
+    const int i = l > 0 ? l - 1 : 0;
+#pragma unroll
+    for (int m = l + 1; m <= (FAR ? N : l + 1); ++m) {
+      const int k = m - l;
+      const float s = P.S[l][k - 1];
+      T d;
+      if (l > 0)
+        d = (zd[m - 1] - zd[i]) + P.Hsum[l][m];
+      else if (z0)
+        d = (zd[m - 1] - *z0) + P.Hsum[l][m];
+      else
+        d = zd[m - 1] + P.Hsum[l][m];
+      T phi, e;  // phi_k, S phi_k'
+      if constexpr (FORM == kExponential) {
+        // charged surfaces: a = e^{-kappa (d - k h*)}, phi = 2 a - a^2,
+        // phi' = 2 kappa a (a - 1)
+        const T a = expv(fmav(d, -P.kappa, P.kappa * ((float)k * P.hstar)));
+        phi = a * (2.f - a);
+        e = (s * (2.f * P.kappa)) * (a * (a - 1.f));
+      } else {
+        const T inv_d = rcp(d);
+        const T r = ((float)k * P.hstar) * inv_d;
+        if constexpr (FORM == kPower32) {
+          const T r2 = r * r;
+          phi = r2 * fmav(r, -2.f, 3.f);
+          e = (k == 1 ? P.Sd[l] : s * P.c_dphi) * ((r2 * (r - 1.f)) * inv_d);
+        } else {
+          const T rm = ipow(r, P.mw), rn = rm * ipow(r, P.nw - P.mw);
+          phi = fmav(rm, (float)P.nw, rn * (-(float)P.mw)) * P.c_phi;
+          e = (s * P.c_dphi) * ((rn - rm) * inv_d);
+        }
+      }
+      // explicit fused updates, so one cell and a packed pair of cells
+      // round identically
+      if (l > 0)
+        e = e * sg[i];
+      else if (sg0)
+        e = e * *sg0;
+      if constexpr (FORM != kPower32) {  // r^64 of a thin film may overflow
+        phi = keep_if(s != 0.f, phi);
+        e = keep_if(s != 0.f, e);
+      }
+      if (l > 0) {
+        ten[i] = fmav(s, phi, ten[i]);
+        pi[i] = pi[i] + e;
+      }
+      pi[m - 1] = pi[m - 1] - e;
+    }
+  }
+}
+
 template <int N, bool W32, class T, bool NN = false>
 __device__ __forceinline__ void neg_pressures(const KParams& P, const T (&zd)[N], const T (&gx)[N],
                                               const T (&gy)[N], const T (&lz)[N], T (&q)[N],
                                               const T* z0 = nullptr, const T* sg0 = nullptr) {
-  T ten[N], pi[N];  // tension of the interface; -Pi of the layer
+  T ten[N], pi[N], sg[N];  // tension of the interface; -Pi of the layer; slope factor
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     ten[i] = Num<T>::splat(P.gamma[i]);
     pi[i] = Num<T>::splat(0.f);
+    sg[i] = fmav(0.5f, fmav(gx[i], gx[i], gy[i] * gy[i]), Num<T>::splat(1.f));
   }
-#pragma unroll
-  for (int l = 0; l < N; ++l) {
-    T sgl;
-    if (l > 0) {
-      const int i = l > 0 ? l - 1 : 0;
-      sgl = fmav(0.5f, fmav(gx[i], gx[i], gy[i] * gy[i]), Num<T>::splat(1.f));
-    }
-#pragma unroll
-    for (int m = l + 1; m <= (NN ? l + 1 : N); ++m) {
-      const int k = m - l;
-      const float s = P.S[l][k - 1];
-      if (NN || s != 0.f) {
-        T d;
-        if (l > 0)
-          d = (zd[m - 1] - zd[l > 0 ? l - 1 : 0]) + P.Hsum[l][m];
-        else if (z0)
-          d = (zd[m - 1] - *z0) + P.Hsum[l][m];
-        else
-          d = zd[m - 1] + P.Hsum[l][m];
-        T phi, e;  // e = S phi'
-        if (!W32 && P.wet_kind == 1) {
-          // charged surfaces: a = e^{-kappa (d - k h*)}, phi = 2 a - a^2,
-          // phi' = 2 kappa a (a - 1)
-          const T a = expv(fmav(d, -P.kappa, P.kappa * ((float)k * P.hstar)));
-          phi = a * (2.f - a);
-          e = s * ((2.f * P.kappa) * (a * (a - 1.f)));
-        } else {
-          const T inv_d = rcp(d);
-          const T r = ((float)k * P.hstar) * inv_d;
-          if constexpr (W32) {
-            const T r2 = r * r;
-            phi = r2 * fmav(r, -2.f, 3.f);
-            e = (NN ? P.Sd[l] : s * P.c_dphi) * ((r2 * (r - 1.f)) * inv_d);
-          } else {
-            const T rm = ipow(r, P.mw), rn = rm * ipow(r, P.nw - P.mw);
-            phi = fmav(rm, (float)P.nw, -(float)P.mw * rn) * P.c_phi;
-            e = s * ((P.c_dphi * (rn - rm)) * inv_d);
-          }
-        }
-        // explicit fused updates, so one cell and a packed pair of cells
-        // round identically
-        if (l > 0) {
-          const int i = l > 0 ? l - 1 : 0;
-          e = e * sgl;
-          ten[i] = fmav(s, phi, ten[i]);
-          pi[i] = pi[i] + e;
-        } else if (sg0) {
-          e = e * *sg0;
-        }
-        pi[m - 1] = pi[m - 1] - e;
-      }
-    }
+  if constexpr (NN && W32) {
+    interface_pairs<N, false, kPower32>(P, zd, sg, z0, sg0, ten, pi);
+  } else if constexpr (W32) {
+    if (P.far_pairs)
+      interface_pairs<N, true, kPower32>(P, zd, sg, z0, sg0, ten, pi);
+    else
+      interface_pairs<N, false, kPower32>(P, zd, sg, z0, sg0, ten, pi);
+  } else if (P.wet_kind == 1) {
+    interface_pairs<N, true, kExponential>(P, zd, sg, z0, sg0, ten, pi);
+  } else if (P.far_pairs) {
+    interface_pairs<N, true, kPower>(P, zd, sg, z0, sg0, ten, pi);
+  } else {
+    interface_pairs<N, false, kPower>(P, zd, sg, z0, sg0, ten, pi);
   }
   T acc = Num<T>::splat(0.f);
 #pragma unroll

@@ -60,11 +60,12 @@ __device__ __forceinline__ long chk_offset(long i, long len) {
 #endif
   return i;
 }
-// global store target: p inside [base, base + len)
-__device__ __forceinline__ float* chk_global(float* base, float* p, long len) {
+// global store target: p[0 .. count) inside [base, base + len), aligned for
+// one access
+__device__ __forceinline__ float* chk_global(float* base, float* p, long len, int count = 1) {
 #ifdef MLSW_DEBUG
   const long i = p - base;
-  if (i < 0 || i >= len) {
+  if (i < 0 || i + count > len || (reinterpret_cast<uintptr_t>(p) & (4 * count - 1)) != 0) {
     note_bounds_violation();
     return base;
   }
@@ -89,11 +90,11 @@ __device__ __forceinline__ void store_edge(float* __restrict__ plane_base, const
                                            int dx, int dy, int xi, int yi, float v) {
   // indices into the plane (not derived pointers), so that the stores keep
   // the base pointer's no-alias guarantee
-  const long r0 = (long)(dy + L.gy) * L.pitch;
+  const long r0 = (long)dy * L.pitch;
   plane_base[chk_offset(r0 + dx + L.gx, L.plane)] = v;
   if (xi != kNoImage) plane_base[chk_offset(r0 + xi + L.gx, L.plane)] = v;
   if (yi != kNoImage) {
-    const long r1 = (long)(yi + L.gy) * L.pitch;
+    const long r1 = (long)yi * L.pitch;
     plane_base[chk_offset(r1 + dx + L.gx, L.plane)] = v;
     if (xi != kNoImage) plane_base[chk_offset(r1 + xi + L.gx, L.plane)] = v;
   }
@@ -199,6 +200,18 @@ __device__ __forceinline__ void collide_d2q9(const KParams& P, T g0, T small, T 
 template <class T>
 __device__ __forceinline__ T moving_sum(const T (&v)[9]) {
   return ((v[1] + v[5]) + (v[3] + v[7])) + ((v[2] + v[6]) + (v[4] + v[8]));
+}
+
+// moments of the nine populations of one layer at a cell (or a pair): the
+// rest population, the sum of the moving ones, the flux
+template <class T>
+struct Moments {
+  T g0, s, jx, jy;
+};
+template <class T>
+__device__ __forceinline__ Moments<T> moments_of(const T (&v)[9]) {
+  return {v[0], moving_sum(v), ((v[1] + v[2]) + v[8]) - ((v[4] + v[5]) + v[6]),
+          ((v[2] + v[3]) + v[4]) - ((v[6] + v[7]) + v[8])};
 }
 
 }  // namespace mlsw

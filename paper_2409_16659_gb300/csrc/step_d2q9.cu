@@ -1,0 +1,103 @@
+// step_d2q9.cu -- the D2Q9 step of one lattice: one warp (one CTA) per unit of
+// work, marching down a strip of 64 columns (march.cuh). This file is
+// compiled once per layer count MLSW_N.
+#include "march.cuh"
+
+#ifndef MLSW_N
+#error "MLSW_N: the layer count of the kernels"
+#endif
+
+namespace mlsw {
+
+// Warps per SM that the registers must allow, in moment form without spills:
+// three layers 12 (168 registers; 16 warps at 128 spill into the 15 KB of L1
+// that the rings leave: 76 us a step against 29 at 1024^2; 8 warps: 97
+// against 89 us at 2048^2), two layers 16, one layer 20, four and five 8.
+constexpr int march_min_warps(int n) { return n == 1 ? 20 : (n == 2 ? 14 : (n == 3 ? 12 : 8)); }
+
+template <int N, int MODE, bool OP>
+__global__ void __launch_bounds__(32, march_min_warps(N))
+    step_d2q9(const __grid_constant__ CUtensorMap map, float* __restrict__ fout,
+              const __grid_constant__ KParams P, int strips, int rows, int* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int strip = (int)(blockIdx.x % strips), ya = (int)(blockIdx.x / strips) * rows;
+  march_unit<N, MODE, OP>(P, &map, fout, strip * kMarchOut, ya, min(ya + rows, P.ny), smem_raw,
+                              status);
+}
+
+// Rows of a unit. A unit costs its rows plus about five rows of warm-up. On
+// a lattice that leaves each warp a scheduler of its own (4 per SM) with at
+// most 3 rows, a row takes the latency of one warp whatever the others do:
+// units are as flat as that allows (three layers, us a step: 256^2 with 1, 2,
+// 3, 4 rows 8.3, 7.8, 7.5, 8.5). Larger lattices run as one wave of the warps
+// that fit (slots), which also spreads them evenly over the SMs: 512^2 with
+// 2, 3, 4 rows 15.9, 12.4, 14.2; 1024^2 with 8, 11, 13 rows 33.3, 28.7, 32.5;
+// 2048^2 with 32, 43, 51 rows 101, 89, 104. Units taller than 64 rows would
+// put neighbouring units further apart in time than the L2 keeps the rows
+// they share; then several waves.
+static int march_rows(int ny, int strips, int num_sms, int slots) {
+  const long total = (long)ny * strips, flat = (total + 4L * num_sms - 1) / (4L * num_sms);
+  if (flat <= 3) return (int)flat;
+  for (long wave = 1;; ++wave) {
+    const long chunks = slots * wave / strips;
+    if (chunks < 1) continue;
+    const long rows = (ny + chunks - 1) / chunks;
+    if (rows <= 64) return (int)rows;
+  }
+}
+
+template <int N, int MODE, bool OP>
+static cudaError_t launch_march(const StepLaunch& a, cudaStream_t st) {
+  using S = MarchShape<N, MODE, OP>;
+  auto kern = step_d2q9<N, MODE, OP>;
+  // raise the dynamic shared-memory limit and count the resident warps once
+  // per device and instantiation
+  static unsigned long long configured = 0;
+  static int per_sm[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 64) return cudaErrorInvalidDevice;
+  if (!((configured >> dev) & 1ull)) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+    if (e != cudaSuccess) return e;
+    int nb = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 32, S::kSmem);
+    if (e != cudaSuccess) return e;
+    per_sm[dev] = nb > 0 ? nb : 1;
+    configured |= 1ull << dev;
+  }
+  const int strips = march_strips(a.P.nx);
+  const int rows = march_rows(a.P.ny, strips, a.num_sms, a.num_sms * per_sm[dev]);
+  const long units = (long)strips * ((a.P.ny + rows - 1) / rows);
+  // launched as a programmatic dependent of the previous kernel on the
+  // stream (see march_unit)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)units);
+  cfg.blockDim = dim3(32);
+  cfg.dynamicSmemBytes = S::kSmem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, *a.fin_map, a.fout, a.P, strips, rows, a.status);
+}
+
+template <>
+cudaError_t launch_step_d2q9<MLSW_N>(const StepLaunch& a, cudaStream_t st) {
+  switch (step_mode(a.P)) {
+    case kGeneral: return launch_march<MLSW_N, kGeneral, true>(a, st);
+    case kFast:
+      return a.to_populations ? launch_march<MLSW_N, kFast, true>(a, st)
+                              : launch_march<MLSW_N, kFast, false>(a, st);
+    default:
+      return a.to_populations ? launch_march<MLSW_N, kTau1, true>(a, st)
+                              : launch_march<MLSW_N, kTau1, false>(a, st);
+  }
+}
+
+MLSW_DEFINE_BOUNDS_READER(MLSW_CAT(bounds_violations_d2q9_, MLSW_N))
+
+}  // namespace mlsw

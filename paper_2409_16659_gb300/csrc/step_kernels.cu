@@ -1,50 +1,29 @@
-// step_kernels.cu -- the fused multilayer shallow-water LBM time step.
-//
-// One launch = one time step over the whole periodic lattice, in one pass
-// over the populations:
-//   M. moments: h_i = H_i + sum_k g_ki (rest population stored shifted by
-//      H_i, see physics.cuh) on the tile plus a two-cell ring, J_i on the
-//      tile -- section LBM;
-//   P. on the tile plus one ring: interfaces z_i, their lattice gradient and
-//      Laplacian, and the layer pressures p_i (Eqs. Laplace_pressure,
-//      disjoining_pressure, p_i = sum_{j>=i} (Lambda_j + Pi_j));
-//   C. on the tile: grad p_i, friction (Eq. friction_force), force
-//      (Eq. force), equilibrium (Eq. equilibrium_distribution), BGK with
-//      forcing (Eq. BGK) and push-streaming into the other buffer, including
-//      the periodic ghost images the next step reads.
-// Algorithmic traffic is one read and one write of every population.
+// step_kernels.cu -- the fused multilayer shallow-water LBM time step of one
+// lattice. One launch = one time step over the whole periodic lattice, in
+// one pass over its state:
+//   * moments: h_i = H_i + g_0 + sum of the moving populations (rest
+//     population stored shifted by H_i, see physics.cuh), J_i -- section LBM;
+//   * interfaces z_i, their lattice gradient and Laplacian, and the layer
+//     pressures p_i (Eqs. Laplace_pressure, disjoining_pressure, p_i =
+//     sum_{j>=i} (Lambda_j + Pi_j));
+//   * grad p_i, friction (Eq. friction_force), force (Eq. force), equilibrium
+//     (Eq. equilibrium_distribution), BGK with forcing (Eq. BGK) and
+//     streaming into the other buffer, including the periodic ghost columns
+//     the next step reads.
 //
 // Discrete derivatives are the isotropic lattice stencils, written as sums
-// of differences from the centre so a constant field gives exactly zero:
+// of differences so a constant field gives exactly zero:
 //   grad phi = (1/c_s^2) sum_k w_k c_k (phi(x + c_k) - phi(x))
 //   lap  phi = (2/c_s^2) sum_k w_k (phi(x + c_k) - phi(x)).
 //
-// D2Q9 runs a persistent kernel, two CTAs per SM, over 32 x TY tiles. The
-// tile plus halo of all n*9 population planes (a box of 40 x (TY + 4) x 9n
-// floats) arrives in shared memory with one TMA bulk tensor copy completing
-// on an mbarrier; each CTA refills its stage with the next tile as soon as
-// the moments of the current one are formed, so copies overlap arithmetic.
-// D1Q3 (small 1-D lattices) uses a plain tiled kernel.
+// D2Q9: one warp per unit of work, marching down a strip of 64 columns
+// (march.cuh, step_d2q9.cu). D1Q3 (small 1-D lattices): plain kernels, here.
 
 #include "kernels.h"
 #include "physics.cuh"
 #include "step_common.cuh"
-#include "d2q9_tile.cuh"
 
 namespace mlsw {
-
-
-template <int N, int MODE>
-__global__ void __launch_bounds__(256, 2)
-    step_d2q9_tma(const __grid_constant__ CUtensorMap fin_map, float* __restrict__ fout,
-                  const __grid_constant__ KParams P, int* __restrict__ status,
-                  int* __restrict__ sched, int rev) {
-  using Tl = D2Tile<N>;
-  const int ntx = (P.nx + Tl::TX - 1) / Tl::TX, nty = (P.ny + Tl::TY - 1) / Tl::TY;
-  const SingleTiles tiles{&P, &fin_map, fout, ntx, ntx * nty, rev};
-  d2q9_tile_loop<N, MODE, Tl::RPT>(tiles, status, sched, (int)blockIdx.x);
-  tile_loop_finish(sched);
-}
 
 // ---------------------------------------------------------------------------
 // D1Q3 cell arithmetic shared by the tiled and the persistent kernels, so
@@ -311,64 +290,22 @@ __global__ void __launch_bounds__(kD1PT)
 // ---------------------------------------------------------------------------
 constexpr int kD1TX = 128;
 
-template <int N, int MODE>
-static cudaError_t launch_d2(const StepLaunch& a, cudaStream_t st) {
-  using T = D2Tile<N>;
-  auto kern = step_d2q9_tma<N, MODE>;
-  // raise the dynamic shared-memory limit and size the persistent grid once
-  // per device and instantiation
-  static unsigned long long configured = 0;
-  static int per_sm[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev >= 64) return cudaErrorInvalidDevice;
-  if (!((configured >> dev) & 1ull)) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::kSmem);
-    if (e != cudaSuccess) return e;
-    int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, T::NT, T::kSmem);
-    if (e != cudaSuccess) return e;
-    per_sm[dev] = nb > 0 ? nb : 1;
-    configured |= 1ull << dev;
-  }
-  const int ntiles = ((a.P.nx + T::TX - 1) / T::TX) * ((a.P.ny + T::TY - 1) / T::TY);
-  const int slots = a.num_sms * per_sm[dev];
-  const int grid = ntiles < slots ? ntiles : slots;
-  // launched as a programmatic dependent of the previous kernel on the
-  // stream (see d2q9_tile_loop)
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(T::NT);
-  cfg.dynamicSmemBytes = T::kSmem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, *a.fin_map, a.fout, a.P, a.status, a.sched, a.reverse);
+int step_mode(const KParams& P) {
+  // the general kernel also takes the lattices whose ghosts need a pass of
+  // their own after every step
+  if (P.omega != 1.f || P.tiny) return kGeneral;
+  const bool w32 = (P.wet_kind == 0 && P.nw == 3 && P.mw == 2);
+  return (w32 && !P.far_pairs && P.sub_amp == 0.f) ? kFast : kTau1;
 }
 
-int step_mode(const KParams& P) {
-  if (P.omega != 1.f) return kGeneral;
-  const bool w32 = (P.wet_kind == 0 && P.nw == 3 && P.mw == 2);
-  bool nn = true;  // spreading coefficients only between neighbouring interfaces
-  for (int l = 0; l < P.n; ++l)
-    for (int k = 2; k <= P.n - l; ++k) nn = nn && (P.S[l][k - 1] == 0.f);
-  return (w32 && nn && P.sub_amp == 0.f) ? kFast : kTau1;
-}
+bool step_moments(const KParams& P) { return step_mode(P) != kGeneral; }
 
 template <int N>
 static cudaError_t launch_n(const StepLaunch& a, cudaStream_t st) {
   const bool tau1 = (a.P.omega == 1.f);
   const bool w32 = (a.P.wet_kind == 0 && a.P.nw == 3 && a.P.mw == 2);
   if (a.lattice == 2) {
-    switch (step_mode(a.P)) {
-      case kGeneral: return launch_d2<N, kGeneral>(a, st);
-      case kFast: return launch_d2<N, kFast>(a, st);
-      default: return launch_d2<N, kTau1>(a, st);
-    }
+    return launch_step_d2q9<N>(a, st);
   }
   dim3 grid((a.P.nx + kD1TX - 1) / kD1TX);
   if (tau1) {
@@ -427,18 +364,7 @@ cudaError_t launch_step(const StepLaunch& a, cudaStream_t st) {
   }
 }
 
-int step_tile_cols(int lattice) { return lattice == 2 ? 32 : kD1TX; }
-
-int step_tile_rows(int n, int lattice) {
-  if (lattice != 2) return 1;
-  switch (n) {
-    case 1: return D2Tile<1>::TY;
-    case 2: return D2Tile<2>::TY;
-    case 3: return D2Tile<3>::TY;
-    case 4: return D2Tile<4>::TY;
-    default: return D2Tile<5>::TY;
-  }
-}
+int step_d1q3_cols() { return kD1TX; }
 
 MLSW_DEFINE_BOUNDS_READER(bounds_violations_step)
 
