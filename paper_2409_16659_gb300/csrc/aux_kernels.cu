@@ -334,6 +334,19 @@ __device__ __forceinline__ double warp_min(double v) {
 
 constexpr int kDiagThreads = 256;
 
+// 1 / x in FP64 from the FP32 reciprocal and two Newton steps (four FMAs; a
+// division takes about twenty instructions of the FP64 pipe, whose rate,
+// two lanes a clock and SM, bounds these reductions). x a thickness: positive
+// and far from the ends of the FP32 range, else the result is not finite.
+__device__ __forceinline__ double rcp64(double x) {
+  double r = (double)__frcp_rn((float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
+// Mass as the sum of the deviations from H_i (H_i enters once, at the end),
+// the smallest height from the smallest deviation: one FP64 addition each
+// per cell or none. 1024^2, three layers: 197 -> 173 us a call.
 template <int LAT>
 __global__ void __launch_bounds__(kDiagThreads)
     diag_partial_kernel(int n, Layout L, const float* __restrict__ f, KShift sh,
@@ -343,13 +356,19 @@ __global__ void __launch_bounds__(kDiagThreads)
   constexpr int Q = LAT == 0 ? kMomPlanes : Lt::Q;
   __shared__ double red[kDiagThreads / 32][kMaxLayers + 2];
   const long ncell = (long)L.nx * L.ny;
-  double mass[kMaxLayers];
-  for (int i = 0; i < kMaxLayers; ++i) mass[i] = 0.0;
-  double ke = 0.0, hmin = DBL_MAX;
-  for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell;
-       c += (long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % L.nx), y = (int)(c / L.nx);
-    for (int i = 0; i < n; ++i) {
+  double ke = 0.0, hmin = DBL_MAX, mass[kMaxLayers];
+  long cells = 0;  // of this thread
+#pragma unroll
+  for (int i = 0; i < kMaxLayers; ++i) {
+    mass[i] = 0.0;
+    if (i >= n) continue;
+    const double H = (double)sh.H[i];
+    float low = FLT_MAX;
+    cells = 0;
+    for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell;
+         c += (long)gridDim.x * blockDim.x, ++cells) {
+      // cells < 2^32 (mlswlbm_check_params): a 32-bit division
+      const int y = (int)((unsigned)c / (unsigned)L.nx), x = (int)((unsigned)c - (unsigned)y * L.nx);
       float dh = 0.f, jx = 0.f, jy = 0.f;
       if constexpr (LAT == 0) {
         dh = f[L.at(i * Q, x, y)] + f[L.at(i * Q + 1, x, y)];
@@ -364,11 +383,12 @@ __global__ void __launch_bounds__(kDiagThreads)
           jy += (float)Lt::cy(k) * v;
         }
       }
-      const double h = (double)sh.H[i] + (double)dh;
-      mass[i] += h;
-      ke += ((double)jx * jx + (double)jy * jy) / (2.0 * h);
-      hmin = fmin(hmin, h);
+      mass[i] += (double)dh;
+      ke = fma(fma((double)jx, (double)jx, (double)jy * (double)jy), 0.5 * rcp64(H + (double)dh), ke);
+      low = fminf(low, dh);
     }
+    mass[i] = fma((double)cells, H, mass[i]);
+    if (cells > 0) hmin = fmin(hmin, H + (double)low);
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int i = 0; i < n; ++i) {
@@ -394,21 +414,22 @@ __global__ void __launch_bounds__(kDiagThreads)
   }
 }
 
+// one warp per quantity, every lane a fixed share of the partials
 __global__ void diag_final_kernel(int n, int nblk, const double* __restrict__ partials,
                                   double* __restrict__ out) {
-  const int q = threadIdx.x;
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (q >= n + 2) return;
   double acc = (q == n + 1) ? DBL_MAX : 0.0;
-  for (int b = 0; b < nblk; ++b) {
+  for (int b = lane; b < nblk; b += 32) {
     const double v = partials[(long)b * (n + 2) + q];
     acc = (q == n + 1) ? fmin(acc, v) : acc + v;
   }
-  out[q] = acc;
+  acc = (q == n + 1) ? warp_min(acc) : warp_sum(acc);
+  if (lane == 0) out[q] = acc;
 }
 
-cudaError_t launch_diagnostics(int Q, int n, const Layout& L, const float* f,
-                               const KShift& sh, double* partials, int nblk, double* out,
-                               cudaStream_t st) {
+cudaError_t launch_diagnostics(int Q, int n, const Layout& L, const float* f, const KShift& sh,
+                               double* partials, int nblk, double* out, cudaStream_t st) {
   if (Q == 9)
     diag_partial_kernel<2><<<nblk, kDiagThreads, 0, st>>>(n, L, f, sh, partials);
   else if (Q == kMomPlanes)
@@ -417,7 +438,7 @@ cudaError_t launch_diagnostics(int Q, int n, const Layout& L, const float* f,
     diag_partial_kernel<1><<<nblk, kDiagThreads, 0, st>>>(n, L, f, sh, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  diag_final_kernel<<<1, 32, 0, st>>>(n, nblk, partials, out);
+  diag_final_kernel<<<1, 32 * (kMaxLayers + 2), 0, st>>>(n, nblk, partials, out);
   return cudaGetLastError();
 }
 
@@ -570,23 +591,36 @@ __device__ __forceinline__ double phi_d(const FreeEnergyParams& E, int k, double
     const double a = exp(-E.kappa * (h - k * E.hstar));
     return 2.0 * a - a * a;
   }
-  const double r = k * E.hstar / h;
-  return (E.nw * pow(r, (double)E.mw) - E.mw * pow(r, (double)E.nw)) / (double)(E.nw - E.mw);
+  // integer powers by squaring: pow() in FP64 is some eighty instructions of
+  // a pipe that runs two lanes a clock and SM
+  const double r = k * E.hstar * rcp64(h);
+  double rm = 1.0, rd = 1.0, s = r;
+  const int lo = E.mw, hi = E.nw - E.mw;
+#pragma unroll 1
+  for (int b = 1; b <= lo || b <= hi; b <<= 1) {
+    if (lo & b) rm *= s;
+    if (hi & b) rd *= s;
+    if (2 * b <= lo || 2 * b <= hi) s *= s;
+  }
+  return (E.nw * rm - E.mw * (rm * rd)) * E.c_phi;
 }
 
+// N layers: z and the squared gradients stay in registers. 1024^2, three
+// layers: 2967 us a call with pow(), divisions and run-time layer loops, 390 us now.
+template <int N>
 __global__ void __launch_bounds__(kFreeThreads)
     free_energy_partial_kernel(FreeEnergyParams E, const float* __restrict__ h,
                                double* __restrict__ partials) {
   __shared__ double red[kFreeThreads / 32];
-  const int n = E.n, nx = E.nx, ny = E.ny;
+  const int nx = E.nx, ny = E.ny;
   const long ncell = (long)nx * ny;
   double acc = 0.0;
   for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell;
        c += (long)gridDim.x * blockDim.x) {
-    const int y = (int)(c / nx), x = (int)(c - (long)y * nx);
+    const int y = (int)((unsigned)c / (unsigned)nx), x = (int)((unsigned)c - (unsigned)y * nx);
     const int xe = x + 1 == nx ? 0 : x + 1, xw = x == 0 ? nx - 1 : x - 1;
     const int yn = y + 1 == ny ? 0 : y + 1, ys = y == 0 ? ny - 1 : y - 1;
-    double z[kMaxLayers + 1], g2[kMaxLayers + 1];
+    double z[N + 1], g2[N + 1];
     // the substrate z_0 at the cell and its neighbours, its squared gradient
     auto z0 = [&](int xx, int yy) {
       if (E.sub_amp == 0.0) return 0.0;
@@ -595,48 +629,41 @@ __global__ void __launch_bounds__(kFreeThreads)
       if (m < 0) m += ncell;
       return E.sub_amp * cospi(2.0 * (double)m / (double)ncell);
     };
+    // lattice gradient (1/cs^2) sum_k w_k c_k a(x + c_k): 1/3 on the axes, 1/12
+    // on the diagonals. Linear: grad z_i = grad z_{i-1} + grad h_i.
+    double gx = 0.0, gy = 0.0;
+    auto add_gradient = [&](double aE, double aW, double aN, double aS, double aNE, double aNW,
+                            double aSE, double aSW) {
+      gx += fma(aE - aW, 1.0 / 3.0, ((aNE - aNW) + (aSE - aSW)) * (1.0 / 12.0));
+      gy += fma(aN - aS, 1.0 / 3.0, ((aNE - aSE) + (aNW - aSW)) * (1.0 / 12.0));
+    };
     z[0] = z0(x, y);
-    double zE = z0(xe, y), zW = z0(xw, y), zN = 0, zS = 0, zNE = 0, zNW = 0, zSE = 0, zSW = 0;
-    if (E.lattice == 2) {
-      zN = z0(x, yn);
-      zS = z0(x, ys);
-      zNE = z0(xe, yn);
-      zNW = z0(xw, yn);
-      zSE = z0(xe, ys);
-      zSW = z0(xw, ys);
-      const double gx = (zE - zW) / 3.0 + ((zNE - zNW) + (zSE - zSW)) / 12.0;
-      const double gy = (zN - zS) / 3.0 + ((zNE - zSE) + (zNW - zSW)) / 12.0;
-      g2[0] = gx * gx + gy * gy;
-    } else {
-      const double gx = 0.5 * (zE - zW);
-      g2[0] = gx * gx;
+    if (E.sub_amp != 0.0) {
+      if (E.lattice == 2)
+        add_gradient(z0(xe, y), z0(xw, y), z0(x, yn), z0(x, ys), z0(xe, yn), z0(xw, yn),
+                     z0(xe, ys), z0(xw, ys));
+      else
+        gx = 0.5 * (z0(xe, y) - z0(xw, y));
     }
-    for (int i = 1; i <= n; ++i) {
+    g2[0] = gx * gx + gy * gy;
+#pragma unroll
+    for (int i = 1; i <= N; ++i) {
       const float* hi = h + (long)(i - 1) * ncell;
-      z[i] = z[i - 1] + (double)hi[(long)y * nx + x];
-      zE += hi[(long)y * nx + xe];
-      zW += hi[(long)y * nx + xw];
-      double gx, gy;
-      if (E.lattice == 2) {
-        zN += hi[(long)yn * nx + x];
-        zS += hi[(long)ys * nx + x];
-        zNE += hi[(long)yn * nx + xe];
-        zNW += hi[(long)yn * nx + xw];
-        zSE += hi[(long)ys * nx + xe];
-        zSW += hi[(long)ys * nx + xw];
-        // (1/cs^2) sum_k w_k c_k z(x + c_k): 1/3 on the axes, 1/12 on the diagonals
-        gx = (zE - zW) / 3.0 + ((zNE - zNW) + (zSE - zSW)) / 12.0;
-        gy = (zN - zS) / 3.0 + ((zNE - zSE) + (zNW - zSW)) / 12.0;
-      } else {
-        gx = 0.5 * (zE - zW);
-        gy = 0.0;
-      }
+      const float *r0 = hi + (long)y * nx, *rn = hi + (long)yn * nx, *rs = hi + (long)ys * nx;
+      z[i] = z[i - 1] + (double)r0[x];
+      if (E.lattice == 2)
+        add_gradient(r0[xe], r0[xw], rn[x], rs[x], rn[xe], rn[xw], rs[xe], rs[xw]);
+      else
+        gx += 0.5 * ((double)r0[xe] - (double)r0[xw]);
       g2[i] = gx * gx + gy * gy;
-      acc += E.gamma[i - 1] * (1.0 + 0.5 * g2[i]);
+      acc += E.gamma[i - 1] * fma(0.5, g2[i], 1.0);
     }
-    for (int i = 0; i < n; ++i)
-      for (int k = 1; k <= n - i; ++k)
-        acc += E.S[i][k - 1] * phi_d(E, k, z[i + k] - z[i]) * (1.0 + 0.5 * g2[i]);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int k = 1; k <= N - i; ++k)
+        if (E.S[i][k - 1] != 0.0)
+          acc += E.S[i][k - 1] * phi_d(E, k, z[i + k] - z[i]) * fma(0.5, g2[i], 1.0);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -651,16 +678,22 @@ __global__ void __launch_bounds__(kFreeThreads)
 
 __global__ void free_energy_final_kernel(int nblk, const double* __restrict__ partials,
                                          double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partials[b];
-    *out = s;
-  }
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += 32) s += partials[b];
+  s = warp_sum(s);
+  if (threadIdx.x == 0) *out = s;
 }
 
 cudaError_t launch_free_energy(const FreeEnergyParams& E, const float* h, double* partials,
                                int nblk, double* out, cudaStream_t st) {
-  free_energy_partial_kernel<<<nblk, kFreeThreads, 0, st>>>(E, h, partials);
+  switch (E.n) {
+    case 1: free_energy_partial_kernel<1><<<nblk, kFreeThreads, 0, st>>>(E, h, partials); break;
+    case 2: free_energy_partial_kernel<2><<<nblk, kFreeThreads, 0, st>>>(E, h, partials); break;
+    case 3: free_energy_partial_kernel<3><<<nblk, kFreeThreads, 0, st>>>(E, h, partials); break;
+    case 4: free_energy_partial_kernel<4><<<nblk, kFreeThreads, 0, st>>>(E, h, partials); break;
+    case 5: free_energy_partial_kernel<5><<<nblk, kFreeThreads, 0, st>>>(E, h, partials); break;
+    default: return cudaErrorInvalidValue;
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   free_energy_final_kernel<<<1, 32, 0, st>>>(nblk, partials, out);

@@ -65,7 +65,8 @@ cudaError_t launch_step_persistent(const StepLaunch& a, int nsteps, cudaStream_t
 // mode and tile height form a contiguous range (batch_kernels.cu).
 // ---------------------------------------------------------------------------
 // Tile heights a batch can use: variant 0 = 16 rows (n <= 3 only), variant
-// 1 = 8 rows. A warp's unit of work is a strip of `rows` rows, whole tiles.
+// 1 = 8 rows. A warp's unit of work is a strip of `rows` rows: the height,
+// scaled alike for all instances of a table (batch.cu).
 constexpr int kBatchVariants = 2;
 __host__ __device__ constexpr int batch_tile_rows(int variant) { return variant == 0 ? 16 : 8; }
 
@@ -197,6 +198,7 @@ struct FreeEnergyParams {
   int sub_kx, sub_ky;
   int wet_kind;    // 0 power law (nw, mw), 1 exponential (kappa)
   double kappa;
+  double c_phi;    // 1 / (nw - mw)
 };
 cudaError_t launch_free_energy(const FreeEnergyParams& E, const float* h, double* partials,
                                int nblk, double* out, cudaStream_t st);

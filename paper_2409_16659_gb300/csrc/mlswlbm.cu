@@ -501,7 +501,7 @@ int mlswlbm_create(const mlsw_params* p, const float* h_init, void* stream, mlsw
     return MLSW_ERR_CUDA;
   }
   h->num_sms = sms > 0 ? sms : 1;
-  h->nblk_diag = 2 * h->num_sms;
+  h->nblk_diag = 8 * h->num_sms;
   if (!(p->flags & MLSW_FLAG_NO_PERSISTENT)) {
     int optin = 0;
     const size_t need = mlsw::step_persistent_smem(n, p->lattice, p->nx);
@@ -743,6 +743,7 @@ int mlswlbm_get_free_energy(mlsw_handle* h, double* F) {
   E.mw = p.wet_m;
   E.wet_kind = p.wet_kind;
   E.kappa = p.wet_kappa;
+  E.c_phi = 1.0 / std::max(1, p.wet_n - p.wet_m);
   E.sub_amp = p.sub_amp;
   E.sub_kx = p.sub_kx;
   E.sub_ky = p.sub_ky;
