@@ -5,6 +5,7 @@
 // over the whole table (batch_kernels.cu), and a timing autotuner for the
 // tile height of every class of alike instances.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <new>
@@ -67,13 +68,53 @@ int planes_of(const KParams& P) { return mlsw::step_moments(P) ? mlsw::kMomPlane
 
 int units_of(const BatchInst& b, int rows) { return b.strips * ((b.P.ny + rows - 1) / rows); }
 
-// Tiles a unit spans: as many (up to 8) as leave three waves of the resident
-// warps. A unit costs its rows plus about five rows of warm-up, and the
-// waves even out the instances' different costs.
-int span_for(long units_one_tile, int warps) {
-  int span = 8;
-  while (span > 1 && units_one_tile / span < 3L * warps) span /= 2;
-  return span;
+// rows of an instance's units: 16-row tiles scaled to r rows, 8-row tiles to
+// half as many, at most 64 (see march_rows in step_d2q9.cu)
+int unit_rows(int variant, int r) {
+  return std::min(64, r * mlsw::batch_tile_rows(variant) / 16 + (variant == 0 ? 0 : r & 1));
+}
+
+// Scale r of the units of a table, by a model of a step's time in units of a
+// row's issue time on one of an SM's four schedulers. A unit costs its rows
+// plus about five rows of warm-up; a warp alone on a scheduler needs 1.75
+// times that time for a row's latencies. Alike instances finish together, in
+// whole waves, and as the schedulers' fullest; uneven ones (work in
+// proportion to n) overlap, and the longest unit may come last. 16 films of
+// 256^2: r = 12 instead of 16 brings a step from 47 to 44 us.
+int scale_for(const mlsw_batch* b, const std::vector<int>& members, const std::vector<int>& variant) {
+  int nmax = 0, nmin = mlsw::kMaxLayers;
+  for (int j : members) {
+    nmax = std::max(nmax, b->hinst[j].P.n);
+    nmin = std::min(nmin, b->hinst[j].P.n);
+  }
+  const int per_sm = mlsw::batch_warps_per_sm(nmax);
+  const double schedulers = 4.0 * b->num_sms, slots = (double)per_sm * b->num_sms;
+  int best_r = 1;
+  double best = 0.0;
+  for (int r = 1; r <= 128; ++r) {
+    double units = 0.0, work = 0.0, longest = 0.0;
+    for (int j : members) {
+      const int rows = unit_rows(variant[j], r);
+      const double u = units_of(b->hinst[j], rows), w = (double)(rows + 5) * b->hinst[j].P.n;
+      units += u;
+      work += u * w;
+      longest = std::max(longest, w);
+    }
+    double cost;
+    if (nmin == nmax) {
+      const double full = per_sm / 4.0;
+      const double q = units <= slots ? std::min(std::ceil(1.05 * units / schedulers), full)
+                                      : std::ceil(units / slots) * full;
+      cost = longest * std::max(1.75, q);
+    } else {
+      cost = work / schedulers + 1.75 * longest;
+    }
+    if (r == 1 || cost < best) {
+      best = cost;
+      best_r = r;
+    }
+  }
+  return best_r;
 }
 
 // the buffer that holds instance j's state now
@@ -121,7 +162,7 @@ int init_all(mlsw_batch* b, const float* const* h_init) {
 // ones to run are short), and the unit rows in the descriptors
 int build_groups(mlsw_batch* b) {
   std::map<std::tuple<int, int, int>, std::vector<int>> members;
-  long tiles = 0;
+  std::vector<int> all;
   b->nmax = 0;
   b->kinds = 0;
   b->tiny.clear();
@@ -129,12 +170,12 @@ int build_groups(mlsw_batch* b) {
     if (!b->selected[j]) continue;
     const BatchInst& bi = b->hinst[j];
     members[std::make_tuple(-bi.P.n, mlsw::step_mode(bi.P), b->variant[j])].push_back(j);
-    tiles += units_of(bi, mlsw::batch_tile_rows(b->variant[j]));
+    all.push_back(j);
     b->nmax = std::max(b->nmax, bi.P.n);
     b->kinds |= 1u << bi.kind;
     if (bi.P.tiny) b->tiny.push_back(j);
   }
-  const int span = span_for(tiles, b->num_sms * mlsw::batch_warps_per_sm(b->nmax));
+  const int r = all.empty() ? 1 : scale_for(b, all, b->variant);
   std::vector<int2> table;
   b->groups.clear();
   for (auto& kv : members) {
@@ -144,7 +185,7 @@ int build_groups(mlsw_batch* b) {
     g.variant = std::get<2>(kv.first);
     g.offset = (int)table.size();
     for (int j : kv.second) {
-      b->hinst[j].rows = mlsw::batch_tile_rows(g.variant) * span;
+      b->hinst[j].rows = unit_rows(g.variant, r);
       const int nu = units_of(b->hinst[j], b->hinst[j].rows);
       for (int t = 0; t < nu; ++t) table.push_back(make_int2(j, t));
     }
@@ -199,10 +240,8 @@ int autotune(mlsw_batch* b) {
     int best_v = 0;
     for (int v = 0; v < mlsw::kBatchVariants && rc == MLSW_OK; ++v) {
       std::vector<int2> table;
-      long tiles = 0;
-      for (int j : kv.second) tiles += units_of(b->hinst[j], mlsw::batch_tile_rows(v));
-      const int span = span_for(tiles, b->num_sms * mlsw::batch_warps_per_sm(n));
-      for (int j : kv.second) b->hinst[j].rows = mlsw::batch_tile_rows(v) * span;
+      const int r = scale_for(b, kv.second, std::vector<int>(b->count, v));
+      for (int j : kv.second) b->hinst[j].rows = unit_rows(v, r);
       for (int j : kv.second)
         for (int t = 0; t < units_of(b->hinst[j], b->hinst[j].rows); ++t)
           table.push_back(make_int2(j, t));

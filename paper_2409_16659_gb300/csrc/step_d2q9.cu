@@ -13,10 +13,13 @@ namespace mlsw {
 // three layers 12 (168 registers; 16 warps at 128 spill into the 15 KB of L1
 // that the rings leave: 76 us a step against 29 at 1024^2; 8 warps: 97
 // against 89 us at 2048^2), two layers 16, one layer 20, four and five 8.
-constexpr int march_min_warps(int n) { return n == 1 ? 20 : (n == 2 ? 14 : (n == 3 ? 12 : 8)); }
+// The other modes carry their options besides: 8 from three layers on.
+constexpr int march_min_warps(int n, int mode) {
+  return n == 1 ? 20 : (n == 2 ? 14 : (n == 3 && mode == kFast ? 12 : 8));
+}
 
 template <int N, int MODE, bool OP>
-__global__ void __launch_bounds__(32, march_min_warps(N))
+__global__ void __launch_bounds__(32, march_min_warps(N, MODE))
     step_d2q9(const __grid_constant__ CUtensorMap map, float* __restrict__ fout,
               const __grid_constant__ KParams P, int strips, int rows, int* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
