@@ -116,28 +116,41 @@ struct ConvArgs {
 // tile's pixels shifted by (sx, sy), and the BN x KC weights of the three
 // taps with that column shift, all by two TMA copies. The three row shifts
 // read the pixels at offsets of 16 rows, whole swizzle atoms.
-template <int KC, int BN>
+//
+// RES: the weights of the CTA's output-channel tile stay in shared memory,
+// copied once per CTA, and the stages hold pixels only. The copies are bound
+// by their rows (about four clocks per row of a box, whatever its bytes): a
+// stage of 32-channel layers is 160 pixel rows and 96 weight rows, of
+// 64-channel ones 160 and 192, which every tile would copy again.
+template <int KC, int BN, bool RES>
 struct ConvShape {
   static constexpr int TW = 16, TH = 8;        // the tile of output pixels
   static constexpr int AROWS = TW * (TH + 2);  // rows of a shifted box
   static constexpr int ABYTES = AROWS * KC * 2, BBYTES = BN * KC * 2;
   static constexpr int ASTRIDE = (ABYTES + 1023) / 1024 * 1024;
   static constexpr int BSTRIDE = BBYTES;       // the weight box's dy blocks are contiguous
-  static constexpr int STAGE = ASTRIDE + (3 * BBYTES + 1023) / 1024 * 1024;
+  static constexpr int WBLK = (3 * BBYTES + 1023) / 1024 * 1024;  // weights of a column shift
+  static constexpr int STAGE = ASTRIDE + (RES ? 0 : WBLK);
   static constexpr int ST0 = 204 * 1024 / STAGE;
   // small stages (the 16- and 32-channel layers): six deep, which measured
   // faster than four with more CTAs per SM
-  static constexpr int ST = STAGE <= 25 * 1024 ? 6 : (STAGE <= 50 * 1024 ? 4 : (ST0 < 2 ? 2 : ST0));
+  static constexpr int ST = RES ? (KC <= 16 ? 6 : 4)
+                                : (STAGE <= 25 * 1024 ? 6 : (STAGE <= 50 * 1024 ? 4 : (ST0 < 2 ? 2 : ST0)));
   static constexpr int ACOLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : 128);
   static constexpr int TCOLS = 2 * ACOLS;          // two accumulators
   static constexpr int CTAS_TMEM = 512 / TCOLS;    // CTAs whose TMEM fits one SM
   static constexpr int kBiasMax = 256;  // output channels whose bias is staged in shared memory
-  static constexpr size_t SMEM_NEED = 1024 + (size_t)ST * STAGE + 8 * (2 * ST + 5) + 16 + 4 * kBiasMax;
-  // ask for enough shared memory that no more CTAs than CTAS_TMEM share an SM
-  static constexpr size_t SMEM_TMEM = 233472 / (CTAS_TMEM + 1) + 1024;
-  static constexpr size_t SMEM = SMEM_NEED > SMEM_TMEM ? SMEM_NEED : SMEM_TMEM;
+  // dynamic shared memory with `wblks` resident weight blocks
+  static constexpr size_t need(int wblks) {
+    return 1024 + (size_t)wblks * WBLK + (size_t)ST * STAGE + 8 * (2 * ST + 6) + 16 + 4 * kBiasMax;
+  }
+  // enough that no more CTAs than CTAS_TMEM share an SM
+  static constexpr size_t smem(int wblks) {
+    const size_t tmem = 233472 / (CTAS_TMEM + 1) + 1024;
+    return need(wblks) > tmem ? need(wblks) : tmem;
+  }
   static_assert(BN <= 128, "output-channel tiles of at most 128");
-  static_assert(SMEM_NEED <= 232448, "stages exceed shared memory");
+  static_assert(need(0) <= 232448, "stages exceed shared memory");
   static_assert(BBYTES % (8 * KC * 2) == 0, "weight blocks are whole swizzle atoms");
 };
 
@@ -149,6 +162,14 @@ __device__ __forceinline__ void st_global_v8(void* dst, const uint32_t (&v)[8]) 
                : "memory");
 }
 
+// Every kernel of a pass is launched as a programmatic dependent of the one
+// before it (launch_dep): its blocks are scheduled while that one ends, do
+// what touches no global memory, and wait here for its results. A pass of
+// one 128^2 sample is 27 launches of 3 to 17 us each.
+__device__ __forceinline__ void wait_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&h);
@@ -157,24 +178,29 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 // Persistent and warp-specialised: warp 0 issues the TMA copies, warp 1
 // the MMAs into one of two TMEM accumulators, warps 2..5 drain a finished
 // accumulator (epilogue) while the next tile accumulates into the other.
-// Work item w of the CTA is tile w / ntn, output-channel tile w % ntn, for
-// w = blockIdx.x, + gridDim.x, ...
-template <int KC, int BN>
-__global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvArgs a, int ntn) {
-  using S = ConvShape<KC, BN>;
+// A CTA keeps one output-channel tile (blockIdx.x % ntn) and takes the pixel
+// tiles blockIdx.x / ntn, + gridDim.x / ntn, ... (gridDim.x a multiple of ntn).
+template <int KC, int BN, bool RES>
+__global__ void __launch_bounds__(192, 1)
+    conv_tc(const __grid_constant__ ConvArgs a, int ntn, int wblks) {
+  using S = ConvShape<KC, BN, RES>;
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+  unsigned char* wres = sm;         // RES: [chunk][column shift] weight blocks
+  sm += RES ? (size_t)wblks * S::WBLK : 0;
   uint64_t* full = (uint64_t*)(sm + S::ST * S::STAGE);
   uint64_t* empty = full + S::ST;
   uint64_t* tfull = empty + S::ST;  // [2] accumulator ready
   uint64_t* tempty = tfull + 2;     // [2] accumulator drained
   uint64_t* drain = tempty + 2;     // every MMA of this CTA has completed
-  uint32_t* tslot = (uint32_t*)(drain + 1);
+  uint64_t* wfull = drain + 1;      // RES: the weights have arrived
+  uint32_t* tslot = (uint32_t*)(wfull + 1);
   float* sbias = (float*)(tslot + 4);  // [cout] (16-byte aligned)
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int W = a.W, H = a.H;
   const int tpr = W / S::TW, tpi = tpr * (H / S::TH);
-  const int nitems = a.B_tiles * ntn;
+  const int n0 = (int)(blockIdx.x % ntn) * BN;
+  const int tile0 = blockIdx.x / ntn, dtile = gridDim.x / ntn;
   const int sgn = a.reverse_taps ? -1 : 1;
 
   if (threadIdx.x == 0) {
@@ -187,9 +213,11 @@ __global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvAr
       mbar_init(&tempty[j], 4);
     }
     mbar_init(drain, 1);
+    mbar_init(wfull, 1);
     mbar_init_fence();
   }
   if (warp == 1) tmem_alloc(tslot, S::TCOLS);
+  wait_previous();
   // the bias, read once per CTA (the epilogue adds it from shared memory)
   if (a.bias)
     for (int c = threadIdx.x; c < a.cout; c += blockDim.x) sbias[c] = a.bias[c];
@@ -200,9 +228,17 @@ __global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvAr
   bool ok = true;
   if (warp == 0) {
     if (lane == 0) {
+      if constexpr (RES) {
+        mbar_arrive_expect_tx(wfull, (uint32_t)(wblks * 3 * S::BBYTES));
+        int w = 0;
+        for (int i = 0; i < a.nin; ++i)
+          for (int c0 = 0; c0 < a.cin[i]; c0 += KC)
+            for (int sx = -1; sx <= 1; ++sx, ++w)
+              tma_load_4d(wres + (size_t)w * S::WBLK, &a.w_map, wfull, a.koff[i] + c0, n0, 0,
+                          sgn * sx + 1);
+      }
       int k = 0;  // stage counter over all items
-      for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        const int tile = item / ntn, n0 = (item % ntn) * BN;
+      for (int tile = tile0; tile < a.B_tiles && ok; tile += dtile) {
         const int b = tile / tpi, r = tile % tpi;
         const int x0 = (r % tpr) * S::TW, y0 = (r / tpr) * S::TH;
         for (int i = 0; i < a.nin && ok; ++i)
@@ -212,13 +248,15 @@ __global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvAr
               if (it > 0) ok = mbar_wait_bounded(&empty[s], (it - 1) & 1);
               if (!ok) break;
               unsigned char* st = sm + s * S::STAGE;
-              mbar_arrive_expect_tx(&full[s], (uint32_t)(S::ABYTES + 3 * S::BBYTES));
+              mbar_arrive_expect_tx(&full[s], (uint32_t)(S::ABYTES + (RES ? 0 : 3 * S::BBYTES)));
               // halo coordinates: real column x0 + sx is x0 + sx + 1, real
               // row y0 - 1 is y0
               tma_load_4d(st, &a.in_map[i], &full[s], c0, x0 + sx + 1, y0, b);
               // the three taps whose pixels are at column shift sx: tap
               // column sgn sx, rows dy = -1, 0, 1 in that order
-              tma_load_4d(st + S::ASTRIDE, &a.w_map, &full[s], a.koff[i] + c0, n0, 0, sgn * sx + 1);
+              if constexpr (!RES)
+                tma_load_4d(st + S::ASTRIDE, &a.w_map, &full[s], a.koff[i] + c0, n0, 0,
+                            sgn * sx + 1);
             }
       }
     }
@@ -226,16 +264,18 @@ __global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvAr
     if (lane == 0) {
       constexpr uint32_t idesc = idesc_bf16_f32(128, BN);
       int k = 0, local = 0;
-      for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++local) {
+      if constexpr (RES) ok = mbar_wait_bounded(wfull, 0);
+      for (int tile = tile0; tile < a.B_tiles && ok; tile += dtile, ++local) {
         const int ab = local & 1, use = local >> 1;
         if (use > 0) ok = mbar_wait_bounded(&tempty[ab], (use - 1) & 1);
         if (!ok) break;
         tc_fence_after();
         const uint32_t acc = tmem + (uint32_t)(ab * S::ACOLS);
         uint32_t accumulate = 0;
+        const unsigned char* wb0 = wres;  // RES: this chunk and shift's weights
         for (int i = 0; i < a.nin && ok; ++i)
           for (int c0 = 0; c0 < a.cin[i] && ok; c0 += KC)
-            for (int sx = 0; sx < 3 && ok; ++sx, ++k) {
+            for (int sx = 0; sx < 3 && ok; ++sx, ++k, wb0 += S::WBLK) {
               const int s = k % S::ST, it = k / S::ST;
               ok = mbar_wait_bounded(&full[s], it & 1);
               if (!ok) break;
@@ -247,7 +287,7 @@ __global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvAr
                 // sgn (sy - 1), block sgn (sy - 1) + 1 of the weight box
                 const int wb = a.reverse_taps ? 2 - sy : sy;
                 const unsigned char* pa = st + sy * S::TW * KC * 2;
-                const unsigned char* pb = st + S::ASTRIDE + wb * S::BSTRIDE;
+                const unsigned char* pb = (RES ? wb0 : st + S::ASTRIDE) + wb * S::BSTRIDE;
 #pragma unroll
                 for (int kk = 0; kk < KC / 16; ++kk) {
                   tc_mma(acc, sdesc_kmajor<KC * 2>(pa + kk * 32), sdesc_kmajor<KC * 2>(pb + kk * 32),
@@ -267,7 +307,7 @@ __global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvAr
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, i.e. pixels
     const int q = warp & 3;
     int local = 0;
-    for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++local) {
+    for (int tile = tile0; tile < a.B_tiles; tile += dtile, ++local) {
       const int ab = local & 1, use = local >> 1;
       const bool dok = mbar_wait_bounded(&tfull[ab], use & 1);
       tc_fence_after();
@@ -275,7 +315,6 @@ __global__ void __launch_bounds__(192, 1) conv_tc(const __grid_constant__ ConvAr
         ok = false;
         break;
       }
-      const int tile = item / ntn, n0 = (item % ntn) * BN;
       const int b = tile / tpi, r = tile % tpi;
       const int x0 = (r % tpr) * S::TW, y0 = (r / tpr) * S::TH;
       const int m = q * 32 + lane;
@@ -418,6 +457,7 @@ __global__ void __launch_bounds__(128) wgrad_tc(const __grid_constant__ WgradArg
     mbar_init_fence();
   }
   if (warp == 0) tmem_alloc(tslot, S::TCOLS);
+  wait_previous();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -495,22 +535,6 @@ __device__ __forceinline__ long hidx(int b, int y, int x, int H, int W, int C) {
   return (((long)b * (H + 2) + y + 1) * (W + 2) + x + 1) * C;
 }
 
-// store one pixel's channel pair (c, c + 1) and its periodic images
-__device__ __forceinline__ void st_pair(bf16* t, int b, int y, int x, int H, int W, int C, int c,
-                                        float v0, float v1) {
-  const __nv_bfloat162 p = __floats2bfloat162_rn(v0, v1);
-  const int xs[2] = {x + 1, x == 0 ? W + 1 : (x == W - 1 ? 0 : -1)};
-  const int ys[2] = {y + 1, y == 0 ? H + 1 : (y == H - 1 ? 0 : -1)};
-  for (int iy = 0; iy < 2; ++iy)
-    for (int ix = 0; ix < 2; ++ix)
-      if (ys[iy] >= 0 && xs[ix] >= 0)
-        *reinterpret_cast<__nv_bfloat162*>(t + (((long)b * (H + 2) + ys[iy]) * (W + 2) + xs[ix]) * C + c) = p;
-}
-
-__device__ __forceinline__ float2 ld_pair(const bf16* t, long off) {
-  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(t + off));
-}
-
 // ---------------------------------------------------------------------------
 // Pooling, upsampling and their gradients work on 8-channel groups (16
 // bytes): a thread takes one group of one output pixel. Tensor sides are
@@ -567,6 +591,7 @@ __device__ __forceinline__ OctIdx oct_idx(long i, int lgH, int lgW, int lgG) {
 // dst (H/2 x W/2, lgH, lgW its sides) = 2 x 2 mean of src (H x W)
 __global__ void pool_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, int B, int lgH,
                             int lgW, int lgG) {
+  wait_previous();
   const int H = 1 << lgH, W = 1 << lgW, C = 8 << lgG;
   const long total = (long)B << (lgH + lgW + lgG);
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -586,6 +611,7 @@ __global__ void pool_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst
 // dst (H x W) = nearest 2x upsampling of src (H/2 x W/2)
 __global__ void up_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, int B, int lgH,
                           int lgW, int lgG) {
+  wait_previous();
   const int H = 1 << lgH, W = 1 << lgW, C = 8 << lgG;
   const long total = (long)B << (lgH + lgW + lgG);
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -597,6 +623,7 @@ __global__ void up_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, 
 // dS (H/2 x W/2, the sides given) = (sum of the 2 x 2 fine pixels of dU) * (S > 0)
 __global__ void up_grad_mask_kernel(const bf16* __restrict__ dU, const bf16* __restrict__ Sact,
                                     bf16* __restrict__ dS, int B, int lgH, int lgW, int lgG) {
+  wait_previous();
   const int H = 1 << lgH, W = 1 << lgW, C = 8 << lgG;
   const long total = (long)B << (lgH + lgW + lgG);
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -618,6 +645,7 @@ __global__ void up_grad_mask_kernel(const bf16* __restrict__ dU, const bf16* __r
 __global__ void pool_grad_add_mask_kernel(const bf16* __restrict__ dP, const bf16* __restrict__ skip,
                                           const bf16* __restrict__ Sact, bf16* __restrict__ dS, int B,
                                           int lgH, int lgW, int lgG) {
+  wait_previous();
   const int H = 1 << lgH, W = 1 << lgW, C = 8 << lgG;
   const long total = (long)B << (lgH + lgW + lgG);
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -649,6 +677,7 @@ __global__ void __launch_bounds__(256) plane_reduce_kernel(const float* __restri
                                                            double* __restrict__ partial,
                                                            unsigned* __restrict__ counter,
                                                            double* __restrict__ out) {
+  wait_previous();
   const int nchunk = HW / kRedChunk, pl = blockIdx.y, ch = blockIdx.x;
   const float4* p = reinterpret_cast<const float4*>(x + (long)pl * HW + (long)ch * kRedChunk);
   const float c = mode ? (float)center[pl] : 0.f;
@@ -699,55 +728,132 @@ __global__ void __launch_bounds__(256) plane_reduce_kernel(const float* __restri
 // 1 / s of a sample, 0 for a flat one (its planes are then all zero)
 __device__ __forceinline__ double inv_or_zero(double s) { return s > 0.0 ? 1.0 / s : 0.0; }
 
-// X0 = (h_i - mean) in_scale / s, parameter planes, zeros (16 channels)
-__global__ void input_kernel(const float* __restrict__ h, const double* __restrict__ mean,
-                             const double* __restrict__ rms, int B, int n, int H, int W,
-                             float in_scale, const float* __restrict__ extra, int n_extra,
-                             bf16* __restrict__ x0) {
-  const long total = (long)B * H * W;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const int x = (int)(i % W);
-    const int y = (int)((i / W) % H), b = (int)(i / ((long)W * H));
+// A double as the sum of two floats, and (x - m) k in that arithmetic: the
+// FP64 pipe (two lanes a clock and SM) bounded these kernels; the product of
+// two-float numbers keeps 45 bits, far below the FP32 rounding of the result.
+struct Two {
+  float hi, lo;
+};
+__device__ __forceinline__ Two two(double v) {
+  const float hi = (float)v;
+  return {hi, (float)(v - (double)hi)};
+}
+__device__ __forceinline__ float centred_times(float x, Two m, Two k) {
+  // x - m.hi exactly, as a sum of two floats
+  const float d = x - m.hi, t = d - x;
+  const float e = (x - (d - t)) - (m.hi + t);
+  const float lo = e - m.lo;
+  const float p = __fmul_rn(d, k.hi);  // the rounded product, not contracted below
+  return p + fmaf(d, k.lo, fmaf(lo, k.hi, fmaf(d, k.hi, -p)));
+}
+
+// the 16 channels of one pixel and their periodic images (32 bytes each)
+__device__ __forceinline__ void st_pixel16(bf16* t, int b, int y, int x, int H, int W,
+                                           const float (&v)[16]) {
+  uint32_t w[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) w[j] = pack_bf16(v[2 * j], v[2 * j + 1]);
+  const int xs[2] = {x + 1, x == 0 ? W + 1 : (x == W - 1 ? 0 : -1)};
+  const int ys[2] = {y + 1, y == 0 ? H + 1 : (y == H - 1 ? 0 : -1)};
+#pragma unroll
+  for (int iy = 0; iy < 2; ++iy)
+#pragma unroll
+    for (int ix = 0; ix < 2; ++ix)
+      if (ys[iy] >= 0 && xs[ix] >= 0)
+        st_global_v8(t + (((long)b * (H + 2) + ys[iy]) * (W + 2) + xs[ix]) * 16, w);
+}
+
+// X0 = (h_i - mean) in_scale / s, parameter planes, zeros (16 channels).
+// blockIdx.y: the sample, whose factors the block forms once; a thread per
+// pixel. Batch 32 of 256^2: 88 -> 27 us.
+__global__ void __launch_bounds__(256) input_kernel(const float* __restrict__ h,
+                                                    const double* __restrict__ mean,
+                                                    const double* __restrict__ rms, int n, int lgH,
+                                                    int lgW, float in_scale,
+                                                    const float* __restrict__ extra, int n_extra,
+                                                    bf16* __restrict__ x0) {
+  static_assert(kCin0 == 16, "one 32-byte store per pixel");
+  __shared__ Two sm[kCin0], sk;
+  __shared__ float se[kCin0];
+  wait_previous();
+  const int H = 1 << lgH, W = 1 << lgW, HW = H * W, b = blockIdx.y;
+  if ((int)threadIdx.x < n) sm[threadIdx.x] = two(mean[b * n + threadIdx.x]);
+  if ((int)threadIdx.x < n_extra) se[threadIdx.x] = extra[threadIdx.x];
+  if (threadIdx.x == 32) sk = two(in_scale * inv_or_zero(rms[b]));
+  __syncthreads();
+  const float* hb = h + (long)b * n * HW;
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < HW; p += gridDim.x * blockDim.x) {
     float v[kCin0];
-    for (int c = 0; c < kCin0; ++c) v[c] = 0.f;
-    const double k = in_scale * inv_or_zero(rms[b]);
-    for (int c = 0; c < n; ++c)
-      v[c] = (float)(((double)h[(((long)b * n + c) * H + y) * W + x] - mean[b * n + c]) * k);
-    for (int j = 0; j < n_extra; ++j) v[n + j] = extra[j];
-    for (int c = 0; c < kCin0; c += 2) st_pair(x0, b, y, x, H, W, kCin0, c, v[c], v[c + 1]);
+#pragma unroll
+    for (int c = 0; c < kCin0; ++c) {
+      v[c] = 0.f;
+      if (c < n)
+        v[c] = centred_times(hb[(long)c * HW + p], sm[c], sk);
+      else if (c < n + n_extra)
+        v[c] = se[c - n];
+    }
+    st_pixel16(x0, b, p >> lgW, p & (W - 1), H, W, v);
   }
 }
 
-// out = h + (y - mean y) s / out_scale per (sample, layer); ymean: means of
-// y, rms: s of every sample
-__global__ void output_kernel(const float* __restrict__ h, const float* __restrict__ y,
-                              const double* __restrict__ ymean, const double* __restrict__ rms,
-                              long total, int n, int HW, float inv_scale, float* __restrict__ out) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x)
-    out[i] = h[i] + (float)(((double)y[i] - ymean[i / HW]) * rms[i / ((long)n * HW)] * inv_scale);
+// out = h + (y - mean y) s / out_scale per (sample, layer) = blockIdx.y;
+// ymean: means of y, rms: s of every sample. HW is a multiple of 4.
+__global__ void __launch_bounds__(256) output_kernel(const float* __restrict__ h,
+                                                     const float* __restrict__ y,
+                                                     const double* __restrict__ ymean,
+                                                     const double* __restrict__ rms, int n, int HW,
+                                                     float inv_scale, int vec,
+                                                     float* __restrict__ out) {
+  wait_previous();
+  const int pl = blockIdx.y;
+  const Two m = two(ymean[pl]), k = two(rms[pl / n] * inv_scale);
+  const long off = (long)pl * HW;
+  if (vec) {  // h and out 16-byte aligned
+    const float4* h4 = reinterpret_cast<const float4*>(h + off);
+    const float4* y4 = reinterpret_cast<const float4*>(y + off);
+    float4* o4 = reinterpret_cast<float4*>(out + off);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < HW / 4; i += gridDim.x * blockDim.x) {
+      const float4 a = h4[i], q = y4[i];
+      o4[i] = make_float4(a.x + centred_times(q.x, m, k), a.y + centred_times(q.y, m, k),
+                          a.z + centred_times(q.z, m, k), a.w + centred_times(q.w, m, k));
+    }
+  } else {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < HW; i += gridDim.x * blockDim.x)
+      out[off + i] = h[off + i] + centred_times(y[off + i], m, k);
+  }
 }
 
 // loss += sum (y - (t - h) out_scale / s)^2 (FP64); dY (NHWC halo, 16
-// channels) = 2 (y - (t - h) out_scale / s) / count
-__global__ void loss_kernel(const float* __restrict__ y, const float* __restrict__ h,
-                            const float* __restrict__ t, const double* __restrict__ rms, int B,
-                            int n, int H, int W, float scale, float inv_count,
-                            double* __restrict__ loss, bf16* __restrict__ dY) {
-  const long total = (long)B * H * W;
+// channels) = 2 (y - (t - h) out_scale / s) / count. blockIdx.y: the sample.
+__global__ void __launch_bounds__(256) loss_kernel(const float* __restrict__ y,
+                                                   const float* __restrict__ h,
+                                                   const float* __restrict__ t,
+                                                   const double* __restrict__ rms, int n, int lgH,
+                                                   int lgW, float scale, float inv_count,
+                                                   double* __restrict__ loss,
+                                                   bf16* __restrict__ dY) {
+  static_assert(kCout == 16, "one 32-byte store per pixel");
+  __shared__ float sks;
+  wait_previous();
+  const int H = 1 << lgH, W = 1 << lgW, HW = H * W, b = blockIdx.y;
+  if (threadIdx.x == 0) sks = (float)(scale * inv_or_zero(rms[b]));
+  __syncthreads();
+  const float ks = sks;
+  const long off = (long)b * n * HW;
   double acc = 0.0;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const int x = (int)(i % W);
-    const int yy = (int)((i / W) % H), b = (int)(i / ((long)W * H));
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < HW; p += gridDim.x * blockDim.x) {
     float g[kCout];
-    for (int c = 0; c < kCout; ++c) g[c] = 0.f;
-    const float ks = (float)(scale * inv_or_zero(rms[b]));
-    for (int c = 0; c < n; ++c) {
-      const long k = (((long)b * n + c) * H + yy) * W + x;
-      const float d = y[k] - (t[k] - h[k]) * ks;
-      acc += (double)d * d;
-      g[c] = 2.f * d * inv_count;
+#pragma unroll
+    for (int c = 0; c < kCout; ++c) {
+      g[c] = 0.f;
+      if (c < n) {
+        const long k = off + (long)c * HW + p;
+        const float d = y[k] - (t[k] - h[k]) * ks;
+        acc += (double)d * d;
+        g[c] = 2.f * d * inv_count;
+      }
     }
-    for (int c = 0; c < kCout; c += 2) st_pair(dY, b, yy, x, H, W, kCout, c, g[c], g[c + 1]);
+    st_pixel16(dY, b, p >> lgW, p & (W - 1), H, W, g);
   }
   __shared__ double red[256];
   red[threadIdx.x] = acc;
@@ -765,6 +871,7 @@ __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict
 // shared memory and adds one atomic per channel.
 __global__ void __launch_bounds__(256) bias_grad_kernel(const bf16* __restrict__ dz, int B, int lgH,
                                                         int lgW, int lgG, float* __restrict__ db) {
+  wait_previous();
   const int H = 1 << lgH, W = 1 << lgW, C = 8 << lgG, g = 1 << lgG;
   const int pp = 256 >> lgG;  // pixels per block and iteration
   const int grp = threadIdx.x & (g - 1), sub = threadIdx.x >> lgG;
@@ -807,6 +914,7 @@ struct AdamArgs {
 // Adam step on the FP32 parameters, then the BF16 copies of every weight:
 // forward layout [o][t][c] and the input-gradient layout [c][t][o]
 __global__ void adam_kernel(const __grid_constant__ AdamArgs a, int do_step) {
+  wait_previous();
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < a.count; i += (long)gridDim.x * blockDim.x) {
     float w = a.p[i];
     if (do_step) {
@@ -913,38 +1021,59 @@ int bn_bwd(int l) {
 int bn_fwd(int l) { return std::min(kNet[l].cout, 128); }
 int bn_wgrad(int cin) { return cin <= 64 ? 64 : 128; }
 
-template <int KC, int BN>
-cudaError_t launch_conv_t(const ConvArgs& a, int ntn, int num_sms, cudaStream_t st) {
-  using S = ConvShape<KC, BN>;
+// launches a kernel as a programmatic dependent of the previous one
+template <class... P, class... A>
+cudaError_t launch_dep(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                       A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+template <int KC, int BN, bool RES>
+cudaError_t launch_conv_t(const ConvArgs& a, int ntn, int wblks, int num_sms, cudaStream_t st) {
+  using S = ConvShape<KC, BN, RES>;
   static bool attr[64] = {};
-  static int per_sm[64] = {};
+  auto kern = conv_tc<KC, BN, RES>;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 64) return cudaErrorInvalidDevice;
   if (!attr[dev]) {
-    e = cudaFuncSetAttribute(conv_tc<KC, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
-    // CTAs per SM by shared memory (228 KB, 1 KB reserved per CTA) and by
-    // tensor memory. Registers can hold fewer (the 16-channel input layer:
-    // 3 of 6), and the grid is then more than one wave; that measured
-    // faster than a grid of only the CTAs resident at once (2.08 against
-    // 1.79 ms per batch-32 prediction): CTAs that finish early make room
-    // for the rest, which balances the uneven tiles better.
-    const int by_smem = 233472 / ((int)S::SMEM + 1024);
-    per_sm[dev] = std::max(1, std::min(by_smem, S::CTAS_TMEM));
     attr[dev] = true;
   }
+  const size_t smem = S::smem(RES ? wblks : 0);
+  // CTAs per SM by shared memory (228 KB, 1 KB reserved per CTA), by tensor
+  // memory and by registers (three of 192 threads): one wave
+  const int by_smem = 233472 / ((int)smem + 1024);
+  const int per_sm = std::max(1, std::min(std::min(by_smem, S::CTAS_TMEM), 3));
   if (a.bias && a.cout > S::kBiasMax) return cudaErrorInvalidValue;
-  const int items = a.B_tiles * ntn;
-  const int grid = std::min(items, num_sms * per_sm[dev]);
-  conv_tc<KC, BN><<<grid, 192, S::SMEM, st>>>(a, ntn);
-  return cudaGetLastError();
+  const int grid = std::min(a.B_tiles * ntn, std::max(ntn, num_sms * per_sm / ntn * ntn));
+  return launch_dep(kern, dim3(grid), 192, smem, st, a, ntn, wblks);
 }
 
+// ntn output-channel tiles of bn channels, kc input channels at a time. The
+// weights stay resident where they leave room for the stages and a CTA has
+// several pixel tiles to use them for.
 cudaError_t launch_conv(int kc, int bn, const ConvArgs& a, int ntn, int num_sms, cudaStream_t st) {
-#define MLSW_CONV_CASE(K, N) \
-  if (kc == K && bn == N) return launch_conv_t<K, N>(a, ntn, num_sms, st);
+  const int wblks = 3 * (a.cin_tot / kc);
+#define MLSW_CONV_CASE(K, N)                                                         \
+  if (kc == K && bn == N) {                                                          \
+    const bool res = ConvShape<K, N, true>::need(wblks) <= 232448 &&                 \
+                     (long)a.B_tiles * ntn > 2L * num_sms;                           \
+    return res ? launch_conv_t<K, N, true>(a, ntn, wblks, num_sms, st)               \
+               : launch_conv_t<K, N, false>(a, ntn, 0, num_sms, st);                 \
+  }
   MLSW_CONV_CASE(16, 32)
   MLSW_CONV_CASE(32, 16)
   MLSW_CONV_CASE(32, 32)
@@ -968,8 +1097,7 @@ cudaError_t launch_wgrad_t(const WgradArgs& a, dim3 grid, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
-  wgrad_tc<BN><<<grid, 128, S::SMEM, st>>>(a);
-  return cudaGetLastError();
+  return launch_dep(wgrad_tc<BN>, grid, 128, S::SMEM, st, a);
 }
 
 int grid_for(long work, int threads) {
@@ -1009,7 +1137,8 @@ struct mlswlbm_unet {
   CUtensorMap act_map[kTensors];          // as a convolution input (KC of its consumer)
   CUtensorMap grad_map[kTensors];         // as an input-gradient convolution input
   CUtensorMap wg_act[kTensors], wg_grad[kTensors];  // weight-gradient operands
-  CUtensorMap wf_map[kLayers], wd_map[kLayers];
+  CUtensorMap wf_map[kLayers], wd_map[kLayers];      // weights, bn_fwd / bn_bwd rows a box
+  CUtensorMap wf_map32[kLayers], wd_map32[kLayers];  // the same, 32 rows (kc = 64 layers)
   int* err;
 };
 
@@ -1051,6 +1180,15 @@ int act_kc(int t) {
   return 0;
 }
 
+// Output channels per tile: 32 instead of bn where the coarse levels of a
+// small batch would leave most SMs idle (one 128^2 sample: 4 and 8 tiles of
+// 128 channels; 75 -> 61 us for its six 128- and 256-channel convolutions). The
+// order of every sum stays.
+int narrow_bn(int kc, int bn, const ConvArgs& a, int num_sms) {
+  const long items = (long)a.B_tiles * (a.cout / bn);
+  return kc == 64 && bn > 32 && 2 * items <= num_sms ? 32 : bn;
+}
+
 cudaError_t conv_forward(mlswlbm_unet* u, int l, int batch) {
   const Layer& N = kNet[l];
   ConvArgs a;
@@ -1079,7 +1217,9 @@ cudaError_t conv_forward(mlswlbm_unet* u, int l, int batch) {
   }
   a.err = u->err;
   a.B_tiles = batch * (a.W / 16) * (a.H / 8);
-  return launch_conv(kc_fwd(l), bn_fwd(l), a, N.cout / bn_fwd(l), u->num_sms, u->stream);
+  const int kc = kc_fwd(l), bn = narrow_bn(kc, bn_fwd(l), a, u->num_sms);
+  if (bn != bn_fwd(l)) a.w_map = u->wf_map32[l];
+  return launch_conv(kc, bn, a, N.cout / bn, u->num_sms, u->stream);
 }
 
 // input gradient of layer l: from grad of its output to the gradients of its
@@ -1111,8 +1251,9 @@ cudaError_t conv_input_grad(mlswlbm_unet* u, int l, int batch, bf16* out0, const
   }
   a.err = u->err;
   a.B_tiles = batch * (a.W / 16) * (a.H / 8);
-  const int bn = bn_bwd(l);
-  return launch_conv(kc_bwd(l), bn, a, a.cout / bn, u->num_sms, u->stream);
+  const int kc = kc_bwd(l), bn = narrow_bn(kc, bn_bwd(l), a, u->num_sms);
+  if (bn != bn_bwd(l)) a.w_map = u->wd_map32[l];
+  return launch_conv(kc, bn, a, a.cout / bn, u->num_sms, u->stream);
 }
 
 cudaError_t weight_grad(mlswlbm_unet* u, int l, int batch) {
@@ -1151,26 +1292,32 @@ cudaError_t weight_grad(mlswlbm_unet* u, int l, int batch) {
   // the output gradient has the layer's cout channels (YG: kCout)
   const int Cz = kTC[tz];
   const int bgrid = (int)std::max(1L, std::min((long)4 * u->num_sms, (long)batch * H * W * (Cz / 8) / 256));
-  bias_grad_kernel<<<bgrid, 256, 0, u->stream>>>(u->grad[tz], batch, ilog2(H), ilog2(W),
-                                                 ilog2(Cz / 8), u->pgrad + u->L[l].b_off);
-  return cudaGetLastError();
+  return launch_dep(bias_grad_kernel, dim3(bgrid), 256, 0, u->stream, u->grad[tz], batch, ilog2(H),
+                    ilog2(W), ilog2(Cz / 8), u->pgrad + u->L[l].b_off);
 }
 
 // plane means (mode 0) or sample RMS deviations about u->means (mode 1) of
 // a [batch][n][H][W] FP32 array
-void plane_reduce(mlswlbm_unet* u, const float* x, int batch, int mode, double* out) {
+cudaError_t plane_reduce(mlswlbm_unet* u, const float* x, int batch, int mode, double* out) {
   const int HW = u->H * u->W;
-  plane_reduce_kernel<<<dim3(HW / kRedChunk, batch * u->n), 256, 0, u->stream>>>(
-      x, batch * u->n, HW, u->n, mode, u->means, u->red_part, u->red_count, out);
+  return launch_dep(plane_reduce_kernel, dim3(HW / kRedChunk, batch * u->n), 256, 0, u->stream, x,
+                    batch * u->n, HW, u->n, mode, u->means, u->red_part, u->red_count, out);
+}
+
+// blocks per sample or plane of `work` items, a few items per thread
+int blocks_for(int work, int groups, int num_sms) {
+  const int most = (work + 255) / 256, want = std::max(1, 16 * num_sms / std::max(1, groups));
+  return std::min(most, want);
 }
 
 cudaError_t forward(mlswlbm_unet* u, const float* h, int batch) {
   const int HW = u->H * u->W;
-  plane_reduce(u, h, batch, 0, u->means);
-  plane_reduce(u, h, batch, 1, u->rms);
-  input_kernel<<<grid_for((long)batch * HW, 256), 256, 0, u->stream>>>(
-      h, u->means, u->rms, batch, u->n, u->H, u->W, u->in_scale, u->extra, u->n_extra, u->act[X0]);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = plane_reduce(u, h, batch, 0, u->means);
+  if (e == cudaSuccess) e = plane_reduce(u, h, batch, 1, u->rms);
+  if (e == cudaSuccess)
+    e = launch_dep(input_kernel, dim3(blocks_for(HW, batch, u->num_sms), batch), 256, 0, u->stream,
+                   h, u->means, u->rms, u->n, ilog2(u->H), ilog2(u->W), u->in_scale, u->extra,
+                   u->n_extra, u->act[X0]);
   if (e != cudaSuccess) return e;
   for (int l = 0; l < kLayers; ++l) {
     // pooling before the first convolution of a level on the way down,
@@ -1182,13 +1329,8 @@ cudaError_t forward(mlswlbm_unet* u, const float* h, int batch) {
       if (p.layer != l) continue;
       const int C = kTC[p.dst], Hd = u->lh[p.dst], Wd = u->lw[p.dst];
       const int grid = grid_for((long)batch * Hd * Wd * C / 8, 256);
-      if (p.up)
-        up_kernel<<<grid, 256, 0, u->stream>>>(u->act[p.src], u->act[p.dst], batch, ilog2(Hd),
-                                               ilog2(Wd), ilog2(C / 8));
-      else
-        pool_kernel<<<grid, 256, 0, u->stream>>>(u->act[p.src], u->act[p.dst], batch, ilog2(Hd),
-                                                 ilog2(Wd), ilog2(C / 8));
-      e = cudaGetLastError();
+      e = launch_dep(p.up ? up_kernel : pool_kernel, dim3(grid), 256, 0, u->stream,
+                     u->act[p.src], u->act[p.dst], batch, ilog2(Hd), ilog2(Wd), ilog2(C / 8));
       if (e != cudaSuccess) return e;
     }
     e = conv_forward(u, l, batch);
@@ -1208,15 +1350,16 @@ cudaError_t backward(mlswlbm_unet* u, int batch) {
   auto Aq = [&](int t) { return (const bf16*)u->act[t]; };
   auto upmask = [&](int dU, int S, int dS) {
     const int C = kTC[S], H = u->lh[dU], W = u->lw[dU];
-    up_grad_mask_kernel<<<grid_for((long)batch * (H / 2) * (W / 2) * C / 8, 256), 256, 0, u->stream>>>(
-        G(dU), Aq(S), G(dS), batch, ilog2(H / 2), ilog2(W / 2), ilog2(C / 8));
-    return cudaGetLastError();
+    return launch_dep(up_grad_mask_kernel,
+                      dim3(grid_for((long)batch * (H / 2) * (W / 2) * C / 8, 256)), 256, 0,
+                      u->stream, G(dU), Aq(S), G(dS), batch, ilog2(H / 2), ilog2(W / 2),
+                      ilog2(C / 8));
   };
   auto poolmask = [&](int dP, int lev, int S) {
     const int C = kTC[S], H = u->lh[S], W = u->lw[S];
-    pool_grad_add_mask_kernel<<<grid_for((long)batch * H * W * C / 8, 256), 256, 0, u->stream>>>(
-        G(dP), u->skipg[lev], Aq(S), G(S), batch, ilog2(H), ilog2(W), ilog2(C / 8));
-    return cudaGetLastError();
+    return launch_dep(pool_grad_add_mask_kernel, dim3(grid_for((long)batch * H * W * C / 8, 256)),
+                      256, 0, u->stream, G(dP), u->skipg[lev], Aq(S), G(S), batch, ilog2(H),
+                      ilog2(W), ilog2(C / 8));
   };
   // layer 14 (out) .. 0, see the table
   MLSW_CK(weight_grad(u, 14, batch));
@@ -1274,8 +1417,7 @@ cudaError_t adam(mlswlbm_unet* u, double lr, int do_step) {
   const double t = (double)(u->adam_t + (do_step ? 1 : 0));
   a.c1 = do_step ? (float)(1.0 / (1.0 - std::pow(0.9, t))) : 1.f;
   a.c2 = do_step ? (float)(1.0 / (1.0 - std::pow(0.999, t))) : 1.f;
-  adam_kernel<<<grid_for(u->nparam, 256), 256, 0, u->stream>>>(a, do_step);
-  return cudaGetLastError();
+  return launch_dep(adam_kernel, dim3(grid_for(u->nparam, 256)), 256, 0, u->stream, a, do_step);
 }
 
 bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
@@ -1431,6 +1573,8 @@ int mlswlbm_unet_create(int n_layers, int nx, int ny, int max_batch, int n_extra
       w += (size_t)9 * L.cout * L.cin;
       ok = map_weights(&u->wf_map[l], L.wf, L.cin, L.cout, kc_fwd(l), bn_fwd(l)) &&
            map_weights(&u->wd_map[l], L.wd, L.cout, L.cin, kc_bwd(l), bn_bwd(l));
+      if (ok && kc_fwd(l) == 64) ok = map_weights(&u->wf_map32[l], L.wf, L.cin, L.cout, 64, 32);
+      if (ok && kc_bwd(l) == 64) ok = map_weights(&u->wd_map32[l], L.wd, L.cout, L.cin, 64, 32);
     }
   }
   for (int t = 0; t < kTensors && ok; ++t) {
@@ -1477,11 +1621,15 @@ int mlswlbm_unet_predict(mlswlbm_unet* u, const float* h, float* out, int batch)
   if (!u || !h || !out || batch < 1 || batch > u->Bmax || out == h) return MLSW_ERR_ARG;
   if (forward(u, h, batch) != cudaSuccess) return MLSW_ERR_CUDA;
   const int HW = u->H * u->W;
-  plane_reduce(u, u->ydense, batch, 0, u->means);
-  const long total = (long)batch * u->n * HW;
-  output_kernel<<<grid_for(total, 256), 256, 0, u->stream>>>(h, u->ydense, u->means, u->rms, total,
-                                                              u->n, HW, 1.f / u->out_scale, out);
-  return cudaGetLastError() == cudaSuccess ? MLSW_OK : MLSW_ERR_CUDA;
+  if (plane_reduce(u, u->ydense, batch, 0, u->means) != cudaSuccess) return MLSW_ERR_CUDA;
+  const int planes = batch * u->n;
+  const int vec = ((reinterpret_cast<uintptr_t>(h) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+  const int work = vec ? HW / 4 : HW;
+  return launch_dep(output_kernel, dim3(blocks_for(work, planes, u->num_sms), planes), 256, 0,
+                    u->stream, h, u->ydense, u->means, u->rms, u->n, HW, 1.f / u->out_scale, vec,
+                    out) == cudaSuccess
+             ? MLSW_OK
+             : MLSW_ERR_CUDA;
 }
 
 int mlswlbm_unet_train_step(mlswlbm_unet* u, const float* h, const float* target, int batch, double lr,
@@ -1492,10 +1640,12 @@ int mlswlbm_unet_train_step(mlswlbm_unet* u, const float* h, const float* target
   if (cudaMemsetAsync(u->dloss, 0, sizeof(double), u->stream) != cudaSuccess ||
       cudaMemsetAsync(u->pgrad, 0, u->nparam * sizeof(float), u->stream) != cudaSuccess)
     return MLSW_ERR_CUDA;
-  loss_kernel<<<grid_for((long)batch * u->H * u->W, 256), 256, 0, u->stream>>>(
-      u->ydense, h, target, u->rms, batch, u->n, u->H, u->W, u->out_scale, 1.f / (float)count,
-      u->dloss, u->grad[YG]);
-  if (cudaGetLastError() != cudaSuccess || backward(u, batch) != cudaSuccess) return MLSW_ERR_CUDA;
+  const int HW = u->H * u->W;
+  if (launch_dep(loss_kernel, dim3(blocks_for(HW, batch, u->num_sms), batch), 256, 0, u->stream,
+                 u->ydense, h, target, u->rms, u->n, ilog2(u->H), ilog2(u->W), u->out_scale,
+                 1.f / (float)count, u->dloss, u->grad[YG]) != cudaSuccess ||
+      backward(u, batch) != cudaSuccess)
+    return MLSW_ERR_CUDA;
   if (adam(u, lr, 1) != cudaSuccess) return MLSW_ERR_CUDA;
   u->adam_t += 1;
   if (loss) {
