@@ -456,8 +456,8 @@ __global__ void friction_eval_kernel(KParams P, long ncell, const float* __restr
     for (int i = 0; i < N; ++i) {
       hh[i] = h[(long)i * ncell + c];
       ih[i] = rcp(hh[i]);
-      jx[i] = Jx[(long)i * ncell + c] * ih[i];  // mean velocities
-      jy[i] = Jy ? Jy[(long)i * ncell + c] * ih[i] : 0.f;
+      jx[i] = mulr(Jx[(long)i * ncell + c], ih[i]);  // mean velocities
+      jy[i] = Jy ? mulr(Jy[(long)i * ncell + c], ih[i]) : 0.f;
     }
     friction<N, true>(P, hh, ih, jx, jy, rx, ry);
 #pragma unroll

@@ -113,7 +113,7 @@ struct KParams {
 __device__ __forceinline__ float substrate_height(const KParams& P, long m, long nc) {
   float s, c;
   sincospif(2.f * (float)((double)m / (double)nc), &s, &c);
-  return P.sub_amp * c;
+  return __fmul_rn(P.sub_amp, c);  // not fused into the sum it starts
 }
 
 // Substrate height at lattice cell (x, y) (any integers: the cosine is
@@ -191,6 +191,14 @@ __device__ __forceinline__ f2 fmav(f2 a, float b, f2 c) { return fmav(a, mk2(b, 
 __device__ __forceinline__ f2 fmav(float a, f2 b, f2 c) { return fmav(mk2(a, a), b, c); }
 __device__ __forceinline__ f2 fmav(f2 a, f2 b, float c) { return fmav(a, b, mk2(c, c)); }
 __device__ __forceinline__ f2 fmav(f2 a, float b, float c) { return fmav(a, mk2(b, b), mk2(c, c)); }
+
+// a product that is rounded by itself: the compiler fuses a scalar product
+// into an addition where it likes, differently from kernel to kernel, and a
+// packed one never. Products that feed additions go through this, so that
+// scalar and packed cells, and all kernels, round identically.
+__device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ f2 mulr(f2 a, f2 b) { return a * b; }
+__device__ __forceinline__ f2 mulr(f2 a, float b) { return a * b; }
 
 // fast reciprocal: the hardware's approximation, at most 1 ulp for normal
 // arguments (here layer thicknesses and friction pivots, far from the ends
@@ -283,26 +291,24 @@ __device__ __forceinline__ void interface_pairs(const KParams& P, const T (&zd)[
         // phi' = 2 kappa a (a - 1)
         const T a = expv(fmav(d, -P.kappa, P.kappa * ((float)k * P.hstar)));
         phi = a * (2.f - a);
-        e = (s * (2.f * P.kappa)) * (a * (a - 1.f));
+        e = mulr(a * (a - 1.f), s * (2.f * P.kappa));
       } else {
         const T inv_d = rcp(d);
         const T r = ((float)k * P.hstar) * inv_d;
         if constexpr (FORM == kPower32) {
           const T r2 = r * r;
           phi = r2 * fmav(r, -2.f, 3.f);
-          e = (k == 1 ? P.Sd[l] : s * P.c_dphi) * ((r2 * (r - 1.f)) * inv_d);
+          e = mulr((r2 * (r - 1.f)) * inv_d, k == 1 ? P.Sd[l] : s * P.c_dphi);
         } else {
-          const T rm = ipow(r, P.mw), rn = rm * ipow(r, P.nw - P.mw);
+          const T rm = ipow(r, P.mw), rn = mulr(rm, ipow(r, P.nw - P.mw));
           phi = fmav(rm, (float)P.nw, rn * (-(float)P.mw)) * P.c_phi;
-          e = (s * P.c_dphi) * ((rn - rm) * inv_d);
+          e = mulr((rn - rm) * inv_d, s * P.c_dphi);
         }
       }
-      // explicit fused updates, so one cell and a packed pair of cells
-      // round identically
       if (l > 0)
-        e = e * sg[i];
+        e = mulr(e, sg[i]);
       else if (sg0)
-        e = e * *sg0;
+        e = mulr(e, *sg0);
       if constexpr (FORM != kPower32) {  // r^64 of a thin film may overflow
         phi = keep_if(s != 0.f, phi);
         e = keep_if(s != 0.f, e);
@@ -384,7 +390,7 @@ __device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], cons
   T na_prev;  // -a_{i-1}
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const T na = h[i] * P.fr_visc[i], s = ih[i] * P.fr_slip2[i];
+    const T na = mulr(h[i], P.fr_visc[i]), s = mulr(ih[i], P.fr_slip2[i]);
     T diag = fmav(na, -2.f, s + P.fr_slip[i]);
     nsup[i] = na + s;
     if (i == 0) {
@@ -404,10 +410,10 @@ __device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], cons
 #pragma unroll
   for (int i = N - 1; i >= 0; --i) {
     const T ox = tx, oy = ty;
-    tx = (i == N - 1 ? bx[i] : fmav(nsup[i], ox, bx[i])) * piv[i];
+    tx = mulr(i == N - 1 ? bx[i] : fmav(nsup[i], ox, bx[i]), piv[i]);
     Rx[i] = i == N - 1 ? tx : tx - ox;
     if constexpr (TWO) {
-      ty = (i == N - 1 ? by[i] : fmav(nsup[i], oy, by[i])) * piv[i];
+      ty = mulr(i == N - 1 ? by[i] : fmav(nsup[i], oy, by[i]), piv[i]);
       Ry[i] = i == N - 1 ? ty : ty - oy;
     }
   }

@@ -68,7 +68,7 @@ __device__ __forceinline__ bool d1q3_collide_cell(const KParams& P, const float 
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     ih[i] = rcp(hh[i]);
-    ux[i] = jx[i] * ih[i];
+    ux[i] = mulr(jx[i], ih[i]);
   }
   friction<N, false>(P, hh, ih, ux, ux, Rx, Rx);
   bool bad = false;
@@ -185,90 +185,94 @@ __global__ void __launch_bounds__(TX)
 
 // ---------------------------------------------------------------------------
 // D1Q3, persistent: one CTA holds the whole lattice in shared memory and
-// runs nsteps steps in one launch, with barriers between the phases of a
-// step instead of kernel launches. Shared memory (floats): two population
-// buffers [3N][nx], z [N][nx], p [N][nx]. The lattice is read from fin and
-// the final state written to fout (which may be fin), ghost images
-// included. Same cell arithmetic as step_d1q3_kernel.
+// runs nsteps steps in one launch. A warp takes 32 neighbouring cells at a
+// time and writes the inner 26: z, the pressures and the streamed populations
+// pass between cells by shuffles, the three cells on each side are computed
+// again by the neighbours, and a step needs one barrier instead of three
+// (512 cells, two layers: 0.88 -> 0.67 us a step; it is bound by the issue of
+// 20 warps on one SM). Shared memory (floats): two population
+// buffers [3N][nx], the substrate [nx]. The lattice is read from fin and the
+// final state written to fout (which may be fin), ghost images included.
+// Same cell arithmetic as step_d1q3_kernel.
 // ---------------------------------------------------------------------------
-constexpr int kD1PT = 256;
+constexpr int kD1Out = 26;  // cells a warp writes
+// threads: 20 warps cover 520 cells at once; more layers need the registers
+constexpr int d1_threads(int n) { return n <= 3 ? 640 : 512; }
 
 template <int N, bool TAU1, bool W32>
-__global__ void __launch_bounds__(kD1PT)
+__global__ void __launch_bounds__(d1_threads(N), 1)
     step_d1q3_persistent(const float* fin, float* fout, const KParams P, int nsteps,
                          int* __restrict__ status) {
   constexpr int Q = 3;
+  constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ __align__(16) float sm[];
   const Layout& L = P.L;
-  const int nx = P.nx, tid = threadIdx.x;
+  const int nx = P.nx, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   float* fa = sm;                     // current populations [i * Q + k][x]
   float* fb = fa + 3 * N * nx;        // next populations
-  float* zsm = fb + 3 * N * nx;       // [i][x]
-  float* psm = zsm + N * nx;          // [i][x]
-  for (int t = tid; t < Q * N * nx; t += kD1PT) {
+  float* z0s = fb + 3 * N * nx;       // [x]
+  for (int t = tid; t < Q * N * nx; t += nt) {
     const int pl = t / nx, x = t - pl * nx;
     *chk_smem(fa + t) = fin[L.at(pl, x, 0)];
   }
+  const bool sub = P.sub_amp != 0.f;
+  if (sub)
+    for (int x = tid; x < nx; x += nt) *chk_smem(z0s + x) = substrate_at(P, x, 0);
   __syncthreads();
   bool bad = false;
   for (int s = 0; s < nsteps; ++s) {
-    // moments -> z
-    for (int x = tid; x < nx; x += kD1PT) {
-      float z = P.sub_amp != 0.f ? substrate_at(P, x, 0) : 0.f;
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        z += *chk_smem(fa + (i * Q + 0) * nx + x) +
-             (*chk_smem(fa + (i * Q + 1) * nx + x) + *chk_smem(fa + (i * Q + 2) * nx + x));
-        *chk_smem(zsm + i * nx + x) = z;
+    for (int c0 = (tid >> 5) * kD1Out; c0 < nx; c0 += (nt >> 5) * kD1Out) {
+      const int xo = c0 - 3 + lane;  // this lane's cell before wrapping
+      int x = xo;
+      if (x < 0 || x >= nx) {
+        x %= nx;
+        x += x < 0 ? nx : 0;
       }
-    }
-    __syncthreads();
-    // pressures
-    for (int x = tid; x < nx; x += kD1PT) {
-      const int xw = x == 0 ? nx - 1 : x - 1, xe = x == nx - 1 ? 0 : x + 1;
-      float zw[N], zc[N], ze[N], p[N];
+      const float z0 = sub ? *chk_smem(z0s + x) : 0.f;
+      float g0[N], sm_[N], hh[N], jx[N], fo[N][Q], fs[N][Q];
+      float zw[N], zc[N], ze[N], pw[N], pc[N], pe[N];
+      float z = z0;
 #pragma unroll
       for (int i = 0; i < N; ++i) {
-        zw[i] = *chk_smem(zsm + i * nx + xw);
-        zc[i] = *chk_smem(zsm + i * nx + x);
-        ze[i] = *chk_smem(zsm + i * nx + xe);
-      }
-      if (P.sub_amp != 0.f)
-        d1q3_pressures<N, W32>(P, zw, zc, ze, p, substrate_at(P, x - 1, 0),
-                               substrate_at(P, x, 0), substrate_at(P, x + 1, 0));
-      else
-        d1q3_pressures<N, W32>(P, zw, zc, ze, p);
 #pragma unroll
-      for (int i = 0; i < N; ++i) *chk_smem(psm + i * nx + x) = p[i];
-    }
-    __syncthreads();
-    // force, collision, streaming into fb
-    for (int x = tid; x < nx; x += kD1PT) {
-      const int xw = x == 0 ? nx - 1 : x - 1, xe = x == nx - 1 ? 0 : x + 1;
-      float g0[N], sm[N], hh[N], jx[N], pw[N], pc[N], pe[N], fo[N][Q], fs[N][Q];
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        const float f0 = *chk_smem(fa + (i * Q + 0) * nx + x);
-        const float f1 = *chk_smem(fa + (i * Q + 1) * nx + x);
-        const float f2 = *chk_smem(fa + (i * Q + 2) * nx + x);
-        const float sum = f0 + (f1 + f2);
-        g0[i] = f0;
-        sm[i] = f1 + f2;
+        for (int k = 0; k < Q; ++k) fo[i][k] = *chk_smem(fa + (i * Q + k) * nx + x);
+        g0[i] = fo[i][0];
+        sm_[i] = fo[i][1] + fo[i][2];
+        const float sum = fo[i][0] + (fo[i][1] + fo[i][2]);
         hh[i] = P.H[i] + sum;
-        jx[i] = f1 - f2;
-        fo[i][0] = f0;
-        fo[i][1] = f1;
-        fo[i][2] = f2;
-        pw[i] = *chk_smem(psm + i * nx + xw);
-        pc[i] = *chk_smem(psm + i * nx + x);
-        pe[i] = *chk_smem(psm + i * nx + xe);
+        jx[i] = fo[i][1] - fo[i][2];
+        z += sum;
+        zc[i] = z;
       }
-      bad |= d1q3_collide_cell<N, TAU1>(P, g0, sm, hh, jx, pw, pc, pe, fo, fs);
-      const int dst[3] = {x, xe, xw};  // c_k = 0, +1, -1
 #pragma unroll
-      for (int i = 0; i < N; ++i)
+      for (int i = 0; i < N; ++i) {
+        zw[i] = __shfl_up_sync(kAll, zc[i], 1);
+        ze[i] = __shfl_down_sync(kAll, zc[i], 1);
+      }
+      if (sub) {
+        const float z0w = __shfl_up_sync(kAll, z0, 1), z0e = __shfl_down_sync(kAll, z0, 1);
+        d1q3_pressures<N, W32>(P, zw, zc, ze, pc, z0w, z0, z0e);
+      } else {
+        d1q3_pressures<N, W32>(P, zw, zc, ze, pc);
+      }
 #pragma unroll
-        for (int k = 0; k < Q; ++k) *chk_smem(fb + (i * Q + k) * nx + dst[k]) = fs[i][k];
+      for (int i = 0; i < N; ++i) {
+        pw[i] = __shfl_up_sync(kAll, pc[i], 1);
+        pe[i] = __shfl_down_sync(kAll, pc[i], 1);
+      }
+      const bool cell_bad = d1q3_collide_cell<N, TAU1>(P, g0, sm_, hh, jx, pw, pc, pe, fo, fs);
+      const bool own = lane >= 3 && lane < 3 + kD1Out && xo < nx;
+      bad |= own && cell_bad;
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const float right = __shfl_up_sync(kAll, fs[i][1], 1);   // c = +1, from x - 1
+        const float left = __shfl_down_sync(kAll, fs[i][2], 1);  // c = -1, from x + 1
+        if (own) {
+          *chk_smem(fb + (i * Q + 0) * nx + x) = fs[i][0];
+          *chk_smem(fb + (i * Q + 1) * nx + x) = right;
+          *chk_smem(fb + (i * Q + 2) * nx + x) = left;
+        }
+      }
     }
     __syncthreads();
     float* t = fa;
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(kD1PT)
     fb = t;
   }
   // final state, real cells and the ghost images x in [-2, nx + 2)
-  for (int t = tid; t < Q * N * (nx + 4); t += kD1PT) {
+  for (int t = tid; t < Q * N * (nx + 4); t += nt) {
     const int pl = t / (nx + 4), x = t - pl * (nx + 4) - 2;
     int sx = x % nx;
     sx += sx < 0 ? nx : 0;
@@ -330,7 +334,9 @@ static cudaError_t launch_d1p(const StepLaunch& a, int nsteps, cudaStream_t st) 
   const size_t smem = step_persistent_smem(N, 1, a.P.nx);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<1, kD1PT, smem, st>>>(a.fin, a.fout, a.P, nsteps, a.status);
+  const int warps = (a.P.nx + kD1Out - 1) / kD1Out;
+  const int threads = 32 * warps < d1_threads(N) ? 32 * warps : d1_threads(N);
+  kern<<<1, threads, smem, st>>>(a.fin, a.fout, a.P, nsteps, a.status);
   return cudaGetLastError();
 }
 

@@ -51,3 +51,19 @@ def test_populations_and_split_runs_at_edge_sizes(nx, ny, n, tau):
         m.step(2)
         m.step(3)
         assert np.array_equal(m.get_heights(1), a.get_heights())
+
+
+@pytest.mark.parametrize("nx", [1, 4, 25, 26, 27, 53, 520, 521, 1100])
+@pytest.mark.parametrize("n,tau,sub", [(1, 1.0, 0.0), (2, 0.8, 0.0), (3, 1.0, 0.1), (5, 1.0, 0.0)])
+def test_d1q3_persistent_cell_groups(nx, n, tau, sub):
+    """The one-CTA D1Q3 kernel at the edges of its groups of 26 cells: the
+    bits of one launch per step, flat and corrugated substrate."""
+    p = workloads.random_params(970 + n, n, B.MLSW_D1Q3, nx, 1, tau=tau)
+    p.update(sub_amp=sub, sub_kx=2)
+    h0 = workloads.random_heights(971, p)
+    q = dict(p, flags=B.MLSW_FLAG_NO_PERSISTENT)
+    with B.Solver(p, h0) as a, B.Solver(q, h0) as b:
+        a.step(12)
+        b.step(12)
+        assert np.array_equal(a.get_state(), b.get_state())
+        assert a.status() == B.MLSW_OK
