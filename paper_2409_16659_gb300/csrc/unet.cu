@@ -134,7 +134,7 @@ struct ConvShape {
   static constexpr int ST0 = 204 * 1024 / STAGE;
   // small stages (the 16- and 32-channel layers): six deep, which measured
   // faster than four with more CTAs per SM
-  static constexpr int ST = RES ? (KC <= 16 ? 6 : 4)
+  static constexpr int ST = RES ? (KC <= 16 || (KC == 64 && BN <= 64) ? 6 : 4)
                                 : (STAGE <= 25 * 1024 ? 6 : (STAGE <= 50 * 1024 ? 4 : (ST0 < 2 ? 2 : ST0)));
   static constexpr int ACOLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : 128);
   static constexpr int TCOLS = 2 * ACOLS;          // two accumulators
@@ -877,12 +877,26 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const bf16* __restrict__
   const int grp = threadIdx.x & (g - 1), sub = threadIdx.x >> lgG;
   const long npix = (long)B << (lgH + lgW);
   float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (long q = (long)blockIdx.x * pp + sub; q < npix; q += (long)gridDim.x * pp) {
+  const long step = (long)gridDim.x * pp;
+  auto load = [&](long q) {
     const int x = (int)(q & (W - 1)), y = (int)((q >> lgW) & (H - 1)), b = (int)(q >> (lgW + lgH));
-    const Oct v = ld_oct(dz, hidx(b, y, x, H, W, C) + grp * 8);
+    return ld_oct(dz, hidx(b, y, x, H, W, C) + grp * 8);
+  };
+  auto add = [&](const Oct& v) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) s[j] += v.v[j];
+  };
+  // four pixels in flight: a read of every gradient tensor once, bound by
+  // the latency of one load per thread without it
+  long q = (long)blockIdx.x * pp + sub;
+  for (; q + 3 * step < npix; q += 4 * step) {
+    const Oct v0 = load(q), v1 = load(q + step), v2 = load(q + 2 * step), v3 = load(q + 3 * step);
+    add(v0);
+    add(v1);
+    add(v2);
+    add(v3);
   }
+  for (; q < npix; q += step) add(load(q));
   __shared__ float red[256][9];
 #pragma unroll
   for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = s[j];
