@@ -34,7 +34,7 @@ __device__ __forceinline__ void run_kind(int kind, const KParams& P, const Batch
   if (kind == K) {
     float* fout = b.f[cur ^ 1];
     __builtin_assume(__isGlobal(fout));
-    march_unit<N, M, M == kGeneral>(P, &b.map[cur], fout, x0, ya, yb, sm, status);
+    march_unit<N, M, M == kGeneral, false>(P, &b.map[cur], fout, x0, ya, yb, sm, status);
   } else if constexpr (K + 1 < 3 * MLSW_BATCH_N) {
     run_kind<K + 1>(kind, P, b, cur, x0, ya, yb, sm, status);
   }
@@ -52,7 +52,9 @@ size_t smem_from(unsigned kinds) {
 }  // namespace
 
 // The instance's parameters are read from a copy in shared memory: in global
-// memory every use after a store would load them again.
+// memory every use after a store would load them again. One row a turn: the
+// kinds' code is long, and the warps of an SM wait for instructions (48 lattices
+// of 2 to 5 layers: 198 us a step with two rows, 182 with one).
 template <int NMAX>
 __global__ void __launch_bounds__(32, kWarps)
     step_d2q9_batch(const BatchInst* __restrict__ inst, const int2* __restrict__ table, int cur,

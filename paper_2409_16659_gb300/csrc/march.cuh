@@ -199,14 +199,15 @@ struct SubstratePhase {
 // column x0, by one warp. sm: MarchShape::kSmem bytes, 128-byte aligned.
 // wait: the programmatic-launch wait for the previous grid (every global
 // access comes after it).
-template <int N, int MODE, bool OP>
+// TWO: two rows a turn of the main loop.
+template <int N, int MODE, bool OP, bool TWO>
 __device__ __forceinline__ void march_unit(const KParams& P, const CUtensorMap* map,
                                            float* __restrict__ fout, int x0, int ya, int yb,
                                            unsigned char* sm, int* __restrict__ status) {
   using S = MarchShape<N, MODE, OP>;
   constexpr bool TAU1 = S::TAU1, W32 = MODE == kFast, NN = MODE == kFast;
   constexpr int Q = 9, RS = S::RS, CW = kMarchCols;
-  constexpr int kTwoRows = N <= 3 ? 2 : 1;  // rows a turn of the main loop (four layers: spills)
+  constexpr int kRows = TWO ? 2 : 1;
   float* ring = reinterpret_cast<float*>(sm);
   float* park = reinterpret_cast<float*>(sm + S::kOffPark) + 2 * (threadIdx.x & 31);
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + S::kOffBar);
@@ -484,7 +485,7 @@ __device__ __forceinline__ void march_unit(const KParams& P, const CUtensorMap* 
       }
       roll_z(zn, sn);
     }
-#pragma unroll kTwoRows
+#pragma unroll kRows
     for (; t < T && ok; ++t) {
       f2 zn[N], pn[N], sn = zero;
       ok = arrive(t, zn, sn);

@@ -24,8 +24,9 @@ __global__ void __launch_bounds__(32, march_min_warps(N, MODE))
               const __grid_constant__ KParams P, int strips, int rows, int* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int strip = (int)(blockIdx.x % strips), ya = (int)(blockIdx.x / strips) * rows;
-  march_unit<N, MODE, OP>(P, &map, fout, strip * kMarchOut, ya, min(ya + rows, P.ny), smem_raw,
-                              status);
+  // (two rows a turn spill from four layers on)
+  march_unit<N, MODE, OP, N <= 3>(P, &map, fout, strip * kMarchOut, ya, min(ya + rows, P.ny),
+                                  smem_raw, status);
 }
 
 // Rows of a unit. A unit costs its rows plus about five rows of warm-up. On
