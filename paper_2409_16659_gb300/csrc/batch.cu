@@ -44,6 +44,8 @@ struct mlsw_batch {
   int2* dtable;  // the unit table, sorted by kind
   int nunits, nmax;    // its length, the largest layer count in it
   unsigned kinds;      // kinds in it
+  int same_params;     // its instances' parameters differ in H and Hsum only
+  KParams params;         // of the first instance in it
   std::vector<int> tiny;  // selected instances whose ghosts need a pass of their own
   float* arena;
   int* dstatus;  // error bits
@@ -83,11 +85,13 @@ int unit_rows(int variant, int r) {
 // 256^2: r = 12 instead of 16 brings a step from 47 to 44 us.
 int scale_for(const mlsw_batch* b, const std::vector<int>& members, const std::vector<int>& variant) {
   int nmax = 0, nmin = mlsw::kMaxLayers;
+  unsigned kinds = 0;
   for (int j : members) {
     nmax = std::max(nmax, b->hinst[j].P.n);
     nmin = std::min(nmin, b->hinst[j].P.n);
+    kinds |= 1u << b->hinst[j].kind;
   }
-  const int per_sm = mlsw::batch_warps_per_sm(nmax);
+  const int per_sm = mlsw::batch_warps_per_sm(kinds);
   const double schedulers = 4.0 * b->num_sms, slots = (double)per_sm * b->num_sms;
   int best_r = 1;
   double best = 0.0;
@@ -157,6 +161,18 @@ int init_all(mlsw_batch* b, const float* const* h_init) {
   return MLSW_OK;
 }
 
+// whether the parameters of the members differ in H and Hsum only
+int same_params(const mlsw_batch* b, const std::vector<int>& members) {
+  for (int j : members) {
+    KParams q = b->hinst[j].P;
+    const KParams& p = b->hinst[members[0]].P;
+    std::memcpy(q.H, p.H, sizeof(q.H));
+    std::memcpy(q.Hsum, p.Hsum, sizeof(q.Hsum));
+    if (std::memcmp(&q, &p, sizeof(q)) != 0) return 0;
+  }
+  return 1;
+}
+
 // the unit table of the groups for the current variant choice, sorted by
 // kind (layer count descending: the dearest units first, so that the last
 // ones to run are short), and the unit rows in the descriptors
@@ -176,6 +192,8 @@ int build_groups(mlsw_batch* b) {
     if (bi.P.tiny) b->tiny.push_back(j);
   }
   const int r = all.empty() ? 1 : scale_for(b, all, b->variant);
+  b->same_params = same_params(b, all);
+  if (!all.empty()) b->params = b->hinst[all[0]].P;
   std::vector<int2> table;
   b->groups.clear();
   for (auto& kv : members) {
@@ -211,6 +229,8 @@ mlsw::BatchLaunch step_launch(const mlsw_batch* b) {
   a.nunits = b->nunits;
   a.nmax = b->nmax;
   a.kinds = b->kinds;
+  a.same_params = b->same_params;
+  a.P = b->params;
   a.cur = b->cur;
   a.status = b->dstatus;
   return a;
@@ -260,6 +280,8 @@ int autotune(mlsw_batch* b) {
       a.nunits = (int)table.size();
       a.nmax = n;
       a.kinds = 1u << mlsw::batch_kind(n, mode);
+      a.same_params = same_params(b, kv.second);
+      a.P = b->hinst[kv.second[0]].P;
       constexpr int kWarm = 2, kTimed = 6;
       float ms = 0.f;
       for (int s = 0; s < kWarm + kTimed && rc == MLSW_OK; ++s) {

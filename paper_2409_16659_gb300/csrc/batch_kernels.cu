@@ -18,11 +18,8 @@ namespace mlsw {
 
 namespace {
 
-constexpr size_t kParBytes = (sizeof(KParams) + 127) / 128 * 128;
-static_assert(sizeof(KParams) % 4 == 0, "parameters are copied as words");
-
-// Warps per SM, as for the single lattice (step_d2q9.cu).
-constexpr int kWarps = MLSW_BATCH_N <= 3 ? 12 : 8;
+// Warps per SM, as for the single lattice.
+constexpr int kWarps = march_warps(MLSW_BATCH_N, kFast);
 
 // The unit, if its kind is K, else the next kinds. Straight-line code: as
 // separate functions the kinds would lose the registers that carry rows.
@@ -34,7 +31,7 @@ __device__ __forceinline__ void run_kind(int kind, const KParams& P, const Batch
   if (kind == K) {
     float* fout = b.f[cur ^ 1];
     __builtin_assume(__isGlobal(fout));
-    march_unit<N, M, M == kGeneral, false>(P, &b.map[cur], fout, x0, ya, yb, sm, status);
+    march_unit<N, M, M == kGeneral, false>(P, P, &b.map[cur], fout, x0, ya, yb, sm, status);
   } else if constexpr (K + 1 < 3 * MLSW_BATCH_N) {
     run_kind<K + 1>(kind, P, b, cur, x0, ya, yb, sm, status);
   }
@@ -62,11 +59,7 @@ __global__ void __launch_bounds__(32, kWarps)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int2 e = table[blockIdx.x];
   const BatchInst& b = inst[e.x];
-  int* dst = reinterpret_cast<int*>(smem_raw);
-  const int* src = reinterpret_cast<const int*>(&b.P);
-  for (int w = threadIdx.x; w < (int)(sizeof(KParams) / 4); w += 32) *chk_smem(dst + w) = src[w];
-  __syncwarp();
-  const KParams& P = *reinterpret_cast<const KParams*>(smem_raw);
+  const KParams& P = stage_params(b, smem_raw);
   const int strip = e.y % b.strips, ya = e.y / b.strips * b.rows;
   run_kind<0>(b.kind, P, b, cur, strip * kMarchOut, ya, min(ya + b.rows, P.ny),
                       smem_raw + kParBytes, status);
@@ -104,10 +97,21 @@ cudaError_t launch_batch_step_n<MLSW_BATCH_N>(const BatchLaunch& a, cudaStream_t
 
 #if MLSW_BATCH_N == 5
 cudaError_t launch_batch_step(const BatchLaunch& a, cudaStream_t st) {
+  // instances of one kind have a kernel of their own
+  for (int k = 0; k < kBatchKinds; ++k)
+    if (a.kinds == 1u << k) return launch_batch_alike(a, k / 3 + 1, k % 3, st);
   return a.nmax <= 3 ? launch_batch_step_n<3>(a, st) : launch_batch_step_n<5>(a, st);
 }
 
-int batch_warps_per_sm(int nmax) { return nmax <= 3 ? 12 : 8; }
+int batch_warps_per_sm(unsigned kinds) {
+  int nmax = 0, alike = 0;
+  for (int k = 0; k < kBatchKinds; ++k) {
+    if (kinds == 1u << k) alike = march_warps(k / 3 + 1, k % 3);
+    if ((kinds >> k) & 1u) nmax = k / 3 + 1;
+  }
+  // (the same number on each of the four schedulers)
+  return (alike ? alike + 3 : march_warps(nmax <= 3 ? 3 : 5, kFast)) / 4 * 4;
+}
 #endif
 
 MLSW_DEFINE_BOUNDS_READER(MLSW_CAT(bounds_violations_batch_, MLSW_BATCH_N))

@@ -98,12 +98,23 @@ struct BatchLaunch {
   int nunits;
   int nmax;        // largest layer count in the table
   unsigned kinds;  // bit k: instances of kind k are in the table
+  int same_params; // the instances' parameters are P's but for H and Hsum
+  KParams P;
   int cur;
   int* status;
 };
 // warps of a batch step resident on one SM
-int batch_warps_per_sm(int nmax);
+int batch_warps_per_sm(unsigned kinds);
 cudaError_t launch_batch_step(const BatchLaunch& a, cudaStream_t st);
+// all of one kind (step_d2q9.cu)
+cudaError_t launch_batch_alike(const BatchLaunch& a, int n, int mode, cudaStream_t st);
+template <int N>
+cudaError_t launch_alike_d2q9(const BatchLaunch& a, int mode, cudaStream_t st);
+template <> cudaError_t launch_alike_d2q9<1>(const BatchLaunch& a, int mode, cudaStream_t st);
+template <> cudaError_t launch_alike_d2q9<2>(const BatchLaunch& a, int mode, cudaStream_t st);
+template <> cudaError_t launch_alike_d2q9<3>(const BatchLaunch& a, int mode, cudaStream_t st);
+template <> cudaError_t launch_alike_d2q9<4>(const BatchLaunch& a, int mode, cudaStream_t st);
+template <> cudaError_t launch_alike_d2q9<5>(const BatchLaunch& a, int mode, cudaStream_t st);
 // the kernel for at most NMAX layers (3: more warps fit an SM; 5)
 template <int NMAX>
 cudaError_t launch_batch_step_n(const BatchLaunch& a, cudaStream_t st);

@@ -195,13 +195,37 @@ struct SubstratePhase {
   }
 };
 
+// Warps per SM that the registers must allow, in moment form without spills:
+// three layers 12 (168 registers; 16 warps at 128 spill into the 15 KB of L1
+// that the rings leave: 76 us a step against 29 at 1024^2; 8 warps: 97
+// against 89 us at 2048^2), two layers 14 (the registers of 16), one layer 20,
+// four and five 8. The other modes carry their options besides: 8 from three
+// layers on.
+__host__ __device__ constexpr int march_warps(int n, int mode) {
+  return n == 1 ? 20 : (n == 2 ? 14 : (n == 3 && mode == kFast ? 12 : 8));
+}
+
+// A batch instance's parameters, copied to the start of the warp's shared
+// memory (kParBytes).
+constexpr size_t kParBytes = (sizeof(KParams) + 127) / 128 * 128;
+static_assert(sizeof(KParams) % 4 == 0, "parameters are copied as words");
+__device__ __forceinline__ const KParams& stage_params(const BatchInst& b, unsigned char* sm) {
+  int* dst = reinterpret_cast<int*>(sm);
+  const int* src = reinterpret_cast<const int*>(&b.P);
+  for (int w = threadIdx.x; w < (int)(sizeof(KParams) / 4); w += 32) *chk_smem(dst + w) = src[w];
+  __syncwarp();
+  return *reinterpret_cast<const KParams*>(sm);
+}
+
 // One unit of work: the output rows [ya, yb) of the strip that starts at
 // column x0, by one warp. sm: MarchShape::kSmem bytes, 128-byte aligned.
 // wait: the programmatic-launch wait for the previous grid (every global
 // access comes after it).
-// TWO: two rows a turn of the main loop.
+// TWO: two rows a turn of the main loop. G: the parameters that hold the
+// rest-population shifts H and Hsum (P itself, or see neg_pressures).
 template <int N, int MODE, bool OP, bool TWO>
-__device__ __forceinline__ void march_unit(const KParams& P, const CUtensorMap* map,
+__device__ __forceinline__ void march_unit(const KParams& P, const KParams& G,
+                                           const CUtensorMap* map,
                                            float* __restrict__ fout, int x0, int ya, int yb,
                                            unsigned char* sm, int* __restrict__ status) {
   using S = MarchShape<N, MODE, OP>;
@@ -332,9 +356,9 @@ __device__ __forceinline__ void march_unit(const KParams& P, const CUtensorMap* 
       f2 g0x, g0y, l0;
       lattice_derivatives<true>(sc, sn - sc, sB, g0x, g0y, l0);
       const f2 sg0 = fmav(0.5f, fmav(g0x, g0x, g0y * g0y), mk2(1.f, 1.f));
-      neg_pressures<N, W32, f2, NN>(P, zd, gx, gy, lz, pn, &sc, &sg0);
+      neg_pressures<N, W32, f2, NN>(P, G, zd, gx, gy, lz, pn, &sc, &sg0);
     } else {
-      neg_pressures<N, W32, f2, NN>(P, zd, gx, gy, lz, pn);
+      neg_pressures<N, W32, f2, NN>(P, G, zd, gx, gy, lz, pn);
     }
   };
   auto roll_z = [&](const f2 (&zn)[N], f2 sn) {
@@ -379,7 +403,7 @@ __device__ __forceinline__ void march_unit(const KParams& P, const CUtensorMap* 
         jx[i] = ld_pair(src + 2 * CW);
         jy[i] = ld_pair(src + 3 * CW);
       }
-      hh[i] = (g0[i] + sm_[i]) + P.H[i];
+      hh[i] = (g0[i] + sm_[i]) + G.H[i];
       ih[i] = rcp(hh[i]);
       ux[i] = jx[i] * ih[i];
       uy[i] = jy[i] * ih[i];

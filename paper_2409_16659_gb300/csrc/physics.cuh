@@ -259,6 +259,8 @@ __device__ __forceinline__ T ipow(T r, int e) {
 // as phi = r^2 (3 - 2 r), phi' = 6 r^2 (r - 1) / d.
 // z0, sg0: the substrate height z_0 (on the scale of zd) and 1 + |grad z_0|^2 / 2
 // at the cell; null for the flat substrate (0 and 1).
+// G: the parameters that hold the reference thicknesses Hsum (P itself, but
+// for alike lattices of a batch, which share the rest).
 //
 // Without NN or W32 the options are run-time values, but uniform ones: the
 // pairs are evaluated in straight-line code for one combination (with or
@@ -268,7 +270,8 @@ __device__ __forceinline__ T ipow(T r, int e) {
 enum PairForm { kPower32, kPower, kExponential };
 
 template <int N, bool FAR, int FORM, class T>
-__device__ __forceinline__ void interface_pairs(const KParams& P, const T (&zd)[N],
+__device__ __forceinline__ void interface_pairs(const KParams& P, const KParams& G,
+                                                const T (&zd)[N],
                                                 const T (&sg)[N], const T* z0, const T* sg0,
                                                 T (&ten)[N], T (&pi)[N]) {
 #pragma unroll
@@ -280,11 +283,11 @@ __device__ __forceinline__ void interface_pairs(const KParams& P, const T (&zd)[
       const float s = P.S[l][k - 1];
       T d;
       if (l > 0)
-        d = (zd[m - 1] - zd[i]) + P.Hsum[l][m];
+        d = (zd[m - 1] - zd[i]) + G.Hsum[l][m];
       else if (z0)
-        d = (zd[m - 1] - *z0) + P.Hsum[l][m];
+        d = (zd[m - 1] - *z0) + G.Hsum[l][m];
       else
-        d = zd[m - 1] + P.Hsum[l][m];
+        d = zd[m - 1] + G.Hsum[l][m];
       T phi, e;  // phi_k, S phi_k'
       if constexpr (FORM == kExponential) {
         // charged surfaces: a = e^{-kappa (d - k h*)}, phi = 2 a - a^2,
@@ -323,7 +326,8 @@ __device__ __forceinline__ void interface_pairs(const KParams& P, const T (&zd)[
 }
 
 template <int N, bool W32, class T, bool NN = false>
-__device__ __forceinline__ void neg_pressures(const KParams& P, const T (&zd)[N], const T (&gx)[N],
+__device__ __forceinline__ void neg_pressures(const KParams& P, const KParams& G,
+                                              const T (&zd)[N], const T (&gx)[N],
                                               const T (&gy)[N], const T (&lz)[N], T (&q)[N],
                                               const T* z0 = nullptr, const T* sg0 = nullptr) {
   T ten[N], pi[N], sg[N];  // tension of the interface; -Pi of the layer; slope factor
@@ -334,18 +338,18 @@ __device__ __forceinline__ void neg_pressures(const KParams& P, const T (&zd)[N]
     sg[i] = fmav(0.5f, fmav(gx[i], gx[i], gy[i] * gy[i]), Num<T>::splat(1.f));
   }
   if constexpr (NN && W32) {
-    interface_pairs<N, false, kPower32>(P, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, false, kPower32>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if constexpr (W32) {
     if (P.far_pairs)
-      interface_pairs<N, true, kPower32>(P, zd, sg, z0, sg0, ten, pi);
+      interface_pairs<N, true, kPower32>(P, G, zd, sg, z0, sg0, ten, pi);
     else
-      interface_pairs<N, false, kPower32>(P, zd, sg, z0, sg0, ten, pi);
+      interface_pairs<N, false, kPower32>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if (P.wet_kind == 1) {
-    interface_pairs<N, true, kExponential>(P, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, true, kExponential>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if (P.far_pairs) {
-    interface_pairs<N, true, kPower>(P, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, true, kPower>(P, G, zd, sg, z0, sg0, ten, pi);
   } else {
-    interface_pairs<N, false, kPower>(P, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, false, kPower>(P, G, zd, sg, z0, sg0, ten, pi);
   }
   T acc = Num<T>::splat(0.f);
 #pragma unroll

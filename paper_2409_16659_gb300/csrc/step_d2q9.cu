@@ -9,24 +9,77 @@
 
 namespace mlsw {
 
-// Warps per SM that the registers must allow, in moment form without spills:
-// three layers 12 (168 registers; 16 warps at 128 spill into the 15 KB of L1
-// that the rings leave: 76 us a step against 29 at 1024^2; 8 warps: 97
-// against 89 us at 2048^2), two layers 16, one layer 20, four and five 8.
-// The other modes carry their options besides: 8 from three layers on.
-constexpr int march_min_warps(int n, int mode) {
-  return n == 1 ? 20 : (n == 2 ? 14 : (n == 3 && mode == kFast ? 12 : 8));
-}
-
 template <int N, int MODE, bool OP>
-__global__ void __launch_bounds__(32, march_min_warps(N, MODE))
+__global__ void __launch_bounds__(32, march_warps(N, MODE))
     step_d2q9(const __grid_constant__ CUtensorMap map, float* __restrict__ fout,
               const __grid_constant__ KParams P, int strips, int rows, int* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int strip = (int)(blockIdx.x % strips), ya = (int)(blockIdx.x / strips) * rows;
   // (two rows a turn spill from four layers on)
-  march_unit<N, MODE, OP, N <= 3>(P, &map, fout, strip * kMarchOut, ya, min(ya + rows, P.ny),
+  march_unit<N, MODE, OP, N <= 3>(P, P, &map, fout, strip * kMarchOut, ya, min(ya + rows, P.ny),
                                   smem_raw, status);
+}
+
+// A step of a batch whose instances are all of this kind (batch_kernels.cu):
+// registers and instructions of one kind only. SAME: they also share every
+// parameter but H and Hsum (the films of a trajectory set), which are then the
+// kernel's, in the constant bank; two rows a turn pay again. 16 films of 256^2:
+// 38.9 us a step in the kernel of all kinds, 35.1 here.
+template <int N, int MODE, bool SAME>
+__global__ void __launch_bounds__(32, march_warps(N, MODE))
+    step_d2q9_alike(const BatchInst* __restrict__ inst, const int2* __restrict__ table,
+                    const __grid_constant__ KParams P, int cur, int* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int2 e = table[blockIdx.x];
+  const BatchInst& b = inst[e.x];
+  const KParams& G = stage_params(b, smem_raw);
+  float* fout = b.f[cur ^ 1];
+  __builtin_assume(__isGlobal(fout));
+  const int strip = e.y % b.strips, ya = e.y / b.strips * b.rows;
+  const KParams& Q = SAME ? P : G;
+  march_unit<N, MODE, MODE == kGeneral, SAME && N <= 3>(Q, G, &b.map[cur], fout,
+                                                        strip * kMarchOut, ya,
+                                                        min(ya + b.rows, Q.ny),
+                                                        smem_raw + kParBytes, status);
+}
+
+template <int N, int MODE, bool SAME>
+static cudaError_t launch_alike(const BatchLaunch& a, cudaStream_t st) {
+  constexpr size_t smem = kParBytes + MarchShape<N, MODE, MODE == kGeneral>::kSmem;
+  auto kern = step_d2q9_alike<N, MODE, SAME>;
+  static unsigned long long configured = 0;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 64) return cudaErrorInvalidDevice;
+  if (!((configured >> dev) & 1ull)) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured |= 1ull << dev;
+  }
+  if (a.nunits <= 0) return cudaSuccess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)a.nunits);
+  cfg.blockDim = dim3(32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a.inst, a.table, a.P, a.cur, a.status);
+}
+
+template <>
+cudaError_t launch_alike_d2q9<MLSW_N>(const BatchLaunch& a, int mode, cudaStream_t st) {
+  switch (mode) {
+    case kGeneral: return launch_alike<MLSW_N, kGeneral, false>(a, st);
+    case kFast:
+      return a.same_params ? launch_alike<MLSW_N, kFast, true>(a, st)
+                           : launch_alike<MLSW_N, kFast, false>(a, st);
+    default: return launch_alike<MLSW_N, kTau1, false>(a, st);
+  }
 }
 
 // Rows of a unit. A unit costs its rows plus about five rows of warm-up. On

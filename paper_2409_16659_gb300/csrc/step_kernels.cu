@@ -48,9 +48,9 @@ __device__ __forceinline__ void d1q3_pressures(const KParams& P, const float (&z
   if (P.sub_amp != 0.f) {
     const float g0 = 0.5f * (z0e - z0w);
     const float sg0 = fmaf(0.5f, g0 * g0, 1.f);
-    neg_pressures<N, W32>(P, zd, gxz, gyz, lz, p, &z0c, &sg0);
+    neg_pressures<N, W32>(P, P, zd, gxz, gyz, lz, p, &z0c, &sg0);
   } else {
-    neg_pressures<N, W32>(P, zd, gxz, gyz, lz, p);
+    neg_pressures<N, W32>(P, P, zd, gxz, gyz, lz, p);
   }
 }
 
@@ -346,6 +346,17 @@ static cudaError_t launch_d1p_n(const StepLaunch& a, int nsteps, cudaStream_t st
   const bool w32 = (a.P.wet_kind == 0 && a.P.nw == 3 && a.P.mw == 2);
   if (tau1) return w32 ? launch_d1p<N, true, true>(a, nsteps, st) : launch_d1p<N, true, false>(a, nsteps, st);
   return launch_d1p<N, false, false>(a, nsteps, st);
+}
+
+cudaError_t launch_batch_alike(const BatchLaunch& a, int n, int mode, cudaStream_t st) {
+  switch (n) {
+    case 1: return launch_alike_d2q9<1>(a, mode, st);
+    case 2: return launch_alike_d2q9<2>(a, mode, st);
+    case 3: return launch_alike_d2q9<3>(a, mode, st);
+    case 4: return launch_alike_d2q9<4>(a, mode, st);
+    case 5: return launch_alike_d2q9<5>(a, mode, st);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_step_persistent(const StepLaunch& a, int nsteps, cudaStream_t st) {
