@@ -102,32 +102,33 @@ __device__ __forceinline__ void lattice_derivatives(f2 c, f2 A, f2 B, f2& gx, f2
 // the strips at their edges column by column. (A strip per lattice edge is
 // most of a small lattice: 16 films of 256^2 step in 38 us instead of 44.)
 struct PairStore {
-  bool own, own2;        // the pair's first / second column belongs to the lattice
-  bool pairs;            // (warp-uniform) even nx >= 8
-  bool edge;             // (warp-uniform) columns with images, or beyond the lattice
-  bool image;            // pairs: this lane's pair has an image
-  bool im[2][2];         // [column][0: + nx, 1: - nx]
-  int ca, nx, gx;
-  unsigned off, off_im;  // bytes from the row's start: the pair, its image
-  __device__ PairStore(int x0, int lane, int nx_, int gx_) {
+  bool own;       // the pair's first column belongs to the lattice (pairs: both)
+  bool image;     // pairs: this lane's pair has an image
+  bool pairs;     // (warp-uniform) even nx >= 8
+  bool edge;      // (warp-uniform) columns with images, or beyond the lattice
+  int nx;
+  unsigned off;   // bytes from the row's start to the pair
+  // pairs: bytes to its image. Else the stores beside the first column's, one
+  // bit each: the second column, then + nx and - nx of each column. (One
+  // register for both: with flags of their own the pairs' path lost 1 to 4 %,
+  // formed at every store the other one 20 %.)
+  unsigned alt;
+  __device__ PairStore(int x0, int lane, int nx_, int gx) {
     nx = nx_;
-    gx = gx_;
-    ca = x0 - kMarchHalo + 2 * lane;
+    const int ca = x0 - kMarchHalo + 2 * lane;
     const bool in = lane >= kMarchHalo / 2 && lane < 32 - kMarchHalo / 2;
     own = in && ca < nx;
-    own2 = in && ca + 1 < nx;
+    const bool own2 = in && ca + 1 < nx;
     pairs = nx % 2 == 0 && nx >= 8;
     edge = x0 < 4 || x0 + kMarchOut > nx - 4;
     image = own2 && (ca < 4 || ca >= nx - 4);
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const bool o = c ? own2 : own;
-      im[c][0] = o && ca + c < 4;
-      im[c][1] = o && ca + c >= nx - 4;
-    }
     off = (unsigned)(gx + ca) * 4u;
-    off_im = (unsigned)(gx + (ca < 4 ? ca + nx : ca - nx)) * 4u;
+    alt = pairs ? (unsigned)(gx + (ca < 4 ? ca + nx : ca - nx)) * 4u
+                : (own2 ? 1u : 0u) | (own && ca < 4 ? 2u : 0u) | (own2 && ca + 1 < 4 ? 4u : 0u) |
+                      (own && ca >= nx - 4 ? 8u : 0u) | (own2 && ca + 1 >= nx - 4 ? 16u : 0u);
   }
+  // the pair's second column belongs to the lattice
+  __device__ __forceinline__ bool own2() const { return pairs ? own : (alt & 1u) != 0u; }
   __device__ __forceinline__ void pair(float* buf, long len, float* row, unsigned at, f2 v) const {
     *reinterpret_cast<float2*>(chk_global(
         buf, reinterpret_cast<float*>(reinterpret_cast<char*>(row) + at), len, 2)) = v.v;
@@ -137,16 +138,16 @@ struct PairStore {
   }
   __device__ __forceinline__ void with_image(float* buf, long len, float* row, f2 v) const {
     if (own) pair(buf, len, row, off, v);
-    if (image) pair(buf, len, row, off_im, v);
+    if (image) pair(buf, len, row, alt, v);
   }
   __device__ __forceinline__ void slow(float* buf, long len, float* row, f2 v) const {
-    float* p = row + gx + ca;
+    float* p = reinterpret_cast<float*>(reinterpret_cast<char*>(row) + off);
     if (own) *chk_global(buf, p, len) = v.v.x;
-    if (own2) *chk_global(buf, p + 1, len) = v.v.y;
-    if (im[0][0]) *chk_global(buf, p + nx, len) = v.v.x;
-    if (im[1][0]) *chk_global(buf, p + 1 + nx, len) = v.v.y;
-    if (im[0][1]) *chk_global(buf, p - nx, len) = v.v.x;
-    if (im[1][1]) *chk_global(buf, p + 1 - nx, len) = v.v.y;
+    if (alt & 1u) *chk_global(buf, p + 1, len) = v.v.y;
+    if (alt & 2u) *chk_global(buf, p + nx, len) = v.v.x;
+    if (alt & 4u) *chk_global(buf, p + 1 + nx, len) = v.v.y;
+    if (alt & 8u) *chk_global(buf, p - nx, len) = v.v.x;
+    if (alt & 16u) *chk_global(buf, p + 1 - nx, len) = v.v.y;
   }
   // one store per plane, by the strip's kind
   // (row(k): its row's start, v(k): its values)
@@ -547,7 +548,7 @@ __device__ __forceinline__ void march_unit(const KParams& P, const KParams& G,
     }
   }
   const bool bad = (put.own && (!(hlow.v.x > 0.f) || isnan(fall.v.x))) ||
-                   (put.own2 && (!(hlow.v.y > 0.f) || isnan(fall.v.y)));
+                   (put.own2() && (!(hlow.v.y > 0.f) || isnan(fall.v.y)));
   if (bad) atomicOr(status, kStatusNonfinite);
 }
 
