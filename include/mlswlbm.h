@@ -370,13 +370,14 @@ int mlswlbm_diagnostics_noalloc(const mlsw_params* p, const float* f, const floa
  * table of every instance's units of work (strips of some rows), in which the
  * instances sharing the layer count, the kernel mode (tau = 1 or not,
  * exponents (3, 2), spreading only between neighbouring interfaces) and the
- * tile height (a group) form a contiguous range. Each instance is stepped
+ * nominal tile height (a group) form a contiguous range. Each instance is stepped
  * with exactly the arithmetic of mlswlbm_step (section LBM, Eq. BGK).
  * ------------------------------------------------------------------------
  */
 typedef struct mlsw_batch mlsw_batch;
 
-/* batch flags */
+/* batch flags. Tile heights are nominal: the rows of an instance's units of
+ * work are 16 or 8, scaled by one factor for the instances stepped together. */
 #define MLSW_BATCH_TILE8 1    /* 8-row tiles for every instance (default: 16 rows for n <= 3) */
 #define MLSW_BATCH_AUTOTUNE 2 /* at create, time 8- and 16-row tiles for every class of
                                  instances with the same n, kernel mode and size (n <= 3)
@@ -385,7 +386,7 @@ typedef struct mlsw_batch mlsw_batch;
 /* Creates a batch of count >= 1 lattices: params[j] and h_init[j] (host,
  * [n_j][ny_j][nx_j]) as for mlswlbm_create, every lattice D2Q9 (else
  * MLSW_ERR_UNSUPPORTED). Errors of an instance are those of mlswlbm_create.
- * One device allocation holds all population buffers. On failure *out is
+ * One device allocation holds all state buffers. On failure *out is
  * NULL and nothing is leaked. */
 int mlswlbm_batch_create(int count, const mlsw_params* params, const float* const* h_init,
                          int flags, void* stream, mlsw_batch** out);
@@ -428,7 +429,7 @@ int mlswlbm_batch_modes(mlsw_batch* b, const int* kx, const int* ky, double* out
  * create or the last query (then cleared); synchronises. */
 int mlswlbm_batch_status(mlsw_batch* b);
 
-/* Tile rows (8 or 16) that instance index runs with, or MLSW_ERR_ARG. */
+/* Nominal tile rows (8 or 16) of instance index, or MLSW_ERR_ARG. */
 int mlswlbm_batch_tile_rows(const mlsw_batch* b, int index);
 
 /* Chooses the instances that mlswlbm_batch_step advances: the nsel distinct

@@ -1,7 +1,7 @@
 // batch.cu -- batches of independent D2Q9 lattices (the C ABI's
-// mlswlbm_batch_*): one population arena, per-instance device descriptors,
+// mlswlbm_batch_*): one arena of states, per-instance device descriptors,
 // one unit table in which the instances that share layer count, kernel mode
-// and tile height (a group) have a contiguous range, one launch per step
+// and nominal tile height (a group) have a contiguous range, one launch per step
 // over the whole table (batch_kernels.cu), and a timing autotuner for the
 // tile height of every class of alike instances.
 #include <algorithm>

@@ -60,9 +60,9 @@ size_t step_persistent_smem(int n, int lattice, int nx);
 cudaError_t launch_step_persistent(const StepLaunch& a, int nsteps, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
-// Batches: many independent D2Q9 lattices stepped by one persistent launch
-// over one tile table, in which the tiles of instances that share n, kernel
-// mode and tile height form a contiguous range (batch_kernels.cu).
+// Batches: many independent D2Q9 lattices stepped by one launch over one
+// table of units, in which the units of instances that share n, kernel mode
+// and nominal tile height form a contiguous range (batch_kernels.cu).
 // ---------------------------------------------------------------------------
 // Tile heights a batch can use: variant 0 = 16 rows (n <= 3 only), variant
 // 1 = 8 rows. A warp's unit of work is a strip of `rows` rows: the height,

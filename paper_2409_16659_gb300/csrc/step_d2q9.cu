@@ -89,7 +89,8 @@ cudaError_t launch_alike_d2q9<MLSW_N>(const BatchLaunch& a, int mode, cudaStream
 // 3, 4 rows 8.3, 7.8, 7.5, 8.5). Larger lattices run as one wave of the warps
 // that fit (slots), which also spreads them evenly over the SMs: 512^2 with
 // 2, 3, 4 rows 15.9, 12.4, 14.2; 1024^2 with 8, 11, 13 rows 33.3, 28.7, 32.5;
-// 2048^2 with 32, 43, 51 rows 101, 89, 104. Units taller than 64 rows would
+// 2048^2 with 32, 43, 51 rows 101, 89, 104 (before image pairs had one store,
+// which took 8 % off each: 26.6 and 80.9 now). Units taller than 64 rows would
 // put neighbouring units further apart in time than the L2 keeps the rows
 // they share; then several waves.
 static int march_rows(int ny, int strips, int num_sms, int slots) {
