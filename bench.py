@@ -3,7 +3,7 @@
 Workload: the three-layer pseudo-3D spinodal film (D2Q9, 1024 x 1024
 periodic cells, means 1.0 / 0.8 / 0.6 plus seeded Gaussian noise 1e-3,
 gamma 0.01 / 0.008 / 0.006, mu = (1, 2, 4) / 6, slip 1, wetting exponents
-(3, 2), h* = 0.07, contact angle 20 degrees), FP32 populations.
+(3, 2), h* = 0.07, contact angle 20 degrees), FP32.
 
 A benchmark step is one LBM time step (one fused kernel launch) over the
 whole lattice. Metric: layer-site updates per second,
@@ -13,12 +13,12 @@ LSU/s = n_layers * nx * ny * steps / time.
 
 Own arm: inputs resident in HBM; K back-to-back steps on the solver's
 stream, bracketed by CUDA events (one before the first step, then one after
-every 50 steps, which also gives the spread). The two population buffers (2 x 113 MB) exceed
-the 129 MB L2, so no flush is needed; a step's dirty lines that the L2
-still holds when it ends are written back inside the next step, as in a
-long run. For context the line also reports single steps with the L2
-flushed before each (a 256 MiB write and read): those exclude that
-write-back and read lower.
+every 50 steps, which also gives the spread). A lattice's state is two
+50 MB buffers, which the 129 MB L2 would hold from step to step, so the K
+steps take four such lattices in turn (408 MB): every step finds its input
+in HBM, as on a lattice larger than the L2. For context the line also
+reports the steps of one lattice in a row (what a run of this size does),
+and single steps with the L2 flushed before each (a 256 MiB write and read).
 The e2e figure goes through the public API with host buffers: every step
 uploads the heights from pinned memory (mlswlbm_set_heights), advances one
 step and reads the heights back (mlswlbm_get_heights).
@@ -30,7 +30,7 @@ Two more workloads are reported beside the main line, under "workloads"
     chip) and heights read back, wall clock;
   * three-layer lens field, D2Q9, 2048 x 2048, lenses of radius 200 (the
     droplet/lens equilibrium workload): LSU/s over event-timed
-    back-to-back steps (its 2 x 906 MB working set exceeds the L2), then
+    back-to-back steps (its 2 x 202 MB working set exceeds the L2), then
     the run until the kinetic energy falls below 1e-12 (at most 500 000
     steps) with the lenses' Neumann angles;
   * batched stability sweep: 512 instances (2..5 layers, sides 64..512,
@@ -68,14 +68,16 @@ import workloads  # noqa: E402
 
 NX = NY = 1024
 N_LAYERS = 3
-Q = 9
-BYTES_PER_LSU = 2 * Q * 4          # read + write of every FP32 population
+BYTES_PER_LSU = 2 * 3 * 4          # read + write of the state at tau = 1: h and J, FP32
 METRIC = "layer-site updates/s"
 UNIT = "LSU/s"
-WORKLOAD = "3-layer D2Q9 spinodal film, 1024x1024 periodic, FP32 populations"
+WORKLOAD = "3-layer D2Q9 spinodal film, 1024x1024 periodic, FP32"
 FALLBACK_HBM_GBS = 6800.0
 CHUNK = 50                         # timed steps between two events
+LATTICES = 4                       # stepped in turn: 408 MB of state, 129 MB of L2
 KERNEL_SOURCES = ["paper_2409_16659_gb300/csrc/step_kernels.cu",
+                  "paper_2409_16659_gb300/csrc/step_d2q9.cu",
+                  "paper_2409_16659_gb300/csrc/step_common.cuh",
                   "paper_2409_16659_gb300/csrc/march.cuh",
                   "paper_2409_16659_gb300/csrc/physics.cuh",
                   "paper_2409_16659_gb300/csrc/tma.cuh"]
@@ -92,8 +94,8 @@ def kernel_hash():
 def config_dict(extra=None):
     c = {"workload": WORKLOAD, "n_layers": N_LAYERS, "lattice": "D2Q9", "nx": NX, "ny": NY,
          "cells": NX * NY, "layer_sites_per_step": N_LAYERS * NX * NY,
-         "l2": "inputs larger than L2: back-to-back steps over two 113 MB population "
-               "buffers (226 MB > 129 MB L2), no flush",
+         "l2": "inputs larger than L2: the steps take four lattices in turn, 4 x 2 state "
+               "buffers of 51 MB (408 MB > 129 MB L2), no flush",
          "parallelism": "replicas (one independent lattice per GPU)"}
     if extra:
         c.update(extra)
@@ -298,7 +300,8 @@ def run_own(args):
     p = workloads.film3_d2q9_params(NX, NY)
     h0 = workloads.film3_d2q9_heights(NX, NY, seed=2 + rank).astype(np.float32)
     stream = torch.cuda.current_stream()
-    solver = B.Solver(p, h0, stream=stream)
+    solvers = [B.Solver(p, h0, stream=stream) for _ in range(LATTICES)]
+    solver = solvers[0]
     lsu_step = N_LAYERS * NX * NY
 
     def barrier():
@@ -309,10 +312,11 @@ def run_own(args):
 
     # ---- warm-up ----------------------------------------------------------
     for _ in range(args.warmup):
-        solver.step(1)
+        for s in solvers:
+            s.step(1)
     torch.cuda.synchronize()
 
-    # ---- timed region: K back-to-back steps ---------------------------------
+    # ---- timed region: K back-to-back steps, the lattices in turn -----------
     # Events only every CHUNK steps: an event recorded between two launches
     # keeps the second from starting while the first drains (programmatic
     # dependent launch), so per-step events would time a slower loop than a
@@ -323,18 +327,27 @@ def run_own(args):
     sampler = ClockSampler(dev) if rank == 0 else None
     if sampler:
         sampler.start()
-    launches0 = solver.launch_count()
+    launches0 = sum(s.launch_count() for s in solvers)
     barrier()
     evs[0].record(stream)
     for j in range(1, len(bounds)):
-        solver.step(bounds[j] - bounds[j - 1])
+        for i in range(bounds[j - 1], bounds[j]):
+            solvers[i % LATTICES].step(1)
         evs[j].record(stream)
     barrier()
-    launches = solver.launch_count() - launches0
+    launches = sum(s.launch_count() for s in solvers) - launches0
     clocks = sampler.stop() if sampler else None
     total_s = evs[0].elapsed_time(evs[-1]) / 1e3
     step_ms = np.array([evs[j - 1].elapsed_time(evs[j]) / (bounds[j] - bounds[j - 1])
                         for j in range(1, len(bounds))])
+
+    # ---- context: one lattice's steps in a row, its state in the L2 ----------
+    barrier()
+    evs[0].record(stream)
+    solver.step(args.steps)
+    evs[-1].record(stream)
+    barrier()
+    resident_ms = evs[0].elapsed_time(evs[-1]) / args.steps
 
     # ---- context: single steps from a flushed L2 ----------------------------
     flush_w = torch.empty(64 * 1024 * 1024, dtype=torch.float32, device="cuda")   # 256 MiB
@@ -371,8 +384,9 @@ def run_own(args):
     t1 = time.perf_counter()
     e2e_s = t1 - t0
     assert np.isfinite(h_out_np).all()
-    status = solver.status()
-    solver.close()
+    status = next((s.status() for s in solvers if s.status() != B.MLSW_OK), B.MLSW_OK)
+    for s in solvers:
+        s.close()
 
     total_s, e2e_s = max_over_ranks([total_s, e2e_s], "cuda")
 
@@ -391,7 +405,7 @@ def run_own(args):
             "config": config_dict(),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": "step_d2q9_tma<3,kFast>",
+                         "kernel": "step_d2q9<3,kFast>",
                          "bytes_per_launch_algorithmic": bytes_alg, "peak_source": peak_src},
             "e2e": {"value": job_rate(ws, lsu_step * k_e2e, e2e_s), "unit": UNIT,
                     "h2d_bytes_per_step": int(h_host.numel() * 4),
@@ -404,6 +418,9 @@ def run_own(args):
                         "p90": float(np.percentile(step_ms, 90)), "max": float(step_ms.max()),
                         "chunks": int(len(step_ms)),
                         "note": "mean time per step of each chunk of %d timed steps" % chunk},
+            "one_lattice": {"ms_per_step": resident_ms, "steps": args.steps,
+                            "note": "context only: consecutive steps of one lattice, whose "
+                                    "102 MB of state the L2 can hold"},
             "flushed_l2": {"ms_per_step_mean": float(flushed_ms.mean()),
                            "ms_per_step_p50": float(np.median(flushed_ms)), "steps": k_fl,
                            "note": "context only: one step after a 256 MiB L2 flush; the "
@@ -473,7 +490,7 @@ def lens_workload(B, torch, max_steps=500000, check_every=5000, ke_stop=1e-12):
         dt = e0.elapsed_time(e1) * 1e-3 / steps
         res.update({"value": lsu / dt, "unit": UNIT, "ms_per_step": 1e3 * dt, "steps": steps,
                     "roofline_frac": BYTES_PER_LSU * lsu / dt / 1e9 / peak,
-                    "l2": "back-to-back steps; 2 x 906 MB working set > 129 MB L2"})
+                    "l2": "back-to-back steps; 2 x 202 MB working set > 129 MB L2"})
         t0 = time.perf_counter()
         done, ke = s.step_until(max_steps, check_every, ke_stop)
         t1 = time.perf_counter()
@@ -702,7 +719,7 @@ def sweep_workload(B, torch):
 
 
 def run_profile_batch(args):
-    """Warm-up then --steps steps of the first 64 sweep instances (~1.4 GB)."""
+    """Warm-up then --steps steps of the first 64 sweep instances (~0.6 GB)."""
     import torch
     torch.cuda.set_device(0)
     from paper_2409_16659_gb300 import mlswlbm as B

@@ -183,6 +183,7 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 mlsw::Layout make_layout(const mlsw_params& p) {
   mlsw::Layout L;
+  std::memset(&L, 0, sizeof(L));  // its padding too: batches compare parameters as bytes
   const bool d2 = p.lattice == MLSW_D2Q9;
   L.nx = p.nx;
   L.ny = p.ny;
