@@ -93,8 +93,31 @@ cudaError_t launch_alike_d2q9<MLSW_N>(const BatchLaunch& a, int mode, cudaStream
 // which took 8 % off each: 26.6 and 80.9 now). Units taller than 64 rows would
 // put neighbouring units further apart in time than the L2 keeps the rows
 // they share; then several waves.
+//
+// One and two layers gain less from warps that share a scheduler (k of them
+// take per_row[k - 1] times one's time for a row): there a wave of the warps
+// that fit is for more than four rows a unit, and below that the height is the
+// cheapest by that model. One layer, 448^2: 8.1 us a step with 1 row (the
+// wave), 5.0 with 3; 25 x 1870 5.1 and 4.4 with 2; two layers, 320^2: 7.3 with
+// 1, 5.8 with 2; 25 x 1870 8.2 and 6.0 with 2.
 static int march_rows(int ny, int strips, int num_sms, int slots) {
   const long total = (long)ny * strips, flat = (total + 4L * num_sms - 1) / (4L * num_sms);
+  if (MLSW_N <= 2 && total <= 4L * slots) {
+    constexpr double per_row[2][5] = {{1.0, 1.12, 1.33, 1.51, 1.95}, {1.0, 1.25, 1.66, 1.95, 2.4}};
+    double best = 0.0;
+    int best_rows = 0;
+    for (int rows = 1; rows <= 8; ++rows) {
+      const long units = (long)strips * ((ny + rows - 1) / rows);
+      const long k = (units + 4L * num_sms - 1) / (4L * num_sms);
+      if (units > slots || k > 5) continue;
+      const double cost = (rows + 5) * per_row[MLSW_N > 1][k - 1];
+      if (best_rows == 0 || cost < best) {
+        best = cost;
+        best_rows = rows;
+      }
+    }
+    if (best_rows > 0) return best_rows;
+  }
   if (flat <= 3) return (int)flat;
   for (long wave = 1;; ++wave) {
     const long chunks = slots * wave / strips;
