@@ -290,6 +290,15 @@ int mlswlbm_status(mlsw_handle* h);
  * memory; synchronises the stream (cudaStream_t or NULL). */
 int mlswlbm_selftest_bounded_wait(int arrive, unsigned limit, void* stream);
 
+/* The same for the wait of a whole warp: one warp waits, as the step's warps
+ * do, on a barrier that has received its arrival; bit i of short_lanes gives
+ * lane i no try at all, so that its wait runs out. A warp goes on together
+ * or not at all: *went_on receives the lanes that would go on, all 32 (and
+ * the call returns MLSW_OK) or none (MLSW_ERR_TIMEOUT, recorded by the kernel
+ * as a step does). 1 <= limit <= 2^22 bounds the other lanes. */
+int mlswlbm_selftest_warp_wait(unsigned short_lanes, unsigned limit, void* stream,
+                               unsigned* went_on);
+
 /* Binds another stream to the handle (cudaStream_t or NULL). The caller
  * orders work already queued on the old stream. */
 int mlswlbm_set_stream(mlsw_handle* h, void* stream);

@@ -726,6 +726,34 @@ cudaError_t launch_wait_selftest(int arrive, unsigned limit, int* status, cudaSt
   return cudaGetLastError();
 }
 
+// One warp waits as the step kernels' warps do, on a barrier that has its
+// arrival; the lanes in short_lanes may try no time at all, so their waits
+// run out. *went_on: the lanes that would go on.
+__global__ void warp_wait_selftest_kernel(unsigned short_lanes, unsigned limit,
+                                          unsigned* __restrict__ went_on,
+                                          int* __restrict__ status) {
+  __shared__ __align__(8) uint64_t bar;
+  const int lane = threadIdx.x;
+  if (lane == 0) {
+    mbar_init(&bar, 1);
+    mbar_init_fence();
+    mbar_arrive_expect_tx(&bar, 0u);
+  }
+  __syncwarp();
+  const bool ok = mbar_wait_bounded_warp(&bar, 0u, (short_lanes >> lane) & 1u ? 0u : limit);
+  const unsigned on = __ballot_sync(0xffffffffu, ok);
+  if (lane == 0) {
+    *went_on = on;
+    if (!ok) atomicOr(status, kStatusTimeout);
+  }
+}
+
+cudaError_t launch_warp_wait_selftest(unsigned short_lanes, unsigned limit, unsigned* went_on,
+                                      int* status, cudaStream_t st) {
+  warp_wait_selftest_kernel<<<1, 32, 0, st>>>(short_lanes, limit, went_on, status);
+  return cudaGetLastError();
+}
+
 MLSW_DEFINE_BOUNDS_READER(bounds_violations_aux)
 
 }  // namespace mlsw

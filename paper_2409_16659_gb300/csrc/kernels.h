@@ -222,6 +222,10 @@ cudaError_t launch_friction_eval(const KParams& P, long ncell, const float* h, c
 // iterations); the barrier gets its arrival only when arrive != 0. A wait
 // that runs out ORs kStatusTimeout into *status.
 cudaError_t launch_wait_selftest(int arrive, unsigned limit, int* status, cudaStream_t st);
+// One warp's wait, whose lanes in short_lanes run out at once: *went_on the
+// lanes that go on (all or none), kStatusTimeout when none does.
+cudaError_t launch_warp_wait_selftest(unsigned short_lanes, unsigned limit, unsigned* went_on,
+                                      int* status, cudaStream_t st);
 
 // Dense layout of a caller-owned population array (no ghosts).
 inline Layout dense_layout(int nx, int ny, int nplanes = 0) {

@@ -321,7 +321,7 @@ __device__ __forceinline__ void march_unit(const KParams& P, const KParams& G,
 
   // Row t arrives: its z; returns false when the bounded wait ran out.
   auto arrive = [&](int t, f2 (&zn)[N], f2& sn) {
-    if (!mbar_wait_bounded(bar + slot, parity)) return false;
+    if (!mbar_wait_bounded_warp(bar + slot, parity)) return false;
     const float* src = ring + slot * S::ROW + 2 * lane;
     f2 z = zero;
     if (sub) {

@@ -941,6 +941,28 @@ int mlswlbm_selftest_bounded_wait(int arrive, unsigned limit, void* stream) {
   return (flag & mlsw::kStatusTimeout) ? MLSW_ERR_TIMEOUT : MLSW_OK;
 }
 
+int mlswlbm_selftest_warp_wait(unsigned short_lanes, unsigned limit, void* stream,
+                               unsigned* went_on) {
+  if (limit == 0 || limit > (1u << 22) || !went_on) return MLSW_ERR_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  unsigned* d = nullptr;
+  if (cudaMalloc(&d, 2 * sizeof(unsigned)) != cudaSuccess) {
+    cudaGetLastError();
+    return MLSW_ERR_NOMEM;
+  }
+  unsigned out[2] = {0, 0};
+  const bool ok =
+      cudaMemsetAsync(d, 0, sizeof(out), st) == cudaSuccess &&
+      mlsw::launch_warp_wait_selftest(short_lanes, limit, d, reinterpret_cast<int*>(d + 1), st) ==
+          cudaSuccess &&
+      cudaMemcpyAsync(out, d, sizeof(out), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+      cudaStreamSynchronize(st) == cudaSuccess;
+  cudaFree(d);
+  if (!ok) return MLSW_ERR_CUDA;
+  *went_on = out[0];
+  return ((int)out[1] & mlsw::kStatusTimeout) ? MLSW_ERR_TIMEOUT : MLSW_OK;
+}
+
 int mlswlbm_debug_bounds_violations(unsigned long long* count) {
   if (!count) return MLSW_ERR_ARG;
 #ifdef MLSW_DEBUG

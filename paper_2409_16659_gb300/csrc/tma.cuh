@@ -57,6 +57,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return false;
 }
 
+// The same wait by a whole warp, with one outcome for all its lanes: the code
+// after a wait shuffles and loads as a warp, and lanes that gave up alone
+// would leave the others in it.
+__device__ __forceinline__ bool mbar_wait_bounded_warp(uint64_t* bar, uint32_t parity,
+                                                       uint32_t limit = (1u << 22)) {
+  return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, limit));
+}
+
 // 3-D tiled bulk copy global -> shared; x must be a multiple of 4 floats
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar,
                                             int x, int y, int z) {

@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(192, 1)
     int local = 0;
     for (int tile = tile0; tile < a.B_tiles; tile += dtile, ++local) {
       const int ab = local & 1, use = local >> 1;
-      const bool dok = mbar_wait_bounded(&tfull[ab], use & 1);
+      const bool dok = mbar_wait_bounded_warp(&tfull[ab], use & 1);
       tc_fence_after();
       if (!dok) {
         ok = false;
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(128) wgrad_tc(const __grid_constant__ WgradArg
     tc_commit(done);
   }
   __syncwarp();
-  const bool dok = nk > 0 ? mbar_wait_bounded(done, 0) : true;
+  const bool dok = nk > 0 ? mbar_wait_bounded_warp(done, 0) : true;
   tc_fence_after();
   if (dok && nk > 0) {
     const int o = m0 + warp * 32 + lane;
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(128) wgrad_tc(const __grid_constant__ WgradArg
         for (int i = 0; i < 16; i += 4) red_add_v4(dst + i, rr + i);
       }
     }
-  } else if (!dok && threadIdx.x == 0) {
+  } else if (!dok && lane == 0) {
     atomicOr(a.err, 1);
   }
   if (!ok) atomicOr(a.err, 2);

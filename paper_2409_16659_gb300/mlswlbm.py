@@ -96,6 +96,8 @@ EXPORTS = {
                                                   ctypes.POINTER(ctypes.c_longlong)]),
     "mlswlbm_fit_cap_angle": (ctypes.c_int, [_D, _D, ctypes.c_int, ctypes.c_double, _D, _D]),
     "mlswlbm_selftest_bounded_wait": (ctypes.c_int, [ctypes.c_int, ctypes.c_uint, ctypes.c_void_p]),
+    "mlswlbm_selftest_warp_wait": (ctypes.c_int, [ctypes.c_uint, ctypes.c_uint, ctypes.c_void_p,
+                                                  ctypes.POINTER(ctypes.c_uint)]),
     "mlswlbm_step_until": (ctypes.c_int, [_H, ctypes.c_long, ctypes.c_long, ctypes.c_double,
                                           ctypes.POINTER(ctypes.c_long), _D]),
     "mlswlbm_set_stream": (ctypes.c_int, [_H, ctypes.c_void_p]),
@@ -611,6 +613,15 @@ def mlswlbm_debug_bounds_violations():
 def selftest_bounded_wait(arrive, limit=256, stream=None):
     """mlswlbm_selftest_bounded_wait: MLSW_OK or MLSW_ERR_TIMEOUT."""
     return lib().mlswlbm_selftest_bounded_wait(int(bool(arrive)), int(limit), _stream_ptr(stream))
+
+
+def selftest_warp_wait(short_lanes, limit=256, stream=None):
+    """mlswlbm_selftest_warp_wait: (MLSW_OK or MLSW_ERR_TIMEOUT, mask of the
+    lanes that would go on)."""
+    on = ctypes.c_uint(0)
+    rc = lib().mlswlbm_selftest_warp_wait(int(short_lanes), int(limit), _stream_ptr(stream),
+                                          ctypes.byref(on))
+    return rc, int(on.value)
 
 
 def fit_cap_angle(profile, area, base):
