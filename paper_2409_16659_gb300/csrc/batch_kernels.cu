@@ -8,6 +8,7 @@
 // run the same kind, so the warps of an SM share its instructions.
 #include <algorithm>
 
+#include "device_once.h"
 #include "march.cuh"
 
 #ifndef MLSW_BATCH_N
@@ -70,17 +71,16 @@ cudaError_t launch_batch_step_n<MLSW_BATCH_N>(const BatchLaunch& a, cudaStream_t
   if (a.nunits <= 0) return cudaSuccess;
   auto kern = step_d2q9_batch<MLSW_BATCH_N>;
   // once per device: the largest shared memory any kind can need
-  static unsigned long long configured = 0;
+  static DeviceOnce configured;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 64) return cudaErrorInvalidDevice;
-  if (!((configured >> dev) & 1ull)) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kParBytes + smem_from<0>(~0u)));
-    if (e != cudaSuccess) return e;
-    configured |= 1ull << dev;
-  }
+  e = configured(dev, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kParBytes + smem_from<0>(~0u)));
+  });
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.nunits);
   cfg.blockDim = dim3(32);

@@ -47,6 +47,7 @@
 #include <vector>
 
 #include "../../include/mlswlbm.h"
+#include "device_once.h"
 #include "tcgen05.cuh"
 
 namespace mlsw {
@@ -972,17 +973,15 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              CUtensorMapFloatOOBfill);
 
 EncodeFn encoder() {
-  static EncodeFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  static const EncodeFn fn = []() -> EncodeFn {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeFn>(p);
-  }
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    return reinterpret_cast<EncodeFn>(p);
+  }();
   return fn;
 }
 
@@ -1055,17 +1054,16 @@ cudaError_t launch_dep(void (*kern)(P...), dim3 grid, int block, size_t smem, cu
 template <int KC, int BN, bool RES>
 cudaError_t launch_conv_t(const ConvArgs& a, int ntn, int wblks, int num_sms, cudaStream_t st) {
   using S = ConvShape<KC, BN, RES>;
-  static bool attr[64] = {};
+  static mlsw::DeviceOnce configured;
   auto kern = conv_tc<KC, BN, RES>;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 64) return cudaErrorInvalidDevice;
-  if (!attr[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr[dev] = true;
-  }
+  e = configured(dev, [&] {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  });
+  if (e != cudaSuccess) return e;
   const size_t smem = S::smem(RES ? wblks : 0);
   // CTAs per SM by shared memory (228 KB, 1 KB reserved per CTA), by tensor
   // memory and by registers (three of 192 threads): one wave
@@ -1102,15 +1100,16 @@ cudaError_t launch_conv(int kc, int bn, const ConvArgs& a, int ntn, int num_sms,
 template <int BN>
 cudaError_t launch_wgrad_t(const WgradArgs& a, dim3 grid, cudaStream_t st) {
   using S = WgShape<BN>;
-  static bool attr[64] = {};
+  static mlsw::DeviceOnce configured;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev < 64 && !attr[dev]) {
-    e = cudaFuncSetAttribute(wgrad_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    if (e != cudaSuccess) return e;
-    attr[dev] = true;
-  }
+  if (dev >= 64) return cudaErrorInvalidDevice;
+  e = configured(dev, [&] {
+    return cudaFuncSetAttribute(wgrad_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)S::SMEM);
+  });
+  if (e != cudaSuccess) return e;
   return launch_dep(wgrad_tc<BN>, grid, 128, S::SMEM, st, a);
 }
 

@@ -1,0 +1,74 @@
+"""Host rules of the launches, compiled from their headers with the host
+compiler: heights of the units of work, and the once-per-device setup that
+they depend on."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2409_16659_gb300", "csrc")
+
+
+def run_cpp(tmp_path, source, *args, timeout=20):
+    """Compiles and runs a C++ program that includes the library's headers;
+    its output lines."""
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text(source)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", CSRC, str(src), "-o", str(exe)],
+                   check=True, timeout=120)
+    r = subprocess.run([str(exe), *map(str, args)], check=True, timeout=timeout,
+                       capture_output=True, text=True)
+    return r.stdout.split()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+def test_unit_heights_end_for_any_number_of_slots(tmp_path, n):
+    """Also for none, which an unset occupancy gives: every height lies in
+    1..64."""
+    out = run_cpp(tmp_path, """
+#include <cstdio>
+#include <cstdlib>
+#include <initializer_list>
+#include "unit_rows.h"
+int main(int, char** a) {
+  for (int slots : {0, 1, 152, 1824})
+    for (int ny : {1, 2, 7, 64, 1024, 5000})
+      for (int strips : {1, 2, 19, 1000})
+        printf("%d ", mlsw::march_rows(atoi(a[1]), ny, strips, 152, slots));
+}""", n)
+    assert len(out) == 4 * 6 * 4 and all(1 <= int(v) <= 64 for v in out)
+
+
+def test_device_setup_is_seen_whole_by_every_thread(tmp_path):
+    """Sixteen threads start together: each finds the value that the setup of
+    its device stored, the setup runs once per device, and one that failed is
+    tried again."""
+    out = run_cpp(tmp_path, """
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "device_once.h"
+int main() {
+  int wrong = 0, runs = 0;
+  for (int trial = 0; trial < 300; ++trial) {
+    mlsw::DeviceOnce once;
+    int value[64] = {};
+    std::atomic<int> count{0}, bad{0}, go{0};
+    std::vector<std::thread> t;
+    for (int k = 0; k < 16; ++k)
+      t.emplace_back([&, k] {
+        const int dev = k % 2 ? 63 : 0;
+        ++go;
+        while (go < 16) {}
+        if (once(dev, [&] { value[dev] = 7; ++count; return 0; }) != 0 || value[dev] != 7) ++bad;
+      });
+    for (auto& x : t) x.join();
+    wrong += bad;
+    runs += count;
+  }
+  mlsw::DeviceOnce once;
+  int a = once(3, [] { return 5; }), b = once(3, [] { return 0; }), c = once(3, [] { return 9; });
+  printf("%d %d %d %d %d", wrong, runs, a, b, c);
+}""")
+    assert out == ["0", "600", "5", "0", "0"]
