@@ -384,18 +384,29 @@ __device__ __forceinline__ void neg_pressures(const KParams& P, const KParams& G
 // elimination needs no pivoting for any n, thicknesses and slips. Solving
 // the full n x n flux-gradient matrix took 2.5 times the arithmetic at n = 3
 // (adjugate), and a pivoted elimination on single cells at n = 4, 5.
+//
+// Back substitution gives T_i = (r_i + (s_i - a_i) T_{i+1}) / d_i from the
+// eliminated right-hand side r_i and pivot d_i. R_i = T_i - T_{i+1} is formed as
+// (r_i - e_i T_{i+1}) / d_i, with e_i = d_i - (s_i - a_i) = 2 a_{i-1} + 3 a_i + b_i
+// less the eliminated term: with slip, a thin layer's s_i = c_i / h_i exceeds
+// the rest of its row, T_i and T_{i+1} then agree to h_i / c_i, and their
+// difference lost as many digits (relative to the forces that the layers'
+// fluxes make one by one: 1e-3 at h = 1e-4 and 1e-1 at 1e-6, 5e-5 at h = 0.05
+// with a slip of 30; now 5e-7 throughout). T_i keeps a formula of its own
+// because it can be the small one. One more addition and two more
+// multiply-adds a layer.
 // ih: 1 / h. TWO: both components (else the y ones are left alone).
 // ---------------------------------------------------------------------------
 template <int N, bool TWO, class T>
 __device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], const T (&ih)[N],
                                          const T (&Ux)[N], const T (&Uy)[N], T (&Rx)[N],
                                          T (&Ry)[N]) {
-  T piv[N], nsup[N], bx[N], by[N];
-  T na_prev;  // -a_{i-1}
+  T piv[N], nsup[N], ne[N], bx[N], by[N];  // ne: -e_i
+  T na_prev;                               // -a_{i-1}
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     const T na = mulr(h[i], P.fr_visc[i]), s = mulr(ih[i], P.fr_slip2[i]);
-    T diag = fmav(na, -2.f, s + P.fr_slip[i]);
+    T rest = fmav(na, -2.f, Num<T>::splat(P.fr_slip[i]));  // d_i - s_i
     nsup[i] = na + s;
     if (i == 0) {
       bx[0] = Ux[0] * -1.f;
@@ -403,11 +414,12 @@ __device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], cons
     } else {
       const int j = i > 0 ? i - 1 : 0;
       const T nf = na_prev * piv[j];
-      diag = fmav(nf, nsup[j] * -1.f, fmav(na_prev, -2.f, diag));
+      rest = fmav(nf, nsup[j] * -1.f, fmav(na_prev, -2.f, rest));
       bx[i] = fmav(nf, bx[j], Ux[j] - Ux[i]);
       if constexpr (TWO) by[i] = fmav(nf, by[j], Uy[j] - Uy[i]);
     }
-    piv[i] = rcp(diag);
+    piv[i] = rcp(rest + s);
+    ne[i] = na - rest;
     na_prev = na;
   }
   T tx, ty;  // T_{i+1}
@@ -415,10 +427,10 @@ __device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], cons
   for (int i = N - 1; i >= 0; --i) {
     const T ox = tx, oy = ty;
     tx = mulr(i == N - 1 ? bx[i] : fmav(nsup[i], ox, bx[i]), piv[i]);
-    Rx[i] = i == N - 1 ? tx : tx - ox;
+    Rx[i] = i == N - 1 ? tx : mulr(fmav(ne[i], ox, bx[i]), piv[i]);
     if constexpr (TWO) {
       ty = mulr(i == N - 1 ? by[i] : fmav(nsup[i], oy, by[i]), piv[i]);
-      Ry[i] = i == N - 1 ? ty : ty - oy;
+      Ry[i] = i == N - 1 ? ty : mulr(fmav(ne[i], oy, by[i]), piv[i]);
     }
   }
 }
