@@ -265,11 +265,12 @@ __device__ __forceinline__ T ipow(T r, int e) {
 // Without NN or W32 the options are run-time values, but uniform ones: the
 // pairs are evaluated in straight-line code for one combination (with or
 // without far pairs, either potential), chosen once, so that the latencies
-// of the pairs overlap. A pair without a coefficient contributes exactly
-// nothing, whatever its potential evaluates to.
+// of the pairs overlap. With SKIP a pair without a coefficient contributes
+// exactly nothing, whatever its potential evaluates to (r^3 of a thin layer
+// overflows, and 0 * inf is NaN; the selects cost no time that shows).
 enum PairForm { kPower32, kPower, kExponential };
 
-template <int N, bool FAR, int FORM, class T>
+template <int N, bool FAR, int FORM, bool SKIP, class T>
 __device__ __forceinline__ void interface_pairs(const KParams& P, const KParams& G,
                                                 const T (&zd)[N],
                                                 const T (&sg)[N], const T* z0, const T* sg0,
@@ -312,7 +313,7 @@ __device__ __forceinline__ void interface_pairs(const KParams& P, const KParams&
         e = mulr(e, sg[i]);
       else if (sg0)
         e = mulr(e, *sg0);
-      if constexpr (FORM != kPower32) {  // r^64 of a thin film may overflow
+      if constexpr (SKIP) {
         phi = keep_if(s != 0.f, phi);
         e = keep_if(s != 0.f, e);
       }
@@ -338,18 +339,18 @@ __device__ __forceinline__ void neg_pressures(const KParams& P, const KParams& G
     sg[i] = fmav(0.5f, fmav(gx[i], gx[i], gy[i] * gy[i]), Num<T>::splat(1.f));
   }
   if constexpr (NN && W32) {
-    interface_pairs<N, false, kPower32>(P, G, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, false, kPower32, false>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if constexpr (W32) {
     if (P.far_pairs)
-      interface_pairs<N, true, kPower32>(P, G, zd, sg, z0, sg0, ten, pi);
+      interface_pairs<N, true, kPower32, true>(P, G, zd, sg, z0, sg0, ten, pi);
     else
-      interface_pairs<N, false, kPower32>(P, G, zd, sg, z0, sg0, ten, pi);
+      interface_pairs<N, false, kPower32, true>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if (P.wet_kind == 1) {
-    interface_pairs<N, true, kExponential>(P, G, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, true, kExponential, true>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if (P.far_pairs) {
-    interface_pairs<N, true, kPower>(P, G, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, true, kPower, true>(P, G, zd, sg, z0, sg0, ten, pi);
   } else {
-    interface_pairs<N, false, kPower>(P, G, zd, sg, z0, sg0, ten, pi);
+    interface_pairs<N, false, kPower, true>(P, G, zd, sg, z0, sg0, ten, pi);
   }
   T acc = Num<T>::splat(0.f);
 #pragma unroll
