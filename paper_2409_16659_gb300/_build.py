@@ -24,7 +24,8 @@ UNITS = ([("batch_kernels.cu", ["-DMLSW_BATCH_N=%d" % n]) for n in (5, 3)]
          + [(s, []) for s in ("unet.cu", "step_kernels.cu", "aux_kernels.cu", "mlswlbm.cu",
                               "noalloc.cu", "batch.cu", "analysis.cu")])
 HEADERS = ["physics.cuh", "step_common.cuh", "march.cuh", "kernels.h", "tma.cuh", "tcgen05.cuh",
-           "host.h", "device_once.h", "unit_rows.h"]
+           "host.h", "device_once.h", "unit_rows.h",
+           "ring_plan.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 CFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",

@@ -17,6 +17,7 @@
 
 #include "kernels.h"
 #include "physics.cuh"
+#include "ring_plan.h"
 
 namespace mlsw {
 
@@ -187,7 +188,7 @@ cudaError_t launch_spectrum(int Q, int n, const Layout& L, const float* f, int n
 // in unit-width rings b = floor(r) around (cx, cy), r the periodic
 // (minimum-image) distance; per-cell heights as the read-out gives them
 // (h_i = H_i + sum of the stored populations, in FP32), interfaces and sums
-// in FP64. A CTA adds its rows into rings in shared memory (SHARED: when
+// in FP64. A CTA adds its cells (ring_plan.h) into rings in shared memory (SHARED: when
 // they fit) and those into sums[m][nbins] and counts[nbins]; every cell
 // adding to the global rings directly put 300 addresses under a million
 // atomics.
@@ -206,7 +207,7 @@ __device__ __forceinline__ int ring_of(double q) {  // floor(sqrt(q))
 template <int Q, int PL, bool SHARED>
 __global__ void __launch_bounds__(256)
     radial_profile_kernel(int n, Layout L, const float* __restrict__ f, KShift sh,
-                          ProfileParams A, double* __restrict__ sums,
+                          ProfileParams A, RingPlan pl, double* __restrict__ sums,
                           unsigned long long* __restrict__ counts) {
   extern __shared__ double rings[];  // [n + 1][nbins], then counts [nbins]
   const int nx = L.nx, ny = L.ny, nb = A.nbins;
@@ -218,11 +219,15 @@ __global__ void __launch_bounds__(256)
   }
   const bool sub = A.sub_amp != 0.0;
   const double inx = 1.0 / nx, iny = 1.0 / ny;
-  for (int y = blockIdx.x; y < ny; y += gridDim.x) {
+  const int tx = 1 << pl.lgx, items = pl.groups * pl.segs;
+  for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    const int group = item / pl.segs, first = (item - group * pl.segs) * pl.seg;
+    const int y = group * pl.tr + (int)(threadIdx.x >> pl.lgx), last = min(nx, first + pl.seg);
+    if (y >= ny) continue;
     double dy = y - A.cy;
     dy -= ny * rint(dy * iny);
     if (!(fabs(dy) < (double)nb)) continue;  // no cell of this row is in a ring
-    for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+    for (int x = first + (int)(threadIdx.x & (tx - 1)); x < last; x += tx) {
       double dx = x - A.cx;
       dx -= nx * rint(dx * inx);
       const double q = fma(dx, dx, dy * dy);
@@ -268,16 +273,16 @@ static cudaError_t profile_q(int n, const Layout& L, const float* f, const KShif
                              const ProfileParams& A, double* sums, unsigned long long* counts,
                              cudaStream_t st) {
   const size_t smem = (size_t)A.nbins * ((n + 1) * sizeof(double) + sizeof(unsigned));
-  const unsigned grid = (unsigned)(L.ny < 608 ? L.ny : 608);
+  const RingPlan pl = ring_plan(L.nx, L.ny);
   if (smem > kProfileShared) {
-    radial_profile_kernel<Q, PL, false><<<grid, 256, 0, st>>>(n, L, f, sh, A, sums, counts);
+    radial_profile_kernel<Q, PL, false><<<pl.blocks, 256, 0, st>>>(n, L, f, sh, A, pl, sums, counts);
     return cudaGetLastError();
   }
   auto kern = radial_profile_kernel<Q, PL, true>;
   const cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProfileShared);
   if (e != cudaSuccess) return e;
-  kern<<<grid, 256, smem, st>>>(n, L, f, sh, A, sums, counts);
+  kern<<<pl.blocks, 256, smem, st>>>(n, L, f, sh, A, pl, sums, counts);
   return cudaGetLastError();
 }
 

@@ -1,6 +1,6 @@
 """Host rules of the launches, compiled from their headers with the host
-compiler: heights of the units of work, and the once-per-device setup that
-they depend on."""
+compiler: heights of the units of work, the once-per-device setup that they
+depend on, and the sharing out of the ring sums."""
 import os
 import subprocess
 
@@ -72,3 +72,44 @@ int main() {
   printf("%d %d %d %d %d", wrong, runs, a, b, c);
 }""")
     assert out == ["0", "600", "5", "0", "0"]
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (8, 100000), (9, 33), (255, 7), (256, 1), (257, 5),
+                                   (1024, 1024), (5000, 3), (100000, 8), (1000000, 1), (1, 4099)])
+def test_ring_sums_are_shared_out_whole_and_evenly(tmp_path, nx, ny):
+    """Every cell belongs to one thread of one block; a block has turns of 256
+    threads, and no block has more than twice the turns that an even split
+    over all of them leaves, rounded up."""
+    out = run_cpp(tmp_path, """
+#include <cstdio>
+#include <cstdlib>
+#include <vector>
+#include "ring_plan.h"
+int main(int, char** a) {
+  const int nx = atoi(a[1]), ny = atoi(a[2]);
+  const mlsw::RingPlan p = mlsw::ring_plan(nx, ny);
+  const int tx = 1 << p.lgx;
+  std::vector<unsigned char> seen((size_t)nx * ny);
+  long twice = 0, most = 0;
+  for (int b = 0; b < p.blocks; ++b) {
+    long turns = 0;
+    for (int item = b; item < p.groups * p.segs; item += p.blocks) {
+      const int g = item / p.segs, first = (item - g * p.segs) * p.seg;
+      const int last = first + p.seg < nx ? first + p.seg : nx;
+      turns += (last - first + tx - 1) / tx;
+      for (int t = 0; t < 256; ++t) {
+        const int y = g * p.tr + (t >> p.lgx);
+        if (y >= ny) continue;
+        for (int x = first + (t & (tx - 1)); x < last; x += tx) twice += seen[(size_t)y * nx + x]++;
+      }
+    }
+    if (turns > most) most = turns;
+  }
+  long missing = 0;
+  for (unsigned char c : seen) missing += c == 0;
+  printf("%ld %ld %ld %d", twice, missing, most, tx * p.tr);
+}""", nx, ny)
+    twice, missing, most, threads = map(int, out)
+    assert (twice, missing, threads) == (0, 0, 256)
+    turns = -(-ny // max(1, 256 // max(8, 1 << (min(nx, 256) - 1).bit_length()))) * -(-nx // 256)
+    assert most <= 2 * -(-turns // 608)
