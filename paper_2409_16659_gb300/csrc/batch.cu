@@ -357,7 +357,7 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
     rc = mlsw_host::prepare_instance(params[j], h_init[j], bi.P, sh);
     if (rc != MLSW_OK) break;
     bi.kind = mlsw::batch_kind(bi.P.n, mlsw::step_mode(bi.P));
-    bi.strips = mlsw::march_strips(bi.P.nx);
+    bi.strips = mlsw::march_strips(bi.P.nx, false);
     const size_t flen = (size_t)bi.P.n * planes_of(bi.P) * bi.P.L.plane;
     off[j] = arena_floats;
     arena_floats += 2 * ((flen + 63) / 64 * 64);  // two buffers, 256-byte aligned
@@ -397,7 +397,7 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
     bi.f[0] = b->arena + off[j];
     bi.f[1] = b->arena + off[j] + (flen + 63) / 64 * 64;
     for (int k = 0; k < 2 && ok; ++k)
-      ok = mlsw_host::make_row_map(&bi.map[k], bi.f[k], bi.P.L, bi.P.n * planes_of(bi.P));
+      ok = mlsw_host::make_row_map(&bi.map[k], bi.f[k], bi.P.L, bi.P.n * planes_of(bi.P), false);
   }
   ok = ok && cudaMemcpy(b->dinst, b->hinst.data(), (size_t)count * sizeof(BatchInst),
                         cudaMemcpyHostToDevice) == cudaSuccess;

@@ -32,7 +32,7 @@ __device__ __forceinline__ void run_kind(int kind, const KParams& P, const Batch
   if (kind == K) {
     float* fout = b.f[cur ^ 1];
     __builtin_assume(__isGlobal(fout));
-    march_unit<N, M, M == kGeneral, false>(P, P, &b.map[cur], fout, x0, ya, yb, sm, status);
+    march_unit<N, M, M == kGeneral, false, f2>(P, P, &b.map[cur], fout, x0, ya, yb, sm, status);
   } else if constexpr (K + 1 < 3 * MLSW_BATCH_N) {
     run_kind<K + 1>(kind, P, b, cur, x0, ya, yb, sm, status);
   }
@@ -42,7 +42,7 @@ __device__ __forceinline__ void run_kind(int kind, const KParams& P, const Batch
 template <int K>
 size_t smem_from(unsigned kinds) {
   constexpr int N = K / 3 + 1, M = K % 3;
-  size_t s = (kinds >> K) & 1u ? MarchShape<N, M, M == kGeneral>::kSmem : 0;
+  size_t s = (kinds >> K) & 1u ? MarchShape<N, M, M == kGeneral, f2>::kSmem : 0;
   if constexpr (K + 1 < 3 * MLSW_BATCH_N) s = std::max(s, smem_from<K + 1>(kinds));
   return s;
 }

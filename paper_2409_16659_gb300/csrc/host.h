@@ -18,8 +18,9 @@ int Qof(int lattice);
 int prepare_instance(const mlsw_params& p, const float* h_init, mlsw::KParams& kp,
                      mlsw::KShift& sh);
 
-// 3-D tensor map of a state buffer of `planes` planes, by rows.
-bool make_row_map(CUtensorMap* m, float* base, const mlsw::Layout& L, int planes);
+// 3-D tensor map of a state buffer of `planes` planes, by rows of the march
+// (solo: one column a lane).
+bool make_row_map(CUtensorMap* m, float* base, const mlsw::Layout& L, int planes, bool solo);
 
 // The device address of a page-locked host buffer, or nullptr.
 const void* mapped_host_ptr(const void* p);

@@ -17,12 +17,25 @@ constexpr int kStatusTimeout = 2;    // a bounded mbarrier wait ran out
 // D2Q9 step: a warp marches down a strip of kMarchCols columns, of which the
 // kMarchHalo on each side only feed the stencils (march.cuh).
 constexpr int kMarchCols = 64, kMarchHalo = 4, kMarchOut = kMarchCols - 2 * kMarchHalo;
-inline int march_strips(int nx) { return (nx + kMarchOut - 1) / kMarchOut; }
+// With one column a lane (march_solo) the strip has 32 columns, and a row's
+// copy 36, from the 16-byte boundary at or before the strip's first column.
+constexpr int kSoloCols = 32, kSoloHalo = 3, kSoloOut = kSoloCols - 2 * kSoloHalo, kSoloBox = 36;
+inline int march_strips(int nx, bool solo) {
+  const int out = solo ? kSoloOut : kMarchOut;
+  return (nx + out - 1) / out;
+}
+inline int march_box(bool solo) { return solo ? kSoloBox : kMarchCols; }
 // A D2Q9 state with tau = 1 is stored as moments: plane 4 i + q holds g_0, s,
 // J_x, J_y (q = 0..3) of layer i; another tau (and a lattice whose ghosts need
 // a pass of their own) as populations, plane 9 i + k. Both in the layout of
 // KParams::L.
 constexpr int kMomPlanes = 4;
+
+// Kernel modes of the D2Q9 step: the general step for tau != 1 and for
+// tau = 1, and a fast step for the case the paper runs (tau = 1, wetting
+// exponents (3, 2), spreading coefficients only between neighbouring
+// interfaces).
+enum StepMode { kGeneral = 0, kTau1 = 1, kFast = 2 };
 
 // Per-layer rest-population shift (see KParams).
 struct KShift {
@@ -36,6 +49,7 @@ struct StepLaunch {
   float* fout;
   const CUtensorMap* fin_map;   // D2Q9: row map of fin (see mlsw_host::make_row_map)
   KParams P;
+  int solo;                     // D2Q9: one column a lane (fin_map then has that box)
   int to_populations;           // D2Q9, moments in: write the populations after the step
   int* status;
   int num_sms;
@@ -80,9 +94,11 @@ struct BatchInst {
   int rows;     // rows of a unit
 };
 
-// Kernel mode of a parameter set: 0 general, 1 tau = 1, 2 fast (tau = 1,
-// exponents (3, 2), spreading only between neighbouring interfaces).
+// Kernel mode of a parameter set.
 int step_mode(const KParams& P);
+// Whether a cell has many terms: tau != 1, far pairs, a substrate or the
+// exponential potential.
+bool step_dear(const KParams& P);
 // Whether a D2Q9 state is stored as moments (else populations).
 bool step_moments(const KParams& P);
 

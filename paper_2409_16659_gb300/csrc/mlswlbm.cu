@@ -12,6 +12,7 @@
 #include "host.h"
 #include "kernels.h"
 #include "physics.cuh"
+#include "unit_rows.h"
 
 using mlsw::KParams;
 
@@ -24,6 +25,7 @@ struct mlsw_handle {
   float* f[2];
   int cur;            // index of the buffer holding the current state
   bool moments;
+  bool solo;          // D2Q9: the march takes one column a lane
   // Moment form only. pop: room for the populations, which the state calls
   // exchange with the host. They are in there (kGiven), or follow from the
   // moments: zero moving populations (kAtRest), or one step on from the other
@@ -227,12 +229,12 @@ EncodeTiledFn encode_fn() {
 // A row map's box is one row of a warp's columns in every plane. Rows are
 // copied one by one (box height 1), so that a warp can wrap them around the
 // periodic lattice.
-bool make_row_map(CUtensorMap* m, float* base, const mlsw::Layout& L, int planes) {
+bool make_row_map(CUtensorMap* m, float* base, const mlsw::Layout& L, int planes, bool solo) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[3] = {(cuuint64_t)L.pitch, (cuuint64_t)L.rows, (cuuint64_t)planes};
   cuuint64_t strides[2] = {(cuuint64_t)L.pitch * 4, (cuuint64_t)L.plane * 4};
-  cuuint32_t box[3] = {(cuuint32_t)mlsw::kMarchCols, 1, (cuuint32_t)planes};
+  cuuint32_t box[3] = {(cuuint32_t)mlsw::march_box(solo), 1, (cuuint32_t)planes};
   cuuint32_t es[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, es,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -287,6 +289,7 @@ cudaError_t populations(mlsw_handle* h, const float** f) {
   a.fin = h->f[h->cur ^ 1];
   a.fin_map = &h->map[h->cur ^ 1];
   a.fout = h->pop;
+  a.solo = h->solo;
   a.to_populations = 1;
   return mlsw::launch_step(a, h->stream);
 }
@@ -500,6 +503,9 @@ int mlswlbm_create(const mlsw_params* p, const float* h_init, void* stream, mlsw
     return MLSW_ERR_CUDA;
   }
   h->num_sms = sms > 0 ? sms : 1;
+  const bool general = mlsw::step_mode(kp) == mlsw::kGeneral;
+  h->solo = p->lattice == MLSW_D2Q9 &&
+            mlsw::march_solo(n, general, mlsw::step_dear(kp), p->nx, p->ny, h->num_sms);
   h->nblk_diag = 8 * h->num_sms;
   if (!(p->flags & MLSW_FLAG_NO_PERSISTENT)) {
     int optin = 0;
@@ -535,7 +541,7 @@ int mlswlbm_create(const mlsw_params* p, const float* h_init, void* stream, mlsw
   }
   if (p->lattice == MLSW_D2Q9) {
     for (int k = 0; k < 2; ++k)
-      if (!make_row_map(&h->map[k], h->f[k], h->kp.L, n * state_planes(h))) {
+      if (!make_row_map(&h->map[k], h->f[k], h->kp.L, n * state_planes(h), h->solo)) {
         mlswlbm_destroy(h);
         return MLSW_ERR_CUDA;
       }
@@ -583,6 +589,7 @@ int mlswlbm_step(mlsw_handle* h, long nsteps) {
   a.P = h->kp;
   a.status = h->status;
   a.num_sms = h->num_sms;
+  a.solo = h->solo;
   a.to_populations = 0;
   if (h->psmem) {
     // whole lattice in one CTA: chunks of steps per launch

@@ -177,7 +177,24 @@ __device__ __forceinline__ f2 operator*(float a, f2 b) { return mk2(a, a) * b; }
 __device__ __forceinline__ f2& operator+=(f2& a, f2 b) { return a = a + b; }
 __device__ __forceinline__ f2& operator-=(f2& a, f2 b) { return a = a - b; }
 
+// One cell in the arithmetic of a pair: every operation rounds by itself, and
+// the compiler contracts nothing, so a cell gets the bits it has in a pair.
+struct f1 {
+  float v;
+};
+__device__ __forceinline__ f1 operator+(f1 a, f1 b) { return {__fadd_rn(a.v, b.v)}; }
+__device__ __forceinline__ f1 operator-(f1 a, f1 b) { return {__fsub_rn(a.v, b.v)}; }
+__device__ __forceinline__ f1 operator*(f1 a, f1 b) { return {__fmul_rn(a.v, b.v)}; }
+__device__ __forceinline__ f1 operator+(f1 a, float b) { return {__fadd_rn(a.v, b)}; }
+__device__ __forceinline__ f1 operator-(f1 a, float b) { return {__fsub_rn(a.v, b)}; }
+__device__ __forceinline__ f1 operator-(float a, f1 b) { return {__fsub_rn(a, b.v)}; }
+__device__ __forceinline__ f1 operator*(f1 a, float b) { return {__fmul_rn(a.v, b)}; }
+__device__ __forceinline__ f1 operator*(float a, f1 b) { return {__fmul_rn(a, b.v)}; }
+
 template <class T> struct Num;
+template <> struct Num<f1> {
+  __device__ static f1 splat(float a) { return {a}; }
+};
 template <> struct Num<float> {
   __device__ static float splat(float a) { return a; }
 };
@@ -191,6 +208,11 @@ __device__ __forceinline__ f2 fmav(f2 a, float b, f2 c) { return fmav(a, mk2(b, 
 __device__ __forceinline__ f2 fmav(float a, f2 b, f2 c) { return fmav(mk2(a, a), b, c); }
 __device__ __forceinline__ f2 fmav(f2 a, f2 b, float c) { return fmav(a, b, mk2(c, c)); }
 __device__ __forceinline__ f2 fmav(f2 a, float b, float c) { return fmav(a, mk2(b, b), mk2(c, c)); }
+__device__ __forceinline__ f1 fmav(f1 a, f1 b, f1 c) { return {__fmaf_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ f1 fmav(f1 a, float b, f1 c) { return {__fmaf_rn(a.v, b, c.v)}; }
+__device__ __forceinline__ f1 fmav(float a, f1 b, f1 c) { return {__fmaf_rn(a, b.v, c.v)}; }
+__device__ __forceinline__ f1 fmav(f1 a, f1 b, float c) { return {__fmaf_rn(a.v, b.v, c)}; }
+__device__ __forceinline__ f1 fmav(f1 a, float b, float c) { return {__fmaf_rn(a.v, b, c)}; }
 
 // a product that is rounded by itself: the compiler fuses a scalar product
 // into an addition where it likes, differently from kernel to kernel, and a
@@ -199,6 +221,8 @@ __device__ __forceinline__ f2 fmav(f2 a, float b, float c) { return fmav(a, mk2(
 __device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ f2 mulr(f2 a, f2 b) { return a * b; }
 __device__ __forceinline__ f2 mulr(f2 a, float b) { return a * b; }
+__device__ __forceinline__ f1 mulr(f1 a, f1 b) { return a * b; }
+__device__ __forceinline__ f1 mulr(f1 a, float b) { return a * b; }
 
 // fast reciprocal: the hardware's approximation, at most 1 ulp for normal
 // arguments (here layer thicknesses and friction pivots, far from the ends
@@ -210,6 +234,8 @@ __device__ __forceinline__ float rcp(float x) {
   return r;
 }
 __device__ __forceinline__ f2 rcp(f2 x) { return mk2(rcp(x.v.x), rcp(x.v.y)); }
+__device__ __forceinline__ f1 rcp(f1 x) { return {rcp(x.v)}; }
+__device__ __forceinline__ f1 expv(f1 x) { return {expf(x.v)}; }
 __device__ __forceinline__ float expv(float x) { return expf(x); }
 __device__ __forceinline__ f2 expv(f2 x) { return mk2(expf(x.v.x), expf(x.v.y)); }
 
@@ -218,6 +244,8 @@ __device__ __forceinline__ float keep_if(bool c, float v) { return c ? v : 0.f; 
 __device__ __forceinline__ f2 keep_if(bool c, f2 v) {
   return mk2(c ? v.v.x : 0.f, c ? v.v.y : 0.f);
 }
+
+__device__ __forceinline__ f1 keep_if(bool c, f1 v) { return {c ? v.v : 0.f}; }
 
 // r^e, e >= 0 a uniform run-time exponent: squares, with the factors of the
 // low three bits chosen by selects (exponents in use are small) and a loop
@@ -406,9 +434,9 @@ __device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], cons
   T na_prev;                               // -a_{i-1}
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    const T na = mulr(h[i], P.fr_visc[i]), s = mulr(ih[i], P.fr_slip2[i]);
+    const T na = mulr(h[i], P.fr_visc[i]);
     T rest = fmav(na, -2.f, Num<T>::splat(P.fr_slip[i]));  // d_i - s_i
-    nsup[i] = na + s;
+    nsup[i] = fmav(ih[i], P.fr_slip2[i], na);
     if (i == 0) {
       bx[0] = Ux[0] * -1.f;
       if constexpr (TWO) by[0] = Uy[0] * -1.f;
@@ -419,7 +447,7 @@ __device__ __forceinline__ void friction(const KParams& P, const T (&h)[N], cons
       bx[i] = fmav(nf, bx[j], Ux[j] - Ux[i]);
       if constexpr (TWO) by[i] = fmav(nf, by[j], Uy[j] - Uy[i]);
     }
-    piv[i] = rcp(rest + s);
+    piv[i] = rcp(fmav(ih[i], P.fr_slip2[i], rest));
     ne[i] = na - rest;
     na_prev = na;
   }

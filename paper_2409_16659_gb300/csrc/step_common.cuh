@@ -9,12 +9,6 @@
 
 namespace mlsw {
 
-// Kernel modes of the D2Q9 step: the general step for tau != 1 and for
-// tau = 1, and a fast step for the case the paper runs (tau = 1, wetting
-// exponents (3, 2), spreading coefficients only between neighbouring
-// interfaces).
-enum StepMode { kGeneral = 0, kTau1 = 1, kFast = 2 };
-
 // ---------------------------------------------------------------------------
 // Bounds checks of the debug build (physics.cuh): a shared-memory pointer
 // must lie in the CTA's dynamic shared memory, an index in its array, a

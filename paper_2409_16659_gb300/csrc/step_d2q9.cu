@@ -11,15 +11,15 @@
 
 namespace mlsw {
 
-template <int N, int MODE, bool OP>
-__global__ void __launch_bounds__(32, march_warps(N, MODE))
+template <int N, int MODE, bool OP, class T>
+__global__ void __launch_bounds__(32, lane_warps<T>(N, MODE))
     step_d2q9(const __grid_constant__ CUtensorMap map, float* __restrict__ fout,
               const __grid_constant__ KParams P, int strips, int rows, int* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int strip = (int)(blockIdx.x % strips), ya = (int)(blockIdx.x / strips) * rows;
   // (two rows a turn spill from four layers on)
-  march_unit<N, MODE, OP, N <= 3>(P, P, &map, fout, strip * kMarchOut, ya, min(ya + rows, P.ny),
-                                  smem_raw, status);
+  march_unit<N, MODE, OP, N <= 3, T>(P, P, &map, fout, strip * MarchLane<T>::kOut, ya,
+                                     min(ya + rows, P.ny), smem_raw, status);
 }
 
 // A step of a batch whose instances are all of this kind (batch_kernels.cu):
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(32, march_warps(N, MODE))
   __builtin_assume(__isGlobal(fout));
   const int strip = e.y % b.strips, ya = e.y / b.strips * b.rows;
   const KParams& Q = SAME ? P : G;
-  march_unit<N, MODE, MODE == kGeneral, SAME && N <= 3>(Q, G, &b.map[cur], fout,
+  march_unit<N, MODE, MODE == kGeneral, SAME && N <= 3, f2>(Q, G, &b.map[cur], fout,
                                                         strip * kMarchOut, ya,
                                                         min(ya + b.rows, Q.ny),
                                                         smem_raw + kParBytes, status);
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(32, march_warps(N, MODE))
 
 template <int N, int MODE, bool SAME>
 static cudaError_t launch_alike(const BatchLaunch& a, cudaStream_t st) {
-  constexpr size_t smem = kParBytes + MarchShape<N, MODE, MODE == kGeneral>::kSmem;
+  constexpr size_t smem = kParBytes + MarchShape<N, MODE, MODE == kGeneral, f2>::kSmem;
   auto kern = step_d2q9_alike<N, MODE, SAME>;
   static DeviceOnce configured;
   int dev = 0;
@@ -83,10 +83,10 @@ cudaError_t launch_alike_d2q9<MLSW_N>(const BatchLaunch& a, int mode, cudaStream
   }
 }
 
-template <int N, int MODE, bool OP>
-static cudaError_t launch_march(const StepLaunch& a, cudaStream_t st) {
-  using S = MarchShape<N, MODE, OP>;
-  auto kern = step_d2q9<N, MODE, OP>;
+template <int N, int MODE, bool OP, class T>
+static cudaError_t launch_march_t(const StepLaunch& a, cudaStream_t st) {
+  using S = MarchShape<N, MODE, OP, T>;
+  auto kern = step_d2q9<N, MODE, OP, T>;
   // raise the dynamic shared-memory limit and count the resident warps once
   // per device and instantiation
   static DeviceOnce configured;
@@ -105,8 +105,12 @@ static cudaError_t launch_march(const StepLaunch& a, cudaStream_t st) {
     return e1;
   });
   if (e != cudaSuccess) return e;
-  const int strips = march_strips(a.P.nx);
-  const int rows = march_rows(N, a.P.ny, strips, a.num_sms, a.num_sms * per_sm[dev]);
+  constexpr bool solo = MarchLane<T>::kPer == 1;
+  const int strips = march_strips(a.P.nx, solo), slots = a.num_sms * per_sm[dev];
+  const bool heavy = N >= (MODE == kGeneral ? 4 : 5) && step_dear(a.P);
+  const int rows =
+      solo ? solo_rows(MODE == kGeneral, a.P.ny, strips, a.num_sms, slots)
+           : march_rows(N, heavy, a.P.ny, strips, a.num_sms, slots);
   const long units = (long)strips * ((a.P.ny + rows - 1) / rows);
   // launched as a programmatic dependent of the previous kernel on the
   // stream (see march_unit)
@@ -121,6 +125,13 @@ static cudaError_t launch_march(const StepLaunch& a, cudaStream_t st) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, *a.fin_map, a.fout, a.P, strips, rows, a.status);
+}
+
+template <int N, int MODE, bool OP>
+static cudaError_t launch_march(const StepLaunch& a, cudaStream_t st) {
+  if constexpr (N >= 4)  // (march_solo)
+    if (a.solo) return launch_march_t<N, MODE, OP, f1>(a, st);
+  return launch_march_t<N, MODE, OP, f2>(a, st);
 }
 
 template <>

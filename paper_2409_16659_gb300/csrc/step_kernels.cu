@@ -302,6 +302,10 @@ int step_mode(const KParams& P) {
   return (w32 && !P.far_pairs && P.sub_amp == 0.f) ? kFast : kTau1;
 }
 
+bool step_dear(const KParams& P) {
+  return step_mode(P) == kGeneral || P.far_pairs || P.sub_amp != 0.f || P.wet_kind != 0;
+}
+
 bool step_moments(const KParams& P) { return step_mode(P) != kGeneral; }
 
 template <int N>

@@ -22,7 +22,12 @@ namespace mlsw {
 // cheapest by that model. One layer, 448^2: 8.1 us a step with 1 row (the
 // wave), 5.0 with 3; 25 x 1870 5.1 and 4.4 with 2; two layers, 320^2: 7.3 with
 // 1, 5.8 with 2; 25 x 1870 8.2 and 6.0 with 2.
-inline int march_rows(int n, int ny, int strips, int num_sms, int slots) {
+//
+// heavy: rows of more than 3 us (four layers with tau != 1, five with many terms a
+// cell, see step_dear): these run as one wave from three rows a unit on (four layers,
+// tau = 0.8, 256^2: 15.1 us a step with 3 rows, 13.3 with 2; five layers, far
+// pairs: 20.1 and 18.8).
+inline int march_rows(int n, bool heavy, int ny, int strips, int num_sms, int slots) {
   if (slots < 1) slots = 1;
   const long total = (long)ny * strips, flat = (total + 4L * num_sms - 1) / (4L * num_sms);
   if (n <= 2 && total <= 4L * slots) {
@@ -41,13 +46,61 @@ inline int march_rows(int n, int ny, int strips, int num_sms, int slots) {
     }
     if (best_rows > 0) return best_rows;
   }
-  if (flat <= 3) return (int)flat;
+  if (flat <= (heavy ? 2 : 3)) return (int)flat;
   for (long wave = 1;; ++wave) {
     const long chunks = (long)slots * wave / strips;
     if (chunks < 1) continue;
     const long rows = (ny + chunks - 1) / chunks;
     if (rows <= 64) return (int)rows;
   }
+}
+
+// Whether the march of an n-layer lattice takes one column a lane (26 columns a
+// strip) instead of a pair (56). Per row and warp that is the shorter chain
+// with half the registers and ring, so more warps; per column it is more
+// instructions. It pays, from four layers on, where
+//   * both forms have one strip: 25 x 1870, us a step with pairs and with single
+//     columns, four layers 12.6 and 9.9 (fast mode), 15.6 and 12.5 (tau = 1
+//     otherwise), 18.1 and 11.5 (tau = 0.8), five 15.3 and 11.3, 20.9 and 16.0, 26.8
+//     and 15.1; 26 x 30000, five layers, tau = 0.8, 270 and 153;
+//   * pairs leave a third of their strips empty (57 to 78 columns) and give a
+//     scheduler two rows or more: 57 x 800, four layers, 14.4 and 12.4 (tau = 1
+//     otherwise); above four rows a scheduler only in the general mode, whose
+//     pairs hold four to six warps an SM (57 x 10000, five layers 171 and 118,
+//     but four layers of the fast mode, 78 x 2500, 18.2 and 19.7);
+//   * pairs have two to three rows a scheduler and every cell many terms (dear:
+//     tau != 1, far pairs, a substrate or the exponential potential): 256^2, five
+//     layers, 20.2 and 18.2 (far pairs), 20.4 and 18.7 (tau = 0.8); without them,
+//     four layers, 10.1 and 10.6.
+// Fewer rows a scheduler go to pairs (130^2: 10.4 and 13.8).
+inline bool march_solo(int n, bool general, bool dear, int nx, int ny, int num_sms) {
+  if (n < 4) return false;
+  const long pairs = (nx + 55) / 56, solo = (nx + 25) / 26, total = pairs * ny, s = 4L * num_sms;
+  if (solo == 1) return true;
+  if (total <= 2 * s) return false;
+  if (2 * solo <= 3 * pairs && (general || total <= 4 * s)) return true;
+  return dear && solo <= 2 * pairs && total <= 3 * s;
+}
+
+// Rows of a unit with one column a lane: the cheapest by rows plus warm-up (five
+// rows, in the general mode one and a half) times what a row takes with k warps
+// on a scheduler; beyond 16 rows one wave of the warps that fit, as for pairs.
+// 25 x 1870, four layers, tau = 1, with 1, 2, 3, 4 rows: 15.2, 12.5, 13.9, 14.4 us.
+inline int solo_rows(bool general, int ny, int strips, int num_sms, int slots) {
+  constexpr double per_row[2][6] = {{1.0, 1.17, 1.38, 1.7, 2.1, 2.5}, {1.0, 1.06, 1.27, 1.6, 2.0, 2.4}};
+  double best = 0.0;
+  int best_rows = 0;
+  for (int rows = 1; rows <= 16; ++rows) {
+    const long units = (long)strips * (((long)ny + rows - 1) / rows);
+    const long k = (units + 4L * num_sms - 1) / (4L * num_sms);
+    if (units > slots || k > 6) continue;
+    const double cost = (rows + (general ? 1.5 : 5.0)) * per_row[general][k - 1];
+    if (best_rows == 0 || cost < best) {
+      best = cost;
+      best_rows = rows;
+    }
+  }
+  return best_rows > 0 ? best_rows : march_rows(4, true, ny, strips, num_sms, slots);
 }
 
 }  // namespace mlsw

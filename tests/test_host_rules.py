@@ -32,12 +32,14 @@ def test_unit_heights_end_for_any_number_of_slots(tmp_path, n):
 #include <initializer_list>
 #include "unit_rows.h"
 int main(int, char** a) {
+  for (bool heavy : {false, true})
   for (int slots : {0, 1, 152, 1824})
     for (int ny : {1, 2, 7, 64, 1024, 5000})
       for (int strips : {1, 2, 19, 1000})
-        printf("%d ", mlsw::march_rows(atoi(a[1]), ny, strips, 152, slots));
+        printf("%d %d ", mlsw::march_rows(atoi(a[1]), heavy, ny, strips, 152, slots),
+               mlsw::solo_rows(heavy, ny, strips, 152, slots));
 }""", n)
-    assert len(out) == 4 * 6 * 4 and all(1 <= int(v) <= 64 for v in out)
+    assert len(out) == 2 * 2 * 4 * 6 * 4 and all(1 <= int(v) <= 64 for v in out)
 
 
 def test_device_setup_is_seen_whole_by_every_thread(tmp_path):
