@@ -386,11 +386,14 @@ int mlswlbm_diagnostics_noalloc(const mlsw_params* p, const float* f, const floa
 typedef struct mlsw_batch mlsw_batch;
 
 /* batch flags. Tile heights are nominal: the rows of an instance's units of
- * work are 16 or 8, scaled by one factor for the instances stepped together. */
-#define MLSW_BATCH_TILE8 1    /* 8-row tiles for every instance (default: 16 rows for n <= 3) */
-#define MLSW_BATCH_AUTOTUNE 2 /* at create, time 8- and 16-row tiles for every class of
-                                 instances with the same n, kernel mode and size (n <= 3)
-                                 and keep the faster; the states are then reset to h_init */
+ * work follow from a model of the step of the instances stepped together. 16
+ * and 8 stand for two heights, the second half of the first (four and five
+ * layers are always 8); beside four and five layers the model is applied to the
+ * proportion that they give. */
+#define MLSW_BATCH_TILE8 1    /* 8 for every instance (default: 16 for n <= 3) */
+#define MLSW_BATCH_AUTOTUNE 2 /* at create, time steps of the batch with 16 and with 8 for
+                                 every layer count (n <= 3) and kernel mode in turn and
+                                 keep the faster; the states are then reset to h_init */
 
 /* Creates a batch of count >= 1 lattices: params[j] and h_init[j] (host,
  * [n_j][ny_j][nx_j]) as for mlswlbm_create, every lattice D2Q9 (else

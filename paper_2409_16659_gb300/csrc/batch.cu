@@ -3,7 +3,7 @@
 // one unit table in which the instances that share layer count, kernel mode
 // and nominal tile height (a group) have a contiguous range, one launch per step
 // over the whole table (batch_kernels.cu), and a timing autotuner for the
-// tile height of every class of alike instances.
+// nominal height of every layer count and mode.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -16,6 +16,7 @@
 #include "host.h"
 #include "kernels.h"
 #include "physics.cuh"
+#include "unit_rows.h"
 
 using mlsw::BatchInst;
 using mlsw::KParams;
@@ -70,26 +71,29 @@ int planes_of(const KParams& P) { return mlsw::step_moments(P) ? mlsw::kMomPlane
 
 int units_of(const BatchInst& b, int rows) { return b.strips * ((b.P.ny + rows - 1) / rows); }
 
-// rows of an instance's units: 16-row tiles scaled to r rows, 8-row tiles to
-// half as many, at most 64 (see march_rows in step_d2q9.cu)
-int unit_rows(int variant, int r) {
-  return std::min(64, r * mlsw::batch_tile_rows(variant) / 16 + (variant == 0 ? 0 : r & 1));
+// Rows of an instance's units at scale r: four and five layers half of r, the
+// others r, or half of it too where the variant is 8 (half).
+int scaled_rows(const BatchInst& b, int r, bool half) {
+  const int rows = b.P.n <= 3 ? r : (r + 1) / 2;
+  return std::min(64, b.P.n <= 3 && half ? mlsw::half_rows(rows) : rows);
 }
 
-// Scale r of the units of a table, by a model of a step's time in units of a
-// row's issue time on one of an SM's four schedulers. A unit costs its rows
-// plus about five rows of warm-up; a warp alone on a scheduler needs 1.75
-// times that time for a row's latencies. Alike instances finish together, in
-// whole waves, and as the schedulers' fullest; uneven ones (work in
-// proportion to n) overlap, and the longest unit may come last. 16 films of
-// 256^2: r = 12 instead of 16 brings a step from 47 to 44 us.
-int scale_for(const mlsw_batch* b, const std::vector<int>& members, const std::vector<int>& variant) {
+// Scale r of the units of a table, by a model of a step's time in units of a row's issue time on one of an SM's four
+// schedulers. A unit costs its rows plus about five rows of warm-up; a warp
+// alone on a scheduler needs 1.75 times that time for a row's latencies.
+// Instances of one layer count finish together, in whole waves, and as the
+// schedulers' fullest (5 % more units than an even split: the SMs are not
+// filled exactly evenly); uneven ones (work in proportion to n) overlap, and the
+// longest unit may come last. Beside four or five layers the variants shift the
+// proportion of the heights, and the scale follows; without them the scale is that
+// of the nominal 16, so that 8 are half of it (a scale for them would give the same
+// heights again). 16 films of 256^2: r = 12 instead of 16 brings
+// a step from 47 to 44 us.
+int scale_for(const mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
   int nmax = 0, nmin = mlsw::kMaxLayers;
-  unsigned kinds = 0;
   for (int j : members) {
     nmax = std::max(nmax, b->hinst[j].P.n);
     nmin = std::min(nmin, b->hinst[j].P.n);
-    kinds |= 1u << b->hinst[j].kind;
   }
   const int per_sm = mlsw::batch_warps_per_sm(kinds);
   const double schedulers = 4.0 * b->num_sms, slots = (double)per_sm * b->num_sms;
@@ -98,7 +102,7 @@ int scale_for(const mlsw_batch* b, const std::vector<int>& members, const std::v
   for (int r = 1; r <= 128; ++r) {
     double units = 0.0, work = 0.0, longest = 0.0;
     for (int j : members) {
-      const int rows = unit_rows(variant[j], r);
+      const int rows = scaled_rows(b->hinst[j], r, nmax > 3 && b->variant[j] == 1);
       const double u = units_of(b->hinst[j], rows), w = (double)(rows + 5) * b->hinst[j].P.n;
       units += u;
       work += u * w;
@@ -119,6 +123,13 @@ int scale_for(const mlsw_batch* b, const std::vector<int>& members, const std::v
     }
   }
   return best_r;
+}
+
+// rows of the members' units: all of the model's for the nominal 16, half for 8
+void choose_rows(mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
+  const int r = scale_for(b, members, kinds);
+  for (int j : members)
+    b->hinst[j].rows = scaled_rows(b->hinst[j], r, b->variant[j] == 1);
 }
 
 // the buffer that holds instance j's state now
@@ -191,7 +202,7 @@ int build_groups(mlsw_batch* b) {
     b->kinds |= 1u << bi.kind;
     if (bi.P.tiny) b->tiny.push_back(j);
   }
-  const int r = all.empty() ? 1 : scale_for(b, all, b->variant);
+  if (!all.empty()) choose_rows(b, all, b->kinds);
   b->same_params = same_params(b, all);
   if (!all.empty()) b->params = b->hinst[all[0]].P;
   std::vector<int2> table;
@@ -203,7 +214,6 @@ int build_groups(mlsw_batch* b) {
     g.variant = std::get<2>(kv.first);
     g.offset = (int)table.size();
     for (int j : kv.second) {
-      b->hinst[j].rows = unit_rows(g.variant, r);
       const int nu = units_of(b->hinst[j], b->hinst[j].rows);
       for (int t = 0; t < nu; ++t) table.push_back(make_int2(j, t));
     }
@@ -215,9 +225,12 @@ int build_groups(mlsw_batch* b) {
   b->dtable = nullptr;
   if (cudaMalloc(&b->dtable, std::max<size_t>(1, table.size()) * sizeof(int2)) != cudaSuccess)
     return MLSW_ERR_NOMEM;
-  CUB(cudaMemcpy(b->dtable, table.data(), table.size() * sizeof(int2), cudaMemcpyHostToDevice));
-  CUB(cudaMemcpy(b->dinst, b->hinst.data(), (size_t)b->count * sizeof(BatchInst),
-                 cudaMemcpyHostToDevice));
+  // on the stream of the steps that read them (pageable sources: staged before
+  // the calls return)
+  CUB(cudaMemcpyAsync(b->dtable, table.data(), table.size() * sizeof(int2), cudaMemcpyHostToDevice,
+                      b->stream));
+  CUB(cudaMemcpyAsync(b->dinst, b->hinst.data(), (size_t)b->count * sizeof(BatchInst),
+                      cudaMemcpyHostToDevice, b->stream));
   return MLSW_OK;
 }
 
@@ -236,73 +249,51 @@ mlsw::BatchLaunch step_launch(const mlsw_batch* b) {
   return a;
 }
 
-// Timing autotuner: for every class of instances with the same n (<= 3),
-// mode and size, time a few steps of the class alone with 16-row and with
-// 8-row tiles and keep the faster. The steps change the states, which the
-// caller resets afterwards.
-int autotune(mlsw_batch* b) {
-  std::map<std::tuple<int, int, int, int>, std::vector<int>> classes;
-  for (int j = 0; j < b->count; ++j) {
-    const KParams& P = b->hinst[j].P;
-    if (P.n <= 3) classes[std::make_tuple(P.n, mlsw::step_mode(P), P.nx, P.ny)].push_back(j);
+// us of a step over the present table, from kTimed steps after a few
+int time_steps(mlsw_batch* b, cudaEvent_t e0, cudaEvent_t e1, float* ms) {
+  constexpr int kWarm = 2, kTimed = 8;
+  for (int s = 0; s < kWarm + kTimed; ++s) {
+    if (s == kWarm) CUB(cudaEventRecord(e0, b->stream));
+    mlsw::BatchLaunch a = step_launch(b);
+    a.cur = s & 1;
+    CUB(mlsw::launch_batch_step(a, b->stream));
+    b->launches += 1;
   }
+  CUB(cudaEventRecord(e1, b->stream));
+  CUB(cudaEventSynchronize(e1));
+  CUB(cudaEventElapsedTime(ms, e0, e1));
+  return MLSW_OK;
+}
+
+// Timing autotuner: for every layer count (<= 3) and mode of the batch in turn,
+// the whole batch is stepped with that class's units at the nominal 16 and 8
+// rows, in the kernel it will run; 8 is kept where it is 0.5 % faster (the spread
+// of the timings; the sweep of 512 lattices: 1097 us a step with 16, 1085 with 8). The steps change the states, which the caller
+// resets afterwards, and leave the table to be built.
+int autotune(mlsw_batch* b) {
+  std::map<int, std::vector<int>> classes;
+  for (int j = 0; j < b->count; ++j)
+    if (b->hinst[j].P.n <= 3) classes[b->hinst[j].kind].push_back(j);
   cudaEvent_t e0, e1;
   CUB(cudaEventCreate(&e0));
   if (cudaEventCreate(&e1) != cudaSuccess) {
     cudaEventDestroy(e0);
     return MLSW_ERR_CUDA;
   }
-  int rc = MLSW_OK;
-  int2* dt = nullptr;
+  float best = 0.f;
+  int rc = build_groups(b);
+  if (rc == MLSW_OK) rc = time_steps(b, e0, e1, &best);
   for (auto& kv : classes) {
-    const int n = std::get<0>(kv.first), mode = std::get<1>(kv.first);
-    float best = 0.f;
-    int best_v = 0;
-    for (int v = 0; v < mlsw::kBatchVariants && rc == MLSW_OK; ++v) {
-      std::vector<int2> table;
-      const int r = scale_for(b, kv.second, std::vector<int>(b->count, v));
-      for (int j : kv.second) b->hinst[j].rows = unit_rows(v, r);
-      for (int j : kv.second)
-        for (int t = 0; t < units_of(b->hinst[j], b->hinst[j].rows); ++t)
-          table.push_back(make_int2(j, t));
-      if (dt) cudaFree(dt);
-      dt = nullptr;
-      if (cudaMalloc(&dt, table.size() * sizeof(int2)) != cudaSuccess ||
-          cudaMemcpy(dt, table.data(), table.size() * sizeof(int2), cudaMemcpyHostToDevice) !=
-              cudaSuccess ||
-          cudaMemcpy(b->dinst, b->hinst.data(), (size_t)b->count * sizeof(BatchInst),
-                     cudaMemcpyHostToDevice) != cudaSuccess) {
-        rc = MLSW_ERR_CUDA;
-        break;
-      }
-      mlsw::BatchLaunch a = step_launch(b);
-      a.table = dt;
-      a.nunits = (int)table.size();
-      a.nmax = n;
-      a.kinds = 1u << mlsw::batch_kind(n, mode);
-      a.same_params = same_params(b, kv.second);
-      a.P = b->hinst[kv.second[0]].P;
-      constexpr int kWarm = 2, kTimed = 6;
-      float ms = 0.f;
-      for (int s = 0; s < kWarm + kTimed && rc == MLSW_OK; ++s) {
-        if (s == kWarm && cudaEventRecord(e0, b->stream) != cudaSuccess) rc = MLSW_ERR_CUDA;
-        a.cur = s & 1;
-        if (mlsw::launch_batch_step(a, b->stream) != cudaSuccess) rc = MLSW_ERR_CUDA;
-        b->launches += 1;
-      }
-      if (rc == MLSW_OK && (cudaEventRecord(e1, b->stream) != cudaSuccess ||
-                            cudaEventSynchronize(e1) != cudaSuccess ||
-                            cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
-        rc = MLSW_ERR_CUDA;
-      if (rc == MLSW_OK && (v == 0 || ms < best)) {
-        best = ms;
-        best_v = v;
-      }
-    }
     if (rc != MLSW_OK) break;
-    for (int j : kv.second) b->variant[j] = best_v;
+    for (int j : kv.second) b->variant[j] = 1;
+    float ms = 0.f;
+    rc = build_groups(b);
+    if (rc == MLSW_OK) rc = time_steps(b, e0, e1, &ms);
+    if (rc == MLSW_OK && ms < 0.995f * best)
+      best = ms;
+    else
+      for (int j : kv.second) b->variant[j] = 0;
   }
-  if (dt) cudaFree(dt);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   return rc;

@@ -78,11 +78,10 @@ cudaError_t launch_step_persistent(const StepLaunch& a, int nsteps, cudaStream_t
 // table of units, in which the units of instances that share n, kernel mode
 // and nominal tile height form a contiguous range (batch_kernels.cu).
 // ---------------------------------------------------------------------------
-// Tile heights a batch can use: variant 0 = 16 rows (n <= 3 only), variant
-// 1 = 8 rows. A warp's unit of work is a strip of `rows` rows: the height,
-// scaled alike for all instances of a table (batch.cu).
+// Nominal tile heights (batch.cu): variant 0 = 16 rows (n <= 3 only), the height
+// of the model, variant 1 = 8 rows, for n <= 3 half of it.
 constexpr int kBatchVariants = 2;
-__host__ __device__ constexpr int batch_tile_rows(int variant) { return variant == 0 ? 16 : 8; }
+constexpr int batch_tile_rows(int variant) { return variant == 0 ? 16 : 8; }
 
 // Device descriptor of one instance (aligned as its tensor maps require).
 struct BatchInst {

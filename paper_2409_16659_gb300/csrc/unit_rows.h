@@ -103,4 +103,8 @@ inline int solo_rows(bool general, int ny, int strips, int num_sms, int slots) {
   return best_rows > 0 ? best_rows : march_rows(4, true, ny, strips, num_sms, slots);
 }
 
+// Batches: the height of nominal 8-row units where that is a choice, half of the
+// model's.
+inline int half_rows(int rows) { return (rows + 1) / 2; }
+
 }  // namespace mlsw

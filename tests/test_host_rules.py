@@ -115,3 +115,15 @@ int main(int, char** a) {
     assert (twice, missing, threads) == (0, 0, 256)
     turns = -(-ny // max(1, 256 // max(8, 1 << (min(nx, 256) - 1).bit_length()))) * -(-nx // 256)
     assert most <= 2 * -(-turns // 608)
+
+
+def test_nominal_heights_of_a_batch_differ(tmp_path):
+    """Units of nominal 8 rows are half as high as those of 16, from two rows on."""
+    out = run_cpp(tmp_path, """
+#include <cstdio>
+#include "unit_rows.h"
+int main() {
+  for (int rows = 1; rows <= 64; ++rows) printf("%d ", mlsw::half_rows(rows));
+}""")
+    assert [int(v) for v in out] == [(r + 1) // 2 for r in range(1, 65)]
+    assert all(int(v) < r for r, v in enumerate(out, 1) if r > 1)
