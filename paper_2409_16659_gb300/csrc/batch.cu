@@ -35,7 +35,8 @@ struct Group {
 struct mlsw_batch {
   int count;
   std::vector<BatchInst> hinst;  // host copies of the descriptors
-  std::vector<int> variant;      // tile-height variant of every instance
+  std::vector<int> variant;      // nominal-height variant of every instance
+  std::vector<char> solo;        // its maps and strips are those of one column a lane
   // instances the step advances (mlswlbm_batch_select; all at create) and,
   // for one left out, the buffer index that holds its state
   std::vector<char> selected;
@@ -43,7 +44,7 @@ struct mlsw_batch {
   std::vector<Group> groups;
   BatchInst* dinst;
   int2* dtable;  // the unit table, sorted by kind
-  int nunits, nmax;    // its length, the largest layer count in it
+  int nunits;          // its length
   unsigned kinds;      // kinds in it
   int same_params;     // its instances' parameters differ in H and Hsum only
   KParams params;         // of the first instance in it
@@ -78,17 +79,40 @@ int scaled_rows(const BatchInst& b, int r, bool half) {
   return std::min(64, b.P.n <= 3 && half ? mlsw::half_rows(rows) : rows);
 }
 
-// Scale r of the units of a table, by a model of a step's time in units of a row's issue time on one of an SM's four
-// schedulers. A unit costs its rows plus about five rows of warm-up; a warp
-// alone on a scheduler needs 1.75 times that time for a row's latencies.
+double weight_of(const BatchInst& b) {
+  return mlsw::batch_weight(b.P.n, b.kind % 3, b.P.sub_amp != 0.f);
+}
+
+unsigned kinds_of(const mlsw_batch* b, const std::vector<int>& members) {
+  unsigned kinds = 0;
+  for (int j : members) kinds |= 1u << b->hinst[j].kind;
+  return kinds;
+}
+
+bool one_kind(unsigned kinds) { return (kinds & (kinds - 1)) == 0; }
+
+// Tables whose units have one height, scaled: those of one kind, of the kernel
+// for at most three layers, or without an instance whose cells have many terms
+// (whose rows take up to four times the others').
+bool scaled_table(const mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
+  if (one_kind(kinds) || mlsw::batch_small(kinds)) return true;
+  for (int j : members)
+    if (mlsw::step_dear(b->hinst[j].P)) return false;
+  return true;
+}
+
+// Scale r of the units of such a table, by a model of a step's time in units of
+// a row's issue time on one of an SM's four schedulers. A unit costs its rows
+// plus about five rows of warm-up; a warp alone on a scheduler needs 1.75 times
+// that time for a row's latencies.
 // Instances of one layer count finish together, in whole waves, and as the
 // schedulers' fullest (5 % more units than an even split: the SMs are not
 // filled exactly evenly); uneven ones (work in proportion to n) overlap, and the
 // longest unit may come last. Beside four or five layers the variants shift the
 // proportion of the heights, and the scale follows; without them the scale is that
 // of the nominal 16, so that 8 are half of it (a scale for them would give the same
-// heights again). 16 films of 256^2: r = 12 instead of 16 brings
-// a step from 47 to 44 us.
+// heights again). 16 films of 256^2: r = 12 instead of 16 brings a step from 47 to
+// 44 us.
 int scale_for(const mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
   int nmax = 0, nmin = mlsw::kMaxLayers;
   for (int j : members) {
@@ -125,11 +149,60 @@ int scale_for(const mlsw_batch* b, const std::vector<int>& members, unsigned kin
   return best_r;
 }
 
+// Duration t (us) of the units of other tables: the same for all kinds, so that
+// none is left running alone (32 lattices of 2 to 5 layers, all modes: 294 us a
+// step with one scaled height, 226).
+double unit_time(const mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
+  const int slots = b->num_sms * mlsw::batch_warps_per_sm(kinds);
+  double best_t = 0.0, best = 0.0;
+  for (int c = 0; c < 128; ++c) {
+    const double t = 3.0 * std::pow(1.035, c);
+    double units = 0.0, work = 0.0, longest = 0.0;
+    for (int j : members) {
+      const double w = weight_of(b->hinst[j]);
+      const int rows = mlsw::batch_rows(w, t);
+      const double u = units_of(b->hinst[j], rows);
+      units += u;
+      work += u * (rows + 5) * w;
+      longest = std::max(longest, (rows + 5) * w);
+    }
+    const double cost = mlsw::batch_cost(units, work, longest, b->num_sms, slots);
+    if (c == 0 || cost < best) {
+      best = cost;
+      best_t = t;
+    }
+  }
+  return best_t;
+}
+
 // rows of the members' units: all of the model's for the nominal 16, half for 8
 void choose_rows(mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
-  const int r = scale_for(b, members, kinds);
-  for (int j : members)
-    b->hinst[j].rows = scaled_rows(b->hinst[j], r, b->variant[j] == 1);
+  const bool scaled = scaled_table(b, members, kinds);
+  const int r = scaled ? scale_for(b, members, kinds) : 1;
+  const double t = scaled ? 0.0 : unit_time(b, members, kinds);
+  for (int j : members) {
+    BatchInst& bi = b->hinst[j];
+    const bool half = b->variant[j] == 1;
+    if (scaled) {
+      bi.rows = scaled_rows(bi, r, half);
+    } else {
+      const int rows = mlsw::batch_rows(weight_of(bi), t);
+      bi.rows = bi.P.n <= 3 && half ? mlsw::half_rows(rows) : rows;
+    }
+  }
+}
+
+// The order of a table of units of equal duration that is sorted by kind and
+// runs as one wave: neighbouring CTAs start on different SMs, so neighbouring
+// entries go num_sms apart, and the warps of an SM share few kinds' instructions
+// (9 lattices of 2 to 5 layers, all modes: 56 us a step in the sorted order, 28; in
+// several waves the sorted order does it, and spreads the work better).
+void order_one_wave(std::vector<int2>& table, int num_sms) {
+  std::vector<int2> out(table.size());
+  size_t u = 0;
+  for (int s = 0; s < num_sms; ++s)
+    for (size_t p = s; p < table.size(); p += num_sms) out[p] = table[u++];
+  table.swap(out);
 }
 
 // the buffer that holds instance j's state now
@@ -153,6 +226,16 @@ int align_buffers(mlsw_batch* b) {
     CUB(cudaMemcpyAsync(b->dinst, b->hinst.data(), (size_t)b->count * sizeof(BatchInst),
                         cudaMemcpyHostToDevice, b->stream));
   return MLSW_OK;
+}
+
+// the row maps of instance j's two buffers, in the form it marches in
+bool map_rows(mlsw_batch* b, int j) {
+  BatchInst& bi = b->hinst[j];
+  bool ok = true;
+  for (int k = 0; k < 2; ++k)
+    ok = ok && mlsw_host::make_row_map(&bi.map[k], bi.f[k], bi.P.L, bi.P.n * planes_of(bi.P),
+                                       b->solo[j]);
+  return ok;
 }
 
 // (re)initialise every instance from its heights: f = f_eq(h, U = 0)
@@ -190,7 +273,6 @@ int same_params(const mlsw_batch* b, const std::vector<int>& members) {
 int build_groups(mlsw_batch* b) {
   std::map<std::tuple<int, int, int>, std::vector<int>> members;
   std::vector<int> all;
-  b->nmax = 0;
   b->kinds = 0;
   b->tiny.clear();
   for (int j = 0; j < b->count; ++j) {
@@ -198,9 +280,17 @@ int build_groups(mlsw_batch* b) {
     const BatchInst& bi = b->hinst[j];
     members[std::make_tuple(-bi.P.n, mlsw::step_mode(bi.P), b->variant[j])].push_back(j);
     all.push_back(j);
-    b->nmax = std::max(b->nmax, bi.P.n);
     b->kinds |= 1u << bi.kind;
     if (bi.P.tiny) b->tiny.push_back(j);
+  }
+  // the strips of the kernel that these instances will run, and its row maps
+  for (int j : all) {
+    BatchInst& bi = b->hinst[j];
+    const bool solo = mlsw::batch_solo(b->kinds, bi.kind);
+    if (solo == b->solo[j]) continue;
+    b->solo[j] = solo;
+    bi.strips = mlsw::march_strips(bi.P.nx, solo);
+    if (!map_rows(b, j)) return MLSW_ERR_CUDA;
   }
   if (!all.empty()) choose_rows(b, all, b->kinds);
   b->same_params = same_params(b, all);
@@ -221,6 +311,8 @@ int build_groups(mlsw_batch* b) {
     b->groups.push_back(g);
   }
   b->nunits = (int)table.size();
+  if (!scaled_table(b, all, b->kinds) && b->nunits <= b->num_sms * mlsw::batch_warps_per_sm(b->kinds))
+    order_one_wave(table, b->num_sms);
   if (b->dtable) cudaFree(b->dtable);
   b->dtable = nullptr;
   if (cudaMalloc(&b->dtable, std::max<size_t>(1, table.size()) * sizeof(int2)) != cudaSuccess)
@@ -240,7 +332,6 @@ mlsw::BatchLaunch step_launch(const mlsw_batch* b) {
   a.inst = b->dinst;
   a.table = b->dtable;
   a.nunits = b->nunits;
-  a.nmax = b->nmax;
   a.kinds = b->kinds;
   a.same_params = b->same_params;
   a.P = b->params;
@@ -331,6 +422,7 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
   try {
     b->hinst.resize(count);
     b->variant.resize(count);
+    b->solo.assign(count, 0);
     b->selected.assign(count, 1);
     b->home.assign(count, 0);
   } catch (...) {
@@ -387,8 +479,7 @@ int mlswlbm_batch_create(int count, const mlsw_params* params, const float* cons
     const size_t flen = (size_t)bi.P.n * planes_of(bi.P) * bi.P.L.plane;
     bi.f[0] = b->arena + off[j];
     bi.f[1] = b->arena + off[j] + (flen + 63) / 64 * 64;
-    for (int k = 0; k < 2 && ok; ++k)
-      ok = mlsw_host::make_row_map(&bi.map[k], bi.f[k], bi.P.L, bi.P.n * planes_of(bi.P), false);
+    ok = map_rows(b, j);
   }
   ok = ok && cudaMemcpy(b->dinst, b->hinst.data(), (size_t)count * sizeof(BatchInst),
                         cudaMemcpyHostToDevice) == cudaSuccess;

@@ -78,8 +78,8 @@ cudaError_t launch_step_persistent(const StepLaunch& a, int nsteps, cudaStream_t
 // table of units, in which the units of instances that share n, kernel mode
 // and nominal tile height form a contiguous range (batch_kernels.cu).
 // ---------------------------------------------------------------------------
-// Nominal tile heights (batch.cu): variant 0 = 16 rows (n <= 3 only), the height
-// of the model, variant 1 = 8 rows, for n <= 3 half of it.
+// Nominal tile heights (batch_rows in unit_rows.h): variant 0 = 16 rows (n <= 3
+// only), the height of the model, variant 1 = 8 rows, for n <= 3 half of it.
 constexpr int kBatchVariants = 2;
 constexpr int batch_tile_rows(int variant) { return variant == 0 ? 16 : 8; }
 
@@ -89,7 +89,7 @@ struct BatchInst {
   KParams P;
   float* f[2];  // buffers, moments or populations
   int kind;     // batch_kind
-  int strips;   // strips of kMarchOut columns
+  int strips;   // strips of its columns
   int rows;     // rows of a unit
 };
 
@@ -111,7 +111,6 @@ struct BatchLaunch {
   const BatchInst* inst;
   const int2* table;
   int nunits;
-  int nmax;        // largest layer count in the table
   unsigned kinds;  // bit k: instances of kind k are in the table
   int same_params; // the instances' parameters are P's but for H and Hsum
   KParams P;
@@ -120,6 +119,17 @@ struct BatchLaunch {
 };
 // warps of a batch step resident on one SM
 int batch_warps_per_sm(unsigned kinds);
+// Whether the kernel for at most three layers takes a table of these kinds.
+constexpr bool batch_small(unsigned kinds) {
+  return kinds < 1u << batch_kind(4, 0) && !((kinds >> batch_kind(3, kGeneral)) & 1u);
+}
+// Whether instances of a kind march with one column a lane in a table of these
+// kinds. Its ring is the launch's: with pairs, five layers in the general mode
+// take 46 KB a warp and leave four warps an SM for every instance (32 lattices
+// of 2 to 5 layers, all modes: 282 us a step with pairs, 226 with single columns).
+constexpr bool batch_solo(unsigned kinds, int kind) {
+  return kinds != 1u << kind && kind % 3 == kGeneral && kind / 3 + 1 >= 4;
+}
 cudaError_t launch_batch_step(const BatchLaunch& a, cudaStream_t st);
 // all of one kind (step_d2q9.cu)
 cudaError_t launch_batch_alike(const BatchLaunch& a, int n, int mode, cudaStream_t st);

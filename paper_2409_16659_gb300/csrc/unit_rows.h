@@ -103,8 +103,36 @@ inline int solo_rows(bool general, int ny, int strips, int num_sms, int slots) {
   return best_rows > 0 ? best_rows : march_rows(4, true, ny, strips, num_sms, slots);
 }
 
-// Batches: the height of nominal 8-row units where that is a choice, half of the
-// model's.
+// Batches whose units are cut to equal duration. What a row takes a warp alone
+// (us), by layers and mode (StepMode; four and five layers of the general one with
+// one column a lane), from the slope of a step's time over unit heights of 1 to 16;
+// a substrate's cosines double it.
+inline double batch_weight(int n, int mode, bool substrate) {
+  constexpr double w[3][5] = {{0.75, 1.3, 2.1, 2.9, 3.9}, {0.6, 1.0, 1.45, 2.45, 3.5}, {0.5, 0.85, 1.3, 1.8, 2.2}};
+  return w[mode][n - 1] * (substrate ? 2.0 : 1.0);
+}
+
+// Rows of a unit that lasts about t (us): rows and about five of warm-up, at
+// most 64 rows.
+inline int batch_rows(double weight, double t) {
+  double r = t / weight - 5.0;
+  r = r < 1.0 ? 1.0 : (r > 64.0 ? 64.0 : r);
+  return (int)(r + 0.5);
+}
+
+// The height of nominal 8-row units where that is a choice: half.
 inline int half_rows(int rows) { return (rows + 1) / 2; }
+
+// What a step takes (us) in units of at most `longest` us, `work` us in all: in one
+// wave the longest unit, stretched by the warps beside it; in several the work at
+// the rate of full schedulers and the longest unit at the end. Coefficients that
+// choose best over 15 batches of 6 to 60 lattices (1 to 5 layers, all modes, sides
+// 16 to 320) stepped with 28 durations each: 3 % from the best duration on average
+// (time at the end of the last wave counted twice as dear, and warps beside one
+// another: 19 %).
+inline double batch_cost(double units, double work, double longest, int num_sms, int slots) {
+  if (units <= slots) return 1.4 * longest;
+  return 0.35 * work / (4.0 * num_sms) + 1.5 * longest;
+}
 
 }  // namespace mlsw
