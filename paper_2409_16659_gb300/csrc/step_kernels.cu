@@ -55,15 +55,17 @@ __device__ __forceinline__ void d1q3_pressures(const KParams& P, const float (&z
 }
 
 // Force, collision with forcing, for one cell: fs[i][k] receives the
-// post-collision populations; f_old is read only when !TAU1. Returns true
-// when a height is not positive or a force not finite.
+// post-collision populations; f_old is read only when !TAU1. hlow: the smallest
+// height so far; fall: 0, or NaN once a force was not finite (0 * inf and 0 * NaN
+// are NaN; a flux that is not finite makes the force so). Both are looked at once,
+// at the end.
 template <int N, bool TAU1>
-__device__ __forceinline__ bool d1q3_collide_cell(const KParams& P, const float (&g0)[N],
+__device__ __forceinline__ void d1q3_collide_cell(const KParams& P, const float (&g0)[N],
                                                   const float (&sm)[N],
                                                   const float (&hh)[N], const float (&jx)[N],
                                                   const float (&pw)[N], const float (&pc)[N],
                                                   const float (&pe)[N], const float (&f_old)[N][3],
-                                                  float (&fs)[N][3]) {
+                                                  float (&fs)[N][3], float& hlow, float& fall) {
   float ih[N], ux[N], Rx[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -71,16 +73,18 @@ __device__ __forceinline__ bool d1q3_collide_cell(const KParams& P, const float 
     ux[i] = mulr(jx[i], ih[i]);
   }
   friction<N, false>(P, hh, ih, ux, ux, Rx, Rx);
-  bool bad = false;
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     const float gqx = 0.5f * ((pe[i] - pc[i]) - (pw[i] - pc[i]));
     const float h = hh[i];
     const float Fx = fmav(h, gqx, Rx[i]);
-    bad |= !(h > 0.f) || !isfinite(Fx) || !isfinite(jx[i]);
+    hlow = fminf(hlow, h);
+    fall = fmaf(Fx, 0.f, fall);
     collide_d1q3<TAU1>(P, g0[i], sm[i], jx[i], ux[i], Fx, f_old[i], fs[i]);
   }
-  return bad;
+}
+__device__ __forceinline__ bool d1q3_bad(float hlow, float fall) {
+  return !(hlow > 0.f) || isnan(fall);
 }
 
 // ---------------------------------------------------------------------------
@@ -162,7 +166,8 @@ __global__ void __launch_bounds__(TX)
 #pragma unroll
     for (int k = 0; k < Q; ++k) fo[i][k] = TAU1 ? 0.f : fin[L.at(i * Q + k, gx, 0)];
   }
-  const bool bad = d1q3_collide_cell<N, TAU1>(P, g0, sm, hh, jx, pw, pc, pe, fo, fs);
+  float hlow = 1.f, fall = 0.f;
+  d1q3_collide_cell<N, TAU1>(P, g0, sm, hh, jx, pw, pc, pe, fo, fs, hlow, fall);
   int dxs[3], xis[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -180,7 +185,7 @@ __global__ void __launch_bounds__(TX)
       store_edge(fout + (long)(i * Q + k) * L.plane, L, dxs[cxi], 0, xis[cxi], kNoImage,
                  fs[i][k]);
     }
-  if (bad) atomicOr(status, kStatusNonfinite);
+  if (d1q3_bad(hlow, fall)) atomicOr(status, kStatusNonfinite);
 }
 
 // ---------------------------------------------------------------------------
@@ -219,12 +224,22 @@ __global__ void __launch_bounds__(d1_threads(N), 1)
   if (sub)
     for (int x = tid; x < nx; x += nt) *chk_smem(z0s + x) = substrate_at(P, x, 0);
   __syncthreads();
-  bool bad = false;
+  float hlow = 1.f, fall = 0.f;
+  const bool inner = lane >= 3 && lane < 3 + kD1Out;
+  // the warp's first cells, and this lane's one wrapped (kept for one and two
+  // layers, whose steps it shortens; three and five layers lose 5 and 10 % to the
+  // register)
+  const int first = (tid >> 5) * kD1Out;
+  int x_first = (first - 3 + lane) % nx;
+  if (x_first < 0) x_first += nx;
   for (int s = 0; s < nsteps; ++s) {
-    for (int c0 = (tid >> 5) * kD1Out; c0 < nx; c0 += (nt >> 5) * kD1Out) {
+    for (int c0 = first; c0 < nx; c0 += (nt >> 5) * kD1Out) {
       const int xo = c0 - 3 + lane;  // this lane's cell before wrapping
       int x = xo;
-      if (x < 0 || x >= nx) {
+      if constexpr (N <= 2) {
+        x = x_first + (c0 - first);  // below 2 nx
+        if (x >= nx) x -= nx;
+      } else if (x < 0 || x >= nx) {
         x %= nx;
         x += x < 0 ? nx : 0;
       }
@@ -260,9 +275,8 @@ __global__ void __launch_bounds__(d1_threads(N), 1)
         pw[i] = __shfl_up_sync(kAll, pc[i], 1);
         pe[i] = __shfl_down_sync(kAll, pc[i], 1);
       }
-      const bool cell_bad = d1q3_collide_cell<N, TAU1>(P, g0, sm_, hh, jx, pw, pc, pe, fo, fs);
-      const bool own = lane >= 3 && lane < 3 + kD1Out && xo < nx;
-      bad |= own && cell_bad;
+      d1q3_collide_cell<N, TAU1>(P, g0, sm_, hh, jx, pw, pc, pe, fo, fs, hlow, fall);
+      const bool own = inner && xo < nx;
 #pragma unroll
       for (int i = 0; i < N; ++i) {
         const float right = __shfl_up_sync(kAll, fs[i][1], 1);   // c = +1, from x - 1
@@ -286,7 +300,8 @@ __global__ void __launch_bounds__(d1_threads(N), 1)
     sx += sx < 0 ? nx : 0;
     fout[L.at(pl, x, 0)] = *chk_smem(fa + pl * nx + sx);
   }
-  if (bad) atomicOr(status, kStatusNonfinite);
+  // (the outer lanes' neighbours are not the lattice's; beyond nx it repeats)
+  if (inner && d1q3_bad(hlow, fall)) atomicOr(status, kStatusNonfinite);
 }
 
 // ---------------------------------------------------------------------------
