@@ -106,8 +106,7 @@ bool scaled_table(const mlsw_batch* b, const std::vector<int>& members, unsigned
 // plus about five rows of warm-up; a warp alone on a scheduler needs 1.75 times
 // that time for a row's latencies.
 // Instances of one layer count finish together, in whole waves, and as the
-// schedulers' fullest (5 % more units than an even split: the SMs are not
-// filled exactly evenly); uneven ones (work in proportion to n) overlap, and the
+// schedulers' fullest; uneven ones (work in proportion to n) overlap, and the
 // longest unit may come last. Beside four or five layers the variants shift the
 // proportion of the heights, and the scale follows; without them the scale is that
 // of the nominal 16, so that 8 are half of it (a scale for them would give the same
@@ -135,7 +134,7 @@ int scale_for(const mlsw_batch* b, const std::vector<int>& members, unsigned kin
     double cost;
     if (nmin == nmax) {
       const double full = per_sm / 4.0;
-      const double q = units <= slots ? std::min(std::ceil(1.05 * units / schedulers), full)
+      const double q = units <= slots ? std::min(std::ceil(units / schedulers), full)
                                       : std::ceil(units / slots) * full;
       cost = longest * std::max(1.75, q);
     } else {
