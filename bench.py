@@ -405,6 +405,8 @@ def run_own(args):
             "config": config_dict(),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
+                         "traffic_note": "DRAM bytes per launch of the same lattices in turn "
+                                         "(ncu, caches not flushed)" if traffic else None,
                          "kernel": "step_d2q9<3,kFast>",
                          "bytes_per_launch_algorithmic": bytes_alg, "peak_source": peak_src},
             "e2e": {"value": job_rate(ws, lsu_step * k_e2e, e2e_s), "unit": UNIT,
@@ -736,18 +738,23 @@ def run_profile_batch(args):
 
 
 def run_profile(args):
-    """Warm-up then --steps back-to-back steps; no flush, e2e or CPU leg."""
+    """Warm-up then --steps steps of the timed region's lattices in turn; no e2e
+    or CPU leg."""
     import torch
     torch.cuda.set_device(0)
     from paper_2409_16659_gb300 import mlswlbm as B
     p = workloads.film3_d2q9_params(NX, NY)
     h0 = workloads.film3_d2q9_heights(NX, NY).astype(np.float32)
-    with B.Solver(p, h0, stream=torch.cuda.current_stream()) as s:
-        s.step(args.warmup)
-        s.step(args.steps)
-        torch.cuda.synchronize()
-        print(json.dumps({"profile_run": True, "launches": s.launch_count(),
-                          "status": B.mlswlbm_strerror(s.status())}), flush=True)
+    st = torch.cuda.current_stream()
+    solvers = [B.Solver(p, h0, stream=st) for _ in range(LATTICES)]
+    for i in range(args.warmup + args.steps):
+        solvers[i % LATTICES].step(1)
+    torch.cuda.synchronize()
+    print(json.dumps({"profile_run": True, "lattices": LATTICES,
+                      "steps_of_each": [s.launch_count() - 1 for s in solvers],
+                      "status": [B.mlswlbm_strerror(s.status()) for s in solvers]}), flush=True)
+    for s in solvers:
+        s.close()
     return 0
 
 
