@@ -140,7 +140,8 @@ __device__ __forceinline__ void lattice_derivatives(f1 c, f1 A, f1 B, f1& gx, f1
 // and has at most one image, as a whole: one predicated 8-byte store each,
 // at 32-bit lane offsets from a warp-uniform address. Other lattices store
 // the strips at their edges column by column. (A strip per lattice edge is
-// most of a small lattice: 16 films of 256^2 step in 38 us instead of 44.)
+// most of a small lattice: 16 films of 256^2, in the kernel of all kinds, step in
+// 38 us instead of 44.)
 struct PairStore {
   bool own;       // the pair's first column belongs to the lattice (pairs: both)
   bool image;     // pairs: this lane's pair has an image

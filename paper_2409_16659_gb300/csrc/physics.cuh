@@ -226,8 +226,8 @@ __device__ __forceinline__ f1 mulr(f1 a, float b) { return a * b; }
 
 // fast reciprocal: the hardware's approximation, at most 1 ulp for normal
 // arguments (here layer thicknesses and friction pivots, far from the ends
-// of the FP32 range). Division intrinsics add five instructions of range
-// scaling to it, which no argument here needs.
+// of the FP32 range). Division intrinsics also scale the range of their
+// arguments, which none here needs.
 __device__ __forceinline__ float rcp(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

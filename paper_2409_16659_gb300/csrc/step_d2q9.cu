@@ -26,7 +26,8 @@ __global__ void __launch_bounds__(32, lane_warps<T>(N, MODE))
 // registers and instructions of one kind only. SAME: they also share every
 // parameter but H and Hsum (the films of a trajectory set), which are then the
 // kernel's, in the constant bank; two rows a turn pay again. 16 films of 256^2:
-// 38.9 us a step in the kernel of all kinds, 35.1 here.
+// 38.9 us a step in the kernel of all kinds, 35.1 here (33.6 with the present
+// friction).
 template <int N, int MODE, bool SAME>
 __global__ void __launch_bounds__(32, march_warps(N, MODE))
     step_d2q9_alike(const BatchInst* __restrict__ inst, const int2* __restrict__ table,

@@ -1003,8 +1003,7 @@ bool map_nhwc(CUtensorMap* m, void* base, int C, int W, int H, int B, int bc, in
          CUDA_SUCCESS;
 }
 
-// 2-D map of a weight matrix [rows][K] (K contiguous), box [kc, bn]
-// weights [rows][tap][K] (tap = 3 (dy + 1) + (dx + 1)) as a 4-D tensor
+// Weights [rows][tap][K] (tap = 3 (dy + 1) + (dx + 1)) as a 4-D tensor
 // [K, rows, 3 dy, 3 dx]; a box [kc, bn, 3, 1] holds one tap column's three
 // taps, each a K-major bn x kc block
 bool map_weights(CUtensorMap* m, void* base, int K, int rows, int kc, int bn) {
