@@ -149,6 +149,9 @@ KParams make_kparams(const mlsw_params& p) {
     for (int kk = 2; kk <= p.n_layers - i; ++kk)
       if (k.S[i][kk - 1] != 0.f) k.far_pairs = 1;
   }
+  for (int i = 0; i < p.n_layers; ++i)
+    for (int kk = 1; kk <= (k.far_pairs ? p.n_layers - i : 1); ++kk)
+      if (k.S[i][kk - 1] == 0.f) k.zero_pairs = 1;
   k.hstar = (float)p.hstar;
   k.nw = p.wet_n;
   k.mw = p.wet_m;

@@ -107,6 +107,9 @@ struct KParams {
   // phi_k(d) = 2 a - a^2, a = e^{-kappa (d - k h*)}
   int wet_kind;
   float kappa;
+  // 1: zero coefficients among the pairs that have a part in the pressures
+  // (all of them with far_pairs, else k = 1)
+  int zero_pairs;
 };
 
 // Substrate height at phase 2 pi m / nc, 0 <= m < nc
@@ -295,7 +298,8 @@ __device__ __forceinline__ T ipow(T r, int e) {
 // without far pairs, either potential), chosen once, so that the latencies
 // of the pairs overlap. With SKIP a pair without a coefficient contributes
 // exactly nothing, whatever its potential evaluates to (r^3 of a thin layer
-// overflows, and 0 * inf is NaN; the selects cost no time that shows).
+// overflows, and 0 * inf is NaN). SKIP false: the host knows that every pair
+// evaluated has one (zero_pairs).
 enum PairForm { kPower32, kPower, kExponential };
 
 template <int N, bool FAR, int FORM, bool SKIP, class T>
@@ -354,7 +358,7 @@ __device__ __forceinline__ void interface_pairs(const KParams& P, const KParams&
   }
 }
 
-template <int N, bool W32, class T, bool NN = false>
+template <int N, bool W32, class T, bool NN = false, bool SKIP = true>
 __device__ __forceinline__ void neg_pressures(const KParams& P, const KParams& G,
                                               const T (&zd)[N], const T (&gx)[N],
                                               const T (&gy)[N], const T (&lz)[N], T (&q)[N],
@@ -370,9 +374,9 @@ __device__ __forceinline__ void neg_pressures(const KParams& P, const KParams& G
     interface_pairs<N, false, kPower32, false>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if constexpr (W32) {
     if (P.far_pairs)
-      interface_pairs<N, true, kPower32, true>(P, G, zd, sg, z0, sg0, ten, pi);
+      interface_pairs<N, true, kPower32, SKIP>(P, G, zd, sg, z0, sg0, ten, pi);
     else
-      interface_pairs<N, false, kPower32, true>(P, G, zd, sg, z0, sg0, ten, pi);
+      interface_pairs<N, false, kPower32, SKIP>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if (P.wet_kind == 1) {
     interface_pairs<N, true, kExponential, true>(P, G, zd, sg, z0, sg0, ten, pi);
   } else if (P.far_pairs) {

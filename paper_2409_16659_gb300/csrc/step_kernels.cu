@@ -30,12 +30,19 @@ namespace mlsw {
 // both give the same bits.
 // ---------------------------------------------------------------------------
 // q_i = p_atm - p_i of one cell from z deviations at x - 1, x, x + 1
-// z0w, z0c, z0e: the substrate at x - 1, x, x + 1 (all 0 when flat)
-template <int N, bool W32>
+// z0w, z0c, z0e: the substrate at x - 1, x, x + 1 (all 0 when flat).
+// FORM: kFull32 exponents (3, 2) and a coefficient on every pair that has a
+// part, kAny32 exponents (3, 2), kAny any potential; chosen by the host. The
+// selects of the second form cost 2 to 4 % from two layers on (us a step, 512
+// cells, two layers 0.635 and 0.662; 420 cells, four 1.525 and 1.585); one layer
+// takes the second form always (500 cells, 0.407, without its selects 0.495).
+enum D1Form { kFull32, kAny32, kAny };
+template <int N, int FORM>
 __device__ __forceinline__ void d1q3_pressures(const KParams& P, const float (&zw)[N],
                                                const float (&zc)[N], const float (&ze)[N],
                                                float (&p)[N], float z0w = 0.f, float z0c = 0.f,
                                                float z0e = 0.f) {
+  constexpr bool W32 = FORM != kAny, SKIP = FORM != kFull32;
   float zd[N], gxz[N], gyz[N], lz[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -48,9 +55,9 @@ __device__ __forceinline__ void d1q3_pressures(const KParams& P, const float (&z
   if (P.sub_amp != 0.f) {
     const float g0 = 0.5f * (z0e - z0w);
     const float sg0 = fmaf(0.5f, g0 * g0, 1.f);
-    neg_pressures<N, W32>(P, P, zd, gxz, gyz, lz, p, &z0c, &sg0);
+    neg_pressures<N, W32, float, false, SKIP>(P, P, zd, gxz, gyz, lz, p, &z0c, &sg0);
   } else {
-    neg_pressures<N, W32>(P, P, zd, gxz, gyz, lz, p);
+    neg_pressures<N, W32, float, false, SKIP>(P, P, zd, gxz, gyz, lz, p);
   }
 }
 
@@ -91,7 +98,7 @@ __device__ __forceinline__ bool d1q3_bad(float hlow, float fall) {
 // D1Q3: tile of TX cells, one cell per thread, plain loads (the padded
 // layout supplies the periodic images in x).
 // ---------------------------------------------------------------------------
-template <int N, int TX, bool TAU1, bool W32>
+template <int N, int TX, bool TAU1, int FORM>
 __global__ void __launch_bounds__(TX)
     step_d1q3_kernel(const float* __restrict__ fin, float* __restrict__ fout, const KParams P,
                      int* __restrict__ status) {
@@ -146,10 +153,10 @@ __global__ void __launch_bounds__(TX)
     }
     if (sub) {
       const int x = x0 - 1 + pc;
-      d1q3_pressures<N, W32>(P, zw, zc, ze, p, substrate_at(P, x - 1, 0), substrate_at(P, x, 0),
+      d1q3_pressures<N, FORM>(P, zw, zc, ze, p, substrate_at(P, x - 1, 0), substrate_at(P, x, 0),
                              substrate_at(P, x + 1, 0));
     } else {
-      d1q3_pressures<N, W32>(P, zw, zc, ze, p);
+      d1q3_pressures<N, FORM>(P, zw, zc, ze, p);
     }
 #pragma unroll
     for (int i = 0; i < N; ++i) ps[i][chk_index(pc, PW)] = p[i];
@@ -204,7 +211,7 @@ constexpr int kD1Out = 26;  // cells a warp writes
 // threads: 20 warps cover 520 cells at once; more layers need the registers
 constexpr int d1_threads(int n) { return n <= 3 ? 640 : 512; }
 
-template <int N, bool TAU1, bool W32>
+template <int N, bool TAU1, int FORM>
 __global__ void __launch_bounds__(d1_threads(N), 1)
     step_d1q3_persistent(const float* fin, float* fout, const KParams P, int nsteps,
                          int* __restrict__ status) {
@@ -266,9 +273,9 @@ __global__ void __launch_bounds__(d1_threads(N), 1)
       }
       if (sub) {
         const float z0w = __shfl_up_sync(kAll, z0, 1), z0e = __shfl_down_sync(kAll, z0, 1);
-        d1q3_pressures<N, W32>(P, zw, zc, ze, pc, z0w, z0, z0e);
+        d1q3_pressures<N, FORM>(P, zw, zc, ze, pc, z0w, z0, z0e);
       } else {
-        d1q3_pressures<N, W32>(P, zw, zc, ze, pc);
+        d1q3_pressures<N, FORM>(P, zw, zc, ze, pc);
       }
 #pragma unroll
       for (int i = 0; i < N; ++i) {
@@ -323,22 +330,26 @@ bool step_dear(const KParams& P) {
 
 bool step_moments(const KParams& P) { return step_mode(P) != kGeneral; }
 
+static D1Form d1_form(const KParams& P) {
+  if (P.wet_kind != 0 || P.nw != 3 || P.mw != 2) return kAny;
+  return P.zero_pairs || P.n == 1 ? kAny32 : kFull32;
+}
+
+// (tau != 1 runs the general form only)
 template <int N>
 static cudaError_t launch_n(const StepLaunch& a, cudaStream_t st) {
-  const bool tau1 = (a.P.omega == 1.f);
-  const bool w32 = (a.P.wet_kind == 0 && a.P.nw == 3 && a.P.mw == 2);
   if (a.lattice == 2) {
     return launch_step_d2q9<N>(a, st);
   }
-  dim3 grid((a.P.nx + kD1TX - 1) / kD1TX);
-  if (tau1) {
-    if (w32)
-      step_d1q3_kernel<N, kD1TX, true, true><<<grid, kD1TX, 0, st>>>(a.fin, a.fout, a.P, a.status);
-    else
-      step_d1q3_kernel<N, kD1TX, true, false><<<grid, kD1TX, 0, st>>>(a.fin, a.fout, a.P, a.status);
-  } else {
-    step_d1q3_kernel<N, kD1TX, false, false><<<grid, kD1TX, 0, st>>>(a.fin, a.fout, a.P, a.status);
+  auto kern = step_d1q3_kernel<N, kD1TX, false, kAny>;
+  if (a.P.omega == 1.f) {
+    switch (d1_form(a.P)) {
+      case kFull32: kern = step_d1q3_kernel<N, kD1TX, true, kFull32>; break;
+      case kAny32: kern = step_d1q3_kernel<N, kD1TX, true, kAny32>; break;
+      default: kern = step_d1q3_kernel<N, kD1TX, true, kAny>; break;
+    }
   }
+  kern<<<(a.P.nx + kD1TX - 1) / kD1TX, kD1TX, 0, st>>>(a.fin, a.fout, a.P, a.status);
   return cudaGetLastError();
 }
 
@@ -347,9 +358,9 @@ size_t step_persistent_smem(int n, int lattice, int nx) {
   return (size_t)8 * n * nx * sizeof(float);
 }
 
-template <int N, bool TAU1, bool W32>
+template <int N, bool TAU1, int FORM>
 static cudaError_t launch_d1p(const StepLaunch& a, int nsteps, cudaStream_t st) {
-  auto kern = step_d1q3_persistent<N, TAU1, W32>;
+  auto kern = step_d1q3_persistent<N, TAU1, FORM>;
   const size_t smem = step_persistent_smem(N, 1, a.P.nx);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -361,10 +372,12 @@ static cudaError_t launch_d1p(const StepLaunch& a, int nsteps, cudaStream_t st) 
 
 template <int N>
 static cudaError_t launch_d1p_n(const StepLaunch& a, int nsteps, cudaStream_t st) {
-  const bool tau1 = (a.P.omega == 1.f);
-  const bool w32 = (a.P.wet_kind == 0 && a.P.nw == 3 && a.P.mw == 2);
-  if (tau1) return w32 ? launch_d1p<N, true, true>(a, nsteps, st) : launch_d1p<N, true, false>(a, nsteps, st);
-  return launch_d1p<N, false, false>(a, nsteps, st);
+  if (a.P.omega != 1.f) return launch_d1p<N, false, kAny>(a, nsteps, st);
+  switch (d1_form(a.P)) {
+    case kFull32: return launch_d1p<N, true, kFull32>(a, nsteps, st);
+    case kAny32: return launch_d1p<N, true, kAny32>(a, nsteps, st);
+    default: return launch_d1p<N, true, kAny>(a, nsteps, st);
+  }
 }
 
 cudaError_t launch_batch_alike(const BatchLaunch& a, int n, int mode, cudaStream_t st) {
