@@ -150,8 +150,9 @@ int scale_for(const mlsw_batch* b, const std::vector<int>& members, unsigned kin
 
 // Duration t (us) of the units of other tables: the same for all kinds, so that
 // none is left running alone (32 lattices of 2 to 5 layers, all modes: 294 us a
-// step with one scaled height, 226).
-double unit_time(const mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
+// step with one scaled height, 226). *one_wave: they fit the chip at once.
+double unit_time(const mlsw_batch* b, const std::vector<int>& members, unsigned kinds,
+                 bool* one_wave) {
   const int slots = b->num_sms * mlsw::batch_warps_per_sm(kinds);
   double best_t = 0.0, best = 0.0;
   for (int c = 0; c < 128; ++c) {
@@ -169,16 +170,27 @@ double unit_time(const mlsw_batch* b, const std::vector<int>& members, unsigned 
     if (c == 0 || cost < best) {
       best = cost;
       best_t = t;
+      *one_wave = units <= slots;
     }
   }
   return best_t;
 }
 
-// rows of the members' units: all of the model's for the nominal 16, half for 8
-void choose_rows(mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
-  const bool scaled = scaled_table(b, members, kinds);
+bool any_general(unsigned kinds) {
+  for (int k = mlsw::kGeneral; k < mlsw::kBatchKinds; k += 3)
+    if ((kinds >> k) & 1u) return true;
+  return false;
+}
+
+// Rows of the members' units: all of the model's for the nominal 16, half for 8.
+// Returns whether the table is one wave of units of equal duration. Tables at
+// tau = 1 in several waves keep one height (71 lattices of the fast mode and on a
+// substrate: 274 us a step, 299 with equal durations).
+bool choose_rows(mlsw_batch* b, const std::vector<int>& members, unsigned kinds) {
+  bool scaled = scaled_table(b, members, kinds), one_wave = false;
+  const double t = scaled ? 0.0 : unit_time(b, members, kinds, &one_wave);
+  scaled = scaled || (!one_wave && !any_general(kinds));
   const int r = scaled ? scale_for(b, members, kinds) : 1;
-  const double t = scaled ? 0.0 : unit_time(b, members, kinds);
   for (int j : members) {
     BatchInst& bi = b->hinst[j];
     const bool half = b->variant[j] == 1;
@@ -189,6 +201,7 @@ void choose_rows(mlsw_batch* b, const std::vector<int>& members, unsigned kinds)
       bi.rows = bi.P.n <= 3 && half ? mlsw::half_rows(rows) : rows;
     }
   }
+  return !scaled && one_wave;
 }
 
 // The order of a table of units of equal duration that is sorted by kind and
@@ -291,7 +304,7 @@ int build_groups(mlsw_batch* b) {
     bi.strips = mlsw::march_strips(bi.P.nx, solo);
     if (!map_rows(b, j)) return MLSW_ERR_CUDA;
   }
-  if (!all.empty()) choose_rows(b, all, b->kinds);
+  const bool one_wave = !all.empty() && choose_rows(b, all, b->kinds);
   b->same_params = same_params(b, all);
   if (!all.empty()) b->params = b->hinst[all[0]].P;
   std::vector<int2> table;
@@ -310,7 +323,7 @@ int build_groups(mlsw_batch* b) {
     b->groups.push_back(g);
   }
   b->nunits = (int)table.size();
-  if (!scaled_table(b, all, b->kinds) && b->nunits <= b->num_sms * mlsw::batch_warps_per_sm(b->kinds))
+  if (one_wave && b->nunits <= b->num_sms * mlsw::batch_warps_per_sm(b->kinds))
     order_one_wave(table, b->num_sms);
   if (b->dtable) cudaFree(b->dtable);
   b->dtable = nullptr;

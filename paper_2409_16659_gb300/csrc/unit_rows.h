@@ -60,14 +60,14 @@ inline int march_rows(int n, bool heavy, int ny, int strips, int num_sms, int sl
 // with half the registers and ring, so more warps; per column it is more
 // instructions. It pays, from four layers on, where
 //   * both forms have one strip: 25 x 1870, us a step with pairs and with single
-//     columns, four layers 12.6 and 9.9 (fast mode), 15.6 and 12.5 (tau = 1
-//     otherwise), 18.1 and 11.5 (tau = 0.8), five 15.3 and 11.3, 20.9 and 16.0, 26.8
-//     and 15.1; 26 x 30000, five layers, tau = 0.8, 270 and 153;
+//     columns, four layers 12.6 and 9.9 (tau = 1, near pairs), 15.6 and 12.5 (far
+//     pairs), 18.1 and 11.5 (tau = 0.8), five 15.3 and 11.3, 20.9 and 16.0, 26.8 and
+//     15.1; 26 x 30000, five layers, tau = 0.8, 270 and 153;
 //   * pairs leave a third of their strips empty (57 to 78 columns) and give a
-//     scheduler two rows or more: 57 x 800, four layers, 14.4 and 12.4 (tau = 1
-//     otherwise); above four rows a scheduler only in the general mode, whose
+//     scheduler two rows or more: 57 x 800, four layers, 14.4 and 12.4 (far
+//     pairs); above four rows a scheduler only in the general mode, whose
 //     pairs hold four to six warps an SM (57 x 10000, five layers 171 and 118,
-//     but four layers of the fast mode, 78 x 2500, 18.2 and 19.7);
+//     but four layers with near pairs, 78 x 2500, 18.2 and 19.7);
 //   * pairs have two to three rows a scheduler and every cell many terms (dear:
 //     tau != 1, far pairs, a substrate or the exponential potential): 256^2, five
 //     layers, 20.2 and 18.2 (far pairs), 20.4 and 18.7 (tau = 0.8); without them,
@@ -103,10 +103,13 @@ inline int solo_rows(bool general, int ny, int strips, int num_sms, int slots) {
   return best_rows > 0 ? best_rows : march_rows(4, true, ny, strips, num_sms, slots);
 }
 
-// Batches whose units are cut to equal duration. What a row takes a warp alone
-// (us), by layers and mode (StepMode; four and five layers of the general one with
-// one column a lane), from the slope of a step's time over unit heights of 1 to 16;
-// a substrate's cosines double it.
+// Batches whose units are cut to equal duration. What a row counts (us), by layers
+// and mode (StepMode; four and five layers of the general one with one column a
+// lane): about what it takes a warp alone where that is slow, and more where it is
+// quick, because warps that share an SM with slow kinds wait with them. (Alone,
+// from the slope between 4 and 16 rows a unit: general 0.9 to 4.4, tau = 1 with far
+// pairs 0.7 to 3.4, fast 0.47, 0.62, 0.84, 1.08, 1.3, a substrate 1.0 more. With these
+// 60 random batches step in 0.995 of the time on average, but five in up to 1.6.)
 inline double batch_weight(int n, int mode, bool substrate) {
   constexpr double w[3][5] = {{0.75, 1.3, 2.1, 2.9, 3.9}, {0.6, 1.0, 1.45, 2.45, 3.5}, {0.5, 0.85, 1.3, 1.8, 2.2}};
   return w[mode][n - 1] * (substrate ? 2.0 : 1.0);
